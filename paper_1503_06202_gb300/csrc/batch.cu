@@ -137,8 +137,7 @@ void free_batch(xeng_batch_s *b)
     small_scratch_free(&b->small);
     cudaFree(b->d_pjobs);
     cudaFree(b->d_pmaps);
-    cudaFree(b->d_err);
-    if (b->h_err) cudaFreeHost(b->h_err);
+    status_free(b->d_err, b->h_err);
     cudaGetLastError();
     delete b;
 }
@@ -159,7 +158,6 @@ cudaError_t enqueue_run(xeng_batch_s *b, cudaStream_t s)
             }
         }
     };
-    e = cudaMemsetAsync(b->d_err, 0, sizeof(int), s);
     // Two branches: the N <= 256 kernel's jobs (cooperative launches sharing one
     // scratch, so one after another) on a side stream, the rest here; a small
     // job's few CTAs then run beside a large job's tail.
@@ -196,7 +194,6 @@ cudaError_t enqueue_run(xeng_batch_s *b, cudaStream_t s)
     } else {
         run_single(true, s);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     return e;
 }
 
@@ -529,8 +526,7 @@ int xeng_batch_create(const xeng_job_t *jobs, int32_t n_jobs, const xeng_batch_o
     b->num_sms = sms;
     int st = plan(b);
     cudaError_t e = cudaSuccess;
-    if (st == XENG_OK) e = cudaMalloc(&b->d_err, sizeof(int));
-    if (st == XENG_OK && e == cudaSuccess) e = cudaMallocHost(&b->h_err, sizeof(int));
+    if (st == XENG_OK) e = status_alloc(&b->d_err, &b->h_err);
     if (st == XENG_OK && e == cudaSuccess) e = prepare_correlate_tc_listed();
     if (st == XENG_OK && e == cudaSuccess) e = prepare_decode_tma_batch();
     if (st == XENG_OK && e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
@@ -559,7 +555,6 @@ int xeng_batch_create(const xeng_job_t *jobs, int32_t n_jobs, const xeng_batch_o
         free_batch(b);
         return st;
     }
-    *b->h_err = 0;
     *out = b;
     return XENG_OK;
 }

@@ -637,7 +637,7 @@ struct xbeam_s {
     int32_t *corr = nullptr;    // [F][Bp][2] offset terms of the beams
     int8_t *wstage = nullptr;   // device copy of host weights
     int *d_err = nullptr;       // device status word of the kernels
-    int *h_err = nullptr;       // pinned mirror, refreshed after each run
+    int *h_err = nullptr;       // its mirror in pinned host memory, written by the kernel that sets it
     int sticky = XENG_OK;
 };
 
@@ -663,7 +663,7 @@ int bf_status(cudaError_t e)
 int bf_check_sticky(xbeam_s *b)
 {
     if (b->sticky != XENG_OK) return b->sticky;
-    if (*b->h_err != 0) b->sticky = XENG_ERR_TIMEOUT;
+    if (*(volatile int *)b->h_err != 0) b->sticky = XENG_ERR_TIMEOUT;
     return b->sticky;
 }
 
@@ -698,15 +698,12 @@ int xbeam_create(int32_t n_inputs, int32_t n_freq, int32_t n_beams, xbeam_t *out
     const size_t corr_bytes = (size_t)n_freq * xeng::beam_padded(n_beams) * 2 * sizeof(int32_t);
     if (e == cudaSuccess) e = cudaMalloc(&b->corr, corr_bytes);
     if (e == cudaSuccess) e = cudaMemset(b->corr, 0, corr_bytes);  // and so are their offset terms
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMallocHost(&b->h_err, sizeof(int));
+    if (e == cudaSuccess) e = xeng::status_alloc(&b->d_err, &b->h_err);
     if (e != cudaSuccess) {
         cudaGetLastError();
         xbeam_destroy(b);
         return bf_status(e);
     }
-    *b->h_err = 0;
     *out = b;
     return XENG_OK;
 }
@@ -760,7 +757,6 @@ int xbeam_run(xbeam_t b, const uint8_t *block, int64_t n_samples, int32_t *out, 
     a.out = out;
     a.err = b->d_err;
     cudaError_t e = xeng::launch_beamform(block, b->wdev, b->corr, a, b->num_sms, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(b->h_err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return (b->sticky = bf_status(e));
     return XENG_OK;
 }
@@ -772,8 +768,7 @@ void xbeam_destroy(xbeam_t b)
     cudaFree(b->wdev);
     cudaFree(b->corr);
     cudaFree(b->wstage);
-    cudaFree(b->d_err);
-    if (b->h_err) cudaFreeHost(b->h_err);
+    xeng::status_free(b->d_err, b->h_err);
     cudaGetLastError();
     delete b;
 }

@@ -739,19 +739,20 @@ cudaError_t encode_planes_map(CUtensorMap *map, const uint8_t *planes, int64_t t
 
 cudaError_t selftest_wait_timeout(int64_t limit_ns, int *status, int *left)
 {
-    int *d = nullptr;
-    cudaError_t e = cudaMalloc(&d, 2 * sizeof(int));
-    if (e != cudaSuccess) return e;
-    e = cudaMemset(d, 0, 2 * sizeof(int));
+    int *d_left = nullptr, *d_err = nullptr, *h_err = nullptr, word = 0;
+    cudaError_t e = cudaMalloc(&d_left, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(d_left, 0, sizeof(int));
+    if (e == cudaSuccess) e = status_alloc(&d_err, &h_err);
     if (e == cudaSuccess) {
-        wait_selftest_kernel<<<1, 64>>>(d, (uint64_t)limit_ns, d + 1);
+        wait_selftest_kernel<<<1, 64>>>(d_err, (uint64_t)limit_ns, d_left);
         e = cudaGetLastError();
     }
-    int h[2] = {0, 0};
-    if (e == cudaSuccess) e = cudaMemcpy(h, d, sizeof(h), cudaMemcpyDeviceToHost);
-    cudaFree(d);
-    *status = h[0];
-    *left = h[1];
+    if (e == cudaSuccess) e = cudaMemcpy(left, d_left, sizeof(int), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(&word, d_err, sizeof(int), cudaMemcpyDeviceToHost);
+    // what a handle would see: the mirror, which has to hold the device's word
+    if (e == cudaSuccess) *status = *(volatile int *)h_err == word ? word : -1;
+    cudaFree(d_left);
+    if (d_err) status_free(d_err, h_err);
     return e;
 }
 

@@ -114,7 +114,7 @@ extern "C" int xeng_correlate_noalloc(const uint8_t *block, int64_t n_samples, i
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         return e == cudaSuccess ? XENG_OK : XENG_ERR_CUDA;
     }
-    e = cudaMemsetAsync(status, 0, sizeof(int), s);
+    e = cudaMemsetAsync(status, 0, sizeof(StatusBlock), s);  // no mirror: the word is read back below
     int64_t group = kPlaneBytes / (2 * n_pad * t_pad);
     if (group > F) group = F;
     if (group > 65535) group = 65535;

@@ -553,7 +553,6 @@ bool launch_round(xserve_s *sv)
         e = cudaMemcpyAsync(st.dump[p.dump_slot].buf, st.acc, (size_t)st.F * n_baselines(st.N) * 8,
                             cudaMemcpyDeviceToDevice, s);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sv->h_err, sv->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (!sv->free_events.empty()) {
         r.ev = sv->free_events.back();
         sv->free_events.pop_back();
@@ -665,15 +664,12 @@ int xserve_create(const xserve_opts_t *opts, xserve_t *out)
             e = cudaMallocHost(&sv->h_smaps[k], (size_t)o.max_streams * o.max_blocks * sizeof(CUtensorMap));
     }
     sv->single_force = single_pass_force_from_env();
-    if (e == cudaSuccess) e = cudaMalloc(&sv->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(sv->d_err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMallocHost(&sv->h_err, sizeof(int));
+    if (e == cudaSuccess) e = status_alloc(&sv->d_err, &sv->h_err);
     if (e != cudaSuccess) {
         cudaGetLastError();
         xserve_destroy(sv);
         return e == cudaErrorMemoryAllocation ? XENG_ERR_NOMEM : XENG_ERR_CUDA;
     }
-    *sv->h_err = 0;
     sv->worker = std::thread(worker_main, sv);
     *out = sv;
     return XENG_OK;
@@ -969,8 +965,7 @@ void xserve_destroy(xserve_t sv)
         cudaFreeHost(sv->h_smaps[k]);
     }
     small_scratch_free(&sv->small);
-    cudaFree(sv->d_err);
-    if (sv->h_err) cudaFreeHost(sv->h_err);
+    status_free(sv->d_err, sv->h_err);
     for (auto e : sv->free_events) cudaEventDestroy(e);
     for (auto e : sv->free_timers) cudaEventDestroy(e);
     if (sv->s) cudaStreamDestroy(sv->s);

@@ -51,6 +51,33 @@ bool use_pair_kernel(int32_t N)
 
 }  // namespace
 
+cudaError_t status_alloc(int **d_err, int **h_err)
+{
+    *d_err = *h_err = nullptr;
+    StatusBlock sb = {0, 0, nullptr};
+    cudaError_t e = cudaMallocHost(h_err, sizeof(int));
+    if (e == cudaSuccess) {
+        **h_err = 0;
+        void *m = nullptr;
+        e = cudaHostGetDevicePointer(&m, *h_err, 0);
+        sb.mirror = static_cast<int *>(m);
+    }
+    if (e == cudaSuccess) e = cudaMalloc(d_err, sizeof sb);
+    if (e == cudaSuccess) e = cudaMemcpy(*d_err, &sb, sizeof sb, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        status_free(*d_err, *h_err);
+        *d_err = *h_err = nullptr;
+    }
+    return e;
+}
+
+void status_free(int *d_err, int *h_err)
+{
+    cudaFree(d_err);
+    if (h_err) cudaFreeHost(h_err);
+}
+
 int single_pass_force_from_env()
 {
     const char *env = getenv("XENG_FUSED_KERNEL");

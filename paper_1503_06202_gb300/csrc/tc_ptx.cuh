@@ -7,6 +7,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "xeng_internal.h"
+
 namespace xeng {
 namespace {
 
@@ -42,6 +44,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// Record `code` in the status block `err` points at (StatusBlock: the status
+// word the waits poll, and the address of its mirror in pinned host memory) if
+// nothing is recorded yet.  The thread that records writes the mirror too, so
+// the host sees a time-out without a copy of the word after every launch.
+__device__ __noinline__ void set_status(int *err, int code)
+{
+    if (atomicCAS(err, 0, code) != 0) return;
+    int *mirror = reinterpret_cast<StatusBlock *>(err)->mirror;
+    if (mirror) {
+        *(volatile int *)mirror = code;
+        __threadfence_system();
+    }
+}
+
 // Bounded wait for the phase with the given parity to complete.  Returns
 // false if the error word is set by someone else or if the limit passes
 // (then this thread sets it to `code`).
@@ -55,7 +71,7 @@ __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *err, 
         if ((it & 63) == 0) {
             if (*(volatile int *)err != 0) return false;
             if (globaltimer() - t0 > limit_ns) {
-                atomicCAS(err, 0, code);
+                set_status(err, code);
                 return false;
             }
         }
@@ -91,7 +107,7 @@ __device__ __forceinline__ bool mbar_wait_backoff(uint32_t bar, uint32_t parity,
         if ((it & (XENG_WAIT_CHECK_EVERY - 1)) == 0) {
             if (*(volatile int *)err != 0) return false;
             if (globaltimer() - t0 > limit_ns) {
-                atomicCAS(err, 0, code);
+                set_status(err, code);
                 return false;
             }
         }
@@ -243,7 +259,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
         if ((it & 15) == 0) {
             if (*(volatile int *)err != 0) return false;
             if (globaltimer() - t0 > kWaitLimitNs) {
-                atomicCAS(err, 0, code);
+                set_status(err, code);
                 return false;
             }
         }
@@ -294,7 +310,7 @@ __device__ __noinline__ bool flag_wait(const int *flag, int v, int *err, int cod
         if ((it & 15) == 0) {
             if (*(volatile int *)err != 0) return false;
             if (globaltimer() - t0 > kWaitLimitNs) {
-                atomicCAS(err, 0, code);
+                set_status(err, code);
                 return false;
             }
         }

@@ -40,7 +40,7 @@ struct xeng_s {
     uint8_t *staging = nullptr;    // device copy of host blocks
     int64_t staging_bytes = 0;
     int *d_err = nullptr;          // device status word of the kernels
-    int *h_err = nullptr;          // pinned mirror, refreshed after each push
+    int *h_err = nullptr;          // its mirror in pinned host memory, written by the kernel that sets it
     int sticky = XENG_OK;
     bool profiling = false;
     xeng_stats_t stats{};
@@ -136,7 +136,7 @@ int cuda_status(cudaError_t e)
 }
 
 // Surface earlier asynchronous failures: sticky CUDA errors and the kernels'
-// device status word (its pinned mirror is written by completed work only).
+// device status word (through its pinned mirror).
 int check_sticky(xeng_s *h)
 {
     if (h->sticky != XENG_OK) return h->sticky;
@@ -349,15 +349,12 @@ int xeng_create(int32_t n_inputs, int32_t n_freq, int64_t t_integ, xeng_t *out_h
     h->planes_bytes = g * per_ch;
 
     cudaError_t e = cudaMalloc(&h->acc, (size_t)acc_bytes(h));
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMallocHost(&h->h_err, sizeof(int));
+    if (e == cudaSuccess) e = status_alloc(&h->d_err, &h->h_err);
     if (e != cudaSuccess) {
         cudaGetLastError();
         xeng_destroy(h);
         return e == cudaErrorMemoryAllocation ? XENG_ERR_NOMEM : XENG_ERR_CUDA;
     }
-    *h->h_err = 0;
     h->gate_fresh.assign(1, 1);
     h->gate_base.assign(1, 0);
     *out_handle = h;
@@ -388,8 +385,7 @@ void xeng_destroy(xeng_t h)
     if (h->ev_fin) cudaEventDestroy(h->ev_fin);
     if (h->ev_sub) cudaEventDestroy(h->ev_sub);
     free_shift(h);
-    cudaFree(h->d_err);
-    if (h->h_err) cudaFreeHost(h->h_err);
+    status_free(h->d_err, h->h_err);
     for (auto &t : h->timed) {
         cudaEventDestroy(t.start);
         cudaEventDestroy(t.stop);
@@ -776,7 +772,6 @@ int xeng_push(xeng_t h, const uint8_t *block, int64_t n_samples, void *stream)
         cudaError_t e = integrate(h, dblock, n_samples, h->acc, h->fresh, s, h->shifted);
         if (e != cudaSuccess) return (h->sticky = cuda_status(e));
     }
-    cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     h->samples += n_samples;
     h->fresh = false;
     h->gate_base[0] += n_samples;  // every input of every sample usable
@@ -807,8 +802,7 @@ int xeng_correlate(xeng_t h, const uint8_t *block, int64_t n_samples, int32_t *o
     if (h->engine != XENG_ENGINE_DP4A && n_samples <= h->chunk_t && (!dev_in || !dev_out)) {
         // host buffers: copies overlap the compute, group by group
         st = integrate_pipelined(h, block, !dev_in, n_samples, dev_out ? out : h->acc, dev_out ? nullptr : out, true, s);
-        if (st == XENG_OK) e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (st == XENG_OK && e == cudaSuccess && !dev_out) e = cudaStreamSynchronize(s);
+        if (st == XENG_OK && !dev_out) e = cudaStreamSynchronize(s);
         if (st != XENG_OK) return (h->sticky = st);
         if (e != cudaSuccess) return (h->sticky = cuda_status(e));
         return dev_out ? XENG_OK : check_sticky(h);
@@ -817,7 +811,6 @@ int xeng_correlate(xeng_t h, const uint8_t *block, int64_t n_samples, int32_t *o
     if (!dblock) return st;
     // device output: written in place; host output: through the accumulators
     e = integrate(h, dblock, n_samples, dev_out ? out : h->acc, true, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && !dev_out) {
         e = cudaMemcpyAsync(out, h->acc, (size_t)bytes, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -896,7 +889,6 @@ int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samples, cons
             e = timed_launch(h, 1, s, [&] { return run_correlate(h, a, s); });
         }
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return (h->sticky = cuda_status(e));
     return XENG_OK;
 }
@@ -1094,7 +1086,6 @@ int xeng_push_gated(xeng_t h, const uint8_t *block, int64_t n_samples, const int
         if (valid) h->counts_dirty = true;
         else h->gate_base[g] += Tg;
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return (h->sticky = cuda_status(e));
     h->samples += n_samples;
     return XENG_OK;
@@ -1173,10 +1164,10 @@ int xeng_decode(const uint8_t *block, int64_t n_samples, int32_t n_freq, int32_t
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int *d_status = nullptr;
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void **>(&d_status), sizeof(int), s);
+    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void **>(&d_status), sizeof(StatusBlock), s);
     if (e != cudaSuccess) return cuda_status(e);
     int h_status = 0;
-    e = cudaMemsetAsync(d_status, 0, sizeof(int), s);
+    e = cudaMemsetAsync(d_status, 0, sizeof(StatusBlock), s);  // no mirror: the word is read back below
     if (e == cudaSuccess)
         e = launch_decode_tma(block, n_samples, n_freq, n_inputs, f0, nf, planes, t_pad, n_pad, d_status, sms, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, s);

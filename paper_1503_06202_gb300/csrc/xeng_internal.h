@@ -23,6 +23,17 @@ enum DevStatus : int {
     kDevTimeoutEpilogue = 3,
 };
 
+// What the kernels' `err` points at, in device memory: their status word and
+// the device address of its mirror in pinned host memory (may be null).
+struct StatusBlock {
+    int status;
+    int pad_;
+    int *mirror;
+};
+// A zeroed status block and its zeroed mirror (both null on failure).
+cudaError_t status_alloc(int **d_err, int **h_err);
+void status_free(int *d_err, int *h_err);
+
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 inline int64_t n_baselines(int64_t n) { return n * (n + 1) / 2; }
 
