@@ -9,35 +9,41 @@
 // cta_group::2 MMA share its B operand, so neither can leave its lower block
 // out.  Here each CTA works alone (cta_group::1, M = 128) on items of equal
 // cost, each two 128 x 128 complex blocks, 512 TMEM columns:
-//   row item of channel c:        A = inputs 0..127, B = inputs 0..255 (one
-//                                 N = 256 MMA per product): blocks (0,0), (0,1)
-//   diagonal item of channels c, c':  block (1,1) of each (one N = 256 and
+//   column item of channel c:     A = inputs 128..255, B = inputs 0..255 (one
+//                                 N = 256 MMA per product): blocks (0,1), (1,1)
+//   diagonal item of channels c, c':  block (0,0) of each (one N = 256 and
 //                                 two N = 128 MMAs per product pair)
 // Up to 128 inputs a channel is one diagonal block, and every item is a
-// diagonal item over two channels' inputs 0..127.  Per stage an item reads two
-// raw tiles of 128 inputs x 128 samples ("X" and "Y": the channel's two input
-// halves, or the two channels' upper halves).
+// diagonal item over two channels.  Per stage an item reads two raw tiles of
+// 128 inputs x 128 samples ("X" and "Y": the channel's two input halves, or the
+// two channels' lower halves).  The A operand holds inputs j and B inputs i, so
+// TMEM lanes are inputs j and a warp's store of column i is one 256-byte run of
+// the triangle's row i.
 //
 // The launch's work -- its items in order, each of n_k stages of 128 samples --
-// is split evenly over the CTAs: CTA b takes stages [b T / G, (b + 1) T / G)
-// of that sequence (T stages in all, G CTAs), so every CTA does the same
-// number of MMAs whether or not the items divide evenly.  An item cut between
-// CTAs is finished by its owner, the CTA holding its first stages (which
-// reaches them last): the CTAs holding its later pieces (which start with
-// them) write their corrected partial blocks to a workspace and raise a flag
-// stamped with the launch's epoch; the owner waits for those flags (bounded),
-// adds the partials to its own and stores.  A cooperative launch keeps every
-// CTA resident, so the waits end.
+// is cut over the CTAs in one of three ways (small_split).  Few items are
+// shared by several CTAs each, at one piece a CTA: all write their corrected
+// partial blocks to a workspace, raise a flag stamped with the launch's epoch,
+// wait (bounded) for the item's other flags, and each adds up and stores its
+// share of the item's 8-column chunks.  Many short items stay whole.  Otherwise
+// the sequence is cut evenly, so every CTA does the same number of MMAs whether
+// or not the items divide evenly: an item cut between CTAs is finished by its
+// owner, the CTA holding its first stages (which reaches them last), which adds
+// the others' partial blocks to its own.  A cooperative launch keeps every CTA
+// resident, so the waits end.  Bound by latency where calls are small: N = 256
+// x 8 channels x 4096 samples (12 items of 32 stages) takes 25 us on 144 CTAs,
+// 54-61 us on the 12 that pieces of 32 stages at least allowed; x 64 channels x
+// 1024 samples 23 us (86 us on 24 CTAs).
 //
 // The TMA writes raw tiles with a 128-byte swizzle: rows are samples, each 128
 // input bytes -- the canonical MN-major layout of an 8-bit tcgen05 operand
 // (inputs along M or N, samples along K).  The converter warps split each byte
 // at its own offset into the Re plane (high nibble) and the Im plane (low
 // nibble) of a plane stage; the raw slots form their own ring, so the TMA runs
-// ahead of the conversion.  The MMAs of a row item's stage
+// ahead of the conversion.  The MMAs of a column item's stage
 // (both operands MN-major; B spans the X and Y tiles, the leading byte offset
 // stepping from one to the other):
-//     Re += A_re B_re^T + A_im B_im^T,   Im += A_im B_re^T + (-A_re) B_im^T;
+//     Re += A_re B_re^T + A_im B_im^T,   Im += A_re B_im^T + (-A_im) B_re^T;
 // a diagonal item's tile against itself: [B_im | B_re] as one N = 256 operand.
 //
 // The planes hold raw nibbles: a byte whose low four bits are u (0..15) and
@@ -63,7 +69,7 @@
 #include <cstring>
 
 #include "tc_ptx.cuh"
-#include "triangle_store.cuh"
+#include "raw_offset.cuh"
 #include "xeng_internal.h"
 
 namespace xeng {
@@ -102,7 +108,15 @@ constexpr int kSBars = 2 * kSRaws + 2 * kSPlanes + 3 + 4;
 constexpr size_t kSSmem =
     1024 + (size_t)kSPlanes * kSPlaneBytes + (size_t)kSRaws * kSRawBytes + kSSums + kSBars * 8 + 16;
 static_assert(kSSmem <= 232448, "shared memory over the per-CTA limit");
-constexpr int kSMinPiece = 32;  // stages per CTA at least (the grid shrinks for small launches)
+constexpr int kSMinPiece = 32;  // evenly cut items: stages per CTA at least
+// Shared items: stages per CTA at least, CTAs per item at most.
+#ifndef XENG_SMALL_MIN_SHARED
+#define XENG_SMALL_MIN_SHARED 2
+#endif
+#ifndef XENG_SMALL_MAX_SHARED
+#define XENG_SMALL_MAX_SHARED 32
+#endif
+constexpr int kSMinShared = XENG_SMALL_MIN_SHARED, kSMaxShared = XENG_SMALL_MAX_SHARED;
 constexpr int kSChunks = 2 * kSBox / 16 / (32 * kSConvWarps);  // 16-byte chunks per converter thread and stage
 static_assert(kSChunks * 32 * kSConvWarps * 16 == 2 * kSBox, "the converter threads cover both tiles");
 constexpr int kSWiden = 16 / kSChunks;  // stages between widenings of the byte-lane sums (<= 240)
@@ -129,10 +143,12 @@ struct SmallArgs {
     int64_t t0, nt;        // samples t0 .. t0 + nt - 1 of the block, nt <= kFusedMaxSamples
     int32_t F, N, f0, nf;  // channels f0 .. f0 + nf - 1
     int32_t n_items, n_k;  // items; stages (of kSKc samples) per item
-    int64_t total;         // n_items * n_k: the launch's (item, stage) sequence, split evenly over the CTAs
+    int32_t split;         // CTAs per item (>= 2: shared items), else kSEven or kSWhole
+    int32_t quot, rest;    // the sequence's n_items * n_k stages (kSEven) or its items (kSWhole) over
+                           // the grid: CTA b takes quot of them, one more if b < rest
     int32_t *acc;          // [nf][N(N+1)/2][2], channel f0 + fl at fl
     int accumulate;        // 0: store, 1: add
-    int2 *ws;              // [grid][2][16][128][8] partial blocks of pieces that do not start their item
+    int2 *ws;              // [grid][2][16][4][128][2] partial blocks: (block, 8-column chunk, column pair, row)
     int *flags;            // [grid]: this launch's epoch once the CTA's partial is in ws
     int *epoch;            // [0]: launches so far on these flags (this launch's epoch is [0] + 1);
                            // [1]: CTAs of this launch finished
@@ -141,41 +157,51 @@ struct SmallArgs {
     int32_t spb;              // the launch's samples running through the blocks in order
 };
 
-// A CTA's work: the stages [lo, hi) of the launch's sequence (item-major),
-// lo = b * total / grid, as pieces (item, stages k0 .. k1 - 1).  A piece with
-// k0 > 0 (only ever a CTA's first) adds its partial block through ws; the CTA
-// whose piece starts the item (its owner) adds them into its own and stores.
+// A CTA's work: the stages [lo, hi) of the launch's sequence (item-major), as
+// pieces (item, stages k0 .. k1 - 1).  How the sequence is cut (small_split):
+//   kSEven      evenly.  A piece with k0 > 0 (only ever a CTA's first) adds its
+//               partial block through ws; the CTA whose piece starts the item
+//               (its owner) adds them into its own and stores.
+//   kSWhole     between items only: no partial blocks.
+//   2 or more   `split` CTAs share each item, one piece each: all of them write
+//               their partials of the chunks the others finish, and each adds up
+//               and stores its share of the item's 8-column chunks.
+constexpr int kSEven = 0, kSWhole = 1;
 struct Piece {
     int it, k0, k1;
 };
 
-__device__ __forceinline__ int64_t range_lo(const SmallArgs &a, int b) { return (int64_t)b * a.total / gridDim.x; }
-
-// The CTA whose range holds stage x of the sequence.
-__device__ __forceinline__ int stage_cta(const SmallArgs &a, int64_t x)
+__device__ __forceinline__ int range_lo(const SmallArgs &a, int b)
 {
-    return (int)(((x + 1) * (int64_t)gridDim.x - 1) / a.total);
+    if (a.split > kSWhole) return (b / a.split) * a.n_k + (b % a.split) * a.n_k / a.split;
+    return (b * a.quot + min(b, a.rest)) * (a.split == kSWhole ? a.n_k : 1);
 }
 
-__device__ __forceinline__ bool next_piece(const SmallArgs &a, int64_t &x, int64_t hi, Piece &p)
+// kSEven: the CTA whose range holds stage x of the sequence.
+__device__ __forceinline__ int stage_cta(const SmallArgs &a, int x)
+{
+    const int more = a.rest * (a.quot + 1);  // stages of the CTAs that take one more
+    return x < more ? x / (a.quot + 1) : a.rest + (x - more) / a.quot;
+}
+
+__device__ __forceinline__ bool next_piece(const SmallArgs &a, int &x, int hi, Piece &p)
 {
     if (x >= hi) return false;
-    p.it = (int)(x / a.n_k);
-    const int64_t first = (int64_t)p.it * a.n_k;
-    p.k0 = (int)(x - first);
-    p.k1 = (int)(hi - first < a.n_k ? hi - first : a.n_k);
+    p.it = x / a.n_k;
+    const int first = p.it * a.n_k;
+    p.k0 = x - first;
+    p.k1 = min(hi - first, a.n_k);
     x = first + p.k1;
     return true;
 }
 
-// Item `it`.  N > 128: per channel pair (2m, 2m + 1) the row item of 2m, the
-// diagonal item of both, the row item of 2m + 1 (an odd last channel: its row
-// item and a diagonal item of it alone).  N <= 128: diagonal items of channel
+// Item `it`.  N > 128: per channel pair (2m, 2m + 1) the column item of 2m, the
+// diagonal item of both, the column item of 2m + 1 (an odd last channel: its
+// column item and a diagonal item of it alone).  N <= 128: diagonal items of channel
 // pairs.  fy < 0: no second channel (its tile repeats the first; nothing stored).
 struct SmallItem {
-    bool row;
-    int fx, fy;  // channels (local) of the X and Y tiles
-    int base;    // first input of both tiles (diagonal items) / of X (row items: Y at 128)
+    bool col;
+    int fx, fy;  // channels (local) of the X and Y tiles: inputs 0..127, but a column item's Y 128..255
 };
 
 __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
@@ -183,28 +209,25 @@ __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
     SmallItem w;
     if (a.N > 128) {
         const int m = it / 3, r = it - 3 * m;
-        w.row = r != 1;
-        if (w.row) {
+        w.col = r != 1;
+        if (w.col) {
             w.fx = w.fy = 2 * m + (r >> 1);
-            w.base = 0;
         } else {
             w.fx = 2 * m;
             w.fy = 2 * m + 1 < a.nf ? 2 * m + 1 : -1;
-            w.base = 128;
         }
     } else {
-        w.row = false;
+        w.col = false;
         w.fx = 2 * it;
         w.fy = 2 * it + 1 < a.nf ? 2 * it + 1 : -1;
-        w.base = 0;
     }
     return w;
 }
 
-// kAdd: add into acc (a.accumulate != 0) instead of storing; a template so that
-// each launch carries only its own triangle-store path (the adding one needs
-// more registers).
-template <bool kAdd>
+// kAdd: add into acc (a.accumulate != 0) instead of storing; kShared: several
+// CTAs per item (a.split >= 2).  Templates so that each launch carries only its
+// own epilogue (the adding one needs more registers).
+template <bool kAdd, bool kShared>
 __global__ void __launch_bounds__(kSThreads, 1)
 correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallArgs a)
 {
@@ -217,6 +240,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
     const uint32_t sums_u = raw0 + kSRaws * kSRawBytes;
     const uint32_t bars = sums_u + kSSums;
     int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][256] (P, Q)
+    float2 *terms = reinterpret_cast<float2 *>(sums);                // in their place: the epilogue's offset terms
     auto plane = [&](int s) { return sbase + (uint32_t)(s * kSPlaneBytes); };
     auto slot = [&](int s) { return raw0 + (uint32_t)(s * kSRawBytes); };
     auto rawf = [&](int s) { return bars + 8u * s; };
@@ -235,7 +259,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int *err = a.err;
-    const int64_t lo = range_lo(a, (int)blockIdx.x), hi = range_lo(a, (int)blockIdx.x + 1);
+    const int lo = range_lo(a, (int)blockIdx.x), hi = range_lo(a, (int)blockIdx.x + 1);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSRaws; s++) {
@@ -274,12 +298,12 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
             int s = 0, issued = 0;
             uint32_t ph = 0;
             bool ok = true;
-            int64_t x = lo;
+            int x = lo;
             Piece pc;
             while (ok && next_piece(a, x, hi, pc)) {
                 const SmallItem w = small_item(a, pc.it);
                 const int fX = a.f0 + w.fx, fY = a.f0 + (w.fy >= 0 ? w.fy : w.fx);
-                const int xX = w.base, xY = w.row ? 128 : w.base;
+                const int xY = w.col ? 128 : 0;
                 for (int kc = pc.k0; kc < pc.k1; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
@@ -292,7 +316,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
                         z = (kc % a.spb) * kSKc;
                     }
                     mbar_expect_tx(rawf(s), kSRawBytes);
-                    tma_load_3d(slot(s), mp, xX, fX, z, rawf(s));
+                    tma_load_3d(slot(s), mp, 0, fX, z, rawf(s));
                     tma_load_3d(slot(s) + kSBox, mp, xY, fY, z, rawf(s));
                     ++issued;
                     if (++s == kSRaws) {
@@ -316,7 +340,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
             int s = 0;
             uint32_t ph = 0, uses = 0;
             bool ok = true;
-            int64_t x = lo;
+            int x = lo;
             Piece pc;
             while (ok && next_piece(a, x, hi, pc)) {
                 const SmallItem w = small_item(a, pc.it);
@@ -330,25 +354,27 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
                     }
                     fence_after();
                     const uint32_t st = plane(s);
-                    if (w.row) {
-                        // A = X rows, B = X and Y columns (the Y plane kSBox after the X
-                        // plane): Re in columns 0..255, Im in 256..511
+                    if (w.col) {
+                        // A = Y rows (TMEM lanes: inputs j), B = X and Y columns (inputs i; the
+                        // Y plane kSBox after the X plane): Re in columns 0..255, Im in 256..511
                         const uint64_t dre = sdesc(st + 2 * kSBox, kSBox), dim = sdesc(st, kSBox);
+                        const uint64_t are = sdesc(st + 3 * kSBox, kSBox), aim = sdesc(st + kSBox, kSBox);
                         #pragma unroll
                         for (int kk = 0; kk < kSKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
                             const uint32_t acc = (kc != pc.k0 || kk != 0) ? 1u : 0u;
                             const uint64_t k4 = 256u * kk;
-                            mma_f8(tmem, dre + k4, dre + k4, small_idesc(256, false), acc);
-                            mma_f8(tmem, dim + k4, dim + k4, small_idesc(256, false), 1u);
-                            mma_f8(tmem + 256u, dim + k4, dre + k4, small_idesc(256, false), acc);
-                            mma_f8(tmem + 256u, dre + k4, dim + k4, small_idesc(256, true), 1u);
+                            mma_f8(tmem, are + k4, dre + k4, small_idesc(256, false), acc);
+                            mma_f8(tmem, aim + k4, dim + k4, small_idesc(256, false), 1u);
+                            mma_f8(tmem + 256u, are + k4, dim + k4, small_idesc(256, false), acc);
+                            mma_f8(tmem + 256u, aim + k4, dre + k4, small_idesc(256, true), 1u);
                         }
                     } else {
                         // each tile against itself, in columns 256h..: one N = 256 MMA of
                         // A_im against [B_im | B_re] (Re_h 16 KB after Im_h) gives
                         // [Im Im^T | Im Re^T]; A_re B_re^T completes Re, and (-A_re) B_im^T
-                        // makes the second half Im Re^T - Re Im^T = Im.  (Four N = 128 MMAs
-                        // per tile instead ran at about 72% of the tensor rate.)
+                        // makes the second half Im Re^T - Re Im^T, minus Im of x_i conj(x_j) with
+                        // A = x_j.  (Four N = 128 MMAs per tile instead ran at about 72% of the
+                        // tensor rate.)
                         #pragma unroll
                         for (int h = 0; h < 2; h++) {
                             const uint64_t dim = sdesc(st + h * kSBox, 2 * kSBox), dre = sdesc(st + (2 + h) * kSBox, 2 * kSBox);
@@ -392,7 +418,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
         int rs = 0, ps = 0, local = 0;
         uint32_t rph = 0, pph = 0;
         bool ok = true;
-        int64_t x = lo;
+        int x = lo;
         Piece pc;
         for (; ok && next_piece(a, x, hi, pc); ++local) {
             // nibble sums of the thread's 16 inputs: byte lanes over up to 16
@@ -514,101 +540,193 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
         const int q = warp & 3;                     // TMEM lane quadrant this warp may access
         const int h = (warp - kSEpiWarp0) >> 2;     // the item's block: columns 128h.. of Re and Im
         const int et = (warp - kSEpiWarp0) * 32 + lane;
-        const int row = q * 32 + lane;              // TMEM lane: row within the block
+        const int row = q * 32 + lane;              // TMEM lane: input j within its 128-input block
         const int N = a.N;                          // <= 256
         const int nt = (int)a.nt;
         const int64_t nb = (int64_t)N * (N + 1) / 2;
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
-        // partial blocks in ws: [CTA][block h][chunk c / 8][row][8 pairs]
-        constexpr int kWs = 2 * 16 * 128 * 8;
-        const int wsi = ((h * 16) * 128 + row) * 8;  // + (c / 8) * 1024
+        // partial blocks in ws: [CTA][block h][chunk c / 8][column pair][row], 16 bytes each,
+        // so that a warp's 32 rows are one 512-byte run
+        constexpr int kWs = 2 * 16 * 4 * 128;    // 16-byte words per CTA
+        const int wsi = h * 16 * 4 * 128 + row;  // + (c / 8) * 512 + 128 per column pair
+        int4 *const ws = reinterpret_cast<int4 *>(a.ws);
         uint32_t uses = 0;
         int local = 0;
-        int64_t x = lo;
+        int x = lo;
         Piece pc;
         while (next_piece(a, x, hi, pc)) {
             const SmallItem w = small_item(a, pc.it);
             const int par = local & 1;
             // the piece's samples inside the launch: 64 n from each of the two products
-            const int n128 = 128 * ((pc.k1 * kSKc < nt ? pc.k1 * kSKc : nt) - pc.k0 * kSKc);
+            const float n128 = (float)(128 * ((pc.k1 * kSKc < nt ? pc.k1 * kSKc : nt) - pc.k0 * kSKc));
             const bool owner = pc.k0 == 0;
             // an owner whose item runs on: the CTAs after it that hold the rest
-            const int c_lo = (int)blockIdx.x + 1;
-            const int c_hi = owner && pc.k1 < a.n_k ? stage_cta(a, (int64_t)(pc.it + 1) * a.n_k - 1) : 0;
+            // (shared items: the item's other CTAs, which this one meets later)
+            const int c_lo = kShared ? pc.it * a.split : (int)blockIdx.x + 1;
+            const int c_hi = kShared ? c_lo + a.split - 1
+                                    : owner && pc.k1 < a.n_k ? stage_cta(a, (pc.it + 1) * a.n_k - 1) : 0;
             bool ok = mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
             ok = ok && mbar_wait_backoff(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
-            if (et == 0)
+            if (et == 0 && !kShared)
                 for (int b = c_lo; ok && b <= c_hi; b++) ok = flag_wait(a.flags + b, *s_epoch, err, kDevTimeoutEpilogue);
             // the barrier ORs the eight warps' failures, so they leave together
             if (bar_any(2, kSEpiWarps * 32, !ok)) break;
             ++uses;
             fence_after();
-            // block geometry: row items (rows 0..127, columns 128h..), diagonal items
-            // (channel fx or fy, rows and columns base..); sums index: X tile 0..127, Y tile 128..
-            const int fl = w.row ? w.fx : (h ? w.fy : w.fx);
-            const int i0 = w.row ? 0 : w.base;
-            const int j0b = w.row ? 128 * h : w.base;
-            const int2 *srow = sums + par * 256 + (w.row ? 0 : 128 * h);
-            const int2 *scol = sums + par * 256 + 128 * h;
-            const int i_warp = i0 + q * 32;
-            const int i = i0 + row;
-            if (fl >= 0 && i_warp < N) {
-                const bool row_ok = i < N;
-                const int2 pq = srow[row];
-                const int si = pq.x + pq.y, di = pq.x - pq.y;
-                const int row_base = i * N - i * (i - 1) / 2 - i;  // pair (i, j) at row_base + j
-                int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
-                // TMEM columns of the block: row items Re at 128h.., Im at 256 + 128h..;
-                // diagonal items Re at 256h.., Im at 256h + 128..
-                const uint32_t cre = w.row ? 128u * h : 256u * h;
-                const uint32_t cim = cre + (w.row ? 256u : 128u);
-                for (int c = 0; c < 128; c += 8) {
-                    const int j0 = j0b + c;
-                    // warp-uniform skips: chunks past the last input or below every row's diagonal
-                    if (j0 >= N) break;
-                    if (j0 + 7 < i_warp) continue;
-                    uint32_t vre[8], vim[8];
-                    tmem_ld8(taddr + cre + c, vre);
-                    tmem_ld8(taddr + cim + c, vim);
-                    tmem_ld_wait();
-                    if (!row_ok) continue;
-                    #pragma unroll
-                    for (int e = 0; e < 8; e++) {  // corrected values in place of the accumulator words
-                        const int2 pj = scol[c + e];  // the same for every lane: a broadcast
-                        // accumulators hold integer sums / 2^18: x 2^18 is exact
-                        vre[e] = (uint32_t)(__float2int_rn(262144.0f * __uint_as_float(vre[e])) -
-                                            8 * (si + pj.x + pj.y) + n128);
-                        vim[e] = (uint32_t)(__float2int_rn(262144.0f * __uint_as_float(vim[e])) +
-                                            8 * (di - (pj.x - pj.y)));
-                    }
-                    const int wo = wsi + (c >> 3) * 1024;
-                    if (!owner) {
-                        // a later piece of the item: the partial goes to this CTA's slot
-                        int4 *d = reinterpret_cast<int4 *>(a.ws + (int64_t)blockIdx.x * kWs + wo);
-                        #pragma unroll
-                        for (int e = 0; e < 8; e += 2)
-                            __stcg(d + e / 2, make_int4((int)vre[e], (int)vim[e], (int)vre[e + 1], (int)vim[e + 1]));
-                        continue;
-                    }
-                    for (int b = c_lo; b <= c_hi; b++) {  // the item's later pieces (none for a whole item)
-                        const int4 *src = reinterpret_cast<const int4 *>(a.ws + (int64_t)b * kWs + wo);
-                        #pragma unroll
-                        for (int e = 0; e < 8; e += 2) {
-                            const int4 v = __ldcg(src + e / 2);
-                            vre[e] += (uint32_t)v.x;
-                            vim[e] += (uint32_t)v.y;
-                            vre[e + 1] += (uint32_t)v.z;
-                            vim[e + 1] += (uint32_t)v.w;
-                        }
-                    }
-                    put8<kAdd>(out + row_base + j0, i - j0, N - j0, vre, vim);
+            // every input's offset terms in place of its sums (read by all the warps)
+            terms[par * 256 + et] = offset_terms(sums[par * 256 + et]);
+            named_bar_sync(2, kSEpiWarps * 32);
+            // Block h: column items' inputs j = 128.. against i = 128h..; diagonal items'
+            // channel fx or fy, both 0..127.  Sums: X tile at 0, Y tile at 128.
+            const int fl = w.col ? w.fx : (h ? w.fy : w.fx);
+            const int j_warp = (w.col ? 128 : 0) + q * 32;
+            const int j = j_warp + lane;
+            const int i_base = w.col ? 128 * h : 0;
+            const float2 *ci = terms + par * 256 + 128 * h;  // inputs i of the columns
+            const float2 tj = terms[par * 256 + (w.col ? 128 : 128 * h) + row];
+            const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
+            const bool lane_ok = j < N;
+            const bool warp_ok = fl >= 0 && j_warp < N;
+            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
+            // TMEM columns of the block: column items Re at 128h.., Im at 256 + 128h..;
+            // diagonal items Re at 256h.., Im (negated) at 256h + 128..
+            const uint32_t tre = taddr + (w.col ? 128u * h : 256u * h);
+            const uint32_t tim = tre + (w.col ? 256u : 128u);
+            const float im_scale = w.col ? kRawScale : -kRawScale;
+            // warp-uniform: columns inside the channel and up to some lane's diagonal
+            auto chunk_ok = [&](const int c) { return c < 128 && i_base + c < N && i_base + c <= j_warp + 31; };
+            // the piece's visibilities in place of the accumulator words of columns c .. c + 7
+            auto correct = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + c + e);  // the same for every lane: a broadcast
+                    vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
+                    vim[e] = raw_to_int(vim[e], im_scale, im_j + t2.y);
+                    vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
+                    vim[e + 1] = raw_to_int(vim[e + 1], im_scale, im_j + t2.w);
                 }
+            };
+            auto put_partial = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                int4 *d = ws + (int64_t)blockIdx.x * kWs + wsi + (c >> 3) * 512;
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2)
+                    __stcg(d + e * 64, make_int4((int)vre[e], (int)vim[e], (int)vre[e + 1], (int)vim[e + 1]));
+            };
+            auto add_partial = [&](const int b, const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                const int4 *src = ws + (int64_t)b * kWs + wsi + (c >> 3) * 512;
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    const int4 v = __ldcg(src + e * 64);
+                    vre[e] += (uint32_t)v.x;
+                    vim[e] += (uint32_t)v.y;
+                    vre[e + 1] += (uint32_t)v.z;
+                    vim[e + 1] += (uint32_t)v.w;
+                }
+            };
+            // Stores or adds columns c .. c + 7: pair (i, j) sits at i*N - i*(i-1)/2 + (j - i)
+            // in the channel's triangle and row i + 1 starts N - i - 1 pairs after row i, so
+            // per column the warp's 32 consecutive inputs j are one 256-byte run.
+            auto put_chunk = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                const int i0 = i_base + c;
+                const int off0 = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                const int last = min(j - i0, N - 1 - i0);  // elements e <= last are pairs of the triangle
+                int2 o[8];
+                if (kAdd) {
+                    int off = off0;
+                    #pragma unroll
+                    for (int e = 0; e < 8; e++) {
+                        if (lane_ok && e <= last) o[e] = __ldcs(out + off);
+                        off += N - (i0 + e) - 1;
+                    }
+                }
+                int off = off0;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (lane_ok && e <= last)
+                        __stcs(out + off, kAdd ? make_int2(o[e].x + (int)vre[e], o[e].y + (int)vim[e])
+                                               : make_int2((int)vre[e], (int)vim[e]));
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            // Calls fn(c, re, im) with the corrected values of the chunks c = c0, c0 + step, ...
+            // Where registers allow, in two sets: the next chunk's TMEM loads run under this
+            // chunk's stores.
+            auto for_chunks = [&](const int c0, const int step, auto &&fn) {
+                if (kAdd || kShared) {
+                    for (int c = c0; warp_ok && chunk_ok(c); c += step) {
+                        uint32_t vre[8], vim[8];
+                        tmem_ld8(tre + c, vre);
+                        tmem_ld8(tim + c, vim);
+                        tmem_ld_wait();
+                        correct(c, vre, vim);
+                        fn(c, vre, vim);
+                    }
+                    return;
+                }
+                uint32_t ra[8], ia[8], rb[8], ib[8];
+                int c = c0;
+                if (!warp_ok || !chunk_ok(c)) return;
+                tmem_ld8(tre + c, ra);
+                tmem_ld8(tim + c, ia);
+                tmem_ld_wait();
+                for (;;) {
+                    const int c1 = c + step;
+                    const bool ok1 = chunk_ok(c1);
+                    if (ok1) {
+                        tmem_ld8(tre + c1, rb);
+                        tmem_ld8(tim + c1, ib);
+                    }
+                    correct(c, ra, ia);
+                    fn(c, ra, ia);
+                    if (!ok1) break;
+                    tmem_ld_wait();
+                    c = c1 + step;
+                    const bool ok2 = chunk_ok(c);
+                    if (ok2) {
+                        tmem_ld8(tre + c, ra);
+                        tmem_ld8(tim + c, ia);
+                    }
+                    correct(c1, rb, ib);
+                    fn(c1, rb, ib);
+                    if (!ok2) break;
+                    tmem_ld_wait();
+                }
+            };
+            if (kShared) {
+                // chunk c of block h is finished by the item's CTA (16 h + c / 8) % split
+                const int part = (int)blockIdx.x - c_lo;
+                for_chunks(0, 8, [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                    if (lane_ok && (16 * h + (c >> 3)) % a.split != part) put_partial(c, vre, vim);
+                });
+                __threadfence();  // the partials are visible at GPU scope before the flag below
+                named_bar_sync(2, kSEpiWarps * 32);
+                if (et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
+                ok = et >= a.split || flag_wait(a.flags + c_lo + et, *s_epoch, err, kDevTimeoutEpilogue);
+                if (bar_any(2, kSEpiWarps * 32, !ok)) break;
+                const int first = (part + a.split - 16 * h % a.split) % a.split;  // 16 h + first = part (mod split)
+                for_chunks(8 * first, 8 * a.split, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                    if (!lane_ok) return;
+                    #pragma unroll 4
+                    for (int p = 1; p < a.split; p++)
+                        add_partial(c_lo + (part + p < a.split ? part + p : part + p - a.split), c, vre, vim);
+                    put_chunk(c, vre, vim);
+                });
+            } else {
+                for_chunks(0, 8, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                    if (!owner) {  // a later piece of the item: the partial goes to this CTA's slot
+                        if (lane_ok) put_partial(c, vre, vim);
+                        return;
+                    }
+                    // the item's later pieces (none for a whole item)
+                    for (int b = c_lo; lane_ok && b <= c_hi; b++) add_partial(b, c, vre, vim);
+                    put_chunk(c, vre, vim);
+                });
             }
-            if (!owner) __threadfence();  // the partial is visible at GPU scope before the flag below
+            if (!owner && !kShared) __threadfence();  // the partial is visible at GPU scope before the flag below
             // every epilogue thread is done with this parity's sums: clear them for
             // the piece after next, then hand TMEM and the buffer back
             named_bar_sync(2, kSEpiWarps * 32);
-            if (!owner && et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
+            if (!owner && !kShared && et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
             sums[par * 256 + et] = make_int2(0, 0);
             fence_before();
             __syncwarp();
@@ -649,6 +767,38 @@ bool small_ok(const uint8_t *block, int32_t N)
     return N >= 1 && N <= 256 && N % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
 }
 
+namespace {
+
+// How a launch's items (n_k stages each) are cut over the CTAs, at most one
+// per SM: *split as SmallArgs::split; returns the grid.
+int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split)
+{
+    // Few items: as many CTAs per item as there are SMs for, each with at least
+    // kSMinShared stages -- unless an even cut would leave a CTA over 16 stages
+    // less to do (GB300, N = 256 x 40 channels x 32,768 samples, 60 items: 162 us
+    // with two CTAs per item on 120 SMs, 159 cut evenly over 152).
+    const int64_t total = n_items * n_k;
+    int64_t s = num_sms / n_items;
+    if (s > n_k / kSMinShared) s = n_k / kSMinShared;
+    if (s > kSMaxShared) s = kSMaxShared;
+    if (s >= 2 && n_k / s <= total / num_sms + 16) {
+        *split = (int32_t)s;
+        return (int)(n_items * s);
+    }
+    // Short items: whole ones, since a partial block costs as much as the stages
+    // that an even cut saves (GB300, N = 256 x 128 channels x 256 samples: 25 us;
+    // cut evenly into pieces of kSMinPiece stages, 209).
+    if (n_k < kSMinPiece) {
+        *split = kSWhole;
+        return (int)(n_items < num_sms ? n_items : num_sms);
+    }
+    *split = kSEven;
+    const int64_t grid = total / kSMinPiece;
+    return (int)(grid < num_sms ? grid : num_sms);
+}
+
+}  // namespace
+
 size_t small_ws_bytes(int num_sms) { return (size_t)num_sms * 2 * 16 * 128 * 8 * sizeof(int2); }
 size_t small_flags_bytes(int num_sms) { return (size_t)(num_sms + 2) * sizeof(int); }
 
@@ -685,6 +835,15 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
         return cudaErrorInvalidValue;
     const int64_t n_items = N > 128 ? (int64_t)nf + (nf + 1) / 2 : (int64_t)(nf + 1) / 2;
     const int n_k = (int)((nt + kSKc - 1) / kSKc);
+    if (n_items * n_k > 2147483647LL) {  // stages are counted in 32 bits
+        const int32_t half = nf / 4 * 2;
+        const cudaError_t e = launch_correlate_small(block, T_block, t0, nt, F, N, f0, half, acc, accumulate, ws, flags,
+                                                     err, num_sms, s, maps, spb);
+        if (e != cudaSuccess) return e;
+        return launch_correlate_small(block, T_block, t0, nt, F, N, f0 + half, nf - half,
+                                      acc + (int64_t)half * N * (N + 1), accumulate, ws, flags, err, num_sms, s, maps,
+                                      spb);
+    }
     CUtensorMap map;
     if (maps) {
         memset(&map, 0, sizeof map);  // not read: the stages take the blocks' maps
@@ -692,7 +851,10 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
         cudaError_t e0 = encode_small_map(&map, block, T_block, F, N);
         if (e0 != cudaSuccess) return e0;
     }
-    auto kern = accumulate ? correlate_small_kernel<true> : correlate_small_kernel<false>;
+    int32_t split = 0;
+    const int grid = small_split(n_items, n_k, num_sms, &split);
+    auto kern = split >= 2 ? (accumulate ? correlate_small_kernel<true, true> : correlate_small_kernel<false, true>)
+                           : (accumulate ? correlate_small_kernel<true, false> : correlate_small_kernel<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmem);
     if (e != cudaSuccess) return e;
     SmallArgs a;
@@ -704,7 +866,6 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     a.nf = nf;
     a.n_items = (int32_t)n_items;
     a.n_k = n_k;
-    a.total = n_items * n_k;
     a.acc = acc;
     a.accumulate = accumulate;
     a.ws = ws;
@@ -713,13 +874,11 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     a.err = err;
     a.maps = maps;
     a.spb = spb;
-    // every CTA gets at least kSMinPiece stages (a piece's epilogue and partial
-    // cost about as much as a few stages of MMAs), at most one CTA per SM
-    int64_t grid = a.total / kSMinPiece;
-    if (grid < 1) grid = 1;
-    if (grid > num_sms) grid = num_sms;
-    // the owner of a split item waits for the CTAs holding its later pieces:
-    // a cooperative launch has every CTA resident at once (or fails)
+    a.split = split;
+    a.quot = (int32_t)((split == kSWhole ? n_items : n_items * n_k) / grid);
+    a.rest = (int32_t)((split == kSWhole ? n_items : n_items * n_k) % grid);
+    // the CTAs of a split item wait for each other's partials: a cooperative
+    // launch has every CTA resident at once (or fails)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid, 1, 1);
     cfg.blockDim = dim3(kSThreads, 1, 1);

@@ -95,6 +95,26 @@ def test_fused_items_split_over_many_ctas(N):
     assert np.array_equal(correlate(blk, pieces=[20000]), want)
 
 
+# How a launch's items (each of ceil(T / 128) stages) are cut over the CTAs:
+# shared by several CTAs (as many as there are SMs for, stages uneven between
+# them, at most 32, at least two stages each), whole, cut evenly, or -- 60 items
+# of 256 stages -- even because two CTAs an item would leave SMs idle.
+@pytest.mark.parametrize("T,F,N", [(257, 1, 128), (511, 1, 256), (512, 7, 16), (1000, 3, 144), (1700, 12, 208),
+                                   (4096, 8, 256), (5000, 25, 160), (9000, 1, 256), (300, 51, 256), (385, 77, 112),
+                                   (3969, 52, 256), (32700, 40, 256)])
+def test_small_items_shared_whole_or_cut(T, F, N):
+    rng = np.random.default_rng(T + F + N)
+    blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    if F > 16 and T > 1000:  # the oracle on the last channels and the first
+        keep = [0, 1, F - 2, F - 1]
+    else:
+        keep = list(range(F))
+    want = oracle.correlate(np.ascontiguousarray(blk[:, keep]))
+    assert np.array_equal(correlate(blk)[keep], want)
+    # the second push adds: its own cut of the rest
+    assert np.array_equal(correlate(blk, pieces=[T // 3])[keep], want)
+
+
 def test_fused_graph_replays_stay_exact():
     # one captured call replayed: the flags that publish split items' partial
     # blocks carry a count the device advances after every launch, so no replay
