@@ -311,7 +311,6 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             uint4 v[8];
             #pragma unroll
             for (int j = 0; j < 8; j++) v[j] = *reinterpret_cast<const uint4 *>(rt + ((j ^ (row & 7)) << 4));
-            mbar_arrive(rawe(r));
             const uint32_t xs = lane_base + (uint32_t)x * kXCols;
             #pragma unroll
             for (int h = 0; h < 8; h++) {  // 16 inputs = 8 columns of (Im, Re) codes per store
@@ -324,6 +323,11 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                 tmem_st8(xs + h * 8, col);
             }
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            // The raw slot goes back only now that the stores have taken the loaded
+            // words: an arrival right after the loads, with nothing waiting for their
+            // data, let the TMA refill the slot under loads still in flight (GB300,
+            // N = 256, 32 beams: half the rows of an item wrong in one run of seven).
+            mbar_arrive(rawe(r));
             fence_before();
             mbar_arrive(xf(x));
         }

@@ -125,3 +125,26 @@ def test_beams_argument_checks():
     torch.cuda.synchronize()
     assert (out == 0).all()
     bf.close()
+
+
+def test_beams_repeat_the_same_bits():
+    # short items of 32 beams, where the raw ring runs fastest: every pass over the
+    # same block gives the bits of the oracle (channel by channel on sampled rows)
+    T, F, N, B = 16384, 128, 256, 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    blk = torch.randint(0, 256, (T, F, N), dtype=torch.uint8, device="cuda", generator=g)
+    rng = np.random.default_rng(4)
+    w_re = rng.integers(-128, 128, size=(F, B, N), dtype=np.int64)
+    w_im = rng.integers(-128, 128, size=(F, B, N), dtype=np.int64)
+    bf = xe.XBeam(N, F, B)
+    bf.set_weights(np.ascontiguousarray(w_re, np.int8), np.ascontiguousarray(w_im, np.int8))
+    first, out = (torch.empty((T, F, B, 2), dtype=torch.int32, device="cuda") for _ in range(2))
+    bf.run(blk, first)
+    for _ in range(60):
+        bf.run(blk, out)
+        assert torch.equal(out, first)
+    ts = np.unique(rng.integers(0, T, 60))
+    want = oracle.beamform(np.ascontiguousarray(blk[torch.from_numpy(ts).cuda()].cpu().numpy()), w_re, w_im)
+    assert np.array_equal(first[torch.from_numpy(ts).cuda()].cpu().numpy().astype(np.int64), want)
+    bf.close()
