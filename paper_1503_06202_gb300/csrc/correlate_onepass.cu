@@ -46,6 +46,7 @@
 //                quadrant taking alternate 8-column chunks
 #include <cstring>
 
+#include "raw_offset.cuh"
 #include "tc_ptx.cuh"
 #include "xeng_internal.h"
 
@@ -164,6 +165,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
     const uint32_t sums_u = raw0 + kORaws * kORawBytes;
     const uint32_t bars = sums_u + kOSums;
     int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][256] (P, Q)
+    float2 *terms = reinterpret_cast<float2 *>(sums);                // in their place: the epilogue's offset terms
     auto plane = [&](int s) { return sbase + (uint32_t)(s * kOPlaneBytes); };
     auto slot = [&](int s) { return raw0 + (uint32_t)(s * kORawBytes); };
     auto rawf = [&](int s) { return bars + 8u * s; };
@@ -443,7 +445,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
         const int et = (warp - kOEpiWarp0) * 32 + lane;
         const int row = q * 32 + lane;                   // TMEM lane: row within the tile
         const int N = a.N;                               // <= 4096: triangle offsets within a channel fit in int
-        const int n128 = 128 * (int)a.nt;                // 64 n from each of the two products
+        const float n128 = 128.0f * (float)(int)a.nt;    // 64 n from each of the two products
         const int64_t nb2 = (int64_t)N * (N + 1) / 2;
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
         int local = 0;
@@ -455,14 +457,17 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
             // the barrier ORs the eight warps' failures, so they leave together
             if (bar_any(2, kOEpiWarps * 32, !ok)) break;
             fence_after();
+            // every input's offset terms in place of its sums (read by all the warps)
+            for (int k = et; k < 256; k += kOEpiWarps * 32) terms[par * 256 + k] = offset_terms(sums[par * 256 + k]);
+            named_bar_sync(2, kOEpiWarps * 32);
             const bool diag = w.I == w.J;
             const int j_warp = w.J * 128 + q * 32;  // the warp's first input j (TMEM lanes: block J)
             const int j = j_warp + lane;
-            const int2 *scol = sums + par * 256 + (diag ? 0 : 128);  // inputs i of the columns (block I)
+            const float2 *ci = terms + par * 256 + (diag ? 0 : 128);  // inputs i of the columns (block I)
             if (j_warp < N) {
                 const bool lane_ok = j < N;
-                const int2 pq = sums[par * 256 + row];
-                const int sj = pq.x + pq.y, dj = pq.x - pq.y;
+                const float2 tj = terms[par * 256 + row];
+                const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
                 int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)w.fl * nb2;
                 const uint32_t tb = taddr + 256u * ab;
                 const int ibase = w.I * 128;
@@ -473,14 +478,13 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
                 auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
                     const int i0 = ibase + c;
                     #pragma unroll
-                    for (int e = 0; e < 8; e++) {  // corrected values in place of the accumulator words
-                        const int2 pi = scol[c + e];  // the same for every lane: a broadcast
-                        // accumulators hold integer sums / 2^18 (x 2^18 is exact); with A = x_j
-                        // the Im half holds minus Im of x_i conj(x_j)
-                        vre[e] = (uint32_t)(__float2int_rn(262144.0f * __uint_as_float(vre[e])) -
-                                            8 * (sj + pi.x + pi.y) + n128);
-                        vim[e] = (uint32_t)(8 * ((pi.x - pi.y) - dj) -
-                                            __float2int_rn(262144.0f * __uint_as_float(vim[e])));
+                    for (int e = 0; e < 8; e += 2) {  // visibilities in place of the accumulator words
+                        const float4 t2 = *reinterpret_cast<const float4 *>(ci + c + e);  // the same for every lane
+                        // with A = x_j the Im half holds minus Im of x_i conj(x_j)
+                        vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
+                        vim[e] = raw_to_int(vim[e], -kRawScale, im_j + t2.y);
+                        vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
+                        vim[e + 1] = raw_to_int(vim[e + 1], -kRawScale, im_j + t2.w);
                     }
                     const int off0 = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
                     const int last = min(j - i0, N - 1 - i0);  // elements e <= last are pairs of the triangle

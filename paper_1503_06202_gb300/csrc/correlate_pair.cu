@@ -55,6 +55,7 @@
 //                each loading its next chunk from TMEM under the current one's stores
 #include <cstring>
 
+#include "raw_offset.cuh"
 #include "tc_ptx.cuh"
 #include "xeng_internal.h"
 
@@ -93,7 +94,7 @@ static_assert(kPEpiWarps % 4 == 0 && kPEpiWarps >= 4, "epilogue warps: a multipl
 constexpr int kPEpiPerQuad = kPEpiWarps / 4;
 constexpr int kPThreads = 32 * (kPEpiWarp0 + kPEpiWarps);
 constexpr uint32_t kPTmemCols = 512;
-constexpr int kPSums = 2 * 384 * 8;     // per item parity: (P, Q) of the CTA's A rows, then all 256 B columns
+constexpr int kPSums = 2 * 384 * 8;     // per item parity: offset terms of the CTA's A rows, then all 256 B columns
 constexpr int kPScratch = 2 * 4 * 128 * 8;  // per tile and warp of it: (P, Q) partials of its 128 inputs
 // barriers: raw full and empty per slot, plane full and empty per stage; acc
 // full, acc empty, drain; sums full and empty per parity
@@ -189,7 +190,7 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
     const uint32_t sums_u = raw0 + kPRaws * kPRawBytes;
     const uint32_t scratch_u = sums_u + kPSums;
     const uint32_t bars = scratch_u + kPScratch;
-    int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));        // [parity][384] (P, Q)
+    float2 *sums = reinterpret_cast<float2 *>(sgen + (sums_u - sbase));    // [parity][384] offset terms of (P, Q)
     int2 *scratch = reinterpret_cast<int2 *>(sgen + (scratch_u - sbase));  // [tile][warp of tile][128] (P, Q)
     auto plane = [&](int s) { return sbase + (uint32_t)(s * kPPlaneBytes); };
     auto slot = [&](int s) { return raw0 + (uint32_t)(s * kPRawBytes); };
@@ -482,14 +483,16 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
                             Q += p2.y;
                         }
                     }
-                    int2 *sp = sums + par * 384;
+                    float2 *sp = sums + par * 384;
+                    const float2 t = offset_terms(make_int2(P, Q));
                     if (g == 0) {
-                        sp[k] = make_int2(P, Q);  // this CTA's A rows
+                        sp[k] = t;  // this CTA's A rows
                     } else {
                         // this CTA's half of the B columns, here and in the peer
                         const int col = 128 + (int)rank * 128 + k;
-                        sp[col] = make_int2(P, Q);
-                        st_cluster_v2(mapa_rank(sums_u + (uint32_t)((par * 384 + col) * 8), peer), P, Q);
+                        sp[col] = t;
+                        st_cluster_v2(mapa_rank(sums_u + (uint32_t)((par * 384 + col) * 8), peer),
+                                      __float_as_int(t.x), __float_as_int(t.y));
                     }
                     __syncwarp();
                     if (lane == 0) {
@@ -516,7 +519,7 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
         for (int it = it_begin; it < a.n_items; it += it_step, ++local) {
             const PairItem w = pair_item<kListed>(a, it);
             const int N = kListed ? a.jobs[w.job].N : a.N;  // <= 4096: triangle offsets within a channel fit in int
-            const int n128 = 128 * (kListed ? a.jobs[w.job].nt : (int)a.nt);  // 64 n from each of the two products
+            const float n128 = 128.0f * (float)(kListed ? a.jobs[w.job].nt : (int)a.nt);  // 64 n from each of the two products
             int32_t *const acc = kListed ? a.jobs[w.job].acc : a.acc;
             const int par = local & 1;
             bool ok = mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
@@ -529,22 +532,21 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
             const int j = j_warp + lane;
             const bool lane_ok = j < N;
             int2 *out = reinterpret_cast<int2 *>(acc) + (int64_t)w.fl * ((int64_t)N * (N + 1) / 2);
-            const int2 *sp = sums + par * 384;
-            const int2 pq = sp[row];  // this lane's input j (A rows of this CTA)
-            const int sj = pq.x + pq.y, dj = pq.x - pq.y;
-            const int2 *cs = sp + 128;  // inputs i of the 256 columns
+            const float2 *sp = sums + par * 384;
+            const float2 tj = sp[row];  // this lane's input j (A rows of this CTA)
+            const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
+            const float2 *ci = sp + 128;  // inputs i of the 256 columns
             const int ibase = w.I2 * 256;
             // Corrects the chunk of columns c..c+7 held in (vre, vim) in place and stores it.
             auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8], const bool add) {
                 const int i0 = ibase + c;
                 #pragma unroll
-                for (int e = 0; e < 8; e++) {  // corrected values in place of the accumulator words
-                    const int2 pi = cs[c + e];  // the same for every lane: a broadcast
-                    // accumulators hold integer sums / 2^18: x 2^18 is exact
-                    vre[e] = (uint32_t)(__float2int_rn(262144.0f * __uint_as_float(vre[e])) -
-                                        8 * (sj + pi.x + pi.y) + n128);
-                    vim[e] = (uint32_t)(__float2int_rn(262144.0f * __uint_as_float(vim[e])) +
-                                        8 * ((pi.x - pi.y) - dj));
+                for (int e = 0; e < 8; e += 2) {  // visibilities in place of the accumulator words
+                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + c + e);  // the same for every lane
+                    vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
+                    vim[e] = raw_to_int(vim[e], kRawScale, im_j + t2.y);
+                    vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
+                    vim[e + 1] = raw_to_int(vim[e + 1], kRawScale, im_j + t2.w);
                 }
                 // pair (i, j) sits at i*N - i*(i-1)/2 + (j - i) in the channel's triangle;
                 // pair (i + 1, j) is N - i - 1 entries further on
