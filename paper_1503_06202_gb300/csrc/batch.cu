@@ -247,7 +247,8 @@ int plan(xeng_batch_s *b)
         int64_t item0 = 0;
         for (size_t k = 0; k < pj.size(); k++) {
             const xeng_job_t &jb = b->jobs[pj[k]];
-            if (encode_pair_map(&pmaps[k], jb.block, jb.n_samples, jb.n_freq, jb.n_inputs) != cudaSuccess)
+            if (encode_raw_map(&pmaps[k], jb.block, jb.n_samples, jb.n_freq, jb.n_inputs, 0, pair_stage_samples()) !=
+                cudaSuccess)
                 return XENG_ERR_CUDA;
             const int32_t nt2 = (jb.n_inputs + 255) / 256;
             PairJob &p = pjobs[k];

@@ -128,6 +128,8 @@ struct OnepassArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int8_t slot[kMaxBlocks];
 };
 
 struct OnepassItem {
@@ -154,7 +156,8 @@ __device__ __forceinline__ OnepassItem onepass_item(const OnepassArgs &a, int it
 // keeps two chunks' TMEM words in registers without spilling.
 template <bool kAdd>
 __global__ void __launch_bounds__(kOThreads, 1)
-correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const OnepassArgs a)
+correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
+                         const OnepassArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -227,6 +230,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
                 const OnepassItem w = onepass_item(a, it);
                 const int f = a.f0 + w.fl;
                 const bool diag = w.I == w.J;
+                const int sJ = a.sub ? a.slot[w.J] : -1, sI = a.sub ? a.slot[w.I] : -1;  // substituted blocks
                 for (int kc = 0; kc < n_k; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
@@ -240,8 +244,13 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
                     }
                     mbar_expect_tx(rawf(s), diag ? kOBox : kORawBytes);
                     // A: block J (TMEM lanes = inputs j), B: block I (columns = inputs i)
-                    tma_load_3d(slot(s), mp, w.J * 128, f, z, rawf(s));
-                    if (!diag) tma_load_3d(slot(s) + kOBox, mp, w.I * 128, f, z, rawf(s));
+                    // (sub_map's channels and samples are the launch's)
+                    if (sJ >= 0) tma_load_3d(slot(s), &sub_map, 128 * sJ, w.fl, kc * kOKc, rawf(s));
+                    else tma_load_3d(slot(s), mp, w.J * 128, f, z, rawf(s));
+                    if (!diag) {
+                        if (sI >= 0) tma_load_3d(slot(s) + kOBox, &sub_map, 128 * sI, w.fl, kc * kOKc, rawf(s));
+                        else tma_load_3d(slot(s) + kOBox, mp, w.I * 128, f, z, rawf(s));
+                    }
                     ++issued;
                     if (++s == kORaws) {
                         s = 0;
@@ -577,28 +586,9 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const Onep
 
 }  // namespace
 
-bool onepass_ok(const uint8_t *block, int32_t N)
+bool onepass_ok(const uint8_t *block, int32_t N, int32_t pitch)
 {
-    return N >= 16 && N <= 4096 && N % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
-}
-
-cudaError_t encode_onepass_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N)
-{
-    EncodeTiledFn enc = encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
-    // raw block: dims (input, channel, sample), boxes of 128 inputs x 1 channel x kOKc
-    // samples with a 128-byte swizzle (the MN-major operand layout); inputs past N and
-    // samples past the block read as zero bytes, nibbles 0 that add nothing (the
-    // converters zero the samples past the launch; rows and columns past N are never
-    // written)
-    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)F, (cuuint64_t)T_block};
-    cuuint64_t strides[2] = {(cuuint64_t)N, (cuuint64_t)N * F};
-    cuuint32_t box[3] = {128, 1, (cuuint32_t)kOKc}, estr[3] = {1, 1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)block, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    return cudaSuccess;
+    return N >= 1 && N <= 4096 && (pitch ? pitch : N) % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
 }
 
 int onepass_stage_samples() { return kOKc; }
@@ -606,21 +596,26 @@ int onepass_stage_samples() { return kOKc; }
 cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                      int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, int *err,
                                      int num_sms, cudaStream_t s,
-                                     const CUtensorMap *maps, int32_t spb)
+                                     const CUtensorMap *maps, int32_t spb,
+                                     int32_t pitch, const SubBlocks *sub)
 {
     if (nf <= 0 || nt <= 0) return cudaSuccess;
-    if (!onepass_ok(maps ? nullptr : block, N) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
+    if (!onepass_ok(maps ? nullptr : block, N, pitch) || (sub && maps) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
         t0 < 0 || t0 + nt > T_block || T_block > 2147483647LL ||
         f0 < 0 || f0 + nf > F || num_sms < 1 || (reinterpret_cast<uintptr_t>(acc) & 7) != 0)
         return cudaErrorInvalidValue;
     const int32_t nb = (N + 127) / 128;
     const int64_t n_items = (int64_t)nf * (nb * (nb + 1) / 2);
     if (n_items > 2147483647LL) return cudaErrorInvalidValue;
-    CUtensorMap map;
-    if (maps) {
-        memset(&map, 0, sizeof map);  // not read: the stages take the blocks' maps
-    } else {
-        cudaError_t e0 = encode_onepass_map(&map, block, T_block, F, N);
+    CUtensorMap map, sub_map;
+    memset(&map, 0, sizeof map);  // not read with `maps`: the stages take the blocks' maps
+    memset(&sub_map, 0, sizeof sub_map);
+    if (!maps) {
+        cudaError_t e0 = encode_raw_map(&map, block, T_block, F, N, pitch, kOKc);
+        if (e0 != cudaSuccess) return e0;
+    }
+    if (sub) {
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kOKc);
         if (e0 != cudaSuccess) return e0;
     }
     auto kernel = accumulate ? correlate_onepass_kernel<true> : correlate_onepass_kernel<false>;
@@ -641,8 +636,10 @@ cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int6
     a.err = err;
     a.maps = maps;
     a.spb = spb;
+    a.sub = sub ? 1 : 0;
+    if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     const int grid = n_items < num_sms ? (int)n_items : num_sms;
-    kernel<<<grid, kOThreads, kOSmem, s>>>(map, a);
+    kernel<<<grid, kOThreads, kOSmem, s>>>(map, sub_map, a);
     return cudaGetLastError();
 }
 

@@ -134,6 +134,8 @@ struct PairArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int8_t slot[kMaxBlocks];
     const PairJob *jobs;      // listed launches: the jobs (items job after job), else unused
     int32_t n_jobs;
 };
@@ -179,7 +181,8 @@ __device__ __forceinline__ PairItem pair_item(const PairArgs &a, int it)
 // keeps two chunks' TMEM words in registers without spilling.
 template <bool kListed, bool kAdd>
 __global__ void __launch_bounds__(kPThreads, 1)
-correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArgs a)
+correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
+                      const PairArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -256,6 +259,8 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
                 const int nk = kListed ? a.jobs[w.job].n_k : n_k;
                 const bool diag = w.I2 == w.J2;
                 const int xa = w.J2 * 256 + (int)rank * 128, xb = w.I2 * 256 + (int)rank * 128;
+                // substituted blocks (a block past the inputs has no slot)
+                const int sa = !kListed && a.sub ? a.slot[xa >> 7] : -1, sb = !kListed && a.sub ? a.slot[xb >> 7] : -1;
                 for (int kc = 0; kc < nk; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
@@ -271,8 +276,13 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
                         z = (kc % a.spb) * kPKc;
                     }
                     mbar_expect_tx(rawf(s), diag ? kPBox : kPRawBytes);
-                    tma_load_3d(slot(s), mp, xa, f, z, rawf(s));
-                    if (!diag) tma_load_3d(slot(s) + kPBox, mp, xb, f, z, rawf(s));
+                    // (sub_map's channels and samples are the launch's)
+                    if (sa >= 0) tma_load_3d(slot(s), &sub_map, 128 * sa, w.fl, kc * kPKc, rawf(s));
+                    else tma_load_3d(slot(s), mp, xa, f, z, rawf(s));
+                    if (!diag) {
+                        if (sb >= 0) tma_load_3d(slot(s) + kPBox, &sub_map, 128 * sb, w.fl, kc * kPKc, rawf(s));
+                        else tma_load_3d(slot(s) + kPBox, mp, xb, f, z, rawf(s));
+                    }
                     ++issued;
                     if (++s == kPRaws) {
                         s = 0;
@@ -640,28 +650,9 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const PairArg
 
 }  // namespace
 
-bool pair_ok(const uint8_t *block, int32_t N)
+bool pair_ok(const uint8_t *block, int32_t N, int32_t pitch)
 {
-    return N >= 16 && N <= 4096 && N % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
-}
-
-cudaError_t encode_pair_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N)
-{
-    EncodeTiledFn enc = encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
-    // raw block: dims (input, channel, sample), boxes of 128 inputs x 1 channel x kPKc
-    // samples with a 128-byte swizzle (the MN-major operand layout); inputs past N and
-    // samples past the block read as zero bytes, nibbles 0 that add nothing (the
-    // converters zero the samples past the launch; rows and columns past N are never
-    // written)
-    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)F, (cuuint64_t)T_block};
-    cuuint64_t strides[2] = {(cuuint64_t)N, (cuuint64_t)N * F};
-    cuuint32_t box[3] = {128, 1, (cuuint32_t)kPKc}, estr[3] = {1, 1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)block, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    return cudaSuccess;
+    return N >= 1 && N <= 4096 && (pitch ? pitch : N) % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
 }
 
 int pair_stage_samples() { return kPKc; }
@@ -669,21 +660,26 @@ int pair_stage_samples() { return kPKc; }
 cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F, int32_t N,
                                   int32_t f0, int32_t nf, int32_t *acc, int accumulate, int *err, int num_sms,
                                   cudaStream_t s,
-                                  const CUtensorMap *maps, int32_t spb)
+                                  const CUtensorMap *maps, int32_t spb,
+                                  int32_t pitch, const SubBlocks *sub)
 {
     if (nf <= 0 || nt <= 0) return cudaSuccess;
-    if (!pair_ok(maps ? nullptr : block, N) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
+    if (!pair_ok(maps ? nullptr : block, N, pitch) || (sub && maps) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
         t0 < 0 || t0 + nt > T_block || T_block > 2147483647LL ||
         f0 < 0 || f0 + nf > F || num_sms < 2 || (reinterpret_cast<uintptr_t>(acc) & 7) != 0)
         return cudaErrorInvalidValue;
     const int32_t nt2 = (N + 255) / 256;
     const int64_t n_items = (int64_t)nf * (nt2 * (nt2 + 1) / 2);
     if (n_items > 2147483647LL) return cudaErrorInvalidValue;
-    CUtensorMap map;
-    if (maps) {
-        memset(&map, 0, sizeof map);  // not read: the stages take the blocks' maps
-    } else {
-        cudaError_t e0 = encode_pair_map(&map, block, T_block, F, N);
+    CUtensorMap map, sub_map;
+    memset(&map, 0, sizeof map);  // not read with `maps`: the stages take the blocks' maps
+    memset(&sub_map, 0, sizeof sub_map);
+    if (!maps) {
+        cudaError_t e0 = encode_raw_map(&map, block, T_block, F, N, pitch, kPKc);
+        if (e0 != cudaSuccess) return e0;
+    }
+    if (sub) {
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kPKc);
         if (e0 != cudaSuccess) return e0;
     }
     auto kernel = accumulate ? correlate_pair_kernel<false, true> : correlate_pair_kernel<false, false>;
@@ -704,6 +700,8 @@ cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t
     a.err = err;
     a.maps = maps;
     a.spb = spb;
+    a.sub = sub ? 1 : 0;
+    if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     const int64_t clusters = n_items < num_sms / 2 ? n_items : num_sms / 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
@@ -719,7 +717,7 @@ cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t
     cfg.numAttrs = 1;
     a.jobs = nullptr;
     a.n_jobs = 0;
-    return cudaLaunchKernelEx(&cfg, kernel, map, a);
+    return cudaLaunchKernelEx(&cfg, kernel, map, sub_map, a);
 }
 
 cudaError_t launch_correlate_pair_listed(const PairJob *jobs, int32_t n_jobs, int64_t n_items, int *err, int num_sms,
@@ -751,7 +749,7 @@ cudaError_t launch_correlate_pair_listed(const PairJob *jobs, int32_t n_jobs, in
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, correlate_pair_kernel<true, false>, unused, a);
+    return cudaLaunchKernelEx(&cfg, correlate_pair_kernel<true, false>, unused, unused, a);
 }
 
 }  // namespace xeng

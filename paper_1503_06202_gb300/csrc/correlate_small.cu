@@ -155,6 +155,8 @@ struct SmallArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int8_t slot[kMaxBlocks];
 };
 
 // A CTA's work: the stages [lo, hi) of the launch's sequence (item-major), as
@@ -229,7 +231,8 @@ __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
 // own epilogue (the adding one needs more registers).
 template <bool kAdd, bool kShared>
 __global__ void __launch_bounds__(kSThreads, 1)
-correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallArgs a)
+correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
+                       const SmallArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -316,8 +319,13 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
                         z = (kc % a.spb) * kSKc;
                     }
                     mbar_expect_tx(rawf(s), kSRawBytes);
-                    tma_load_3d(slot(s), mp, 0, fX, z, rawf(s));
-                    tma_load_3d(slot(s) + kSBox, mp, xY, fY, z, rawf(s));
+                    // input block 0 of channel fx, and block 0 or 1 of fy; a substituted block
+                    // comes from its slot of sub_map, whose channels and samples are the launch's
+                    const int sX = a.sub ? a.slot[0] : -1, sY = a.sub ? a.slot[xY >> 7] : -1;
+                    if (sX >= 0) tma_load_3d(slot(s), &sub_map, 128 * sX, fX - a.f0, kc * kSKc, rawf(s));
+                    else tma_load_3d(slot(s), mp, 0, fX, z, rawf(s));
+                    if (sY >= 0) tma_load_3d(slot(s) + kSBox, &sub_map, 128 * sY, fY - a.f0, kc * kSKc, rawf(s));
+                    else tma_load_3d(slot(s) + kSBox, mp, xY, fY, z, rawf(s));
                     ++issued;
                     if (++s == kSRaws) {
                         s = 0;
@@ -762,9 +770,9 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const SmallA
 
 }  // namespace
 
-bool small_ok(const uint8_t *block, int32_t N)
+bool small_ok(const uint8_t *block, int32_t N, int32_t pitch)
 {
-    return N >= 1 && N <= 256 && N % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
+    return N >= 1 && N <= 256 && (pitch ? pitch : N) % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
 }
 
 namespace {
@@ -802,53 +810,40 @@ int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split)
 size_t small_ws_bytes(int num_sms) { return (size_t)num_sms * 2 * 16 * 128 * 8 * sizeof(int2); }
 size_t small_flags_bytes(int num_sms) { return (size_t)(num_sms + 2) * sizeof(int); }
 
-cudaError_t encode_small_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N)
-{
-    EncodeTiledFn enc = encode_tiled();
-    if (!enc) return cudaErrorNotSupported;
-    // raw block: dims (input, channel, sample), boxes of 128 inputs x 1 channel x kSKc
-    // samples with a 128-byte swizzle (the MN-major operand layout); inputs past N and
-    // samples past the block read as zero bytes, nibbles 0 that add nothing (the
-    // converters zero the samples past the launch; rows and columns past N are never
-    // written)
-    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)F, (cuuint64_t)T_block};
-    cuuint64_t strides[2] = {(cuuint64_t)N, (cuuint64_t)N * F};
-    cuuint32_t box[3] = {128, 1, (cuuint32_t)kSKc}, estr[3] = {1, 1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)block, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    return cudaSuccess;
-}
-
 int small_stage_samples() { return kSKc; }
 
 cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F, int32_t N,
                                    int32_t f0, int32_t nf, int32_t *acc, int accumulate, int2 *ws, int *flags,
                                    int *err, int num_sms, cudaStream_t s,
-                                   const CUtensorMap *maps, int32_t spb)
+                                   const CUtensorMap *maps, int32_t spb,
+                                   int32_t pitch, const SubBlocks *sub)
 {
     if (nf <= 0 || nt <= 0) return cudaSuccess;
-    if (!small_ok(maps ? nullptr : block, N) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
+    if (!small_ok(maps ? nullptr : block, N, pitch) || (sub && maps) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
         t0 < 0 || t0 + nt > T_block || T_block > 2147483647LL ||
         f0 < 0 || f0 + nf > F || num_sms < 1 || (reinterpret_cast<uintptr_t>(acc) & 7) != 0 || !ws || !flags)
         return cudaErrorInvalidValue;
     const int64_t n_items = N > 128 ? (int64_t)nf + (nf + 1) / 2 : (int64_t)(nf + 1) / 2;
     const int n_k = (int)((nt + kSKc - 1) / kSKc);
+    if (n_items * n_k > 2147483647LL && sub) return cudaErrorInvalidValue;
     if (n_items * n_k > 2147483647LL) {  // stages are counted in 32 bits
         const int32_t half = nf / 4 * 2;
         const cudaError_t e = launch_correlate_small(block, T_block, t0, nt, F, N, f0, half, acc, accumulate, ws, flags,
-                                                     err, num_sms, s, maps, spb);
+                                                     err, num_sms, s, maps, spb, pitch, nullptr);
         if (e != cudaSuccess) return e;
         return launch_correlate_small(block, T_block, t0, nt, F, N, f0 + half, nf - half,
                                       acc + (int64_t)half * N * (N + 1), accumulate, ws, flags, err, num_sms, s, maps,
-                                      spb);
+                                      spb, pitch, nullptr);
     }
-    CUtensorMap map;
-    if (maps) {
-        memset(&map, 0, sizeof map);  // not read: the stages take the blocks' maps
-    } else {
-        cudaError_t e0 = encode_small_map(&map, block, T_block, F, N);
+    CUtensorMap map, sub_map;
+    memset(&map, 0, sizeof map);  // not read with `maps`: the stages take the blocks' maps
+    memset(&sub_map, 0, sizeof sub_map);
+    if (!maps) {
+        cudaError_t e0 = encode_raw_map(&map, block, T_block, F, N, pitch, kSKc);
+        if (e0 != cudaSuccess) return e0;
+    }
+    if (sub) {
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kSKc);
         if (e0 != cudaSuccess) return e0;
     }
     int32_t split = 0;
@@ -874,6 +869,8 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     a.err = err;
     a.maps = maps;
     a.spb = spb;
+    a.sub = sub ? 1 : 0;
+    if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     a.split = split;
     a.quot = (int32_t)((split == kSWhole ? n_items : n_items * n_k) / grid);
     a.rest = (int32_t)((split == kSWhole ? n_items : n_items * n_k) % grid);
@@ -889,7 +886,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, map, a);
+    return cudaLaunchKernelEx(&cfg, kern, map, sub_map, a);
 }
 
 }  // namespace xeng

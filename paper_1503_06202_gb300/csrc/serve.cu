@@ -354,7 +354,7 @@ bool launch_round(xserve_s *sv)
                 st.queue.pop_front();
                 part.arrivals.push_back(qb.arrival);
                 st.last_arrival = std::max(st.last_arrival, qb.arrival);
-                if (encode_single_pass_map(sk, sv->h_smaps[slot] + n_smaps++, qb.ptr, st.block_samples, st.F, st.N) !=
+                if (encode_raw_map(sv->h_smaps[slot] + n_smaps++, qb.ptr, st.block_samples, st.F, st.N, 0, single_pass_stage(sk)) !=
                     cudaSuccess) {
                     sv->sticky = XENG_ERR_CUDA;  // never launch with a descriptor that failed to encode
                     return false;

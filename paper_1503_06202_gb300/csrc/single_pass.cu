@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "tc_ptx.cuh"
 #include "xeng_internal.h"
 
 namespace xeng {
@@ -88,14 +89,14 @@ int single_pass_force_from_env()
     return 0;
 }
 
-int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded)
+int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded, int32_t pitch)
 {
     if (force == kSingleNone || (bounded && N > XENG_FUSED_MAX_N)) return 0;
     const int k = force ? force : N <= 256 ? kSingleSmall : use_pair_kernel(N) ? kSinglePair : kSingleOnepass;
     switch (k) {
-    case kSingleSmall: return XENG_FUSED_SMALL && small_ok(block, N) ? k : 0;
-    case kSinglePair: return pair_ok(block, N) ? k : 0;
-    default: return onepass_ok(block, N) ? k : 0;
+    case kSingleSmall: return XENG_FUSED_SMALL && small_ok(block, N, pitch) ? k : 0;
+    case kSinglePair: return pair_ok(block, N, pitch) ? k : 0;
+    default: return onepass_ok(block, N, pitch) ? k : 0;
     }
 }
 
@@ -122,30 +123,42 @@ void small_scratch_free(SmallScratch *sc)
 
 cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, SmallScratch *sc,
-                               int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps, int32_t spb)
+                               int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps, int32_t spb,
+                               int32_t pitch, const SubBlocks *sub)
 {
     if (kernel == kSingleSmall) {
         cudaError_t e = small_scratch_alloc(sc, num_sms, s);
         if (e != cudaSuccess) return e;
         return launch_correlate_small(block, T_block, t0, nt, F, N, f0, nf, acc, accumulate, sc->ws, sc->flags, err,
-                                      num_sms, s, maps, spb);
+                                      num_sms, s, maps, spb, pitch, sub);
     }
     if (kernel == kSinglePair)
         return launch_correlate_pair(block, T_block, t0, nt, F, N, f0, nf, acc, accumulate, err, num_sms, s, maps,
-                                     spb);
+                                     spb, pitch, sub);
     if (kernel == kSingleOnepass)
         return launch_correlate_onepass(block, T_block, t0, nt, F, N, f0, nf, acc, accumulate, err, num_sms, s, maps,
-                                        spb);
+                                        spb, pitch, sub);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t encode_single_pass_map(int kernel, CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F,
-                                   int32_t N)
+cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N,
+                           int32_t pitch, int stage)
 {
-    if (kernel == kSingleSmall) return encode_small_map(map, block, T_block, F, N);
-    if (kernel == kSinglePair) return encode_pair_map(map, block, T_block, F, N);
-    if (kernel == kSingleOnepass) return encode_onepass_map(map, block, T_block, F, N);
-    return cudaErrorInvalidValue;
+    EncodeTiledFn enc = encode_tiled();
+    if (!enc) return cudaErrorNotSupported;
+    // a 128-byte swizzle gives the MN-major operand layout; inputs past N and
+    // samples past the block read as zero bytes, nibbles 0 that add nothing (the
+    // converters zero the samples past the launch; rows and columns past N are never
+    // written)
+    const cuuint64_t p = (cuuint64_t)(pitch ? pitch : N);
+    cuuint64_t dims[3] = {(cuuint64_t)N, (cuuint64_t)F, (cuuint64_t)T_block};
+    cuuint64_t strides[2] = {p, p * F};
+    cuuint32_t box[3] = {128, 1, (cuuint32_t)stage}, estr[3] = {1, 1, 1};
+    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)block, dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
 }
 
 int single_pass_stage(int kernel)

@@ -30,6 +30,8 @@ struct xeng_s {
     int32_t *acc = nullptr;        // [F][N(N+1)/2][2]
     uint8_t *planes = nullptr;     // decode buffer of the tensor engine
     int64_t planes_bytes = 0;
+    uint8_t *packed = nullptr;     // samples rearranged for the single-pass kernels (pack.cu)
+    int64_t packed_bytes = 0;
     int2 *partials = nullptr;      // raw-nibble planes: per-tile nibble sums [group_f][n_tb][n_pad]
     int2 *sums = nullptr;          // raw-nibble planes: (S, D) per input [group_f][n_pad]
     SmallScratch small;            // single-pass kernel up to 256 inputs: partial blocks of split items,
@@ -57,6 +59,8 @@ struct xeng_s {
     // time shifting: delays, history of the delayed inputs (ping-pong), their list
     bool shifted = false;
     int32_t *d_delay = nullptr, *d_slot = nullptr, *d_chunk_delay = nullptr, *d_shift_inputs = nullptr;
+    int32_t *d_shift_chunks = nullptr;  // 16-input chunks of the 128-input blocks that hold a delayed input
+    SubBlocks shift_blocks{};           // those blocks (n of them; `packed` is set per launch)
     uint8_t *hist[2] = {nullptr, nullptr};
     int hist_cur = 0;
     int64_t hist_H = 0;
@@ -118,9 +122,10 @@ void free_shift(xeng_s *h)
     cudaFree(h->d_slot);
     cudaFree(h->d_chunk_delay);
     cudaFree(h->d_shift_inputs);
+    cudaFree(h->d_shift_chunks);
     cudaFree(h->hist[0]);
     cudaFree(h->hist[1]);
-    h->d_delay = h->d_slot = h->d_chunk_delay = h->d_shift_inputs = nullptr;
+    h->d_delay = h->d_slot = h->d_chunk_delay = h->d_shift_inputs = h->d_shift_chunks = nullptr;
     h->hist[0] = h->hist[1] = nullptr;
     h->shifted = false;
     h->hist_H = 0;
@@ -259,6 +264,28 @@ cudaError_t launch_fused(xeng_s *h, const uint8_t *block, int64_t T_block, int64
                               &h->small, h->d_err, h->num_sms, s);
 }
 
+// The single-pass kernel for samples that are rearranged first (pack.cu), so
+// that neither N nor the block's alignment matters; 0: decode to planes.
+int packed_kernel(const xeng_s *h)
+{
+    const int32_t pitch = (int32_t)round_up(h->N, 16);
+    if (h->engine == XENG_ENGINE_TENSOR) return single_pass_kernel(nullptr, h->N, h->fused_force, true, pitch);
+    if (h->engine == XENG_ENGINE_TENSOR_FUSED)
+        return single_pass_kernel(nullptr, h->N, h->fused_force == kSingleNone ? 0 : h->fused_force, false, pitch);
+    return 0;
+}
+
+cudaError_t ensure_packed(xeng_s *h)
+{
+    if (h->packed) return cudaSuccess;
+    cudaError_t e = cudaMalloc(&h->packed, (size_t)h->packed_bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h->packed = nullptr;
+    }
+    return e;
+}
+
 // Run one kernel launch, bracketed by events when profiling.
 template <class F>
 cudaError_t timed_launch(xeng_s *h, int kind, cudaStream_t s, F &&fn)
@@ -347,6 +374,12 @@ int xeng_create(int32_t n_inputs, int32_t n_freq, int64_t t_integ, xeng_t *out_h
     if (g > 65535) g = 65535;
     h->group_f = (int32_t)g;
     h->planes_bytes = g * per_ch;
+    {
+        // the same budget for rearranged samples: rounds of channels x at most
+        // kFusedMaxSamples samples x whole 128-input blocks
+        const int64_t per = std::min<int64_t>(h->chunk_t, kFusedMaxSamples) * round_up(n_inputs, kTile);
+        h->packed_bytes = std::min<int64_t>(n_freq, std::max<int64_t>(1, budget / per)) * per;
+    }
 
     cudaError_t e = cudaMalloc(&h->acc, (size_t)acc_bytes(h));
     if (e == cudaSuccess) e = status_alloc(&h->d_err, &h->h_err);
@@ -367,6 +400,7 @@ void xeng_destroy(xeng_t h)
     cudaDeviceSynchronize();
     cudaFree(h->acc);
     cudaFree(h->planes);
+    cudaFree(h->packed);
     cudaFree(h->partials);
     cudaFree(h->sums);
     small_scratch_free(&h->small);
@@ -432,11 +466,25 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
         if (same) chunk[c] = delays[c * 16];
     }
     const int32_t S = (int32_t)inputs.size();
+    // the 128-input blocks that hold a delayed input, one after another
+    SubBlocks sub;
+    sub.packed = nullptr;
+    sub.n = 0;
+    std::fill(sub.slot, sub.slot + kMaxBlocks, (int8_t)-1);
+    std::vector<int32_t> chunks;
+    for (int32_t i : inputs)
+        if (sub.slot[i / kTile] < 0) {
+            sub.slot[i / kTile] = (int8_t)sub.n++;
+            for (int32_t c = 0; c < kTile / 16; c++) chunks.push_back(i / kTile * (kTile / 16) + c);
+        }
     const int64_t hist_bytes = (int64_t)H * h->F * S;
     cudaError_t e = cudaMalloc(&h->d_delay, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_slot, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_chunk_delay, sizeof(int32_t) * chunk.size());
     if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_inputs, sizeof(int32_t) * S);
+    if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_chunks, sizeof(int32_t) * chunks.size());
+    if (e == cudaSuccess)
+        e = cudaMemcpy(h->d_shift_chunks, chunks.data(), sizeof(int32_t) * chunks.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMalloc(&h->hist[0], (size_t)hist_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->hist[1], (size_t)hist_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_delay, delays, sizeof(int32_t) * N, cudaMemcpyHostToDevice);
@@ -454,6 +502,7 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
     }
     h->hist_H = H;
     h->hist_S = S;
+    h->shift_blocks = sub;
     h->shifted = true;
     return XENG_OK;
 }
@@ -488,6 +537,104 @@ const uint8_t *device_block(xeng_s *h, const uint8_t *block, int64_t bytes, cuda
     return h->staging;
 }
 
+// Integrate samples of the device block into `target` ([F][B][2] int32; the
+// first launch stores when `fresh`, every later one adds) through pack.cu and a
+// single-pass kernel: rounds of at most kFusedMaxSamples samples and as many
+// channels as the buffer holds.  The samples are 0 .. n - 1 of the block, or rows
+// idx[0 .. n) of it (device memory), with flags `valid` and usable-sample
+// `counts` [F][N] (either may be null).  Channels f0 .. f0 + nf - 1 of the block
+// (F_block channels) go to channels 0 .. nf - 1 of `target`.
+cudaError_t integrate_packed(xeng_s *h, int kernel, const uint8_t *dblock, int32_t F_block, int32_t f0, int32_t nf,
+                             int64_t n, const int32_t *idx, const uint8_t *valid, int32_t *counts, int32_t *target,
+                             bool fresh, cudaStream_t s)
+{
+    const int64_t nb2 = (int64_t)h->N * (h->N + 1);
+    cudaError_t e = ensure_packed(h);
+    PackArgs p;
+    p.block = dblock;
+    p.F = F_block;
+    p.N = h->N;
+    p.pitch = (int32_t)round_up(h->N, 16);
+    p.out = h->packed;
+    p.valid = valid;
+    for (int64_t t0 = 0; t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
+        p.nt = std::min<int64_t>(kFusedMaxSamples, n - t0);
+        p.t0 = t0;
+        p.idx = idx ? idx + t0 : nullptr;
+        const int64_t group = std::min<int64_t>(65535, h->packed_bytes / (p.nt * p.pitch));
+        for (int64_t c0 = 0; c0 < nf && e == cudaSuccess; c0 += group) {
+            p.f0 = f0 + (int32_t)c0;
+            p.nf = (int32_t)std::min<int64_t>(group, nf - c0);
+            p.counts = counts ? counts + c0 * h->N : nullptr;
+            e = timed_launch(h, 0, s, [&] { return launch_pack(p, h->num_sms, s); });
+            if (e != cudaSuccess) break;
+            e = timed_launch(h, 1, s, [&] {
+                return launch_single_pass(kernel, h->packed, p.nt, 0, p.nt, p.nf, h->N, 0, p.nf, target + c0 * nb2,
+                                          fresh && t0 == 0 ? 0 : 1, &h->small, h->d_err, h->num_sms, s, nullptr, 0,
+                                          p.pitch);
+            });
+        }
+    }
+    return e;
+}
+
+// The same with the handle's delays applied to samples 0 .. n - 1 of the block:
+// where TMA can address the block's rows only the 128-input blocks that hold a
+// delayed input are rearranged, else every input.
+cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int64_t n, int32_t *target, bool fresh,
+                              cudaStream_t s)
+{
+    const int32_t N = h->N, F = h->F;
+    const int64_t nb2 = (int64_t)N * (N + 1);
+    const bool direct = single_pass_kernel(dblock, N, kernel, false) == kernel;
+    cudaError_t e = ensure_packed(h);
+    ShiftArgs sa;
+    sa.delay = h->d_delay;
+    sa.slot = h->d_slot;
+    sa.chunk_delay = h->d_chunk_delay;
+    sa.hist = h->hist[h->hist_cur];
+    sa.H = h->hist_H;
+    sa.S = h->hist_S;
+    PackArgs p;
+    p.block = dblock;
+    p.F = F;
+    p.N = N;
+    p.out = h->packed;
+    p.chunks = direct ? h->d_shift_chunks : nullptr;
+    p.pitch = direct ? h->shift_blocks.n * kTile : (int32_t)round_up(N, 16);
+    SubBlocks sub = h->shift_blocks;
+    sub.packed = h->packed;
+    for (int64_t t0 = 0; t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
+        p.nt = std::min<int64_t>(kFusedMaxSamples, n - t0);
+        p.t0 = t0;
+        const int64_t group = std::min<int64_t>(65535, h->packed_bytes / (p.nt * p.pitch));
+        for (int64_t f0 = 0; f0 < F && e == cudaSuccess; f0 += group) {
+            p.f0 = (int32_t)f0;
+            p.nf = (int32_t)std::min<int64_t>(group, F - f0);
+            const int accumulate = fresh && t0 == 0 ? 0 : 1;
+            e = timed_launch(h, 0, s, [&] { return launch_pack_shifted(p, sa, h->num_sms, s); });
+            if (e != cudaSuccess) break;
+            e = timed_launch(h, 1, s, [&] {
+                return direct ? launch_single_pass(kernel, dblock, n, t0, p.nt, F, N, p.f0, p.nf, target + f0 * nb2,
+                                                   accumulate, &h->small, h->d_err, h->num_sms, s, nullptr, 0, 0, &sub)
+                              : launch_single_pass(kernel, h->packed, p.nt, 0, p.nt, p.nf, N, 0, p.nf,
+                                                   target + f0 * nb2, accumulate, &h->small, h->d_err, h->num_sms, s,
+                                                   nullptr, 0, p.pitch);
+            });
+        }
+    }
+    return e;
+}
+
+// New history of the delayed inputs after n samples of the block.
+cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t n, cudaStream_t s)
+{
+    cudaError_t e = launch_shift_history(h->hist[h->hist_cur], dblock, n, h->F, h->N, h->d_shift_inputs, h->hist_S,
+                                         h->hist_H, h->hist[h->hist_cur ^ 1], s);
+    if (e == cudaSuccess) h->hist_cur ^= 1;
+    return e;
+}
+
 // Integrate n samples of the device block into `target` ([F][B][2] int32):
 // the first launch stores when `fresh`, every later one adds.  Work is
 // ordered after earlier work on `s` and before later work on `s`.
@@ -513,6 +660,13 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
             });
         }
         return e;
+    }
+    if (const int kernel = packed_kernel(h)) {
+        if (!apply_shift)
+            return integrate_packed(h, kernel, dblock, (int32_t)F, 0, (int32_t)F, n_samples, nullptr, nullptr, nullptr,
+                                    target, fresh, s);
+        e = integrate_shifted(h, kernel, dblock, n_samples, target, fresh, s);
+        return e == cudaSuccess ? advance_history(h, dblock, n_samples, s) : e;
     }
     e = ensure_planes(h);
     for (int64_t t0 = 0; t0 < n_samples && e == cudaSuccess; t0 += h->chunk_t) {
@@ -563,11 +717,7 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
             e = timed_launch(h, 1, s, [&] { return run_correlate(h, a, s); });
         }
     }
-    if (e == cudaSuccess && apply_shift) {
-        e = launch_shift_history(h->hist[h->hist_cur], dblock, n_samples, (int32_t)F, (int32_t)N, h->d_shift_inputs,
-                                 h->hist_S, h->hist_H, h->hist[h->hist_cur ^ 1], s);
-        if (e == cudaSuccess) h->hist_cur ^= 1;
-    }
+    if (e == cudaSuccess && apply_shift) e = advance_history(h, dblock, n_samples, s);
     return e;
 }
 
@@ -689,10 +839,14 @@ int integrate_pipelined(xeng_s *h, const uint8_t *src, bool host_in, int64_t n, 
         // correlation earlier and end as much sooner after the last one.
         const int32_t subs = host_out ? std::min<int32_t>(XENG_PIPE_SUBGROUPS, nf) : 1;
         const int32_t per = (nf + subs - 1) / subs;
-        if (fused_ok(h, blk)) {
+        const int pk = fused_ok(h, blk) ? 0 : packed_kernel(h);
+        if (pk || fused_ok(h, blk)) {
             for (int32_t c0 = 0; c0 < nf && e == cudaSuccess; c0 += per) {
                 const int32_t nc = std::min<int32_t>(per, nf - c0);
-                for (int64_t t0 = 0; t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
+                if (pk)
+                    e = integrate_packed(h, pk, blk, bf, bf0 + c0, nc, n, nullptr, nullptr, nullptr,
+                                         target + (f0 + c0) * nb2, fresh, s);
+                for (int64_t t0 = 0; !pk && t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
                     const int64_t nt = (n - t0) < kFusedMaxSamples ? (n - t0) : kFusedMaxSamples;
                     e = timed_launch(h, 1, s, [&] {
                         return launch_fused(h, blk, n, t0, nt, bf, bf0 + c0, nc, target + (f0 + c0) * nb2,
@@ -856,7 +1010,8 @@ int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samples, cons
         if (e != cudaSuccess) return (h->sticky = cuda_status(e));
         h->gidx_cap = (int64_t)idx.size();
     }
-    e = ensure_planes(h);
+    const int pk = packed_kernel(h);
+    e = pk ? ensure_packed(h) : ensure_planes(h);
     if (e != cudaSuccess) return (h->sticky = cuda_status(e));
     e = cudaMemcpyAsync(h->gidx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // idx is pageable and goes out of scope
@@ -866,6 +1021,11 @@ int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samples, cons
         int32_t *out_g = out + (int64_t)g * F * nb2;
         if (Tg == 0) {
             e = cudaMemsetAsync(out_g, 0, (size_t)(F * nb2 * 4), s);
+            continue;
+        }
+        if (pk) {
+            e = integrate_packed(h, pk, block, (int32_t)F, 0, (int32_t)F, Tg, h->gidx + cnt[g], valid,
+                                 counts ? counts + (int64_t)g * F * N : nullptr, out_g, true, s);
             continue;
         }
         const int64_t t_pad = round_up(Tg, kTile);
@@ -1048,7 +1208,8 @@ int xeng_push_gated(xeng_t h, const uint8_t *block, int64_t n_samples, const int
         if (e != cudaSuccess) return (h->sticky = cuda_status(e));
         h->gidx_cap = (int64_t)idx.size();
     }
-    e = ensure_planes(h);
+    const int pk = packed_kernel(h);
+    e = pk ? ensure_packed(h) : ensure_planes(h);
     // the list is rewritten by the next gated call: this call's launches read it first
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e == cudaSuccess)
@@ -1058,6 +1219,14 @@ int xeng_push_gated(xeng_t h, const uint8_t *block, int64_t n_samples, const int
         const int64_t Tg = cnt[g + 1] - cnt[g];
         if (Tg == 0) continue;
         int32_t *set = h->acc + (int64_t)g * F * nb2;
+        if (pk) {
+            e = integrate_packed(h, pk, block, (int32_t)F, 0, (int32_t)F, Tg, h->gidx + cnt[g], valid,
+                                 valid ? h->counts + (int64_t)g * F * N : nullptr, set, set_fresh(h, g), s);
+            mark_set_used(h, g);
+            if (valid) h->counts_dirty = true;
+            else h->gate_base[g] += Tg;
+            continue;
+        }
         // rounds of at most chunk_t samples of the set: exact f32 sums per launch
         for (int64_t k0 = 0; k0 < Tg && e == cudaSuccess; k0 += h->chunk_t) {
             const int64_t nk = std::min<int64_t>(h->chunk_t, Tg - k0);

@@ -143,7 +143,45 @@ cudaError_t launch_shift_fixup(const uint8_t *block, int64_t t0, int64_t nt, int
 cudaError_t launch_shift_history(const uint8_t *hist_old, const uint8_t *block, int64_t n, int32_t F, int32_t N,
                                  const int32_t *inputs, int32_t S, int64_t H, uint8_t *hist_new, cudaStream_t s);
 
-// Decode fused into the correlation for N <= 256 (small_ok: N % 16 == 0, block
+// Raw samples rearranged into rows of `pitch` bytes (a multiple of 16) per
+// channel, out[nt][nf][pitch], for a single-pass launch: row t is the block's
+// sample t0 + t, or idx[t] where idx (device memory) is given; channels
+// f0 .. f0 + nf - 1.  launch_pack (pitch >= N) also replaces samples whose
+// `valid` byte is 0 by 0x88 and adds the usable samples to counts[nf][N]; both
+// may be null.  launch_pack_shifted applies the delays of `sa`; `chunks` (device
+// memory, pitch / 16 entries) names the 16-input chunks of the block that make
+// up a row, null all of them.  nt <= kMaxChunkSamples.
+struct PackArgs {
+    const uint8_t *block = nullptr;
+    int64_t t0 = 0, nt = 0;
+    int32_t F = 0, N = 0, f0 = 0, nf = 0;
+    const int32_t *idx = nullptr;
+    const uint8_t *valid = nullptr;
+    int32_t *counts = nullptr;
+    const int32_t *chunks = nullptr;
+    int32_t pitch = 0;
+    uint8_t *out = nullptr;
+};
+cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s);
+cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_sms, cudaStream_t s);
+
+// What the three single-pass launches below share.  A block's rows are `pitch`
+// bytes per channel (0: N), a multiple of 16; N itself need not be one.  With
+// `sub`, the 128-input blocks b with slot[b] >= 0 are read from packed
+// [nt][nf][128 n] (16-byte aligned) instead, at inputs 128 slot[b] ..: the
+// launch's samples and channels, rearranged (launch_pack_shifted).
+constexpr int kMaxBlocks = 32;  // 128-input blocks of 4096 inputs
+struct SubBlocks {
+    const uint8_t *packed;
+    int32_t n;
+    int8_t slot[kMaxBlocks];
+};
+// The raw block's tensor map of their stages (3D: input, channel, sample; boxes of
+// 128 inputs x 1 channel x `stage` samples, 128-byte swizzle).
+cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N,
+                           int32_t pitch, int stage);
+
+// Decode fused into the correlation for N <= 256 (small_ok: pitch % 16 == 0, block
 // 16-byte aligned): samples t0 .. t0 + nt - 1 (nt <= kFusedMaxSamples) of the
 // block (T_block samples), channels f0 .. f0 + nf - 1, stored (accumulate = 0)
 // or added into acc [nf][N(N+1)/2][2] (8-byte aligned); no decoded planes.
@@ -153,43 +191,40 @@ cudaError_t launch_shift_history(const uint8_t *hist_old, const uint8_t *block, 
 // and flags (small_flags_bytes(num_sms), zeroed once: a flag per CTA, the
 // count of launches on them and an arrival counter, with which the last CTA of
 // each launch advances the count, so replays of a captured launch stay apart).
-bool small_ok(const uint8_t *block, int32_t N);
+bool small_ok(const uint8_t *block, int32_t N, int32_t pitch = 0);
 size_t small_ws_bytes(int num_sms);
 size_t small_flags_bytes(int num_sms);
 cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F, int32_t N,
                                    int32_t f0, int32_t nf, int32_t *acc, int accumulate, int2 *ws, int *flags,
                                    int *err, int num_sms, cudaStream_t s,
-                                   const CUtensorMap *maps = nullptr, int32_t spb = 0);
-// The raw-block tensor map launch_correlate_small uses (3D: input, channel, sample;
-// its stage's box, 128-byte swizzle), and its stage in samples.
-cudaError_t encode_small_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N);
-int small_stage_samples();
+                                   const CUtensorMap *maps = nullptr, int32_t spb = 0,
+                                   int32_t pitch = 0, const SubBlocks *sub = nullptr);
+int small_stage_samples();  // its stage
 
-// One pass over the raw bytes for N a multiple of 16 up to 4096 (block 16-byte
-// aligned; used above 256 inputs): single CTAs over every channel's
+// One pass over the raw bytes for N up to 4096 (rows of 16-byte multiples, block
+// 16-byte aligned; used above 256 inputs): single CTAs over every channel's
 // upper-triangle pairs of 128-input blocks, the nibble split and each pair's
 // nibble sums in shared memory; nt <= kFusedMaxSamples, acc 8-byte aligned.
-bool onepass_ok(const uint8_t *block, int32_t N);
+bool onepass_ok(const uint8_t *block, int32_t N, int32_t pitch = 0);
 cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                      int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, int *err,
                                      int num_sms, cudaStream_t s,
-                                     const CUtensorMap *maps = nullptr, int32_t spb = 0);
-// The raw-block tensor map launch_correlate_onepass uses (3D: input, channel, sample;
-// its stage's box, 128-byte swizzle), and its stage in samples.
-cudaError_t encode_onepass_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N);
-int onepass_stage_samples();
+                                     const CUtensorMap *maps = nullptr, int32_t spb = 0,
+                                     int32_t pitch = 0, const SubBlocks *sub = nullptr);
+int onepass_stage_samples();  // its stage
 
-// Decode fused into the correlation for 16 <= N <= 4096 (N % 16 == 0, block
+// Decode fused into the correlation for N <= 4096 (rows of 16-byte multiples, block
 // 16-byte aligned), as launch_correlate_small: 2-CTA clusters over every
 // channel's upper-triangle pairs of 256-input blocks, nibble sums in shared
 // memory; nt <= kFusedMaxSamples, acc 8-byte aligned.
-bool pair_ok(const uint8_t *block, int32_t N);
+bool pair_ok(const uint8_t *block, int32_t N, int32_t pitch = 0);
 cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F, int32_t N,
                                   int32_t f0, int32_t nf, int32_t *acc, int accumulate, int *err, int num_sms,
                                   cudaStream_t s,
-                                  const CUtensorMap *maps = nullptr, int32_t spb = 0);
+                                  const CUtensorMap *maps = nullptr, int32_t spb = 0,
+                                  int32_t pitch = 0, const SubBlocks *sub = nullptr);
 // One job of a listed launch of the pair kernel (a batch's jobs in one
-// persistent launch): its raw block's tensor map (encode_pair_map, in device
+// persistent launch): its raw block's tensor map (encode_raw_map, in device
 // memory, 64-byte aligned), its output [F][N(N+1)/2][2] (stored) and sizes: nt
 // <= kFusedMaxSamples samples in n_k stages, nt2 256-input blocks and
 // pairs_per_ch upper-triangle block pairs per channel, its items item0 ..
@@ -201,22 +236,20 @@ struct PairJob {
 };
 cudaError_t launch_correlate_pair_listed(const PairJob *jobs, int32_t n_jobs, int64_t n_items, int *err, int num_sms,
                                          cudaStream_t s);
-// The raw-block tensor map launch_correlate_pair uses (3D: input, channel, sample;
-// its stage's box, 128-byte swizzle), and its stage in samples.
-cudaError_t encode_pair_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N);
-int pair_stage_samples();
+int pair_stage_samples();  // its stage
 
 // The single-pass kernel (single_pass.cu) that takes a block of N inputs:
 // kSingleSmall (N <= 256), kSingleOnepass or kSinglePair (above, by the
 // measured cost of their block pairs), or 0 where none applies (N not a
-// multiple of 16, block not 16-byte aligned, a kernel switched off, or
+// multiple of 16 (where `pitch` is not given), block not 16-byte aligned, a kernel
+// switched off, or
 // `bounded` and N above the build's XENG_FUSED_MAX_N, where two passes are
 // faster).  `force`: 0, a kernel to take for every N it covers, or kSingleNone.
 enum SinglePass { kSingleNone = -1, kSingleSmall = 1, kSingleOnepass = 2, kSinglePair = 3 };
 // The environment variable XENG_FUSED_KERNEL: "pair", "onepass" (force that
 // kernel), "none" (no single pass for the default engine and batches), else 0.
 int single_pass_force_from_env();
-int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded);
+int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded, int32_t pitch = 0);
 // Scratch of the N <= 256 kernel, allocated at its first launch (flags zeroed
 // on the stream) and owned by the caller.
 struct SmallScratch {
@@ -229,14 +262,12 @@ void small_scratch_free(SmallScratch *sc);
 // (nt <= kFusedMaxSamples) and channels f0 .. f0 + nf - 1 of the block.  With
 // `maps` (device memory, 64-byte aligned), the samples come instead from
 // consecutive blocks of spb stages each, block k through maps[k] (made by
-// encode_single_pass_map); block is then unused and t0 must be 0.
+// encode_raw_map); block is then unused and t0 must be 0.
 cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, SmallScratch *sc,
                                int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps = nullptr,
-                               int32_t spb = 0);
-// A block's tensor map for `kernel`'s stage tables, and the kernel's stage.
-cudaError_t encode_single_pass_map(int kernel, CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F,
-                                   int32_t N);
+                               int32_t spb = 0, int32_t pitch = 0, const SubBlocks *sub = nullptr);
+// A kernel's stage in samples.
 int single_pass_stage(int kernel);
 
 // Beamforming (Sec. IV-C-3).  The host fills T, F, N, B, out and err; the
