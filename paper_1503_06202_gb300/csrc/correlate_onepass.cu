@@ -48,6 +48,7 @@
 
 #include "raw_offset.cuh"
 #include "tc_ptx.cuh"
+#include "triangle_add.cuh"
 #include "xeng_internal.h"
 
 namespace xeng {
@@ -89,7 +90,8 @@ constexpr int kOChunks = kOBox / 16 / kOCT;   // 16-byte chunks of a tile per co
 static_assert(kOConvWarps == 8 || kOConvWarps == 16, "8 or 16 converter warps");
 static_assert(kOEpiWarps == 4 || kOEpiWarps == 8, "4 or 8 epilogue warps");
 constexpr uint32_t kOTmemCols = 512;
-constexpr int kOSums = 2 * 256 * 8;  // per item parity: (P, Q) of block I's inputs, then block J's
+constexpr int kOSumPar = sum_slot(256);  // entries per item parity
+constexpr int kOSums = 2 * kOSumPar * 8;  // per item parity: (P, Q) of block J's inputs, then block I's (sum_slot)
 // barriers: raw full and empty per slot, plane full and empty per stage; acc full
 // and empty per accumulator; drain; sums full and empty per parity
 constexpr int kOBars = 2 * kORaws + 2 * kOPlanes + 4 + 1 + 4;
@@ -157,7 +159,7 @@ __device__ __forceinline__ OnepassItem onepass_item(const OnepassArgs &a, int it
 template <bool kAdd>
 __global__ void __launch_bounds__(kOThreads, 1)
 correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
-                         const OnepassArgs a)
+                         const __grid_constant__ OnepassArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -167,7 +169,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
     const uint32_t raw0 = sbase + kOPlanes * kOPlaneBytes;
     const uint32_t sums_u = raw0 + kORaws * kORawBytes;
     const uint32_t bars = sums_u + kOSums;
-    int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][256] (P, Q)
+    int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][sum_slot] (P, Q)
     float2 *terms = reinterpret_cast<float2 *>(sums);                // in their place: the epilogue's offset terms
     auto plane = [&](int s) { return sbase + (uint32_t)(s * kOPlaneBytes); };
     auto slot = [&](int s) { return raw0 + (uint32_t)(s * kORawBytes); };
@@ -209,7 +211,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&raw_map) : "memory");
     }
-    for (int k = threadIdx.x; k < 2 * 256; k += kOThreads) sums[k] = make_int2(0, 0);
+    for (int k = threadIdx.x; k < 2 * kOSumPar; k += kOThreads) sums[k] = make_int2(0, 0);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kOTmemCols));
@@ -230,27 +232,28 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 const OnepassItem w = onepass_item(a, it);
                 const int f = a.f0 + w.fl;
                 const bool diag = w.I == w.J;
-                const int sJ = a.sub ? a.slot[w.J] : -1, sI = a.sub ? a.slot[w.I] : -1;  // substituted blocks
+                // where each block's tiles are: map, input, channel, first sample (a substituted
+                // block's in sub_map, whose channels and samples are the launch's)
+                const int sJ = a.sub ? a.slot[w.J] : -1, sI = a.sub ? a.slot[w.I] : -1;
+                const CUtensorMap *mJ = sJ >= 0 ? &sub_map : &raw_map, *mI = sI >= 0 ? &sub_map : &raw_map;
+                const int xJ = 128 * (sJ >= 0 ? sJ : w.J), xI = 128 * (sI >= 0 ? sI : w.I);
+                const int fJ = sJ >= 0 ? w.fl : f, fI = sI >= 0 ? w.fl : f;
+                int zJ = sJ >= 0 ? 0 : (int)a.t0, zI = sI >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < n_k; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
                         break;
                     }
-                    const CUtensorMap *mp = &raw_map;
-                    int z = (int)(a.t0 + (int64_t)kc * kOKc);
                     if (a.maps) {  // blocks of spb stages, each with its own map
-                        mp = a.maps + kc / a.spb;
-                        z = (kc % a.spb) * kOKc;
+                        mJ = mI = a.maps + kc / a.spb;
+                        zJ = zI = (kc % a.spb) * kOKc;
                     }
                     mbar_expect_tx(rawf(s), diag ? kOBox : kORawBytes);
                     // A: block J (TMEM lanes = inputs j), B: block I (columns = inputs i)
-                    // (sub_map's channels and samples are the launch's)
-                    if (sJ >= 0) tma_load_3d(slot(s), &sub_map, 128 * sJ, w.fl, kc * kOKc, rawf(s));
-                    else tma_load_3d(slot(s), mp, w.J * 128, f, z, rawf(s));
-                    if (!diag) {
-                        if (sI >= 0) tma_load_3d(slot(s) + kOBox, &sub_map, 128 * sI, w.fl, kc * kOKc, rawf(s));
-                        else tma_load_3d(slot(s) + kOBox, mp, w.I * 128, f, z, rawf(s));
-                    }
+                    tma_load_3d(slot(s), mJ, xJ, fJ, zJ, rawf(s));
+                    if (!diag) tma_load_3d(slot(s) + kOBox, mI, xI, fI, zI, rawf(s));
+                    zJ += kOKc;
+                    zI += kOKc;
                     ++issued;
                     if (++s == kORaws) {
                         s = 0;
@@ -436,7 +439,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 break;
             }
             if (active && (r0 & 3) == 0) {
-                int *sp = reinterpret_cast<int *>(sums + par * 256 + g * 128 + lc * 16);
+                int *sp = reinterpret_cast<int *>(sums + par * kOSumPar + sum_slot(g * 128 + lc * 16));
                 #pragma unroll
                 for (int m = 0; m < 16; m++) {
                     atomicAdd(sp + 2 * m, (int)P32[m]);
@@ -461,75 +464,91 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
         for (int it = it_begin; it < a.n_items; it += it_step, ++local) {
             const OnepassItem w = onepass_item(a, it);
             const int par = local & 1, ab = local & 1;  // sums buffer and accumulator
+            const int j_warp = w.J * 128 + q * 32;  // the warp's first input j (TMEM lanes: block J)
+            const int j = j_warp + lane;
+            const bool lane_ok = j < N;
+            const int ibase = w.I * 128;
+            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)w.fl * nb2;
+            // warp-uniform: columns inside the channel and up to some lane's diagonal
+            auto chunk_ok = [&](const int c) {
+                return j_warp < N && c < 128 && ibase + c < N && ibase + c <= j_warp + 31;
+            };
+            // the triangle's values of columns c .. c + 7 (adding launches)
+            auto load_old = [&](const int c, int2 (&o)[8]) {
+                const int i0 = ibase + c;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last) o[e] = __ldcg(out + off);
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            int2 old0[8], old1[8];  // of the warp's next two chunks
+            if (kAdd && it + it_step < a.n_items) {  // the next pair's values, to L2
+                const OnepassItem nx = onepass_item(a, it + it_step);
+                prefetch_triangle(reinterpret_cast<const int2 *>(a.acc) + (int64_t)nx.fl * nb2, N, nx.J * 128 + q * 32,
+                                  nx.I * 128 + 8 * half, nx.I * 128 + 128, 8 * kPerQuad, lane);
+            }
+            if (kAdd && chunk_ok(8 * half)) load_old(8 * half, old0);  // under the wait for the accumulator
+            if (kAdd && chunk_ok(8 * half + 8 * kPerQuad)) load_old(8 * half + 8 * kPerQuad, old1);
             bool ok = mbar_wait_backoff(accf(ab), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
             ok = ok && mbar_wait_backoff(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
             // the barrier ORs the eight warps' failures, so they leave together
             if (bar_any(2, kOEpiWarps * 32, !ok)) break;
             fence_after();
             // every input's offset terms in place of its sums (read by all the warps)
-            for (int k = et; k < 256; k += kOEpiWarps * 32) terms[par * 256 + k] = offset_terms(sums[par * 256 + k]);
+            for (int k = et; k < 256; k += kOEpiWarps * 32) {
+                const int m = par * kOSumPar + sum_slot(k);
+                terms[m] = offset_terms(sums[m]);
+            }
             named_bar_sync(2, kOEpiWarps * 32);
             const bool diag = w.I == w.J;
-            const int j_warp = w.J * 128 + q * 32;  // the warp's first input j (TMEM lanes: block J)
-            const int j = j_warp + lane;
-            const float2 *ci = terms + par * 256 + (diag ? 0 : 128);  // inputs i of the columns (block I)
+            const float2 *ci = terms + par * kOSumPar + (diag ? 0 : sum_slot(128));  // inputs i of the columns (block I)
             if (j_warp < N) {
-                const bool lane_ok = j < N;
-                const float2 tj = terms[par * 256 + row];
+                const float2 tj = terms[par * kOSumPar + sum_slot(row)];
                 const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
-                int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)w.fl * nb2;
                 const uint32_t tb = taddr + 256u * ab;
-                const int ibase = w.I * 128;
                 // Corrects the chunk of columns c..c+7 held in (vre, vim) in place and stores
                 // or adds it: pair (i, j) sits at i*N - i*(i-1)/2 + (j - i) in the channel's
                 // triangle and row i + 1 starts N - i - 1 pairs after row i, so per column
                 // the warp's 32 consecutive inputs j are one 256-byte run.
-                auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8], const int2 (&old)[8]) {
                     const int i0 = ibase + c;
                     #pragma unroll
                     for (int e = 0; e < 8; e += 2) {  // visibilities in place of the accumulator words
-                        const float4 t2 = *reinterpret_cast<const float4 *>(ci + c + e);  // the same for every lane
+                        const float4 t2 = *reinterpret_cast<const float4 *>(ci + sum_slot(c) + e);  // the same for every lane
                         // with A = x_j the Im half holds minus Im of x_i conj(x_j)
                         vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
                         vim[e] = raw_to_int(vim[e], -kRawScale, im_j + t2.y);
                         vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
                         vim[e + 1] = raw_to_int(vim[e + 1], -kRawScale, im_j + t2.w);
                     }
-                    const int off0 = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
-                    const int last = min(j - i0, N - 1 - i0);  // elements e <= last are pairs of the triangle
-                    if (kAdd) {
-                        int2 o[8];
-                        int off = off0;
-                        #pragma unroll
-                        for (int e = 0; e < 8; e++) {
-                            if (lane_ok && e <= last) o[e] = __ldcs(out + off);
-                            off += N - (i0 + e) - 1;
-                        }
-                        off = off0;
-                        #pragma unroll
-                        for (int e = 0; e < 8; e++) {
-                            if (lane_ok && e <= last) __stcs(out + off, make_int2(o[e].x + (int)vre[e], o[e].y + (int)vim[e]));
-                            off += N - (i0 + e) - 1;
-                        }
-                    } else {
-                        int off = off0;
-                        #pragma unroll
-                        for (int e = 0; e < 8; e++) {
-                            if (lane_ok && e <= last) __stcs(out + off, make_int2((int)vre[e], (int)vim[e]));
-                            off += N - (i0 + e) - 1;
-                        }
+                    const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;  // elements e <= last are pairs of the triangle
+                    int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                    #pragma unroll
+                    for (int e = 0; e < 8; e++) {
+                        if (e <= last)
+                            __stcs(out + off, kAdd ? make_int2(old[e].x + (int)vre[e], old[e].y + (int)vim[e])
+                                                   : make_int2((int)vre[e], (int)vim[e]));
+                        off += N - (i0 + e) - 1;
                     }
                 };
-                // warp-uniform: columns inside the channel and up to some lane's diagonal
-                auto chunk_ok = [&](const int c) { return c < 128 && ibase + c < N && ibase + c <= j_warp + 31; };
                 constexpr int kStep = 8 * kPerQuad;
-                if (kAdd) {  // adding to the triangle: one chunk at a time
-                    for (int c = 8 * half; chunk_ok(c); c += kStep) {
+                if (kAdd) {
+                    // adding to the triangle: two chunks' old values are in flight
+                    auto add_chunk = [&](const int c, int2 (&o)[8]) {
                         uint32_t vre[8], vim[8];
                         tmem_ld8(tb + c, vre);
                         tmem_ld8(tb + 128u + c, vim);
                         tmem_ld_wait();
-                        put_chunk(c, vre, vim);
+                        put_chunk(c, vre, vim, o);
+                        if (chunk_ok(c + 2 * kStep)) load_old(c + 2 * kStep, o);
+                    };
+                    for (int c = 8 * half; chunk_ok(c); c += 2 * kStep) {
+                        add_chunk(c, old0);
+                        if (!chunk_ok(c + kStep)) break;
+                        add_chunk(c + kStep, old1);
                     }
                 } else {
                     // two register sets: the next chunk's TMEM loads run under this chunk's stores
@@ -547,7 +566,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                             tmem_ld8(tb + c1, rb);
                             tmem_ld8(tb + 128u + c1, ib);
                         }
-                        put_chunk(c, ra, ia);
+                        put_chunk(c, ra, ia, old0);
                         tmem_ld_wait();
                         if (!ok1) break;
                         const int c2 = c1 + kStep;
@@ -556,7 +575,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                             tmem_ld8(tb + c2, ra);
                             tmem_ld8(tb + 128u + c2, ia);
                         }
-                        put_chunk(c1, rb, ib);
+                        put_chunk(c1, rb, ib, old0);
                         tmem_ld_wait();
                         c = c2;
                     }
@@ -566,7 +585,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
             // with this parity's sums: clear them for the item after next
             fence_before();
             named_bar_sync(2, kOEpiWarps * 32);
-            for (int k = et; k < 256; k += kOEpiWarps * 32) sums[par * 256 + k] = make_int2(0, 0);
+            for (int k = et; k < kOSumPar; k += kOEpiWarps * 32) sums[par * kOSumPar + k] = make_int2(0, 0);
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(acce(ab));

@@ -57,6 +57,7 @@
 
 #include "raw_offset.cuh"
 #include "tc_ptx.cuh"
+#include "triangle_add.cuh"
 #include "xeng_internal.h"
 
 namespace xeng {
@@ -182,7 +183,7 @@ __device__ __forceinline__ PairItem pair_item(const PairArgs &a, int it)
 template <bool kListed, bool kAdd>
 __global__ void __launch_bounds__(kPThreads, 1)
 correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
-                      const PairArgs a)
+                      const __grid_constant__ PairArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -259,30 +260,28 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                 const int nk = kListed ? a.jobs[w.job].n_k : n_k;
                 const bool diag = w.I2 == w.J2;
                 const int xa = w.J2 * 256 + (int)rank * 128, xb = w.I2 * 256 + (int)rank * 128;
-                // substituted blocks (a block past the inputs has no slot)
+                // where each tile's block is: map, input, channel, first sample (a substituted
+                // block's in sub_map, whose channels and samples are the launch's; a block past
+                // the inputs has no slot)
                 const int sa = !kListed && a.sub ? a.slot[xa >> 7] : -1, sb = !kListed && a.sub ? a.slot[xb >> 7] : -1;
+                const CUtensorMap *ma = sa >= 0 ? &sub_map : kListed ? a.jobs[w.job].map : &raw_map;
+                const CUtensorMap *mb = sb >= 0 ? &sub_map : kListed ? a.jobs[w.job].map : &raw_map;
+                const int fa = sa >= 0 ? w.fl : f, fb = sb >= 0 ? w.fl : f;
+                int za = kListed || sa >= 0 ? 0 : (int)a.t0, zb = kListed || sb >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < nk; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
                         break;
                     }
-                    const CUtensorMap *mp = &raw_map;
-                    int z = (int)(a.t0 + (int64_t)kc * kPKc);
-                    if (kListed) {  // the job's own map
-                        mp = a.jobs[w.job].map;
-                        z = kc * kPKc;
-                    } else if (a.maps) {  // blocks of spb stages, each with its own map
-                        mp = a.maps + kc / a.spb;
-                        z = (kc % a.spb) * kPKc;
+                    if (!kListed && a.maps) {  // blocks of spb stages, each with its own map
+                        ma = mb = a.maps + kc / a.spb;
+                        za = zb = (kc % a.spb) * kPKc;
                     }
                     mbar_expect_tx(rawf(s), diag ? kPBox : kPRawBytes);
-                    // (sub_map's channels and samples are the launch's)
-                    if (sa >= 0) tma_load_3d(slot(s), &sub_map, 128 * sa, w.fl, kc * kPKc, rawf(s));
-                    else tma_load_3d(slot(s), mp, xa, f, z, rawf(s));
-                    if (!diag) {
-                        if (sb >= 0) tma_load_3d(slot(s) + kPBox, &sub_map, 128 * sb, w.fl, kc * kPKc, rawf(s));
-                        else tma_load_3d(slot(s) + kPBox, mp, xb, f, z, rawf(s));
-                    }
+                    tma_load_3d(slot(s), ma, sa >= 0 ? 128 * sa : xa, fa, za, rawf(s));
+                    if (!diag) tma_load_3d(slot(s) + kPBox, mb, sb >= 0 ? 128 * sb : xb, fb, zb, rawf(s));
+                    za += kPKc;
+                    zb += kPKc;
                     ++issued;
                     if (++s == kPRaws) {
                         s = 0;
@@ -532,23 +531,47 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
             const float n128 = 128.0f * (float)(kListed ? a.jobs[w.job].nt : (int)a.nt);  // 64 n from each of the two products
             int32_t *const acc = kListed ? a.jobs[w.job].acc : a.acc;
             const int par = local & 1;
+            const int j_warp = w.J2 * 256 + (int)rank * 128 + q * 32;  // the warp's first input j
+            const int j = j_warp + lane;
+            const bool lane_ok = j < N;
+            int2 *out = reinterpret_cast<int2 *>(acc) + (int64_t)w.fl * ((int64_t)N * (N + 1) / 2);
+            const int ibase = w.I2 * 256;
+            // warp-uniform: columns inside the channel and up to some lane's diagonal
+            auto chunk_ok = [&](const int c) {
+                return j_warp < N && c < 256 && ibase + c < N && ibase + c <= j_warp + 31;
+            };
+            // the triangle's values of columns c .. c + 7 (adding launches)
+            auto load_old = [&](const int c, int2 (&o)[8]) {
+                const int i0 = ibase + c;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last) o[e] = __ldcg(out + off);
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            int2 old0[8], old1[8];  // of the warp's next two chunks
+            if (kAdd && it + it_step < a.n_items) {  // the next pair's values, to L2
+                const PairItem nx = pair_item<kListed>(a, it + it_step);
+                prefetch_triangle(reinterpret_cast<const int2 *>(acc) + (int64_t)nx.fl * ((int64_t)N * (N + 1) / 2), N,
+                                  nx.J2 * 256 + (int)rank * 128 + q * 32, nx.I2 * 256 + cbeg, nx.I2 * 256 + 256,
+                                  8 * kPEpiPerQuad, lane);
+            }
+            if (kAdd && chunk_ok(cbeg)) load_old(cbeg, old0);  // under the wait for the accumulator
+            if (kAdd && chunk_ok(cbeg + 8 * kPEpiPerQuad)) load_old(cbeg + 8 * kPEpiPerQuad, old1);
             bool ok = mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
             ok = ok && mbar_wait_cluster(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue);
             // the barrier ORs the eight warps' failures, so they leave together
             if (bar_any(2, kPEpiWarps * 32, !ok)) break;
             ++uses;
             fence_after();
-            const int j_warp = w.J2 * 256 + (int)rank * 128 + q * 32;  // the warp's first input j
-            const int j = j_warp + lane;
-            const bool lane_ok = j < N;
-            int2 *out = reinterpret_cast<int2 *>(acc) + (int64_t)w.fl * ((int64_t)N * (N + 1) / 2);
             const float2 *sp = sums + par * 384;
             const float2 tj = sp[row];  // this lane's input j (A rows of this CTA)
             const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
             const float2 *ci = sp + 128;  // inputs i of the 256 columns
-            const int ibase = w.I2 * 256;
             // Corrects the chunk of columns c..c+7 held in (vre, vim) in place and stores it.
-            auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8], const bool add) {
+            auto put_chunk = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8], const int2 (&old)[8]) {
                 const int i0 = ibase + c;
                 #pragma unroll
                 for (int e = 0; e < 8; e += 2) {  // visibilities in place of the accumulator words
@@ -560,41 +583,31 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                 }
                 // pair (i, j) sits at i*N - i*(i-1)/2 + (j - i) in the channel's triangle;
                 // pair (i + 1, j) is N - i - 1 entries further on
-                const int off0 = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
-                const int last = min(j - i0, N - 1 - i0);  // elements e <= last are pairs of the triangle
-                if (add) {
-                    int2 o[8];
-                    int off = off0;
-                    #pragma unroll
-                    for (int e = 0; e < 8; e++) {
-                        if (lane_ok && e <= last) o[e] = __ldcs(out + off);
-                        off += N - (i0 + e) - 1;
-                    }
-                    off = off0;
-                    #pragma unroll
-                    for (int e = 0; e < 8; e++) {
-                        if (lane_ok && e <= last) __stcs(out + off, make_int2(o[e].x + (int)vre[e], o[e].y + (int)vim[e]));
-                        off += N - (i0 + e) - 1;
-                    }
-                } else {
-                    int off = off0;
-                    #pragma unroll
-                    for (int e = 0; e < 8; e++) {
-                        if (lane_ok && e <= last) __stcs(out + off, make_int2((int)vre[e], (int)vim[e]));
-                        off += N - (i0 + e) - 1;
-                    }
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;  // elements e <= last are pairs of the triangle
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last)
+                        __stcs(out + off, kAdd ? make_int2(old[e].x + (int)vre[e], old[e].y + (int)vim[e])
+                                               : make_int2((int)vre[e], (int)vim[e]));
+                    off += N - (i0 + e) - 1;
                 }
             };
-            // warp-uniform: columns inside the channel and up to some lane's diagonal
-            auto chunk_ok = [&](const int c) { return c < 256 && ibase + c < N && ibase + c <= j_warp + 31; };
             constexpr int kStep = 8 * kPEpiPerQuad;
-            if (kAdd && j_warp < N) {  // adding to the triangle: one chunk at a time
-                for (int c = cbeg; chunk_ok(c); c += kStep) {
+            if (kAdd) {
+                // adding to the triangle: two chunks' old values are in flight
+                auto add_chunk = [&](const int c, int2 (&o)[8]) {
                     uint32_t vre[8], vim[8];
                     tmem_ld8(taddr + c, vre);
                     tmem_ld8(taddr + 256 + c, vim);
                     tmem_ld_wait();
-                    put_chunk(c, vre, vim, true);
+                    put_chunk(c, vre, vim, o);
+                    if (chunk_ok(c + 2 * kStep)) load_old(c + 2 * kStep, o);
+                };
+                for (int c = cbeg; chunk_ok(c); c += 2 * kStep) {
+                    add_chunk(c, old0);
+                    if (!chunk_ok(c + kStep)) break;
+                    add_chunk(c + kStep, old1);
                 }
             } else if (j_warp < N) {
                 // two register sets: the next chunk's TMEM loads run under this chunk's stores
@@ -613,7 +626,7 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                         tmem_ld8(taddr + c1, rb);
                         tmem_ld8(taddr + 256 + c1, ib);
                     }
-                    put_chunk(c, ra, ia, false);
+                    put_chunk(c, ra, ia, old0);
                     tmem_ld_wait();
                     if (!ok1) break;
                     const int c2 = c1 + kStep;
@@ -622,7 +635,7 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                         tmem_ld8(taddr + c2, ra);
                         tmem_ld8(taddr + 256 + c2, ia);
                     }
-                    put_chunk(c1, rb, ib, false);
+                    put_chunk(c1, rb, ib, old0);
                     tmem_ld_wait();
                     c = c2;
                 }

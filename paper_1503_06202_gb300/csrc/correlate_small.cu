@@ -69,6 +69,7 @@
 #include <cstring>
 
 #include "tc_ptx.cuh"
+#include "triangle_add.cuh"
 #include "raw_offset.cuh"
 #include "xeng_internal.h"
 
@@ -101,7 +102,8 @@ constexpr int kSConvWarp0 = 2, kSConvWarps = 8;
 constexpr int kSEpiWarp0 = kSConvWarp0 + kSConvWarps, kSEpiWarps = 8;
 constexpr int kSThreads = 32 * (kSEpiWarp0 + kSEpiWarps);
 constexpr uint32_t kSTmemCols = 512;
-constexpr int kSSums = 2 * 256 * 8;  // per item parity: (P, Q) of the item's 256 inputs (X tile, then Y tile)
+constexpr int kSSumPar = sum_slot(256);  // entries per item parity
+constexpr int kSSums = 2 * kSSumPar * 8;  // per item parity: (P, Q) of the item's 256 inputs (X tile, then Y tile; sum_slot)
 // barriers: raw full and empty per slot, plane full and empty per stage; acc full,
 // acc empty, drain; sums full and empty per parity
 constexpr int kSBars = 2 * kSRaws + 2 * kSPlanes + 3 + 4;
@@ -232,7 +234,7 @@ __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
 template <bool kAdd, bool kShared>
 __global__ void __launch_bounds__(kSThreads, 1)
 correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
-                       const SmallArgs a)
+                       const __grid_constant__ SmallArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -242,7 +244,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
     const uint32_t raw0 = sbase + kSPlanes * kSPlaneBytes;
     const uint32_t sums_u = raw0 + kSRaws * kSRawBytes;
     const uint32_t bars = sums_u + kSSums;
-    int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][256] (P, Q)
+    int2 *sums = reinterpret_cast<int2 *>(sgen + (sums_u - sbase));  // [parity][sum_slot] (P, Q)
     float2 *terms = reinterpret_cast<float2 *>(sums);                // in their place: the epilogue's offset terms
     auto plane = [&](int s) { return sbase + (uint32_t)(s * kSPlaneBytes); };
     auto slot = [&](int s) { return raw0 + (uint32_t)(s * kSRawBytes); };
@@ -284,7 +286,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
         asm volatile("prefetch.tensormap [%0];" ::"l"(&raw_map) : "memory");
         *s_epoch = *(volatile int *)a.epoch + 1;
     }
-    for (int k = threadIdx.x; k < 2 * 256; k += kSThreads) sums[k] = make_int2(0, 0);
+    for (int k = threadIdx.x; k < 2 * kSSumPar; k += kSThreads) sums[k] = make_int2(0, 0);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kSTmemCols));
@@ -306,26 +308,28 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             while (ok && next_piece(a, x, hi, pc)) {
                 const SmallItem w = small_item(a, pc.it);
                 const int fX = a.f0 + w.fx, fY = a.f0 + (w.fy >= 0 ? w.fy : w.fx);
-                const int xY = w.col ? 128 : 0;
+                // where each tile's block is: map, input, channel, sample (block 0 of channel fx,
+                // and block 0 or 1 of fy; a substituted block's in sub_map, whose channels and
+                // samples are the launch's)
+                const int sX = a.sub ? a.slot[0] : -1, sY = a.sub ? a.slot[w.col ? 1 : 0] : -1;
+                const CUtensorMap *mX = sX >= 0 ? &sub_map : &raw_map, *mY = sY >= 0 ? &sub_map : &raw_map;
+                const int xX = sX >= 0 ? 128 * sX : 0, xY = sY >= 0 ? 128 * sY : w.col ? 128 : 0;
+                const int cX = sX >= 0 ? fX - a.f0 : fX, cY = sY >= 0 ? fY - a.f0 : fY;
+                int zX = (sX >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc, zY = (sY >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc;
                 for (int kc = pc.k0; kc < pc.k1; kc++) {
                     if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
                         ok = false;
                         break;
                     }
-                    const CUtensorMap *mp = &raw_map;
-                    int z = (int)(a.t0 + (int64_t)kc * kSKc);
                     if (a.maps) {  // blocks of spb stages, each with its own map
-                        mp = a.maps + kc / a.spb;
-                        z = (kc % a.spb) * kSKc;
+                        mX = mY = a.maps + kc / a.spb;
+                        zX = zY = (kc % a.spb) * kSKc;
                     }
                     mbar_expect_tx(rawf(s), kSRawBytes);
-                    // input block 0 of channel fx, and block 0 or 1 of fy; a substituted block
-                    // comes from its slot of sub_map, whose channels and samples are the launch's
-                    const int sX = a.sub ? a.slot[0] : -1, sY = a.sub ? a.slot[xY >> 7] : -1;
-                    if (sX >= 0) tma_load_3d(slot(s), &sub_map, 128 * sX, fX - a.f0, kc * kSKc, rawf(s));
-                    else tma_load_3d(slot(s), mp, 0, fX, z, rawf(s));
-                    if (sY >= 0) tma_load_3d(slot(s) + kSBox, &sub_map, 128 * sY, fY - a.f0, kc * kSKc, rawf(s));
-                    else tma_load_3d(slot(s) + kSBox, mp, xY, fY, z, rawf(s));
+                    tma_load_3d(slot(s), mX, xX, cX, zX, rawf(s));
+                    tma_load_3d(slot(s) + kSBox, mY, xY, cY, zY, rawf(s));
+                    zX += kSKc;
+                    zY += kSKc;
                     ++issued;
                     if (++s == kSRaws) {
                         s = 0;
@@ -533,7 +537,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                 break;
             }
             if ((r0 & 3) == 0) {
-                int *sp = reinterpret_cast<int *>(sums + par * 256 + g * 128 + lc * 16);
+                int *sp = reinterpret_cast<int *>(sums + par * kSSumPar + sum_slot(g * 128 + lc * 16));
                 #pragma unroll
                 for (int m = 0; m < 16; m++) {
                     atomicAdd(sp + 2 * m, (int)P32[m]);
@@ -573,6 +577,45 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             const int c_lo = kShared ? pc.it * a.split : (int)blockIdx.x + 1;
             const int c_hi = kShared ? c_lo + a.split - 1
                                     : owner && pc.k1 < a.n_k ? stage_cta(a, (pc.it + 1) * a.n_k - 1) : 0;
+            // Block h: column items' inputs j = 128.. against i = 128h..; diagonal items'
+            // channel fx or fy, both 0..127.  Sums: X tile at 0, Y tile at 128.
+            const int fl = w.col ? w.fx : (h ? w.fy : w.fx);
+            const int j_warp = (w.col ? 128 : 0) + q * 32;
+            const int j = j_warp + lane;
+            const int i_base = w.col ? 128 * h : 0;
+            const bool lane_ok = j < N;
+            const bool warp_ok = fl >= 0 && j_warp < N;
+            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
+            // warp-uniform: columns inside the channel and up to some lane's diagonal
+            auto chunk_ok = [&](const int c) { return c < 128 && i_base + c < N && i_base + c <= j_warp + 31; };
+            // the triangle's values of columns c .. c + 7 (adding launches): pair (i, j) sits
+            // at i*N - i*(i-1)/2 + (j - i) in the channel's triangle and row i + 1 starts
+            // N - i - 1 pairs after row i, so per column the warp's 32 consecutive inputs j
+            // are one 256-byte run
+            auto load_old = [&](const int c, int2 (&o)[8]) {
+                const int i0 = i_base + c;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last) o[e] = __ldcg(out + off);
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            int2 old[8];
+            if (kAdd && !kShared) {
+                int nx = x;
+                Piece np;
+                if (next_piece(a, nx, hi, np)) {  // the next item's values, to L2
+                    const SmallItem nw = small_item(a, np.it);
+                    const int nfl = nw.col ? nw.fx : (h ? nw.fy : nw.fx);
+                    if (nfl >= 0 && np.k0 == 0)
+                        prefetch_triangle(reinterpret_cast<const int2 *>(a.acc) + (int64_t)nfl * nb, N,
+                                          (nw.col ? 128 : 0) + q * 32, nw.col ? 128 * h : 0,
+                                          min(N, nw.col ? 128 * h + 128 : 128), 8, lane);
+                }
+                if (owner && warp_ok && chunk_ok(0)) load_old(0, old);  // under the wait for the accumulator
+            }
             bool ok = mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
             ok = ok && mbar_wait_backoff(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
             if (et == 0 && !kShared)
@@ -582,32 +625,24 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             ++uses;
             fence_after();
             // every input's offset terms in place of its sums (read by all the warps)
-            terms[par * 256 + et] = offset_terms(sums[par * 256 + et]);
+            {
+                const int m = par * kSSumPar + sum_slot(et);
+                terms[m] = offset_terms(sums[m]);
+            }
             named_bar_sync(2, kSEpiWarps * 32);
-            // Block h: column items' inputs j = 128.. against i = 128h..; diagonal items'
-            // channel fx or fy, both 0..127.  Sums: X tile at 0, Y tile at 128.
-            const int fl = w.col ? w.fx : (h ? w.fy : w.fx);
-            const int j_warp = (w.col ? 128 : 0) + q * 32;
-            const int j = j_warp + lane;
-            const int i_base = w.col ? 128 * h : 0;
-            const float2 *ci = terms + par * 256 + 128 * h;  // inputs i of the columns
-            const float2 tj = terms[par * 256 + (w.col ? 128 : 128 * h) + row];
+            const float2 *ci = terms + par * kSSumPar + sum_slot(128 * h);  // inputs i of the columns
+            const float2 tj = terms[par * kSSumPar + sum_slot((w.col ? 128 : 128 * h) + row)];
             const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
-            const bool lane_ok = j < N;
-            const bool warp_ok = fl >= 0 && j_warp < N;
-            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
             // TMEM columns of the block: column items Re at 128h.., Im at 256 + 128h..;
             // diagonal items Re at 256h.., Im (negated) at 256h + 128..
             const uint32_t tre = taddr + (w.col ? 128u * h : 256u * h);
             const uint32_t tim = tre + (w.col ? 256u : 128u);
             const float im_scale = w.col ? kRawScale : -kRawScale;
-            // warp-uniform: columns inside the channel and up to some lane's diagonal
-            auto chunk_ok = [&](const int c) { return c < 128 && i_base + c < N && i_base + c <= j_warp + 31; };
             // the piece's visibilities in place of the accumulator words of columns c .. c + 7
             auto correct = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
                 #pragma unroll
                 for (int e = 0; e < 8; e += 2) {
-                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + c + e);  // the same for every lane: a broadcast
+                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + sum_slot(c) + e);  // the same for every lane: a broadcast
                     vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
                     vim[e] = raw_to_int(vim[e], im_scale, im_j + t2.y);
                     vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
@@ -631,27 +666,15 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                     vim[e + 1] += (uint32_t)v.w;
                 }
             };
-            // Stores or adds columns c .. c + 7: pair (i, j) sits at i*N - i*(i-1)/2 + (j - i)
-            // in the channel's triangle and row i + 1 starts N - i - 1 pairs after row i, so
-            // per column the warp's 32 consecutive inputs j are one 256-byte run.
+            // Stores columns c .. c + 7, or adds them to the values in `old`.
             auto put_chunk = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
                 const int i0 = i_base + c;
-                const int off0 = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
-                const int last = min(j - i0, N - 1 - i0);  // elements e <= last are pairs of the triangle
-                int2 o[8];
-                if (kAdd) {
-                    int off = off0;
-                    #pragma unroll
-                    for (int e = 0; e < 8; e++) {
-                        if (lane_ok && e <= last) o[e] = __ldcs(out + off);
-                        off += N - (i0 + e) - 1;
-                    }
-                }
-                int off = off0;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;  // elements e <= last are pairs of the triangle
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
                 #pragma unroll
                 for (int e = 0; e < 8; e++) {
-                    if (lane_ok && e <= last)
-                        __stcs(out + off, kAdd ? make_int2(o[e].x + (int)vre[e], o[e].y + (int)vim[e])
+                    if (e <= last)
+                        __stcs(out + off, kAdd ? make_int2(old[e].x + (int)vre[e], old[e].y + (int)vim[e])
                                                : make_int2((int)vre[e], (int)vim[e]));
                     off += N - (i0 + e) - 1;
                 }
@@ -661,13 +684,21 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             // chunk's stores.
             auto for_chunks = [&](const int c0, const int step, auto &&fn) {
                 if (kAdd || kShared) {
+                    // adding: the next chunk's old values are loaded under this chunk's TMEM
+                    // loads and stores
                     for (int c = c0; warp_ok && chunk_ok(c); c += step) {
                         uint32_t vre[8], vim[8];
+                        int2 next[8];
                         tmem_ld8(tre + c, vre);
                         tmem_ld8(tim + c, vim);
+                        if (kAdd && !kShared && owner && chunk_ok(c + step)) load_old(c + step, next);
                         tmem_ld_wait();
                         correct(c, vre, vim);
                         fn(c, vre, vim);
+                        if (kAdd && !kShared) {
+                            #pragma unroll
+                            for (int e = 0; e < 8; e++) old[e] = next[e];
+                        }
                     }
                     return;
                 }
@@ -714,6 +745,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                 const int first = (part + a.split - 16 * h % a.split) % a.split;  // 16 h + first = part (mod split)
                 for_chunks(8 * first, 8 * a.split, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
                     if (!lane_ok) return;
+                    if (kAdd) load_old(c, old);
                     #pragma unroll 4
                     for (int p = 1; p < a.split; p++)
                         add_partial(c_lo + (part + p < a.split ? part + p : part + p - a.split), c, vre, vim);
@@ -735,7 +767,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             // the piece after next, then hand TMEM and the buffer back
             named_bar_sync(2, kSEpiWarps * 32);
             if (!owner && !kShared && et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
-            sums[par * 256 + et] = make_int2(0, 0);
+            for (int k = et; k < kSSumPar; k += kSEpiWarps * 32) sums[par * kSSumPar + k] = make_int2(0, 0);
             fence_before();
             __syncwarp();
             if (lane == 0) {

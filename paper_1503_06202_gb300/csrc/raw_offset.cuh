@@ -23,6 +23,12 @@ constexpr float kRawScale = 262144.0f;         // accumulators hold integer sums
 constexpr float kFloatToInt = 12582912.0f;     // M = 1.5 x 2^23
 constexpr uint32_t kFloatToIntBits = 0x4B400000u;
 
+// Where the sums of input k (and the terms in their place) of an item lie in
+// shared memory: two entries more after every 16 inputs, so that the eight lanes
+// of a converter warp that add the sums of inputs 16 l + m (l their lane's chunk)
+// hit eight banks and not one.
+__host__ __device__ constexpr int sum_slot(int k) { return k + 2 * (k >> 4); }
+
 // An input's terms (-8 S, 8 D) of its nibble sums (P, Q).
 __device__ __forceinline__ float2 offset_terms(int2 pq)
 {

@@ -541,8 +541,10 @@ bool launch_round(xserve_s *sv)
         for (int b0 = 0; b0 < sg.nblocks && e == cudaSuccess; b0 += per) {
             const int nb = std::min(per, sg.nblocks - b0);
             const int64_t nt = (int64_t)nb * st.block_samples;
-            e = launch_single_pass(sg.kernel, nullptr, nt, 0, nt, st.F, st.N, 0, st.F, st.acc,
-                                   (sg.store && b0 == 0) ? 0 : 1, &sv->small, sv->d_err, sv->num_sms, s,
+            const int accumulate = (sg.store && b0 == 0) ? 0 : 1;
+            const int k = sv->single_force ? sg.kernel
+                                           : single_pass_by_shape(sg.kernel, st.N, st.F, nt, accumulate, sv->num_sms);
+            e = launch_single_pass(k, nullptr, nt, 0, nt, st.F, st.N, 0, st.F, st.acc, accumulate, &sv->small, sv->d_err, sv->num_sms, s,
                                    sv->d_smaps[slot] + sg.map0 + b0, spb);
         }
     }

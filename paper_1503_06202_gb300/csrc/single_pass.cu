@@ -100,6 +100,36 @@ int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded,
     }
 }
 
+int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms)
+{
+    // Rounds of the grid times an item's time in ns, fitted to launches of 2 .. 256
+    // stages of 128 samples (GB300; us per item at 2 / 8 / 64 / 256 stages, storing:
+    // pair kernel 8.4 / 16.8 / 83.5 / 314, one pass 3.0 / 7.8 / 52 / 204, N <= 256
+    // kernel 7.9 / 14.9 / --; adding: 14.7 / -- / 87 / --, 5.3 / 9.3 / 55 / --,
+    // 14.9 / 24.8 / --).  At 64 stages and many rounds the first two are in the ratio
+    // of XENG_PAIR_COST and XENG_ONEPASS_COST.  A few rounds, and short launches,
+    // favour the one pass, whose items are the smallest and whose epilogue overlaps
+    // the next item (us a call, the N-only choice / the one pass: N = 1024 x 4
+    // channels x 32,768 samples 322 / 207; 512 x 256 x 256 100 / 65; 256 x 256 x 256
+    // 32 / 25); above about 1900 inputs and many channels its items take a quarter
+    // longer.
+    const int64_t n_k = (nt + 127) / 128;
+    auto rounds = [](int64_t items, int64_t units) { return (items + units - 1) / units; };
+    const int64_t b2 = (N + 255) / 256, b1 = (N + 127) / 128;
+    const int64_t ones = rounds(nf * (b1 * (b1 + 1) / 2), num_sms);
+    int64_t t_one = ones * (770 * n_k + (accumulate ? 3200 : 1600));
+    if (N > 1900 && ones > 8 && n_k > 32) t_one += t_one / 4;
+    if (kernel == kSingleSmall) {
+        // only against its whole items: it shares few items, and cuts long ones, evenly
+        const int64_t items = N > 128 ? nf + (nf + 1) / 2 : (nf + 1) / 2;
+        if (n_k >= 32 || 2 * items <= num_sms) return kernel;
+        return rounds(items, num_sms) * (1000 * n_k + (accumulate ? 13500 : 6000)) <= t_one ? kernel : kSingleOnepass;
+    }
+    if (kernel != kSinglePair && kernel != kSingleOnepass) return kernel;
+    const int64_t t_pair = rounds(nf * (b2 * (b2 + 1) / 2), num_sms / 2) * (1200 * n_k + (accumulate ? 12300 : 7400));
+    return t_pair < t_one ? kSinglePair : kSingleOnepass;
+}
+
 cudaError_t small_scratch_alloc(SmallScratch *sc, int num_sms, cudaStream_t s)
 {
     if (sc->ws) return cudaSuccess;

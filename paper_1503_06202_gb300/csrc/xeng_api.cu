@@ -257,10 +257,16 @@ int fused_kernel(const xeng_s *h, const uint8_t *block)
 
 bool fused_ok(const xeng_s *h, const uint8_t *block) { return fused_kernel(h, block) != 0; }
 
+// The kernel of one launch (XENG_FUSED_KERNEL's choice stands).
+int shaped(const xeng_s *h, int kernel, int64_t nf, int64_t nt, int accumulate)
+{
+    return h->fused_force ? kernel : single_pass_by_shape(kernel, h->N, nf, nt, accumulate, h->num_sms);
+}
+
 cudaError_t launch_fused(xeng_s *h, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                          int32_t f0, int32_t nf, int32_t *acc, int accumulate, cudaStream_t s)
 {
-    return launch_single_pass(fused_kernel(h, block), block, T_block, t0, nt, F, h->N, f0, nf, acc, accumulate,
+    return launch_single_pass(shaped(h, fused_kernel(h, block), nf, nt, accumulate), block, T_block, t0, nt, F, h->N, f0, nf, acc, accumulate,
                               &h->small, h->d_err, h->num_sms, s);
 }
 
@@ -568,9 +574,11 @@ cudaError_t integrate_packed(xeng_s *h, int kernel, const uint8_t *dblock, int32
             p.counts = counts ? counts + c0 * h->N : nullptr;
             e = timed_launch(h, 0, s, [&] { return launch_pack(p, h->num_sms, s); });
             if (e != cudaSuccess) break;
+            const int accumulate = fresh && t0 == 0 ? 0 : 1;
+            const int k = shaped(h, kernel, p.nf, p.nt, accumulate);
             e = timed_launch(h, 1, s, [&] {
-                return launch_single_pass(kernel, h->packed, p.nt, 0, p.nt, p.nf, h->N, 0, p.nf, target + c0 * nb2,
-                                          fresh && t0 == 0 ? 0 : 1, &h->small, h->d_err, h->num_sms, s, nullptr, 0,
+                return launch_single_pass(k, h->packed, p.nt, 0, p.nt, p.nf, h->N, 0, p.nf, target + c0 * nb2, accumulate,
+                                          &h->small, h->d_err, h->num_sms, s, nullptr, 0,
                                           p.pitch);
             });
         }
@@ -614,10 +622,11 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
             const int accumulate = fresh && t0 == 0 ? 0 : 1;
             e = timed_launch(h, 0, s, [&] { return launch_pack_shifted(p, sa, h->num_sms, s); });
             if (e != cudaSuccess) break;
+            const int k = shaped(h, kernel, p.nf, p.nt, accumulate);
             e = timed_launch(h, 1, s, [&] {
-                return direct ? launch_single_pass(kernel, dblock, n, t0, p.nt, F, N, p.f0, p.nf, target + f0 * nb2,
+                return direct ? launch_single_pass(k, dblock, n, t0, p.nt, F, N, p.f0, p.nf, target + f0 * nb2,
                                                    accumulate, &h->small, h->d_err, h->num_sms, s, nullptr, 0, 0, &sub)
-                              : launch_single_pass(kernel, h->packed, p.nt, 0, p.nt, p.nf, N, 0, p.nf,
+                              : launch_single_pass(k, h->packed, p.nt, 0, p.nt, p.nf, N, 0, p.nf,
                                                    target + f0 * nb2, accumulate, &h->small, h->d_err, h->num_sms, s,
                                                    nullptr, 0, p.pitch);
             });

@@ -250,6 +250,11 @@ enum SinglePass { kSingleNone = -1, kSingleSmall = 1, kSingleOnepass = 2, kSingl
 // kernel), "none" (no single pass for the default engine and batches), else 0.
 int single_pass_force_from_env();
 int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded, int32_t pitch = 0);
+// For one launch of nf channels x nt samples, storing or adding, whose kernel is
+// not forced: the kernel whose rounds of the grid take less time -- of the two over
+// block pairs, or (kernel = kSingleSmall) of that one and the one pass.  All three
+// read the same stages.
+int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);
 // Scratch of the N <= 256 kernel, allocated at its first launch (flags zeroed
 // on the stream) and owned by the caller.
 struct SmallScratch {
