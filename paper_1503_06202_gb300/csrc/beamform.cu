@@ -39,8 +39,9 @@
 //                 shared memory, splits it into E2M3 nibble codes and writes them,
 //                 real and imaginary parts interleaved along K, into the
 //                 group's TMEM slot with tcgen05.st
-//   warps 14..17  epilogue: TMEM -> int32 beams [T][F][B][2] in HBM
-//   warp 18       TMA producer of the raw tiles (128 samples x 128 inputs of one
+//   warps 14..21  epilogue: TMEM -> int32 beams [T][F][B][2] in HBM, two warps per
+//                 TMEM lane quadrant taking half the beams each
+//   warp 22       TMA producer of the raw tiles (128 samples x 128 inputs of one
 //                 channel, 128-byte swizzle) into a six-slot ring
 // Shared memory then carries only the weight slices; decoded planes written to
 // and read back from shared memory made the MMAs shared-memory bound at small
@@ -64,8 +65,9 @@ namespace {
 // used by one group only, in order, so its barriers never run two phases apart).
 constexpr int kGroups = 3;
 constexpr int kConvWarps = 4 * kGroups;              // warps 2 .. 13
-constexpr int kEpiWarp0 = 2 + kConvWarps;            // 4 epilogue warps (one per TMEM lane quadrant)
-constexpr int kRawProdWarp = kEpiWarp0 + 4;          // TMA producer of the raw tiles
+constexpr int kEpiWarp0 = 2 + kConvWarps;            // epilogue warps: two per TMEM lane quadrant
+constexpr int kEpiWarps = 8;
+constexpr int kRawProdWarp = kEpiWarp0 + kEpiWarps;  // TMA producer of the raw tiles
 constexpr int kBfThreads = 32 * (kRawProdWarp + 1);
 constexpr int kRawBytes = 128 * 128;                 // 128 samples x 128 inputs of one channel
 // Raw-tile ring slots asked for (a build parameter); each configuration takes
@@ -131,14 +133,14 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
                  : "memory");
 }
 
-__device__ __forceinline__ void bf_item(const BfArgs &a, int64_t it, int &f, int &tt)
+__device__ __forceinline__ void bf_item(const BfArgs &a, int it, int &f, int &tt)
 {
     if (a.f_fastest) {
-        f = (int)(it % a.F);
-        tt = (int)(it / a.F);
+        f = it % a.F;
+        tt = it / a.F;
     } else {
-        tt = (int)(it % a.n_tt);
-        f = (int)(it / a.n_tt);
+        tt = it % a.n_tt;
+        f = it / a.n_tt;
     }
 }
 
@@ -162,15 +164,12 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
     const uint32_t drain_bar = bars + 8u * (2 * C::kXS + 2 * C::kSW + 2 * C::kAcc);
     auto rawf = [&](int r) { return bars + 8u * (2 * C::kXS + 2 * C::kSW + 2 * C::kAcc + 1 + r); };       // tile landed
     auto rawe = [&](int r) { return bars + 8u * (2 * C::kXS + 2 * C::kSW + 2 * C::kAcc + 1 + C::kR + r); };  // tile read
-    // step n of this CTA belongs to group n % kGroups, which uses its slots in
-    // turn: slot (n / kGroups) % kSlots of the group, phase (n / kGroups / kSlots) & 1
-    auto xslot = [&](int64_t n) { return (int)(n % kGroups) * C::kSlots + (int)((n / kGroups) % C::kSlots); };
-    auto xphase = [&](int64_t n) { return (uint32_t)((n / kGroups / C::kSlots) & 1); };
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem_raw + (bars + 8u * C::kBars - raw));
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int *err = a.err;
-    const int64_t n_seq = ((a.n_items - blockIdx.x + gridDim.x - 1) / gridDim.x) * a.n_kc;
+    const int n_items = (int)a.n_items, it0 = (int)blockIdx.x, it_step = (int)gridDim.x;
+    const int n_seq = (n_items - it0 + it_step - 1) / it_step * a.n_kc;  // steps of this CTA
 
     if (threadIdx.x == 0) {
         for (int x = 0; x < C::kXS; x++) {
@@ -183,7 +182,7 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
         }
         for (int b = 0; b < C::kAcc; b++) {
             mbar_init(accf(b), 1);
-            mbar_init(acce(b), 128);
+            mbar_init(acce(b), 32 * kEpiWarps);
         }
         mbar_init(drain_bar, 1);
         for (int r = 0; r < C::kR; r++) {
@@ -210,7 +209,7 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             int s = 0, issued = 0;
             uint32_t ps = 0;
             bool ok = true;
-            for (int64_t it = blockIdx.x; ok && it < a.n_items; it += gridDim.x) {
+            for (int it = it0; ok && it < n_items; it += it_step) {
                 int f, tt;
                 bf_item(a, it, f, tt);
                 for (int k = 0; k < a.n_kc; k++) {
@@ -249,7 +248,7 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             int sw = 0, local = 0, c = 0;  // c = step index modulo the X slots
             uint32_t pw = 0, pxs = 0;
             bool ok = true;
-            for (int64_t it = blockIdx.x; ok && it < a.n_items; it += gridDim.x, ++local) {
+            for (int it = it0; ok && it < n_items; it += it_step, ++local) {
                 const int ab = C::kAcc == 2 ? (local & 1) : 0;
                 // the accumulator's earlier uses: local / kAcc (a counter array indexed by ab would live in local memory)
                 const uint32_t used = (uint32_t)(C::kAcc == 2 ? (local >> 1) : local);
@@ -299,12 +298,14 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
         const int q = warp & 3;  // TMEM lane quadrant this warp may access
         const int row = q * 32 + lane;
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + C::kXCol0;
-        for (int64_t n = g; n < n_seq; n += kGroups) {
-            const int r = (int)(n % C::kR);
-            const uint32_t pr = (uint32_t)((n / C::kR) & 1);
-            const int x = xslot(n);
+        // step n belongs to group n % kGroups, which uses its raw slots (g, g + kGroups,
+        // ...: step n's is n % kR) and its X slots in turn
+        int r = g, xk = 0;
+        uint32_t pr = 0, px = 0;
+        for (int n = g; n < n_seq; n += kGroups) {
+            const int x = g * C::kSlots + xk;
             const bool ok = mbar_wait_backoff(rawf(r), pr, err, kDevTimeoutProducer, XENG_CONV_SLEEP_NS) &&
-                            mbar_wait_backoff(xe(x), xphase(n) ^ 1u, err, kDevTimeoutProducer, XENG_CONV_SLEEP_NS);
+                            mbar_wait_backoff(xe(x), px ^ 1u, err, kDevTimeoutProducer, XENG_CONV_SLEEP_NS);
             if (!__all_sync(0xffffffffu, ok)) break;  // keep the warp converged for tcgen05.st
             fence_after();
             const uint8_t *rt = rgen + r * kRawBytes + row * 128;
@@ -330,24 +331,37 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             mbar_arrive(rawe(r));
             fence_before();
             mbar_arrive(xf(x));
+            r += kGroups;
+            if (r >= C::kR) {
+                r -= C::kR;
+                pr ^= 1u;
+            }
+            if (++xk == C::kSlots) {
+                xk = 0;
+                px ^= 1u;
+            }
         }
     } else if (warp < kRawProdWarp) {
-        // ---------------- epilogue (warps 14..17) ----------------
+        // ---------------- epilogue (warps 14..21) ----------------
         // The offset terms of an item's channel are loaded by the first
         // epilogue warp while the MMAs run and staged in shared memory (two
-        // items' worth, alternating), where the four warps read them as
-        // broadcasts; a barrier over the four warps publishes them and also
-        // ORs the warps' wait results, so that all four leave together.
+        // items' worth, alternating), where the eight warps read them as
+        // broadcasts; a barrier over the eight warps publishes them and also
+        // ORs the warps' wait results, so that all leave together.
         const int q = warp & 3;  // TMEM lane quadrant this warp may access
+        // this warp's beams [bb, bb + kMine): half of them, but all of four
+        constexpr int kMine = kBp >= 8 ? kBp / 2 : kBp;
+        const int bb = (warp - kEpiWarp0) >> 2 ? kBp / 2 : 0;
+        const bool idle = kBp < 8 && bb != 0;
         const int row = q * 32 + lane;
         const bool stager = warp == kEpiWarp0;
         // [2][kBp], 16-byte aligned for the paired loads (the barrier area ends 8 bytes off a 16-byte boundary
         // when the barrier count is odd)
         int2 *corr_s = reinterpret_cast<int2 *>(smem_raw + (((bars + 8u * C::kBars + 16 + 15) & ~15u) - raw));
-        constexpr int G = kBp < 16 ? kBp : 16;
+        constexpr int G = kMine < 16 ? kMine : 16;
         constexpr int kPer = (kBp + 31) / 32;  // offset terms per lane of the staging warp
         int local = 0;
-        for (int64_t it = blockIdx.x; it < a.n_items; it += gridDim.x, ++local) {
+        for (int it = it0; it < n_items; it += it_step, ++local) {
             int f, tt;
             bf_item(a, it, f, tt);
             const int ab = C::kAcc == 2 ? (local & 1) : 0;
@@ -374,18 +388,20 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             uint32_t any_fail;
             asm volatile(
                 "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
-                "bar.red.or.pred p, 1, 128, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                "bar.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                 : "=r"(any_fail)
-                : "r"(ok ? 0u : 1u)
+                : "r"(ok ? 0u : 1u), "n"(32 * kEpiWarps)
                 : "memory");
-            if (any_fail) break;  // all four warps, converged for tcgen05.ld
+            if (any_fail) break;  // all the warps, converged for tcgen05.ld
             fence_after();
             const int64_t t = (int64_t)tt * 128 + row;
             int2 *o = reinterpret_cast<int2 *>(a.out) + (t * a.F + f) * a.B;
             int4 *o4 = reinterpret_cast<int4 *>(o);  // two beams per store when B is even
             const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * C::kN);
             #pragma unroll
-            for (int b0 = 0; b0 < kBp; b0 += G) {
+            for (int bk = 0; bk < kMine; bk += G) {
+                if (idle) break;
+                const int b0 = bb + bk;
                 uint32_t hre[G], him[G], lre[G], lim[G];
                 #pragma unroll
                 for (int c = 0; c < G; c += 4) {
@@ -415,7 +431,16 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                         const uint32_t bli = __float_as_uint(__uint_as_float(lim[e]) + kMagic);
                         y[e] = make_int2((int)(16u * bhr + blr - (uint32_t)c.x), (int)(16u * bhi + bli - (uint32_t)c.y));
                     }
-                    if (a.vec16) {
+                    if (G >= 4 && a.vec == 2) {  // four beams, a 32-byte sector, per store
+                        #pragma unroll
+                        for (int e = 0; e + 3 < G; e += 4)
+                            if (b0 + e < a.B)
+                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                             ::"l"(o + b0 + e), "r"(y[e].x), "r"(y[e].y), "r"(y[e + 1].x),
+                                               "r"(y[e + 1].y), "r"(y[e + 2].x), "r"(y[e + 2].y), "r"(y[e + 3].x),
+                                               "r"(y[e + 3].y)
+                                             : "memory");
+                    } else if (a.vec) {
                         #pragma unroll
                         for (int e = 0; e < G; e += 2)
                             if (b0 + e < a.B) o4[(b0 + e) >> 1] = make_int4(y[e].x, y[e].y, y[e + 1].x, y[e + 1].y);
@@ -431,25 +456,33 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
         }
     } else if (lane == 0) {
         // ---------------- TMA producer: raw tiles (warp 18) ----------------
-        int issued = 0;
+        int r = 0, issued = 0;
+        uint32_t ph = 0;
         bool ok = true;
-        for (int64_t n = 0; n < n_seq; n++) {
-            const int r = (int)(n % C::kR);
-            if (!mbar_wait(rawe(r), (uint32_t)((n / C::kR) & 1) ^ 1u, err, kDevTimeoutProducer)) {
-                ok = false;
-                break;
-            }
-            const int64_t it = blockIdx.x + (n / a.n_kc) * (int64_t)gridDim.x;
+        for (int it = it0; ok && it < n_items; it += it_step) {
             int f, tt;
             bf_item(a, it, f, tt);
-            mbar_expect_tx(rawf(r), kRawBytes);
-            tma_load_3d(rbase + r * kRawBytes, &raw_map, (int)(n % a.n_kc) * 128, f, tt * 128, rawf(r));
-            ++issued;
+            for (int k = 0; k < a.n_kc; k++) {
+                if (!mbar_wait(rawe(r), ph ^ 1u, err, kDevTimeoutProducer)) {
+                    ok = false;
+                    break;
+                }
+                mbar_expect_tx(rawf(r), kRawBytes);
+                tma_load_3d(rbase + r * kRawBytes, &raw_map, k * 128, f, tt * 128, rawf(r));
+                ++issued;
+                if (++r == C::kR) {
+                    r = 0;
+                    ph ^= 1u;
+                }
+            }
         }
         if (!ok) {
             // Let the copies already issued land before the CTA can exit.
-            for (int64_t n = issued - 1; n >= 0 && n >= issued - C::kR; n--)
-                (void)mbar_wait(rawf((int)(n % C::kR)), (uint32_t)((n / C::kR) & 1), err, kDevTimeoutProducer);
+            for (int k = 1; k <= C::kR && k <= issued; k++) {
+                int q = r - k, p = (int)ph;
+                if (q < 0) { q += C::kR; p ^= 1; }
+                (void)mbar_wait(rawf(q), (uint32_t)p, err, kDevTimeoutProducer);
+            }
         }
     }
 
@@ -618,7 +651,9 @@ cudaError_t launch_beamform(const uint8_t *block, const uint8_t *wdev, const int
     // needs every channel's weights in L2, else one channel at a time
     a.f_fastest = ((int64_t)a.F * 8 * bp * n_pad <= ((int64_t)48 << 20)) ? 1 : 0;
     a.block = block;
-    a.vec16 = (a.B % 2 == 0 && (reinterpret_cast<uintptr_t>(a.out) & 15) == 0) ? 1 : 0;
+    const uintptr_t oa = reinterpret_cast<uintptr_t>(a.out);
+    a.vec = a.B % 4 == 0 && (oa & 31) == 0 ? 2 : a.B % 2 == 0 && (oa & 15) == 0 ? 1 : 0;
+    if (a.n_items > 2147483647LL) return cudaErrorInvalidValue;  // more than the device's memory could hold
     const int grid = (int)(a.n_items < num_sms ? a.n_items : num_sms);
     switch (bp) {
         case 4: return launch_bf<4>(rm, wm, a, grid, s);
