@@ -240,32 +240,31 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
-            // Per step: two waits, eight MMAs, two commits; the bookkeeping is
-            // kept to a few integer operations since each step carries little
-            // tensor work (N = 4 Bp).
-            int sw = 0, local = 0, c = 0;  // c = step index modulo the X slots
-            uint32_t pw = 0, pxs = 0;
-            bool ok = true;
-            for (int it = it0; ok && it < n_items; it += it_step, ++local) {
-                const int ab = C::kAcc == 2 ? (local & 1) : 0;
-                // the accumulator's earlier uses: local / kAcc (a counter array indexed by ab would live in local memory)
-                const uint32_t used = (uint32_t)(C::kAcc == 2 ? (local >> 1) : local);
-                if (!mbar_wait_backoff(acce(ab), (used & 1u) ^ 1u, err, kDevTimeoutMma, 0)) break;
+        // ---------------- MMA issuer (the whole warp, one elected lane issuing) ----------------
+        // Per step: two waits, eight MMAs, two commits; the bookkeeping is
+        // kept to a few integer operations since each step carries little
+        // tensor work (N = 4 Bp).
+        int sw = 0, local = 0, c = 0;  // c = step index modulo the X slots
+        uint32_t pw = 0, pxs = 0;
+        bool ok = true;
+        for (int it = it0; ok && it < n_items; it += it_step, ++local) {
+            const int ab = C::kAcc == 2 ? (local & 1) : 0;
+            // the accumulator's earlier uses: local / kAcc (a counter array indexed by ab would live in local memory)
+            const uint32_t used = (uint32_t)(C::kAcc == 2 ? (local >> 1) : local);
+            ok = __all_sync(0xffffffffu, mbar_wait_backoff(acce(ab), (used & 1u) ^ 1u, err, kDevTimeoutMma, 0));
+            if (!ok) break;
+            fence_after();
+            const uint32_t d = tmem + (uint32_t)(ab * C::kN);
+            for (int k = 0; k < a.n_kc; k++) {
+                const int x = (c % kGroups) * C::kSlots + c / kGroups;
+                ok = __all_sync(0xffffffffu, mbar_wait_backoff(wf(sw), pw, err, kDevTimeoutMma, 0) &&
+                                                 mbar_wait_backoff(xf(x), pxs, err, kDevTimeoutMma, 0));
+                if (!ok) break;
                 fence_after();
-                const uint32_t d = tmem + (uint32_t)(ab * C::kN);
-                for (int k = 0; k < a.n_kc; k++) {
-                    const int x = (c % kGroups) * C::kSlots + c / kGroups;
-                    if (!mbar_wait_backoff(wf(sw), pw, err, kDevTimeoutMma, 0) ||
-                        !mbar_wait_backoff(xf(x), pxs, err, kDevTimeoutMma, 0)) {
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t xs = tmem + C::kXCol0 + (uint32_t)x * kXCols;
-                    const uint32_t w0 = wbase + sw * C::kWStageBytes;
-                    const uint64_t b0 = bf_desc(w0), b1 = bf_desc(w0 + C::kWBytes);
+                const uint32_t xs = tmem + C::kXCol0 + (uint32_t)x * kXCols;
+                const uint32_t w0 = wbase + sw * C::kWStageBytes;
+                const uint64_t b0 = bf_desc(w0), b1 = bf_desc(w0 + C::kWBytes);
+                if (elect_one()) {
                     #pragma unroll
                     for (int kk = 0; kk < 8; kk++) {  // +32 bytes along K = +2 in the descriptor's address field
                         const uint64_t bk = (kk < 4 ? b0 : b1) + 2 * (kk & 3);
@@ -273,22 +272,22 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                     }
                     mma_commit(xe(x));
                     mma_commit(we(sw));
-                    if (++sw == C::kSW) {
-                        sw = 0;
-                        pw ^= 1u;
-                    }
-                    if (++c == C::kXS) {
-                        c = 0;
-                        pxs ^= 1u;
-                    }
                 }
-                if (!ok) break;
-                mma_commit(accf(ab));
+                if (++sw == C::kSW) {
+                    sw = 0;
+                    pw ^= 1u;
+                }
+                if (++c == C::kXS) {
+                    c = 0;
+                    pxs ^= 1u;
+                }
             }
-            // Drain: every MMA issued above has finished once this completes.
-            mma_commit(drain_bar);
-            (void)mbar_wait(drain_bar, 0u, err, kDevTimeoutMma);
+            if (!ok) break;
+            if (elect_one()) mma_commit(accf(ab));
         }
+        // Drain: every MMA issued above has finished once this completes.
+        if (elect_one()) mma_commit(drain_bar);
+        (void)mbar_wait(drain_bar, 0u, err, kDevTimeoutMma);
     } else if (warp < kEpiWarp0) {
         // ---------------- converters: raw tile (smem) -> E2M3 nibble codes in TMEM ----------------
         // Thread = one sample row of a step (its TMEM lane): the row's 128

@@ -190,6 +190,17 @@ __device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap *map, int x, i
                  : "memory");
 }
 
+// True for one lane of a converged warp.  A warp that stays converged around its
+// MMAs keeps their descriptors in uniform registers, which the instruction
+// takes; from one lane of a divergent branch each operand is moved there first
+// (GB300, beamformer: about 56 cycles an MMA).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // ---- clusters of two CTAs (cta_group::2 pair MMAs) ----
 __device__ __forceinline__ uint32_t cluster_rank()
 {
