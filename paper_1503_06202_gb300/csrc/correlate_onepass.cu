@@ -271,8 +271,8 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
+        {
+            // ---------------- MMA issuer (the whole warp, one elected lane issuing) ----------------
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -282,39 +282,41 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 const bool diag = w.I == w.J;
                 // accumulator ab = local % 2, used for the (local / 2)-th time
                 const int ab = local & 1;
-                if (!mbar_wait(acce(ab), (uint32_t)((local >> 1) & 1) ^ 1u, err, kDevTimeoutMma)) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(acce(ab), (uint32_t)((local >> 1) & 1) ^ 1u, err, kDevTimeoutMma)))
+                    break;
                 fence_after();
                 const uint32_t d = tmem + 256u * ab;
                 for (int kc = 0; kc < n_k; kc++) {
-                    if (!mbar_try_wait(full(s), ph) && !mbar_wait(full(s), ph, err, kDevTimeoutMma)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(full(s), ph) ||
+                                                     mbar_wait(full(s), ph, err, kDevTimeoutMma));
+                    if (!ok) break;
                     fence_after();
                     const uint32_t st = plane(s);
                     // A: block J (Im plane, Re kOBox on); B: block I, or J itself on the diagonal
                     const uint64_t da_im = odesc(st), da_re = odesc(st + kOBox);
                     const uint64_t db_im = diag ? da_im : odesc(st + 2 * kOBox);
                     const uint64_t db_re = diag ? da_re : odesc(st + 3 * kOBox);
-                    #pragma unroll
-                    for (int kk = 0; kk < kOKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
-                        const uint32_t acc = (kc != 0 || kk != 0) ? 1u : 0u;
-                        const uint64_t k4 = 256u * kk;
-                        mma_f8(d, da_im + k4, db_im + k4, op_idesc(256, false), acc);
-                        mma_f8(d, da_re + k4, db_re + k4, op_idesc(128, false), 1u);
-                        mma_f8(d + 128u, da_re + k4, db_im + k4, op_idesc(128, true), 1u);
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int kk = 0; kk < kOKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
+                            const uint32_t acc = (kc != 0 || kk != 0) ? 1u : 0u;
+                            const uint64_t k4 = 256u * kk;
+                            mma_f8(d, da_im + k4, db_im + k4, op_idesc(256, false), acc);
+                            mma_f8(d, da_re + k4, db_re + k4, op_idesc(128, false), 1u);
+                            mma_f8(d + 128u, da_re + k4, db_im + k4, op_idesc(128, true), 1u);
+                        }
+                        mma_commit(empty(s));
                     }
-                    mma_commit(empty(s));
                     if (++s == kOPlanes) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
                 if (!ok) break;
-                mma_commit(accf(ab));
+                if (elect_one()) mma_commit(accf(ab));
             }
             // Drain: every MMA issued above has finished once this completes.
-            mma_commit(drain);
+            if (elect_one()) mma_commit(drain);
             (void)mbar_wait(drain, 0u, err, kDevTimeoutMma);
         }
     } else if (warp < kOEpiWarp0) {

@@ -299,8 +299,8 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
-            // ---------------- MMA issuer (leader CTA) ----------------
+        if (leader) {
+            // ---------------- MMA issuer (leader CTA: the whole warp, one elected lane issuing) ----------------
             int s = 0;
             uint32_t ph = 0, uses = 0;
             bool ok = true;
@@ -309,39 +309,40 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                 const PairItem w = pair_item<kListed>(a, it);
                 const bool diag = w.I2 == w.J2;
                 const int nk = kListed ? a.jobs[w.job].n_k : n_k;
-                if (!mbar_wait(acce, (uses & 1u) ^ 1u, err, kDevTimeoutMma)) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(acce, (uses & 1u) ^ 1u, err, kDevTimeoutMma))) break;
                 ++uses;
                 fence_after();
                 for (int kc = 0; kc < nk; kc++) {
-                    if (!mbar_try_wait(full(s), ph) && !mbar_wait_cluster(full(s), ph, err, kDevTimeoutMma)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(full(s), ph) ||
+                                                     mbar_wait_cluster(full(s), ph, err, kDevTimeoutMma));
+                    if (!ok) break;
                     fence_after();
                     const uint32_t st = plane(s);
                     const uint64_t dai = pdesc(st), dar = pdesc(st + kPBox);
                     const uint64_t dbi = diag ? dai : pdesc(st + 2 * kPBox);
                     const uint64_t dbr = diag ? dar : pdesc(st + 3 * kPBox);
-                    #pragma unroll
-                    for (int kk = 0; kk < kPKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
-                        const uint32_t acc = (kc != 0 || kk != 0) ? 1u : 0u;
-                        const uint64_t k4 = 256u * kk;
-                        mma_f8_cg2(d_re, dar + k4, dbr + k4, pair_idesc(false), acc);
-                        mma_f8_cg2(d_re, dai + k4, dbi + k4, pair_idesc(false), 1u);
-                        mma_f8_cg2(d_im, dar + k4, dbi + k4, pair_idesc(false), acc);
-                        mma_f8_cg2(d_im, dai + k4, dbr + k4, pair_idesc(true), 1u);
+                    if (elect_one()) {
+                        #pragma unroll
+                        for (int kk = 0; kk < kPKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
+                            const uint32_t acc = (kc != 0 || kk != 0) ? 1u : 0u;
+                            const uint64_t k4 = 256u * kk;
+                            mma_f8_cg2(d_re, dar + k4, dbr + k4, pair_idesc(false), acc);
+                            mma_f8_cg2(d_re, dai + k4, dbi + k4, pair_idesc(false), 1u);
+                            mma_f8_cg2(d_im, dar + k4, dbi + k4, pair_idesc(false), acc);
+                            mma_f8_cg2(d_im, dai + k4, dbr + k4, pair_idesc(true), 1u);
+                        }
+                        mma_commit_cg2(empty(s), kBoth);
                     }
-                    mma_commit_cg2(empty(s), kBoth);
                     if (++s == kPPlanes) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
                 if (!ok) break;
-                mma_commit_cg2(accf, kBoth);
+                if (elect_one()) mma_commit_cg2(accf, kBoth);
             }
             // Drain: every MMA issued above has finished once this completes.
-            mma_commit_cg2(drain, 0x1);
+            if (elect_one()) mma_commit_cg2(drain, 0x1);
             (void)mbar_wait(drain, 0u, err, kDevTimeoutMma);
         }
     } else if (warp < kPEpiWarp0) {

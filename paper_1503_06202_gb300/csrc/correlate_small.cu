@@ -347,8 +347,8 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer ----------------
+        {
+            // ---------------- MMA issuer (the whole warp, one elected lane issuing) ----------------
             int s = 0;
             uint32_t ph = 0, uses = 0;
             bool ok = true;
@@ -356,62 +356,63 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             Piece pc;
             while (ok && next_piece(a, x, hi, pc)) {
                 const SmallItem w = small_item(a, pc.it);
-                if (!mbar_wait(acce, (uses & 1u) ^ 1u, err, kDevTimeoutMma)) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(acce, (uses & 1u) ^ 1u, err, kDevTimeoutMma))) break;
                 ++uses;
                 fence_after();
                 for (int kc = pc.k0; kc < pc.k1; kc++) {
-                    if (!mbar_try_wait(full(s), ph) && !mbar_wait(full(s), ph, err, kDevTimeoutMma)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(full(s), ph) ||
+                                                     mbar_wait(full(s), ph, err, kDevTimeoutMma));
+                    if (!ok) break;
                     fence_after();
                     const uint32_t st = plane(s);
-                    if (w.col) {
-                        // A = Y rows (TMEM lanes: inputs j), B = X and Y columns (inputs i; the
-                        // Y plane kSBox after the X plane): Re in columns 0..255, Im in 256..511
-                        const uint64_t dre = sdesc(st + 2 * kSBox, kSBox), dim = sdesc(st, kSBox);
-                        const uint64_t are = sdesc(st + 3 * kSBox, kSBox), aim = sdesc(st + kSBox, kSBox);
-                        #pragma unroll
-                        for (int kk = 0; kk < kSKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
-                            const uint32_t acc = (kc != pc.k0 || kk != 0) ? 1u : 0u;
-                            const uint64_t k4 = 256u * kk;
-                            mma_f8(tmem, are + k4, dre + k4, small_idesc(256, false), acc);
-                            mma_f8(tmem, aim + k4, dim + k4, small_idesc(256, false), 1u);
-                            mma_f8(tmem + 256u, are + k4, dim + k4, small_idesc(256, false), acc);
-                            mma_f8(tmem + 256u, aim + k4, dre + k4, small_idesc(256, true), 1u);
-                        }
-                    } else {
-                        // each tile against itself, in columns 256h..: one N = 256 MMA of
-                        // A_im against [B_im | B_re] (Re_h 16 KB after Im_h) gives
-                        // [Im Im^T | Im Re^T]; A_re B_re^T completes Re, and (-A_re) B_im^T
-                        // makes the second half Im Re^T - Re Im^T, minus Im of x_i conj(x_j) with
-                        // A = x_j.  (Four N = 128 MMAs per tile instead ran at about 72% of the
-                        // tensor rate.)
-                        #pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            const uint64_t dim = sdesc(st + h * kSBox, 2 * kSBox), dre = sdesc(st + (2 + h) * kSBox, 2 * kSBox);
-                            const uint32_t d = tmem + 256u * h;
+                    if (elect_one()) {
+                        if (w.col) {
+                            // A = Y rows (TMEM lanes: inputs j), B = X and Y columns (inputs i; the
+                            // Y plane kSBox after the X plane): Re in columns 0..255, Im in 256..511
+                            const uint64_t dre = sdesc(st + 2 * kSBox, kSBox), dim = sdesc(st, kSBox);
+                            const uint64_t are = sdesc(st + 3 * kSBox, kSBox), aim = sdesc(st + kSBox, kSBox);
                             #pragma unroll
-                            for (int kk = 0; kk < kSKc / 32; kk++) {
+                            for (int kk = 0; kk < kSKc / 32; kk++) {  // +32 samples = +4 KB = +256 in the address field
                                 const uint32_t acc = (kc != pc.k0 || kk != 0) ? 1u : 0u;
                                 const uint64_t k4 = 256u * kk;
-                                mma_f8(d, dim + k4, dim + k4, small_idesc(256, false), acc);
-                                mma_f8(d, dre + k4, dre + k4, small_idesc(128, false), 1u);
-                                mma_f8(d + 128u, dre + k4, dim + k4, small_idesc(128, true), 1u);
+                                mma_f8(tmem, are + k4, dre + k4, small_idesc(256, false), acc);
+                                mma_f8(tmem, aim + k4, dim + k4, small_idesc(256, false), 1u);
+                                mma_f8(tmem + 256u, are + k4, dim + k4, small_idesc(256, false), acc);
+                                mma_f8(tmem + 256u, aim + k4, dre + k4, small_idesc(256, true), 1u);
+                            }
+                        } else {
+                            // each tile against itself, in columns 256h..: one N = 256 MMA of
+                            // A_im against [B_im | B_re] (Re_h 16 KB after Im_h) gives
+                            // [Im Im^T | Im Re^T]; A_re B_re^T completes Re, and (-A_re) B_im^T
+                            // makes the second half Im Re^T - Re Im^T, minus Im of x_i conj(x_j) with
+                            // A = x_j.  (Four N = 128 MMAs per tile instead ran at about 72% of the
+                            // tensor rate.)
+                            #pragma unroll
+                            for (int h = 0; h < 2; h++) {
+                                const uint64_t dim = sdesc(st + h * kSBox, 2 * kSBox), dre = sdesc(st + (2 + h) * kSBox, 2 * kSBox);
+                                const uint32_t d = tmem + 256u * h;
+                                #pragma unroll
+                                for (int kk = 0; kk < kSKc / 32; kk++) {
+                                    const uint32_t acc = (kc != pc.k0 || kk != 0) ? 1u : 0u;
+                                    const uint64_t k4 = 256u * kk;
+                                    mma_f8(d, dim + k4, dim + k4, small_idesc(256, false), acc);
+                                    mma_f8(d, dre + k4, dre + k4, small_idesc(128, false), 1u);
+                                    mma_f8(d + 128u, dre + k4, dim + k4, small_idesc(128, true), 1u);
+                                }
                             }
                         }
+                        mma_commit(empty(s));
                     }
-                    mma_commit(empty(s));
                     if (++s == kSPlanes) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
                 if (!ok) break;
-                mma_commit(accf);
+                if (elect_one()) mma_commit(accf);
             }
             // Drain: every MMA issued above has finished once this completes.
-            mma_commit(drain);
+            if (elect_one()) mma_commit(drain);
             (void)mbar_wait(drain, 0u, err, kDevTimeoutMma);
         }
     } else if (warp < kSEpiWarp0) {
