@@ -223,8 +223,8 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer ----------------
+        {
+            // ---------------- TMA producer (the whole warp, one elected lane issuing) ----------------
             int s = 0, issued = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -240,18 +240,19 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 const int fJ = sJ >= 0 ? w.fl : f, fI = sI >= 0 ? w.fl : f;
                 int zJ = sJ >= 0 ? 0 : (int)a.t0, zI = sI >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < n_k; kc++) {
-                    if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
+                                                     mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer));
+                    if (!ok) break;
                     if (a.maps) {  // blocks of spb stages, each with its own map
                         mJ = mI = a.maps + kc / a.spb;
                         zJ = zI = (kc % a.spb) * kOKc;
                     }
-                    mbar_expect_tx(rawf(s), diag ? kOBox : kORawBytes);
-                    // A: block J (TMEM lanes = inputs j), B: block I (columns = inputs i)
-                    tma_load_3d(slot(s), mJ, xJ, fJ, zJ, rawf(s));
-                    if (!diag) tma_load_3d(slot(s) + kOBox, mI, xI, fI, zI, rawf(s));
+                    if (elect_one()) {
+                        mbar_expect_tx(rawf(s), diag ? kOBox : kORawBytes);
+                        // A: block J (TMEM lanes = inputs j), B: block I (columns = inputs i)
+                        tma_load_3d(slot(s), mJ, xJ, fJ, zJ, rawf(s));
+                        if (!diag) tma_load_3d(slot(s) + kOBox, mI, xI, fI, zI, rawf(s));
+                    }
                     zJ += kOKc;
                     zI += kOKc;
                     ++issued;

@@ -249,8 +249,8 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer (both CTAs: each its own tiles) ----------------
+        {
+            // ---------------- TMA producer (both CTAs, each its own tiles; one elected lane issuing) ----------------
             int s = 0, issued = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -269,17 +269,18 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                 const int fa = sa >= 0 ? w.fl : f, fb = sb >= 0 ? w.fl : f;
                 int za = kListed || sa >= 0 ? 0 : (int)a.t0, zb = kListed || sb >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < nk; kc++) {
-                    if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
+                                                     mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer));
+                    if (!ok) break;
                     if (!kListed && a.maps) {  // blocks of spb stages, each with its own map
                         ma = mb = a.maps + kc / a.spb;
                         za = zb = (kc % a.spb) * kPKc;
                     }
-                    mbar_expect_tx(rawf(s), diag ? kPBox : kPRawBytes);
-                    tma_load_3d(slot(s), ma, sa >= 0 ? 128 * sa : xa, fa, za, rawf(s));
-                    if (!diag) tma_load_3d(slot(s) + kPBox, mb, sb >= 0 ? 128 * sb : xb, fb, zb, rawf(s));
+                    if (elect_one()) {
+                        mbar_expect_tx(rawf(s), diag ? kPBox : kPRawBytes);
+                        tma_load_3d(slot(s), ma, sa >= 0 ? 128 * sa : xa, fa, za, rawf(s));
+                        if (!diag) tma_load_3d(slot(s) + kPBox, mb, sb >= 0 ? 128 * sb : xb, fb, zb, rawf(s));
+                    }
                     za += kPKc;
                     zb += kPKc;
                     ++issued;

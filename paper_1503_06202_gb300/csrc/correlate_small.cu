@@ -298,8 +298,8 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------- TMA producer ----------------
+        {
+            // ---------------- TMA producer (the whole warp, one elected lane issuing) ----------------
             int s = 0, issued = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -317,17 +317,18 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                 const int cX = sX >= 0 ? fX - a.f0 : fX, cY = sY >= 0 ? fY - a.f0 : fY;
                 int zX = (sX >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc, zY = (sY >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc;
                 for (int kc = pc.k0; kc < pc.k1; kc++) {
-                    if (!mbar_try_wait(rawe(s), ph ^ 1u) && !mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
+                                                     mbar_wait(rawe(s), ph ^ 1u, err, kDevTimeoutProducer));
+                    if (!ok) break;
                     if (a.maps) {  // blocks of spb stages, each with its own map
                         mX = mY = a.maps + kc / a.spb;
                         zX = zY = (kc % a.spb) * kSKc;
                     }
-                    mbar_expect_tx(rawf(s), kSRawBytes);
-                    tma_load_3d(slot(s), mX, xX, cX, zX, rawf(s));
-                    tma_load_3d(slot(s) + kSBox, mY, xY, cY, zY, rawf(s));
+                    if (elect_one()) {
+                        mbar_expect_tx(rawf(s), kSRawBytes);
+                        tma_load_3d(slot(s), mX, xX, cX, zX, rawf(s));
+                        tma_load_3d(slot(s) + kSBox, mY, xY, cY, zY, rawf(s));
+                    }
                     zX += kSKc;
                     zY += kSKc;
                     ++issued;
