@@ -233,8 +233,8 @@ __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
 // own epilogue (the adding one needs more registers).
 template <bool kAdd, bool kShared>
 __global__ void __launch_bounds__(kSThreads, 1)
-correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
-                       const __grid_constant__ SmallArgs a)
+correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap diag_map,
+                       const __grid_constant__ CUtensorMap sub_map, const __grid_constant__ SmallArgs a)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -312,7 +312,8 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                 // and block 0 or 1 of fy; a substituted block's in sub_map, whose channels and
                 // samples are the launch's)
                 const int sX = a.sub ? a.slot[0] : -1, sY = a.sub ? a.slot[w.col ? 1 : 0] : -1;
-                const CUtensorMap *mX = sX >= 0 ? &sub_map : &raw_map, *mY = sY >= 0 ? &sub_map : &raw_map;
+                const CUtensorMap *own = w.col ? &raw_map : &diag_map;
+                const CUtensorMap *mX = sX >= 0 ? &sub_map : own, *mY = sY >= 0 ? &sub_map : own;
                 const int xX = sX >= 0 ? 128 * sX : 0, xY = sY >= 0 ? 128 * sY : w.col ? 128 : 0;
                 const int cX = sX >= 0 ? fX - a.f0 : fX, cY = sY >= 0 ? fY - a.f0 : fY;
                 int zX = (sX >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc, zY = (sY >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc;
@@ -869,11 +870,16 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
                                       acc + (int64_t)half * N * (N + 1), accumulate, ws, flags, err, num_sms, s, maps,
                                       spb, pitch, nullptr);
     }
-    CUtensorMap map, sub_map;
+    CUtensorMap map, diag_map, sub_map;
     memset(&map, 0, sizeof map);  // not read with `maps`: the stages take the blocks' maps
+    memset(&diag_map, 0, sizeof diag_map);
     memset(&sub_map, 0, sizeof sub_map);
     if (!maps) {
         cudaError_t e0 = encode_raw_map(&map, block, T_block, F, N, pitch, kSKc);
+        // Above 128 inputs a diagonal item reads a channel's first 128 only: fetching
+        // 256 bytes there brings in the rest for nothing (GB300, full Pathfinder band,
+        // whose time the board's power sets: 3.25 ms, 3.15 without).
+        if (e0 == cudaSuccess) e0 = encode_raw_map(&diag_map, block, T_block, F, N, pitch, kSKc, N <= 128);
         if (e0 != cudaSuccess) return e0;
     }
     if (sub) {
@@ -920,7 +926,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, map, sub_map, a);
+    return cudaLaunchKernelEx(&cfg, kern, map, diag_map, sub_map, a);
 }
 
 }  // namespace xeng

@@ -172,7 +172,7 @@ cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block
 }
 
 cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N,
-                           int32_t pitch, int stage)
+                           int32_t pitch, int stage, bool wide)
 {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return cudaErrorNotSupported;
@@ -185,7 +185,8 @@ cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_blo
     cuuint64_t strides[2] = {p, p * F};
     cuuint32_t box[3] = {128, 1, (cuuint32_t)stage}, estr[3] = {1, 1, 1};
     if (enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)block, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            wide ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     return cudaSuccess;

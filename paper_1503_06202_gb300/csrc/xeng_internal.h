@@ -177,9 +177,10 @@ struct SubBlocks {
     int8_t slot[kMaxBlocks];
 };
 // The raw block's tensor map of their stages (3D: input, channel, sample; boxes of
-// 128 inputs x 1 channel x `stage` samples, 128-byte swizzle).
+// 128 inputs x 1 channel x `stage` samples, 128-byte swizzle).  `wide`: L2 fetches
+// 256 bytes for a miss, for launches that read the next 128 inputs too.
 cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_block, int32_t F, int32_t N,
-                           int32_t pitch, int stage);
+                           int32_t pitch, int stage, bool wide = true);
 
 // Decode fused into the correlation for N <= 256 (small_ok: pitch % 16 == 0, block
 // 16-byte aligned): samples t0 .. t0 + nt - 1 (nt <= kFusedMaxSamples) of the
