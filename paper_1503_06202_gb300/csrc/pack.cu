@@ -6,8 +6,8 @@
 //   gates and flags (paper Sec. IV-C-4, Sec. IV-A): the rows of one gate, in
 //   order, a flagged sample replaced by the byte 0x88 (value 0 + 0i) and the
 //   usable samples per (channel, input) counted;
-//   time shifts (Sec. IV-C-5): inputs read d samples late, from the block or,
-//   before it, from the history of the delayed inputs.
+//   time shifts (Sec. IV-C-5): the delayed inputs read d samples late from their
+//   history.
 // Decoding such blocks to planes instead moves a byte in and two out, and the
 // correlation reads those two (three times over, at 256 inputs); here it is a
 // byte in, a byte out, and a byte read by the kernel that splits nibbles in
@@ -24,45 +24,63 @@ constexpr int kPackSpan = 256;     // rows per thread at most (byte-lane counts 
 
 // The 16 bytes at p, any alignment, of which the first n are wanted (the rest
 // may come out as anything): only 16-byte words that hold a wanted byte are read.
-__device__ __forceinline__ uint4 load16(const uint8_t *p, int n)
+// Without branches, so that several rows' loads are in flight at once.
+struct Loaded16 {
+    uint4 lo, hi;
+    int a;
+};
+__device__ __forceinline__ Loaded16 load16(const uint8_t *p, int n)
 {
-    const int a = (int)(reinterpret_cast<uintptr_t>(p) & 15);
-    const uint4 *q = reinterpret_cast<const uint4 *>(p - a);
-    const uint4 lo = __ldg(q);
-    if (a == 0) return lo;
-    const uint4 hi = a + n > 16 ? __ldg(q + 1) : lo;
-    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    if (a & 8) {
-        #pragma unroll
-        for (int k = 0; k < 6; k++) w[k] = w[k + 2];
-    }
-    if (a & 4) {
-        #pragma unroll
-        for (int k = 0; k < 5; k++) w[k] = w[k + 1];
-    }
-    const int s = 8 * (a & 3);
+    Loaded16 l;
+    l.a = (int)(reinterpret_cast<uintptr_t>(p) & 15);
+    const uint4 *q = reinterpret_cast<const uint4 *>(p - l.a);
+    l.lo = __ldg(q);
+    l.hi = __ldg(q + (l.a + n > 16 ? 1 : 0));
+    return l;
+}
+
+__device__ __forceinline__ uint4 value16(const Loaded16 &l)
+{
+    uint32_t w[8] = {l.lo.x, l.lo.y, l.lo.z, l.lo.w, l.hi.x, l.hi.y, l.hi.z, l.hi.w};
+    #pragma unroll
+    for (int k = 0; k < 6; k++) w[k] = l.a & 8 ? w[k + 2] : w[k];
+    #pragma unroll
+    for (int k = 0; k < 5; k++) w[k] = l.a & 4 ? w[k + 1] : w[k];
+    const int s = 8 * (l.a & 3);
     return make_uint4(__funnelshift_r(w[0], w[1], s), __funnelshift_r(w[1], w[2], s),
                       __funnelshift_r(w[2], w[3], s), __funnelshift_r(w[3], w[4], s));
 }
 
+// Column `col` of a row's chunks: channel c, 16-byte chunk j of the packed row,
+// inputs ic .. of the block.
+__device__ __forceinline__ void pack_column(const PackArgs &a, int64_t col, int &c, int &j, int &ic)
+{
+    const int per = a.chunks ? a.n_chunks : a.pitch / 16;
+    c = (int)(col / per);
+    const int k = (int)(col - (int64_t)c * per);
+    j = a.chunks ? a.chunks[k].x : k;
+    ic = 16 * (a.chunks ? a.chunks[k].y : k);
+}
+
 // kAligned: every source chunk is 16-byte aligned.  Thread = (row of the block's
-// rows, chunk): chunk `col` of the [nf][pitch / 16] chunks of a sample.
+// rows, chunk of a sample).
 template <bool kAligned, bool kValid>
 __global__ void __launch_bounds__(kPackThreads)
-pack_kernel(const PackArgs a, int cols_per_block, int rows_per_block, int span)
+pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_block, int span)
 {
-    const int cpr = a.pitch / 16;
+    constexpr int kRows = !kAligned && kValid ? kPackRows / 2 : kPackRows;  // registers
     const int64_t col = (int64_t)blockIdx.x * cols_per_block + threadIdx.x % cols_per_block;
     const int rsub = threadIdx.x / cols_per_block;
-    if (col >= (int64_t)a.nf * cpr || rsub >= rows_per_block) return;
-    const int c = (int)(col / cpr), ic = (int)(col % cpr) * 16;
+    if (col >= cols || rsub >= rows_per_block) return;
+    int c, j, ic;
+    pack_column(a, col, c, j, ic);
     const int n = min(16, a.N - ic);
     const int64_t row_bytes = (int64_t)a.F * a.N;
     const int64_t off = (int64_t)(a.f0 + c) * a.N + ic;
     const int64_t out_row = (int64_t)a.nf * a.pitch;
     const int64_t first = (int64_t)blockIdx.y * span * rows_per_block + rsub;
     const int64_t last = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
-    uint8_t *out = a.out + col * 16;
+    uint8_t *out = a.out + (int64_t)c * a.pitch + j * 16;
     uint32_t acc[4] = {0, 0, 0, 0};                       // usable samples, a byte per input
     uint32_t acc16[8] = {0, 0, 0, 0, 0, 0, 0, 0};         // the same, 16-bit lanes
     int rows = 0, pending = 0;
@@ -75,24 +93,27 @@ pack_kernel(const PackArgs a, int cols_per_block, int rows_per_block, int span)
         }
         pending = 0;
     };
-    for (int64_t t = first; t < last; t += (int64_t)kPackRows * rows_per_block) {
-        uint4 x[kPackRows], v[kPackRows];
+    for (int64_t t = first; t < last; t += (int64_t)kRows * rows_per_block) {
+        Loaded16 x[kRows], v[kRows];
         #pragma unroll
-        for (int k = 0; k < kPackRows; k++) {
+        for (int k = 0; k < kRows; k++) {
             const int64_t tk = t + (int64_t)k * rows_per_block;
             if (tk >= last) break;
             const int64_t src = (a.idx ? (int64_t)__ldg(a.idx + tk) : a.t0 + tk) * row_bytes + off;
-            x[k] = kAligned ? __ldg(reinterpret_cast<const uint4 *>(a.block + src)) : load16(a.block + src, n);
-            if (kValid)
-                v[k] = kAligned ? __ldg(reinterpret_cast<const uint4 *>(a.valid + src)) : load16(a.valid + src, n);
+            if (kAligned) x[k].lo = __ldg(reinterpret_cast<const uint4 *>(a.block + src));
+            else x[k] = load16(a.block + src, n);
+            if (kValid && kAligned) v[k].lo = __ldg(reinterpret_cast<const uint4 *>(a.valid + src));
+            else if (kValid) v[k] = load16(a.valid + src, n);
         }
         #pragma unroll
-        for (int k = 0; k < kPackRows; k++) {
+        for (int k = 0; k < kRows; k++) {
             const int64_t tk = t + (int64_t)k * rows_per_block;
             if (tk >= last) break;
-            uint32_t w[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+            const uint4 xv = kAligned ? x[k].lo : value16(x[k]);
+            uint32_t w[4] = {xv.x, xv.y, xv.z, xv.w};
             if (kValid) {
-                const uint32_t vw[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+                const uint4 vv = kAligned ? v[k].lo : value16(v[k]);
+                const uint32_t vw[4] = {vv.x, vv.y, vv.z, vv.w};
                 #pragma unroll
                 for (int j = 0; j < 4; j++) {
                     const uint32_t z = __vcmpeq4(vw[j], 0u);  // 0xFF in each flagged byte
@@ -103,7 +124,7 @@ pack_kernel(const PackArgs a, int cols_per_block, int rows_per_block, int span)
             ++rows;
             *reinterpret_cast<uint4 *>(out + tk * out_row) = make_uint4(w[0], w[1], w[2], w[3]);
         }
-        if (kValid && (pending += kPackRows) > 240 - kPackRows) widen();
+        if (kValid && (pending += kRows) > 240 - kRows) widen();
     }
     if (!a.counts) return;
     if (kValid) widen();
@@ -115,63 +136,88 @@ pack_kernel(const PackArgs a, int cols_per_block, int rows_per_block, int span)
     }
 }
 
-// Shifted rows: chunk j of a row is the block's 16-input chunk a.chunks[j] (or j
-// where a.chunks is null).  A chunk without delayed inputs is copied, one whose
-// inputs share a delay is copied from that many samples earlier, others byte by
-// byte where an input is delayed.
+// The chunks that hold a delayed input: copied, with the delayed inputs' samples
+// from the history's ring, which holds the launch's too -- their rows are dense
+// there, so that reading them d samples back stays in L2, where the block's rows
+// do not.  Launched over these chunks alone: among plain ones they kept whole
+// warps waiting (N = 496 x 188 channels x 30,415 samples, 7 inputs delayed, 1.9 ms
+// for all chunks in one launch).
 __global__ void __launch_bounds__(kPackThreads)
-pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int cols_per_block, int rows_per_block, int span)
+pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols_per_block, int rows_per_block, int span)
 {
-    const int cpr = a.pitch / 16;
     const int64_t col = (int64_t)blockIdx.x * cols_per_block + threadIdx.x % cols_per_block;
     const int rsub = threadIdx.x / cols_per_block;
-    if (col >= (int64_t)a.nf * cpr || rsub >= rows_per_block) return;
-    const int c = (int)(col / cpr), j = (int)(col % cpr);
-    const int ic = (a.chunks ? a.chunks[j] : j) * 16;
-    if (ic >= a.N) return;  // past the inputs: never read
+    if (col >= cols || rsub >= rows_per_block) return;
+    int c, j, ic;
+    pack_column(a, col, c, j, ic);
     const int n = min(16, a.N - ic);
     const int64_t f = a.f0 + c;
+    const int64_t row_bytes = (int64_t)a.F * a.N, ring_bytes = (int64_t)a.F * sa.S;
+    const uint8_t *blk = a.block + a.t0 * row_bytes + f * a.N + ic;
     const int64_t out_row = (int64_t)a.nf * a.pitch;
     const int64_t first = (int64_t)blockIdx.y * span * rows_per_block + rsub;
     const int64_t last = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
-    const int cd = n == 16 ? sa.chunk_delay[ic >> 4] : -1;
-    uint32_t delayed = 0;  // inputs of a mixed chunk that are
-    if (cd < 0)
-        for (int m = 0; m < n; m++) delayed |= (sa.delay[ic + m] > 0 ? 1u : 0u) << m;
-    uint8_t *out = a.out + col * 16;
-    for (int64_t t = first; t < last; t += rows_per_block) {
-        const int64_t tt = a.t0 + t;  // sample of the block before the shift
-        uint32_t todo = cd > tt ? (1u << n) - 1u : delayed;  // a shared delay reaching before the block: byte by byte
-        const int64_t from = cd > 0 && cd <= tt ? tt - cd : tt;
-        const uint4 x = load16(a.block + (from * a.F + f) * a.N + ic, n);
-        uint32_t w[4] = {x.x, x.y, x.z, x.w};
-        while (todo) {
-            const int m = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int i = ic + m;
-            const int64_t src = tt - sa.delay[i];
-            const uint32_t byte = src >= 0 ? a.block[(src * a.F + f) * a.N + i]
-                                           : sa.hist[((sa.H + src) * a.F + f) * sa.S + sa.slot[i]];
-            #pragma unroll
-            for (int k = 0; k < 4; k++)
-                if (k == m >> 2) w[k] = (w[k] & ~(0xFFu << (8 * (m & 3)))) | (byte << (8 * (m & 3)));
+    int slot0 = -1;        // ring column of the chunk's first delayed input
+    uint32_t delayed = 0;  // its delayed inputs
+    for (int m = 0; m < n; m++)
+        if (sa.delay[ic + m] > 0) {
+            if (slot0 < 0) slot0 = sa.slot[ic + m];
+            delayed |= 1u << m;
         }
-        *reinterpret_cast<uint4 *>(out + t * out_row) = make_uint4(w[0], w[1], w[2], w[3]);
+    const uint8_t *ring = sa.hist + f * sa.S + slot0;
+    uint8_t *out = a.out + (int64_t)c * a.pitch + j * 16;
+    for (int64_t t = first; t < last; t += (int64_t)kPackRows * rows_per_block) {
+        Loaded16 x[kPackRows];
+        uint32_t w[kPackRows][4];
+        #pragma unroll
+        for (int k = 0; k < kPackRows; k++)
+            x[k] = load16(blk + min(t + (int64_t)k * rows_per_block, last - 1) * row_bytes, n);
+        #pragma unroll
+        for (int k = 0; k < kPackRows; k++) {
+            const uint4 xv = value16(x[k]);
+            w[k][0] = xv.x;
+            w[k][1] = xv.y;
+            w[k][2] = xv.z;
+            w[k][3] = xv.w;
+        }
+        int s = 0;
+        for (uint32_t todo = delayed; todo; todo &= todo - 1, ++s) {
+            const int m = __ffs(todo) - 1;
+            const int64_t d = sa.delay[ic + m];
+            const uint32_t byte = 0xFFu << (8 * (m & 3));
+            uint32_t b[kPackRows];
+            #pragma unroll
+            for (int k = 0; k < kPackRows; k++)
+                b[k] = 0x01010101u * __ldg(ring + sa.row(min(t + (int64_t)k * rows_per_block, last - 1) - d) * ring_bytes + s);
+            #pragma unroll
+            for (int k = 0; k < kPackRows; k++) {
+                #pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const uint32_t here = q == m >> 2 ? byte : 0u;
+                    w[k][q] = (w[k][q] & ~here) | (b[k] & here);
+                }
+            }
+        }
+        #pragma unroll
+        for (int k = 0; k < kPackRows; k++) {
+            const int64_t tk = t + (int64_t)k * rows_per_block;
+            if (tk >= last) break;
+            *reinterpret_cast<uint4 *>(out + tk * out_row) = make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]);
+        }
     }
 }
 
-// Blocks of 256 threads over the chunks of a row (all of them, or 256) and, where
-// a row is shorter, several rows; each thread walks at most kPackSpan rows, fewer
+// Blocks of 256 threads over the `cols` columns of a row (all of them, or 256) and,
+// where a row is shorter, several rows; each thread walks at most kPackSpan rows, fewer
 // where that would leave SMs without a few blocks each.
 struct PackGrid {
     dim3 grid;
     int cols, rows, span;
 };
 
-PackGrid pack_grid(const PackArgs &a, int num_sms)
+PackGrid pack_grid(const PackArgs &a, int64_t cols, int num_sms)
 {
     PackGrid g;
-    const int64_t cols = (int64_t)a.nf * (a.pitch / 16);
     g.cols = (int)(cols < kPackThreads ? cols : kPackThreads);
     g.rows = kPackThreads / g.cols;
     const int64_t bx = (cols + g.cols - 1) / g.cols;
@@ -192,23 +238,25 @@ bool pack_args_ok(const PackArgs &a)
 
 cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s)
 {
-    if (a.nf <= 0 || a.nt <= 0) return cudaSuccess;
-    if (!pack_args_ok(a) || a.pitch < a.N || a.chunks) return cudaErrorInvalidValue;
-    const PackGrid g = pack_grid(a, num_sms);
+    const int64_t cols = (int64_t)a.nf * (a.chunks ? a.n_chunks : a.pitch / 16);
+    if (cols <= 0 || a.nt <= 0) return cudaSuccess;
+    if (!pack_args_ok(a) || (!a.chunks && a.pitch < a.N)) return cudaErrorInvalidValue;
+    const PackGrid g = pack_grid(a, cols, num_sms);
     const bool aligned = a.N % 16 == 0 && (reinterpret_cast<uintptr_t>(a.block) & 15) == 0 &&
                          (reinterpret_cast<uintptr_t>(a.valid) & 15) == 0;
     auto kernel = a.valid ? (aligned ? pack_kernel<true, true> : pack_kernel<false, true>)
                           : (aligned ? pack_kernel<true, false> : pack_kernel<false, false>);
-    kernel<<<g.grid, kPackThreads, 0, s>>>(a, g.cols, g.rows, g.span);
+    kernel<<<g.grid, kPackThreads, 0, s>>>(a, cols, g.cols, g.rows, g.span);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_sms, cudaStream_t s)
 {
-    if (a.nf <= 0 || a.nt <= 0) return cudaSuccess;
-    if (!pack_args_ok(a) || (!a.chunks && a.pitch < a.N)) return cudaErrorInvalidValue;
-    const PackGrid g = pack_grid(a, num_sms);
-    pack_shifted_kernel<<<g.grid, kPackThreads, 0, s>>>(a, sa, g.cols, g.rows, g.span);
+    const int64_t cols = (int64_t)a.nf * a.n_chunks;
+    if (cols <= 0 || a.nt <= 0) return cudaSuccess;
+    if (!pack_args_ok(a) || !a.chunks) return cudaErrorInvalidValue;
+    const PackGrid g = pack_grid(a, cols, num_sms);
+    pack_shifted_kernel<<<g.grid, kPackThreads, 0, s>>>(a, sa, cols, g.cols, g.rows, g.span);
     return cudaGetLastError();
 }
 

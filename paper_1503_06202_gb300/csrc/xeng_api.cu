@@ -56,14 +56,16 @@ struct xeng_s {
     int64_t pstage_bytes = 0;
     int32_t *gidx = nullptr;       // sample indices of the gates of a gated call
     int64_t gidx_cap = 0;
-    // time shifting: delays, history of the delayed inputs (ping-pong), their list
+    // time shifting: delays, history of the delayed inputs (a ring of rows), their list
     bool shifted = false;
     int32_t *d_delay = nullptr, *d_slot = nullptr, *d_chunk_delay = nullptr, *d_shift_inputs = nullptr;
-    int32_t *d_shift_chunks = nullptr;  // 16-input chunks of the 128-input blocks that hold a delayed input
+    // 16-byte chunks of rearranged rows (PackArgs::chunks): of the 128-input blocks that hold a
+    // delayed input, and of whole rows; first 64-byte lines without, then those with a delayed input
+    int2 *d_shift_chunks = nullptr;
+    int32_t n_shift_chunks[4] = {0, 0, 0, 0};
     SubBlocks shift_blocks{};           // those blocks (n of them; `packed` is set per launch)
-    uint8_t *hist[2] = {nullptr, nullptr};
-    int hist_cur = 0;
-    int64_t hist_H = 0;
+    uint8_t *hist = nullptr;
+    int64_t hist_cap = 0, hist_head = 0;
     int32_t hist_S = 0;
     bool decode_tma = false;       // decode through the TMA pipeline where the block allows it
     int fused_force = 0;           // single_pass_kernel's force: XENG_FUSED_KERNEL at handle creation
@@ -123,14 +125,14 @@ void free_shift(xeng_s *h)
     cudaFree(h->d_chunk_delay);
     cudaFree(h->d_shift_inputs);
     cudaFree(h->d_shift_chunks);
-    cudaFree(h->hist[0]);
-    cudaFree(h->hist[1]);
-    h->d_delay = h->d_slot = h->d_chunk_delay = h->d_shift_inputs = h->d_shift_chunks = nullptr;
-    h->hist[0] = h->hist[1] = nullptr;
+    cudaFree(h->hist);
+    h->d_delay = h->d_slot = h->d_chunk_delay = h->d_shift_inputs = nullptr;
+    h->d_shift_chunks = nullptr;
+    h->hist = nullptr;
     h->shifted = false;
-    h->hist_H = 0;
+    h->hist_cap = 0;
     h->hist_S = 0;
-    h->hist_cur = 0;
+    h->hist_head = 0;
 }
 
 int cuda_status(cudaError_t e)
@@ -477,36 +479,47 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
     sub.packed = nullptr;
     sub.n = 0;
     std::fill(sub.slot, sub.slot + kMaxBlocks, (int8_t)-1);
-    std::vector<int32_t> chunks;
     for (int32_t i : inputs)
-        if (sub.slot[i / kTile] < 0) {
-            sub.slot[i / kTile] = (int8_t)sub.n++;
-            for (int32_t c = 0; c < kTile / 16; c++) chunks.push_back(i / kTile * (kTile / 16) + c);
+        if (sub.slot[i / kTile] < 0) sub.slot[i / kTile] = (int8_t)sub.n++;
+    std::vector<int2> chunks;
+    for (int list = 0; list < 4; list++) {
+        const size_t before = chunks.size();
+        for (int32_t c = 0; c * 16 < N; c++) {
+            const int8_t b = sub.slot[c * 16 / kTile];
+            if (list < 2 && b < 0) continue;
+            // the chunks of a 64-byte line go together: parts of it written by two launches
+            // are read back from HBM in between
+            bool has = false;
+            for (int32_t i = c / 4 * 64; i < std::min(N, c / 4 * 64 + 64); i++) has = has || delays[i] > 0;
+            if (has == (list % 2 == 1)) chunks.push_back(make_int2(list < 2 ? b * (kTile / 16) + c % (kTile / 16) : c, c));
         }
-    const int64_t hist_bytes = (int64_t)H * h->F * S;
+        h->n_shift_chunks[list] = (int32_t)(chunks.size() - before);
+    }
+    // the ring holds a round's samples besides the H before them
+    const int64_t cap = H + std::min<int64_t>(h->t_integ, kFusedMaxSamples);
+    const int64_t hist_bytes = cap * h->F * S;
     cudaError_t e = cudaMalloc(&h->d_delay, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_slot, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_chunk_delay, sizeof(int32_t) * chunk.size());
     if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_inputs, sizeof(int32_t) * S);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_chunks, sizeof(int32_t) * chunks.size());
+    if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_chunks, sizeof(int2) * chunks.size());
     if (e == cudaSuccess)
-        e = cudaMemcpy(h->d_shift_chunks, chunks.data(), sizeof(int32_t) * chunks.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&h->hist[0], (size_t)hist_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&h->hist[1], (size_t)hist_bytes);
+        e = cudaMemcpy(h->d_shift_chunks, chunks.data(), sizeof(int2) * chunks.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&h->hist, (size_t)hist_bytes);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_delay, delays, sizeof(int32_t) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_slot, slot.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_chunk_delay, chunk.data(), sizeof(int32_t) * chunk.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_shift_inputs, inputs.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(h->hist[0], 0x88, (size_t)hist_bytes);  // value 0 + 0i
+    if (e == cudaSuccess) e = cudaMemset(h->hist, 0x88, (size_t)hist_bytes);  // value 0 + 0i
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cudaGetLastError();
         free_shift(h);
         return e == cudaErrorMemoryAllocation ? XENG_ERR_NOMEM : XENG_ERR_CUDA;
     }
-    h->hist_H = H;
+    h->hist_cap = cap;
     h->hist_S = S;
     h->shift_blocks = sub;
     h->shifted = true;
@@ -586,9 +599,21 @@ cudaError_t integrate_packed(xeng_s *h, int kernel, const uint8_t *dblock, int32
     return e;
 }
 
+// Samples t0 .. t0 + n - 1 of the block into the history of the delayed inputs (the
+// last of them, where it holds no more).
+cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t t0, int64_t n, cudaStream_t s)
+{
+    const int64_t m = std::min(n, h->hist_cap);
+    cudaError_t e = launch_shift_history(h->hist, dblock, t0 + n - m, m, h->F, h->N, h->d_shift_inputs, h->hist_S,
+                                         h->hist_cap, h->hist_head, s);
+    if (e == cudaSuccess) h->hist_head = (h->hist_head + m) % h->hist_cap;
+    return e;
+}
+
 // The same with the handle's delays applied to samples 0 .. n - 1 of the block:
 // where TMA can address the block's rows only the 128-input blocks that hold a
-// delayed input are rearranged, else every input.
+// delayed input are rearranged, else every input.  Each round's samples enter the
+// history first.
 cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int64_t n, int32_t *target, bool fresh,
                               cudaStream_t s)
 {
@@ -600,27 +625,38 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
     sa.delay = h->d_delay;
     sa.slot = h->d_slot;
     sa.chunk_delay = h->d_chunk_delay;
-    sa.hist = h->hist[h->hist_cur];
-    sa.H = h->hist_H;
+    sa.hist = h->hist;
+    sa.cap = h->hist_cap;
     sa.S = h->hist_S;
     PackArgs p;
     p.block = dblock;
     p.F = F;
     p.N = N;
     p.out = h->packed;
-    p.chunks = direct ? h->d_shift_chunks : nullptr;
+    const int32_t *nc = h->n_shift_chunks + (direct ? 0 : 2);
+    const int2 *plain = h->d_shift_chunks + (direct ? 0 : h->n_shift_chunks[0] + h->n_shift_chunks[1]);
     p.pitch = direct ? h->shift_blocks.n * kTile : (int32_t)round_up(N, 16);
     SubBlocks sub = h->shift_blocks;
     sub.packed = h->packed;
     for (int64_t t0 = 0; t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
         p.nt = std::min<int64_t>(kFusedMaxSamples, n - t0);
         p.t0 = t0;
+        sa.head = h->hist_head;
+        e = advance_history(h, dblock, t0, p.nt, s);
         const int64_t group = std::min<int64_t>(65535, h->packed_bytes / (p.nt * p.pitch));
         for (int64_t f0 = 0; f0 < F && e == cudaSuccess; f0 += group) {
             p.f0 = (int32_t)f0;
             p.nf = (int32_t)std::min<int64_t>(group, F - f0);
             const int accumulate = fresh && t0 == 0 ? 0 : 1;
-            e = timed_launch(h, 0, s, [&] { return launch_pack_shifted(p, sa, h->num_sms, s); });
+            e = timed_launch(h, 0, s, [&] {
+                p.chunks = plain;
+                p.n_chunks = nc[0];
+                const cudaError_t e2 = launch_pack(p, h->num_sms, s);
+                if (e2 != cudaSuccess) return e2;
+                p.chunks = plain + nc[0];
+                p.n_chunks = nc[1];
+                return launch_pack_shifted(p, sa, h->num_sms, s);
+            });
             if (e != cudaSuccess) break;
             const int k = shaped(h, kernel, p.nf, p.nt, accumulate);
             e = timed_launch(h, 1, s, [&] {
@@ -632,15 +668,6 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
             });
         }
     }
-    return e;
-}
-
-// New history of the delayed inputs after n samples of the block.
-cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t n, cudaStream_t s)
-{
-    cudaError_t e = launch_shift_history(h->hist[h->hist_cur], dblock, n, h->F, h->N, h->d_shift_inputs, h->hist_S,
-                                         h->hist_H, h->hist[h->hist_cur ^ 1], s);
-    if (e == cudaSuccess) h->hist_cur ^= 1;
     return e;
 }
 
@@ -674,8 +701,7 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
         if (!apply_shift)
             return integrate_packed(h, kernel, dblock, (int32_t)F, 0, (int32_t)F, n_samples, nullptr, nullptr, nullptr,
                                     target, fresh, s);
-        e = integrate_shifted(h, kernel, dblock, n_samples, target, fresh, s);
-        return e == cudaSuccess ? advance_history(h, dblock, n_samples, s) : e;
+        return integrate_shifted(h, kernel, dblock, n_samples, target, fresh, s);
     }
     e = ensure_planes(h);
     for (int64_t t0 = 0; t0 < n_samples && e == cudaSuccess; t0 += h->chunk_t) {
@@ -691,8 +717,9 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
                 sa.delay = h->d_delay;
                 sa.slot = h->d_slot;
                 sa.chunk_delay = h->d_chunk_delay;
-                sa.hist = h->hist[h->hist_cur];
-                sa.H = h->hist_H;
+                sa.hist = h->hist;
+                sa.cap = h->hist_cap;
+                sa.head = h->hist_head;
                 sa.S = h->hist_S;
                 e = timed_launch(h, 0, s, [&] {
                     if (h->decode_tma && decode_tma_ok(src, (int32_t)N)) {
@@ -726,7 +753,7 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
             e = timed_launch(h, 1, s, [&] { return run_correlate(h, a, s); });
         }
     }
-    if (e == cudaSuccess && apply_shift) e = advance_history(h, dblock, n_samples, s);
+    if (e == cudaSuccess && apply_shift) e = advance_history(h, dblock, 0, n_samples, s);
     return e;
 }
 

@@ -90,11 +90,20 @@ inline int64_t decode_ctas(int64_t t_pad, int64_t n_pad, int64_t F) { return (t_
 // samples late; the samples before the block come from the history.
 struct ShiftArgs {
     const int32_t *delay = nullptr;        // [N] delay of input i, samples
-    const int32_t *slot = nullptr;         // [N] history column of input i (-1: not delayed)
+    const int32_t *slot = nullptr;         // [N] history column of input i (-1: not delayed), in the inputs' order
     const int32_t *chunk_delay = nullptr;  // [ceil(N/16)] delay shared by inputs 16c..16c+15, or -1
-    const uint8_t *hist = nullptr;         // [H][F][S] the H samples before the block, delayed inputs only
-    int64_t H = 0;
+    // [cap][F][S] samples of the delayed inputs, a ring of rows: sample 0 of the
+    // block (or of the launch, see launch_pack_shifted) belongs at row head, and
+    // every sample from max(delay) before it on is there
+    const uint8_t *hist = nullptr;
+    int64_t cap = 0, head = 0;
     int32_t S = 0;
+    // the ring's row of sample src, |src| <= cap
+    __host__ __device__ int64_t row(int64_t src) const
+    {
+        const int64_t r = head + src;
+        return r < 0 ? r + cap : r >= cap ? r - cap : r;
+    }
 };
 // Decode samples t0 .. t0 + nt - 1 of the block (T_block samples) with the
 // shift applied, channels f0 .. f0 + nf - 1, into planes as launch_decode.
@@ -138,19 +147,21 @@ cudaError_t launch_decode_tma_batch(const CUtensorMap *maps, const DecTmaJob *jo
 cudaError_t launch_shift_fixup(const uint8_t *block, int64_t t0, int64_t nt, int32_t F, int32_t N, int32_t f0,
                                int32_t nf, const ShiftArgs &sa, const int32_t *inputs, uint8_t *planes, int64_t t_pad,
                                int64_t n_pad, cudaStream_t s);
-// New history after a block of n samples: the last H samples of (old history,
-// block) for the S delayed inputs listed in `inputs`.
-cudaError_t launch_shift_history(const uint8_t *hist_old, const uint8_t *block, int64_t n, int32_t F, int32_t N,
-                                 const int32_t *inputs, int32_t S, int64_t H, uint8_t *hist_new, cudaStream_t s);
+// Samples t0 .. t0 + m - 1 of the block's S delayed inputs, listed in `inputs`,
+// into the ring's rows head, head + 1, ... (modulo cap; m <= cap).
+cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0, int64_t m, int32_t F, int32_t N,
+                                 const int32_t *inputs, int32_t S, int64_t cap, int64_t head, cudaStream_t s);
 
 // Raw samples rearranged into rows of `pitch` bytes (a multiple of 16) per
 // channel, out[nt][nf][pitch], for a single-pass launch: row t is the block's
 // sample t0 + t, or idx[t] where idx (device memory) is given; channels
 // f0 .. f0 + nf - 1.  launch_pack (pitch >= N) also replaces samples whose
 // `valid` byte is 0 by 0x88 and adds the usable samples to counts[nf][N]; both
-// may be null.  launch_pack_shifted applies the delays of `sa`; `chunks` (device
-// memory, pitch / 16 entries) names the 16-input chunks of the block that make
-// up a row, null all of them.  nt <= kMaxChunkSamples.
+// may be null.  `chunks` (device memory): only these 16-byte chunks of the rows, as
+// (position in the packed row, 16-input chunk of the block); null: chunk k is
+// chunk k.  launch_pack_shifted takes the chunks that hold delayed inputs and
+// applies the delays of `sa`, whose ring has to hold the launch's samples already
+// (head: row of sample t0).  nt <= kMaxChunkSamples.
 struct PackArgs {
     const uint8_t *block = nullptr;
     int64_t t0 = 0, nt = 0;
@@ -158,7 +169,8 @@ struct PackArgs {
     const int32_t *idx = nullptr;
     const uint8_t *valid = nullptr;
     int32_t *counts = nullptr;
-    const int32_t *chunks = nullptr;
+    const int2 *chunks = nullptr;
+    int32_t n_chunks = 0;
     int32_t pitch = 0;
     uint8_t *out = nullptr;
 };
