@@ -91,19 +91,25 @@ struct BfCfg {
     // step while the MMAs of the previous one run), else one
     static constexpr int kSlots = (kTmemCols - kXCol0) / (kGroups * kXCols) >= 2 ? 2 : 1;
     static_assert(kXCol0 + kGroups * kSlots * kXCols <= kTmemCols, "TMEM: accumulators + X slots");
+    // output staging: per epilogue warp 32 rows of kRowBytes, the beams it forms at once
+    static constexpr int kMine = kBp >= 8 ? kBp / 2 : kBp;       // beams of an epilogue warp: half, but all of four
+    static constexpr int kG = kMine < 16 ? kMine : 16;           // ... formed at once
+    static constexpr int kRowBytes = 8 * kG;
+    static constexpr int kOutBytes = kEpiWarps * 32 * kRowBytes;
     // raw ring: a multiple of the groups, so each slot has one user
-    static constexpr int kRFit = (232448 - 1024 - 512 - 2 * kBp * 8 - 2 * kWStageBytes) / kRawBytes / kGroups * kGroups;
+    static constexpr int kRFit =
+        (232448 - 1024 - 512 - 2 * kBp * 8 - kOutBytes - 2 * kWStageBytes) / kRawBytes / kGroups * kGroups;
     static constexpr int kRWant = XENG_BF_RAW_SLOTS / kGroups * kGroups;
     static constexpr int kR = kRWant < kRFit ? kRWant : kRFit;
     static_assert(kR >= kGroups, "raw ring needs a slot per converter group");
     static constexpr int kCorrBytes = 2 * kBp * 8;                // offset terms of two items, staged for the epilogue
-    static constexpr int kSWFit = (232448 - 1024 - 512 - kCorrBytes - kR * kRawBytes) / kWStageBytes;
+    static constexpr int kSWFit = (232448 - 1024 - 512 - kCorrBytes - kOutBytes - kR * kRawBytes) / kWStageBytes;
     static constexpr int kSW = kSWFit > 8 ? 8 : kSWFit;          // weight ring stages (L2 latency off the path)
     static_assert(kSW >= 2, "weight ring needs two stages");
     static constexpr int kXS = kGroups * kSlots;                 // X slots in all
     static constexpr int kBars = 2 * kR + 2 * kXS + 2 * kSW + 2 * kAcc + 1;
     static constexpr size_t kSmem =
-        1024 + (size_t)kR * kRawBytes + (size_t)kSW * kWStageBytes + kBars * 8 + 16 + 8 + kCorrBytes;
+        1024 + (size_t)kR * kRawBytes + kOutBytes + (size_t)kSW * kWStageBytes + kBars * 8 + 16 + 8 + kCorrBytes;
     // kind::f8f6f4, D f32, A and B E2M3 (type 3) K-major, N and M = 128
     static constexpr uint32_t kIdesc = (1u << 4) | (3u << 7) | (3u << 10) | ((uint32_t)(kN >> 3) << 17) |
                                        ((uint32_t)(128 >> 4) << 24);
@@ -146,14 +152,16 @@ __device__ __forceinline__ void bf_item(const BfArgs &a, int it, int &f, int &tt
 
 template <int kBp>
 __global__ void __launch_bounds__(kBfThreads, 1)
-beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap w_map, const BfArgs a)
+beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap w_map,
+                const __grid_constant__ CUtensorMap out_map, const __grid_constant__ BfArgs a)
 {
     using C = BfCfg<kBp>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t rbase = (raw + 1023u) & ~1023u;                  // raw ring
     const uint8_t *rgen = smem_raw + (rbase - raw);                 // generic view of it
-    const uint32_t wbase = rbase + C::kR * kRawBytes;                  // weight ring
+    const uint32_t obase = rbase + C::kR * kRawBytes;                  // output staging
+    const uint32_t wbase = obase + C::kOutBytes;                       // weight ring
     const uint32_t bars = wbase + C::kSW * C::kWStageBytes;
     auto xf = [&](int x) { return bars + 8u * x; };                           // X slot x written
     auto xe = [&](int x) { return bars + 8u * (C::kXS + x); };                // X slot x consumed
@@ -349,15 +357,19 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
         // ORs the warps' wait results, so that all leave together.
         const int q = warp & 3;  // TMEM lane quadrant this warp may access
         // this warp's beams [bb, bb + kMine): half of them, but all of four
-        constexpr int kMine = kBp >= 8 ? kBp / 2 : kBp;
+        constexpr int kMine = C::kMine;
+        // its staging rows; their 16-byte chunks swizzled as the output's map says (by the
+        // 128-byte lines of the tile: rows of 128, 64 or 32 bytes)
+        const uint32_t stage = obase + (uint32_t)((warp - kEpiWarp0) * 32 * C::kRowBytes);
+        uint8_t *const srow = smem_raw + (stage - raw) + lane * C::kRowBytes;
+        const int sw_row = C::kRowBytes == 128 ? lane & 7 : C::kRowBytes == 64 ? (lane >> 1) & 3 : (lane >> 2) & 1;
         const int bb = (warp - kEpiWarp0) >> 2 ? kBp / 2 : 0;
         const bool idle = kBp < 8 && bb != 0;
-        const int row = q * 32 + lane;
         const bool stager = warp == kEpiWarp0;
         // [2][kBp], 16-byte aligned for the paired loads (the barrier area ends 8 bytes off a 16-byte boundary
         // when the barrier count is odd)
         int2 *corr_s = reinterpret_cast<int2 *>(smem_raw + (((bars + 8u * C::kBars + 16 + 15) & ~15u) - raw));
-        constexpr int G = kMine < 16 ? kMine : 16;
+        constexpr int G = C::kG;
         constexpr int kPer = (kBp + 31) / 32;  // offset terms per lane of the staging warp
         int local = 0;
         for (int it = it0; it < n_items; it += it_step, ++local) {
@@ -393,9 +405,6 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                 : "memory");
             if (any_fail) break;  // all the warps, converged for tcgen05.ld
             fence_after();
-            const int64_t t = (int64_t)tt * 128 + row;
-            int2 *o = reinterpret_cast<int2 *>(a.out) + (t * a.F + f) * a.B;
-            int4 *o4 = reinterpret_cast<int4 *>(o);  // two beams per store when B is even
             const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * C::kN);
             #pragma unroll
             for (int bk = 0; bk < kMine; bk += G) {
@@ -410,7 +419,10 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                     tmem_ld4(ta + 3 * kBp + b0 + c, *reinterpret_cast<uint32_t(*)[4]>(lim + c));
                 }
                 tmem_ld_wait();
-                if (t < a.T) {
+                // the rows staged last time have been read
+                if (a.tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+                {
                     // An accumulator holds S / 64 for an integer |S| < 2^22; adding 1.5 * 2^17
                     // (ulp 2^-6) is exact and leaves S + kMagicBits in the sum's bit pattern,
                     // so y = 16 S_hi + S_lo - offset needs no float-to-int conversion.
@@ -430,29 +442,40 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                         const uint32_t bli = __float_as_uint(__uint_as_float(lim[e]) + kMagic);
                         y[e] = make_int2((int)(16u * bhr + blr - (uint32_t)c.x), (int)(16u * bhi + bli - (uint32_t)c.y));
                     }
-                    if (G >= 4 && a.vec == 2) {  // four beams, a 32-byte sector, per store
-                        #pragma unroll
-                        for (int e = 0; e + 3 < G; e += 4)
-                            if (b0 + e < a.B)
-                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                             ::"l"(o + b0 + e), "r"(y[e].x), "r"(y[e].y), "r"(y[e + 1].x),
-                                               "r"(y[e + 1].y), "r"(y[e + 2].x), "r"(y[e + 2].y), "r"(y[e + 3].x),
-                                               "r"(y[e + 3].y)
-                                             : "memory");
-                    } else if (a.vec) {
-                        #pragma unroll
-                        for (int e = 0; e < G; e += 2)
-                            if (b0 + e < a.B) o4[(b0 + e) >> 1] = make_int4(y[e].x, y[e].y, y[e + 1].x, y[e + 1].y);
+                    // Staged, then stored in whole runs of a row: a lane's own row is F * B beams
+                    // from the next lane's.  By TMA where rows are multiples of 16 bytes (B even);
+                    // rows past T and beams past B are clipped.
+                    #pragma unroll
+                    for (int e = 0; e < G; e += 2)
+                        *reinterpret_cast<int4 *>(srow + (((e >> 1) ^ sw_row) << 4)) =
+                            make_int4(y[e].x, y[e].y, y[e + 1].x, y[e + 1].y);
+                    const int64_t t_warp = (int64_t)tt * 128 + q * 32;
+                    if (a.tma_out) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0 && t_warp < a.T && b0 < a.B) {
+                            tma_store_3d(&out_map, 2 * b0, f, (int)t_warp, stage);
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
                     } else {
-                        #pragma unroll
-                        for (int e = 0; e < G; e++)
-                            if (b0 + e < a.B) o[b0 + e] = y[e];
+                        __syncwarp();
+                        const uint8_t *tile = srow - lane * C::kRowBytes;
+                        int2 *o = reinterpret_cast<int2 *>(a.out) + (t_warp * a.F + f) * a.B + b0;
+                        #pragma unroll 4
+                        for (int k = lane; k < 32 * G; k += 32) {
+                            const int r = k / G, e = k % G;
+                            const int sw = C::kRowBytes == 128 ? r & 7 : C::kRowBytes == 64 ? (r >> 1) & 3 : (r >> 2) & 1;
+                            if (b0 + e < a.B && t_warp + r < a.T)
+                                o[(int64_t)r * a.F * a.B + e] = *reinterpret_cast<const int2 *>(
+                                    tile + r * C::kRowBytes + (((e >> 1) ^ sw) << 4) + (e & 1) * 8);
+                        }
                     }
                 }
             }
             fence_before();
             mbar_arrive(acce(ab));
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // staging read, beams written
     } else if (lane == 0) {
         // ---------------- TMA producer: raw tiles (warp 18) ----------------
         int r = 0, issued = 0;
@@ -582,10 +605,26 @@ template <int kBp>
 cudaError_t launch_bf(const CUtensorMap &rm, const CUtensorMap &wm, const BfArgs &a, int grid, cudaStream_t s)
 {
     using C = BfCfg<kBp>;
+    CUtensorMap om;
+    memset(&om, 0, sizeof om);
+    if (a.tma_out) {
+        // beams as int32: dims (2 B, channel, sample), boxes of one warp's rows
+        cuuint64_t dims[3] = {(cuuint64_t)(2 * a.B), (cuuint64_t)a.F, (cuuint64_t)a.T};
+        cuuint64_t strides[2] = {(cuuint64_t)a.B * 8, (cuuint64_t)a.F * a.B * 8};
+        cuuint32_t box[3] = {(cuuint32_t)(2 * C::kG), 1, 32}, estr[3] = {1, 1, 1};
+        const CUtensorMapSwizzle sw = C::kRowBytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                                      : C::kRowBytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                           : CU_TENSOR_MAP_SWIZZLE_32B;
+        EncodeTiledFn enc = encode_tiled();
+        if (!enc) return cudaErrorNotSupported;
+        if (enc(&om, CU_TENSOR_MAP_DATA_TYPE_INT32, 3, a.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
     cudaError_t e = cudaFuncSetAttribute(beamform_kernel<kBp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)C::kSmem);
     if (e != cudaSuccess) return e;
-    beamform_kernel<kBp><<<grid, kBfThreads, C::kSmem, s>>>(rm, wm, a);
+    beamform_kernel<kBp><<<grid, kBfThreads, C::kSmem, s>>>(rm, wm, om, a);
     return cudaGetLastError();
 }
 
@@ -651,7 +690,7 @@ cudaError_t launch_beamform(const uint8_t *block, const uint8_t *wdev, const int
     a.f_fastest = ((int64_t)a.F * 8 * bp * n_pad <= ((int64_t)48 << 20)) ? 1 : 0;
     a.block = block;
     const uintptr_t oa = reinterpret_cast<uintptr_t>(a.out);
-    a.vec = a.B % 4 == 0 && (oa & 31) == 0 ? 2 : a.B % 2 == 0 && (oa & 15) == 0 ? 1 : 0;
+    a.tma_out = a.B % 2 == 0 && (oa & 15) == 0 ? 1 : 0;  // TMA rows are 16-byte multiples
     if (a.n_items > 2147483647LL) return cudaErrorInvalidValue;  // more than the device's memory could hold
     const int grid = (int)(a.n_items < num_sms ? a.n_items : num_sms);
     switch (bp) {
