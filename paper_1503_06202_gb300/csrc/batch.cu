@@ -68,6 +68,7 @@ struct xeng_batch_s {
     int n_sjobs = 0;
     int64_t sum_entries = 0;
     std::vector<std::pair<int, int>> single;  // (job, single-pass kernel) in job order
+    std::vector<int64_t> packed;                // per job: offset in planes of its rearranged samples, or -1
     std::vector<char> listed;                   // per job: in the pair kernel's listed launch
     PairJob *d_pjobs = nullptr;                 // that launch's jobs and their maps
     CUtensorMap *d_pmaps = nullptr;
@@ -88,6 +89,12 @@ struct xeng_batch_s {
 };
 
 namespace {
+
+// From this many bytes on, a job whose rows TMA cannot address is rearranged
+// (pack.cu) and takes a single-pass kernel: two launches of its own, 15 us, where
+// decoding it with the others costs it about 1 us per MB more (GB300, N = 203 x 64
+// channels x 10007 samples, 130 MB: 146 us against 269).
+constexpr int64_t kBatchPackBytes = (int64_t)16 << 20;
 
 int status_of(cudaError_t e)
 {
@@ -153,6 +160,21 @@ cudaError_t enqueue_run(xeng_batch_s *b, cudaStream_t s)
             const xeng_job_t &jb = b->jobs[jk.first];
             for (int64_t t0 = 0; t0 < jb.n_samples && e == cudaSuccess; t0 += kFusedMaxSamples) {
                 const int64_t nt = std::min<int64_t>(kFusedMaxSamples, jb.n_samples - t0);
+                if (b->packed[jk.first] >= 0) {
+                    PackArgs p;
+                    p.block = jb.block;
+                    p.t0 = t0;
+                    p.nt = nt;
+                    p.F = p.nf = jb.n_freq;
+                    p.N = jb.n_inputs;
+                    p.pitch = (int32_t)round_up(jb.n_inputs, 16);
+                    p.out = b->planes + b->packed[jk.first];
+                    e = launch_pack(p, b->num_sms, st);
+                    if (e == cudaSuccess)
+                        e = launch_single_pass(jk.second, p.out, nt, 0, nt, jb.n_freq, jb.n_inputs, 0, jb.n_freq, jb.out,
+                                               t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st, nullptr, 0, p.pitch);
+                    continue;
+                }
                 e = launch_single_pass(jk.second, jb.block, jb.n_samples, t0, nt, jb.n_freq, jb.n_inputs, 0,
                                        jb.n_freq, jb.out, t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st);
             }
@@ -226,7 +248,9 @@ int plan(xeng_batch_s *b)
     std::vector<char> single(n, 0);
     const int force = single_pass_force_from_env();
     b->listed.assign(n, 0);
+    b->packed.assign(n, -1);
     std::vector<int> pj;  // the pair kernel's listed jobs
+    int64_t total = 0;    // bytes of rearranged samples and planes
     for (int j = 0; j < n; j++) {
         const int k = single_pass_kernel(b->jobs[j].block, b->jobs[j].n_inputs, force, true);
         if (k) {
@@ -236,6 +260,16 @@ int plan(xeng_batch_s *b)
                 b->listed[j] = 1;
                 pj.push_back(j);
             }
+            continue;
+        }
+        const xeng_job_t &jb = b->jobs[j];
+        const int32_t pitch = (int32_t)round_up(jb.n_inputs, 16);
+        const int kp = single_pass_kernel(nullptr, jb.n_inputs, force, true, pitch);
+        if (kp && jb.n_samples * jb.n_freq * jb.n_inputs >= kBatchPackBytes) {
+            single[j] = 1;
+            b->single.push_back({j, kp});
+            b->packed[j] = total;
+            total += round_up(std::min<int64_t>(jb.n_samples, kFusedMaxSamples) * jb.n_freq * pitch, 1024);
         }
     }
     if (!pj.empty()) {
@@ -270,7 +304,7 @@ int plan(xeng_batch_s *b)
         b->n_pjobs = (int)pj.size();
         b->p_items = item0;
     }
-    int64_t total = 0, ptotal = 0, stotal = 0;
+    int64_t ptotal = 0, stotal = 0;
     for (int j = 0; j < n; j++) {
         if (single[j]) continue;
         const xeng_job_t &jb = b->jobs[j];
@@ -576,7 +610,7 @@ int xeng_batch_info(xeng_batch_t b, xeng_batch_info_t *info)
     if (!b || !info) return XENG_ERR_ARG;
     info->n_jobs = (int32_t)b->jobs.size();
     info->n_items = b->n_items;
-    info->grid = b->grid;
+    info->grid = b->grid ? b->grid : b->num_sms;  // no planned launch: the single-pass kernels' own
     info->decode_ctas = b->dec_ctas + b->dtiles;
     info->planes_bytes = b->planes_bytes;
     info->max_chunks_per_item = b->opts.max_chunks_per_item;
