@@ -130,7 +130,8 @@ struct OnepassArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
-    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map,
+    int32_t sub_f0;           // channel fl of the launch at its channel sub_f0 + fl
     int8_t slot[kMaxBlocks];
 };
 
@@ -233,11 +234,11 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 const int f = a.f0 + w.fl;
                 const bool diag = w.I == w.J;
                 // where each block's tiles are: map, input, channel, first sample (a substituted
-                // block's in sub_map, whose channels and samples are the launch's)
+                // block's in sub_map, whose samples are the launch's)
                 const int sJ = a.sub ? a.slot[w.J] : -1, sI = a.sub ? a.slot[w.I] : -1;
                 const CUtensorMap *mJ = sJ >= 0 ? &sub_map : &raw_map, *mI = sI >= 0 ? &sub_map : &raw_map;
                 const int xJ = 128 * (sJ >= 0 ? sJ : w.J), xI = 128 * (sI >= 0 ? sI : w.I);
-                const int fJ = sJ >= 0 ? w.fl : f, fI = sI >= 0 ? w.fl : f;
+                const int fJ = sJ >= 0 ? a.sub_f0 + w.fl : f, fI = sI >= 0 ? a.sub_f0 + w.fl : f;
                 int zJ = sJ >= 0 ? 0 : (int)a.t0, zI = sI >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < n_k; kc++) {
                     ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
@@ -637,7 +638,7 @@ cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int6
         if (e0 != cudaSuccess) return e0;
     }
     if (sub) {
-        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kOKc);
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, sub->F, 128 * sub->n, 0, kOKc);
         if (e0 != cudaSuccess) return e0;
     }
     auto kernel = accumulate ? correlate_onepass_kernel<true> : correlate_onepass_kernel<false>;
@@ -659,6 +660,7 @@ cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int6
     a.maps = maps;
     a.spb = spb;
     a.sub = sub ? 1 : 0;
+    a.sub_f0 = sub ? sub->f0 : 0;
     if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     const int grid = n_items < num_sms ? (int)n_items : num_sms;
     kernel<<<grid, kOThreads, kOSmem, s>>>(map, sub_map, a);

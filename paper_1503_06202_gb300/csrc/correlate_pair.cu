@@ -135,7 +135,8 @@ struct PairArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
-    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map,
+    int32_t sub_f0;           // channel fl of the launch at its channel sub_f0 + fl
     int8_t slot[kMaxBlocks];
     const PairJob *jobs;      // listed launches: the jobs (items job after job), else unused
     int32_t n_jobs;
@@ -261,12 +262,12 @@ correlate_pair_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_
                 const bool diag = w.I2 == w.J2;
                 const int xa = w.J2 * 256 + (int)rank * 128, xb = w.I2 * 256 + (int)rank * 128;
                 // where each tile's block is: map, input, channel, first sample (a substituted
-                // block's in sub_map, whose channels and samples are the launch's; a block past
+                // block's in sub_map, whose samples are the launch's; a block past
                 // the inputs has no slot)
                 const int sa = !kListed && a.sub ? a.slot[xa >> 7] : -1, sb = !kListed && a.sub ? a.slot[xb >> 7] : -1;
                 const CUtensorMap *ma = sa >= 0 ? &sub_map : kListed ? a.jobs[w.job].map : &raw_map;
                 const CUtensorMap *mb = sb >= 0 ? &sub_map : kListed ? a.jobs[w.job].map : &raw_map;
-                const int fa = sa >= 0 ? w.fl : f, fb = sb >= 0 ? w.fl : f;
+                const int fa = sa >= 0 ? a.sub_f0 + w.fl : f, fb = sb >= 0 ? a.sub_f0 + w.fl : f;
                 int za = kListed || sa >= 0 ? 0 : (int)a.t0, zb = kListed || sb >= 0 ? 0 : (int)a.t0;
                 for (int kc = 0; kc < nk; kc++) {
                     ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
@@ -694,7 +695,7 @@ cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t
         if (e0 != cudaSuccess) return e0;
     }
     if (sub) {
-        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kPKc);
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, sub->F, 128 * sub->n, 0, kPKc);
         if (e0 != cudaSuccess) return e0;
     }
     auto kernel = accumulate ? correlate_pair_kernel<false, true> : correlate_pair_kernel<false, false>;
@@ -716,6 +717,7 @@ cudaError_t launch_correlate_pair(const uint8_t *block, int64_t T_block, int64_t
     a.maps = maps;
     a.spb = spb;
     a.sub = sub ? 1 : 0;
+    a.sub_f0 = sub ? sub->f0 : 0;
     if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     const int64_t clusters = n_items < num_sms / 2 ? n_items : num_sms / 2;
     cudaLaunchConfig_t cfg = {};

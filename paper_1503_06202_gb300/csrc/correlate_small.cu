@@ -157,7 +157,8 @@ struct SmallArgs {
     int *err;
     const CUtensorMap *maps;  // null: raw_map over one block; else a map per block of spb stages,
     int32_t spb;              // the launch's samples running through the blocks in order
-    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map
+    int32_t sub;              // != 0: the 128-input blocks b with slot[b] >= 0 come from sub_map,
+    int32_t sub_f0;           // channel fl of the launch at its channel sub_f0 + fl
     int8_t slot[kMaxBlocks];
 };
 
@@ -309,13 +310,13 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
                 const SmallItem w = small_item(a, pc.it);
                 const int fX = a.f0 + w.fx, fY = a.f0 + (w.fy >= 0 ? w.fy : w.fx);
                 // where each tile's block is: map, input, channel, sample (block 0 of channel fx,
-                // and block 0 or 1 of fy; a substituted block's in sub_map, whose channels and
+                // and block 0 or 1 of fy; a substituted block's in sub_map, whose
                 // samples are the launch's)
                 const int sX = a.sub ? a.slot[0] : -1, sY = a.sub ? a.slot[w.col ? 1 : 0] : -1;
                 const CUtensorMap *own = w.col ? &raw_map : &diag_map;
                 const CUtensorMap *mX = sX >= 0 ? &sub_map : own, *mY = sY >= 0 ? &sub_map : own;
                 const int xX = sX >= 0 ? 128 * sX : 0, xY = sY >= 0 ? 128 * sY : w.col ? 128 : 0;
-                const int cX = sX >= 0 ? fX - a.f0 : fX, cY = sY >= 0 ? fY - a.f0 : fY;
+                const int cX = sX >= 0 ? a.sub_f0 + fX - a.f0 : fX, cY = sY >= 0 ? a.sub_f0 + fY - a.f0 : fY;
                 int zX = (sX >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc, zY = (sY >= 0 ? 0 : (int)a.t0) + pc.k0 * kSKc;
                 for (int kc = pc.k0; kc < pc.k1; kc++) {
                     ok = __all_sync(0xffffffffu, mbar_try_wait(rawe(s), ph ^ 1u) ||
@@ -883,7 +884,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
         if (e0 != cudaSuccess) return e0;
     }
     if (sub) {
-        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, nf, 128 * sub->n, 0, kSKc);
+        cudaError_t e0 = encode_raw_map(&sub_map, sub->packed, nt, sub->F, 128 * sub->n, 0, kSKc);
         if (e0 != cudaSuccess) return e0;
     }
     int32_t split = 0;
@@ -910,6 +911,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     a.maps = maps;
     a.spb = spb;
     a.sub = sub ? 1 : 0;
+    a.sub_f0 = sub ? sub->f0 : 0;
     if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     a.split = split;
     a.quot = (int32_t)((split == kSWhole ? n_items : n_items * n_k) / grid);

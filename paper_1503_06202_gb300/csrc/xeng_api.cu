@@ -259,17 +259,23 @@ int fused_kernel(const xeng_s *h, const uint8_t *block)
 
 bool fused_ok(const xeng_s *h, const uint8_t *block) { return fused_kernel(h, block) != 0; }
 
-// The kernel of one launch (XENG_FUSED_KERNEL's choice stands).
-int shaped(const xeng_s *h, int kernel, int64_t nf, int64_t nt, int accumulate)
+// One single-pass launch, its kernel by the launch's shape (XENG_FUSED_KERNEL's
+// choice stands).
+cudaError_t launch_shaped(xeng_s *h, int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
+                          int32_t f0, int32_t nf, int32_t *acc, int accumulate, cudaStream_t s, int32_t pitch = 0,
+                          const SubBlocks *sub = nullptr)
 {
-    return h->fused_force ? kernel : single_pass_by_shape(kernel, h->N, nf, nt, accumulate, h->num_sms);
+    if (h->fused_force)
+        return launch_single_pass(kernel, block, T_block, t0, nt, F, h->N, f0, nf, acc, accumulate, &h->small, h->d_err,
+                                  h->num_sms, s, nullptr, 0, pitch, sub);
+    return launch_single_pass_shaped(kernel, block, T_block, t0, nt, F, h->N, f0, nf, acc, accumulate, &h->small,
+                                     h->d_err, h->num_sms, s, pitch, sub, &h->stats.launches);
 }
 
 cudaError_t launch_fused(xeng_s *h, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                          int32_t f0, int32_t nf, int32_t *acc, int accumulate, cudaStream_t s)
 {
-    return launch_single_pass(shaped(h, fused_kernel(h, block), nf, nt, accumulate), block, T_block, t0, nt, F, h->N, f0, nf, acc, accumulate,
-                              &h->small, h->d_err, h->num_sms, s);
+    return launch_shaped(h, fused_kernel(h, block), block, T_block, t0, nt, F, f0, nf, acc, accumulate, s);
 }
 
 // The single-pass kernel for samples that are rearranged first (pack.cu), so
@@ -477,7 +483,7 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
     // the 128-input blocks that hold a delayed input, one after another
     SubBlocks sub;
     sub.packed = nullptr;
-    sub.n = 0;
+    sub.n = sub.F = sub.f0 = 0;
     std::fill(sub.slot, sub.slot + kMaxBlocks, (int8_t)-1);
     for (int32_t i : inputs)
         if (sub.slot[i / kTile] < 0) sub.slot[i / kTile] = (int8_t)sub.n++;
@@ -587,12 +593,9 @@ cudaError_t integrate_packed(xeng_s *h, int kernel, const uint8_t *dblock, int32
             p.counts = counts ? counts + c0 * h->N : nullptr;
             e = timed_launch(h, 0, s, [&] { return launch_pack(p, h->num_sms, s); });
             if (e != cudaSuccess) break;
-            const int accumulate = fresh && t0 == 0 ? 0 : 1;
-            const int k = shaped(h, kernel, p.nf, p.nt, accumulate);
             e = timed_launch(h, 1, s, [&] {
-                return launch_single_pass(k, h->packed, p.nt, 0, p.nt, p.nf, h->N, 0, p.nf, target + c0 * nb2, accumulate,
-                                          &h->small, h->d_err, h->num_sms, s, nullptr, 0,
-                                          p.pitch);
+                return launch_shaped(h, kernel, h->packed, p.nt, 0, p.nt, p.nf, 0, p.nf, target + c0 * nb2,
+                                     fresh && t0 == 0 ? 0 : 1, s, p.pitch);
             });
         }
     }
@@ -653,18 +656,18 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
                 p.n_chunks = nc[0];
                 const cudaError_t e2 = launch_pack(p, h->num_sms, s);
                 if (e2 != cudaSuccess) return e2;
+                if (nc[0] > 0) h->stats.launches++;
                 p.chunks = plain + nc[0];
                 p.n_chunks = nc[1];
                 return launch_pack_shifted(p, sa, h->num_sms, s);
             });
             if (e != cudaSuccess) break;
-            const int k = shaped(h, kernel, p.nf, p.nt, accumulate);
+            sub.F = p.nf;
             e = timed_launch(h, 1, s, [&] {
-                return direct ? launch_single_pass(k, dblock, n, t0, p.nt, F, N, p.f0, p.nf, target + f0 * nb2,
-                                                   accumulate, &h->small, h->d_err, h->num_sms, s, nullptr, 0, 0, &sub)
-                              : launch_single_pass(k, h->packed, p.nt, 0, p.nt, p.nf, N, 0, p.nf,
-                                                   target + f0 * nb2, accumulate, &h->small, h->d_err, h->num_sms, s,
-                                                   nullptr, 0, p.pitch);
+                return direct ? launch_shaped(h, kernel, dblock, n, t0, p.nt, F, p.f0, p.nf, target + f0 * nb2, accumulate,
+                                              s, 0, &sub)
+                              : launch_shaped(h, kernel, h->packed, p.nt, 0, p.nt, p.nf, 0, p.nf, target + f0 * nb2,
+                                              accumulate, s, p.pitch);
             });
         }
     }

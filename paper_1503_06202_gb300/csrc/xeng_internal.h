@@ -180,12 +180,13 @@ cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_
 // What the three single-pass launches below share.  A block's rows are `pitch`
 // bytes per channel (0: N), a multiple of 16; N itself need not be one.  With
 // `sub`, the 128-input blocks b with slot[b] >= 0 are read from packed
-// [nt][nf][128 n] (16-byte aligned) instead, at inputs 128 slot[b] ..: the
-// launch's samples and channels, rearranged (launch_pack_shifted).
+// [nt][F][128 n] (16-byte aligned) instead, at inputs 128 slot[b] ..: the
+// launch's samples, rearranged (launch_pack_shifted), the launch's channels from
+// its channel f0 on.
 constexpr int kMaxBlocks = 32;  // 128-input blocks of 4096 inputs
 struct SubBlocks {
     const uint8_t *packed;
-    int32_t n;
+    int32_t n, F, f0;
     int8_t slot[kMaxBlocks];
 };
 // The raw block's tensor map of their stages (3D: input, channel, sample; boxes of
@@ -285,6 +286,13 @@ cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block
                                int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, SmallScratch *sc,
                                int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps = nullptr,
                                int32_t spb = 0, int32_t pitch = 0, const SubBlocks *sub = nullptr);
+// The same launch with the kernel chosen by its shape (single_pass_by_shape); what
+// would be a last round of the pair kernel with few items may go to the one pass,
+// as a second launch (counted in *launches).
+cudaError_t launch_single_pass_shaped(int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt,
+                                      int32_t F, int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate,
+                                      SmallScratch *sc, int *err, int num_sms, cudaStream_t s, int32_t pitch = 0,
+                                      const SubBlocks *sub = nullptr, int64_t *launches = nullptr);
 // A kernel's stage in samples.
 int single_pass_stage(int kernel);
 

@@ -115,6 +115,43 @@ def test_small_items_shared_whole_or_cut(T, F, N):
     assert np.array_equal(correlate(blk, pieces=[T // 3])[keep], want)
 
 
+# Launches whose kernel is chosen by their shape: a few stages over many pairs (one
+# pass, N = 128 and 256 too), one round (one pass) and, at N = 512 x 26 channels, 78
+# items for 76 clusters: 25 channels by the pair kernel, the last by the one pass.
+@pytest.mark.parametrize("T,F,N", [(130, 40, 512), (1500, 26, 512), (700, 3, 1024), (200, 300, 128), (256, 90, 256)])
+def test_kernel_by_launch_shape(T, F, N):
+    rng = np.random.default_rng(T * 3 + F + N)
+    blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    keep = sorted({0, 1, F // 2, F - 2, F - 1})
+    want = oracle.correlate(np.ascontiguousarray(blk[:, keep]))
+    assert np.array_equal(correlate(blk)[keep], want)
+    # the later pushes add, the last of them a few samples
+    assert np.array_equal(correlate(blk, pieces=[T // 2, T // 2 - 3])[keep], want)
+
+
+# Samples rearranged first (pack.cu): rows off 16 bytes, fewer inputs than a chunk,
+# a block off a 16-byte boundary, several rounds (more than 32,768 samples)
+@pytest.mark.parametrize("T,F,N,skip", [(1, 1, 1, 0), (300, 5, 7, 0), (1031, 3, 203, 0), (700, 26, 509, 0),
+                                        (500, 2, 1025, 0), (33000, 1, 33, 0), (600, 3, 272, 1), (600, 3, 128, 8)])
+def test_unaligned_rows_and_blocks(T, F, N, skip):
+    rng = np.random.default_rng(T + 7 * F + N)
+    blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    want = oracle.correlate(blk)
+    flat = torch.zeros(blk.size + 64, dtype=torch.uint8, device="cuda")
+    src = flat[skip:skip + blk.size].view(T, F, N)
+    src.copy_(torch.from_numpy(blk))
+    eng = xe.XEngine(N, F, T)
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    eng.correlate(src, out, T)
+    assert np.array_equal(out.cpu().numpy().astype(np.int64), want)
+    eng.push(src, T // 3)
+    eng.push(src[T // 3:], T - T // 3)
+    eng.dump(out)
+    assert np.array_equal(out.cpu().numpy().astype(np.int64), want)
+    eng.close()
+    assert np.array_equal(correlate(blk, host=True), want)
+
+
 def test_fused_graph_replays_stay_exact():
     # one captured call replayed: the flags that publish split items' partial
     # blocks carry a count the device advances after every launch, so no replay

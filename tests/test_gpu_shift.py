@@ -143,3 +143,17 @@ def test_shift_argument_checks_and_removal():
     eng.set_engine(xe.XENG_ENGINE_DP4A)
     assert xe.xeng_set_delays(eng.h, d) == xe.XENG_ERR_UNSUPPORTED
     eng.close()
+
+
+# Delayed inputs in some 128-input blocks only (copied, the others read in place),
+# whole 16-input chunks and single inputs, pushes longer and shorter than the
+# delays and across the ring's end; 26 channels of 512 inputs run as two launches
+@pytest.mark.parametrize("N,F,delays", [(512, 26, {0: 5, 130: 700, 131: 700}), (272, 2, {i: 40 for i in range(16, 32)}),
+                                        (256, 3, {3: 1, 255: 999}), (1040, 1, {1039: 300, 500: 1}),
+                                        (61, 4, {60: 17, 0: 1000})])
+def test_shift_some_blocks(N, F, delays):
+    d = np.zeros(N, np.int32)
+    for i, v in delays.items():
+        d[i] = v
+    stream, got = run_stream(N, F, 2000, d, [900, 100, 700, 200, 1000], {1, 3, 4}, seed=N + F)
+    check(stream, d, got)
