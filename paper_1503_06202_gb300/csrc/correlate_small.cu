@@ -145,8 +145,8 @@ struct SmallArgs {
     int64_t t0, nt;        // samples t0 .. t0 + nt - 1 of the block, nt <= kFusedMaxSamples
     int32_t F, N, f0, nf;  // channels f0 .. f0 + nf - 1
     int32_t n_items, n_k;  // items; stages (of kSKc samples) per item
-    int32_t split;         // CTAs per item (>= 2: shared items), else kSEven or kSWhole
-    int32_t quot, rest;    // the sequence's n_items * n_k stages (kSEven) or its items (kSWhole) over
+    int32_t split;         // CTAs per item (>= 2: shared items), else kSmallEven or kSmallWhole
+    int32_t quot, rest;    // the sequence's n_items * n_k stages (kSmallEven) or its items (kSmallWhole) over
                            // the grid: CTA b takes quot of them, one more if b < rest
     int32_t *acc;          // [nf][N(N+1)/2][2], channel f0 + fl at fl
     int accumulate;        // 0: store, 1: add
@@ -164,25 +164,24 @@ struct SmallArgs {
 
 // A CTA's work: the stages [lo, hi) of the launch's sequence (item-major), as
 // pieces (item, stages k0 .. k1 - 1).  How the sequence is cut (small_split):
-//   kSEven      evenly.  A piece with k0 > 0 (only ever a CTA's first) adds its
+//   kSmallEven  evenly.  A piece with k0 > 0 (only ever a CTA's first) adds its
 //               partial block through ws; the CTA whose piece starts the item
 //               (its owner) adds them into its own and stores.
-//   kSWhole     between items only: no partial blocks.
+//   kSmallWhole between items only: no partial blocks.
 //   2 or more   `split` CTAs share each item, one piece each: all of them write
 //               their partials of the chunks the others finish, and each adds up
 //               and stores its share of the item's 8-column chunks.
-constexpr int kSEven = 0, kSWhole = 1;
 struct Piece {
     int it, k0, k1;
 };
 
 __device__ __forceinline__ int range_lo(const SmallArgs &a, int b)
 {
-    if (a.split > kSWhole) return (b / a.split) * a.n_k + (b % a.split) * a.n_k / a.split;
-    return (b * a.quot + min(b, a.rest)) * (a.split == kSWhole ? a.n_k : 1);
+    if (a.split > kSmallWhole) return (b / a.split) * a.n_k + (b % a.split) * a.n_k / a.split;
+    return (b * a.quot + min(b, a.rest)) * (a.split == kSmallWhole ? a.n_k : 1);
 }
 
-// kSEven: the CTA whose range holds stage x of the sequence.
+// kSmallEven: the CTA whose range holds stage x of the sequence.
 __device__ __forceinline__ int stage_cta(const SmallArgs &a, int x)
 {
     const int more = a.rest * (a.quot + 1);  // stages of the CTAs that take one more
@@ -813,8 +812,8 @@ bool small_ok(const uint8_t *block, int32_t N, int32_t pitch)
 
 namespace {
 
-// How a launch's items (n_k stages each) are cut over the CTAs, at most one
-// per SM: *split as SmallArgs::split; returns the grid.
+}  // namespace
+
 int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split)
 {
     // Few items: as many CTAs per item as there are SMs for, each with at least
@@ -833,15 +832,13 @@ int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split)
     // that an even cut saves (GB300, N = 256 x 128 channels x 256 samples: 25 us;
     // cut evenly into pieces of kSMinPiece stages, 209).
     if (n_k < kSMinPiece) {
-        *split = kSWhole;
+        *split = kSmallWhole;
         return (int)(n_items < num_sms ? n_items : num_sms);
     }
-    *split = kSEven;
+    *split = kSmallEven;
     const int64_t grid = total / kSMinPiece;
     return (int)(grid < num_sms ? grid : num_sms);
 }
-
-}  // namespace
 
 size_t small_ws_bytes(int num_sms) { return (size_t)num_sms * 2 * 16 * 128 * 8 * sizeof(int2); }
 size_t small_flags_bytes(int num_sms) { return (size_t)(num_sms + 2) * sizeof(int); }
@@ -914,8 +911,8 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     a.sub_f0 = sub ? sub->f0 : 0;
     if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     a.split = split;
-    a.quot = (int32_t)((split == kSWhole ? n_items : n_items * n_k) / grid);
-    a.rest = (int32_t)((split == kSWhole ? n_items : n_items * n_k) % grid);
+    a.quot = (int32_t)((split == kSmallWhole ? n_items : n_items * n_k) / grid);
+    a.rest = (int32_t)((split == kSmallWhole ? n_items : n_items * n_k) % grid);
     // the CTAs of a split item wait for each other's partials: a cooperative
     // launch has every CTA resident at once (or fails)
     cudaLaunchConfig_t cfg = {};

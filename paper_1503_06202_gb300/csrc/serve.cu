@@ -542,8 +542,10 @@ bool launch_round(xserve_s *sv)
             const int nb = std::min(per, sg.nblocks - b0);
             const int64_t nt = (int64_t)nb * st.block_samples;
             const int accumulate = (sg.store && b0 == 0) ? 0 : 1;
-            const int k = sv->single_force ? sg.kernel
-                                           : single_pass_by_shape(sg.kernel, st.N, st.F, nt, accumulate, sv->num_sms);
+            // the maps' boxes and spb are those of sg.kernel's stages
+            int k = sv->single_force ? sg.kernel
+                                     : single_pass_by_shape(sg.kernel, st.N, st.F, nt, accumulate, sv->num_sms);
+            if (single_pass_stage(k) != single_pass_stage(sg.kernel)) k = sg.kernel;
             e = launch_single_pass(k, nullptr, nt, 0, nt, st.F, st.N, 0, st.F, st.acc, accumulate, &sv->small, sv->d_err, sv->num_sms, s,
                                    sv->d_smaps[slot] + sg.map0 + b0, spb);
         }

@@ -139,10 +139,24 @@ int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accu
     int64_t t_one = ones * (770 * n_k + (accumulate ? 3200 : 1600));
     if (N > 1900 && ones > 8 && n_k > 32) t_one += t_one / 4;
     if (kernel == kSingleSmall) {
-        // only against its whole items: it shares few items, and cuts long ones, evenly
+        // By how it cuts its items: between CTAs (an exchange of partial blocks, then
+        // the stages of one CTA) or whole.  The exchange costs more than the stages it
+        // takes off the CTAs of a short launch (us a call, the N <= 256 kernel / the
+        // one pass: N = 256 x 8 channels x 1024 samples 22.3 / 14.3, x 2048 22.5 / 19.2,
+        // x 4096 26.1 / 30.6; 256 x 48 x 4096 37.9 / 31.3, x 8192 56.0 / 54.4; 160 x 2
+        // x 256 15.0 / 9.0; 128 x 152 x 4096 39.5 / 27.7, x 32,768 168 / 191).
         const int64_t items = N > 128 ? nf + (nf + 1) / 2 : (nf + 1) / 2;
-        if (n_k >= 32 || 2 * items <= num_sms) return kernel;
-        return rounds(items, num_sms) * (1000 * n_k + (accumulate ? 13500 : 6000)) <= t_one ? kernel : kSingleOnepass;
+        const int64_t n_one = accumulate ? 3200 : 1600;
+        int32_t split;
+        const int grid = small_split(items, (int)n_k, num_sms, &split);
+        int64_t t_small;
+        if (split == kSmallWhole)
+            t_small = 2000 + rounds(items, num_sms) * (1100 * n_k + (accumulate ? 13500 : 5000));
+        else if (split == kSmallEven)  // one item a CTA is as good as whole
+            t_small = (grid == items ? 6000 : 18000) + 1200 * (items * n_k / grid) + (accumulate ? 11000 * items / grid : 0);
+        else
+            t_small = 9000 + 25 * N + 1100 * n_k / split + (accumulate ? 5500 : 0);
+        return t_small <= ones * ((N > 128 ? 770 : 680) * n_k + n_one) ? kernel : kSingleOnepass;
     }
     if (kernel != kSinglePair && kernel != kSingleOnepass) return kernel;
     return rounds(nf * (b2 * (b2 + 1) / 2), num_sms / 2) * (1200 * n_k + (accumulate ? 12300 : 7400)) < t_one

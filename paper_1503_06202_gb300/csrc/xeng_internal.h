@@ -269,6 +269,11 @@ int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded,
 // block pairs, or (kernel = kSingleSmall) of that one and the one pass.  All three
 // read the same stages.
 int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);
+// How a launch of the N <= 256 kernel cuts its items (n_k stages each) over the
+// CTAs, at most one per SM: *split CTAs share each item (2 or more), or all stages
+// are cut evenly (kSmallEven), or the items stay whole (kSmallWhole); returns the grid.
+constexpr int kSmallEven = 0, kSmallWhole = 1;
+int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split);
 // Scratch of the N <= 256 kernel, allocated at its first launch (flags zeroed
 // on the stream) and owned by the caller.
 struct SmallScratch {

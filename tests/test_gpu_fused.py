@@ -99,9 +99,9 @@ def test_fused_items_split_over_many_ctas(N):
 # shared by several CTAs (as many as there are SMs for, stages uneven between
 # them, at most 32, at least two stages each), whole, cut evenly, or -- 60 items
 # of 256 stages -- even because two CTAs an item would leave SMs idle.
-@pytest.mark.parametrize("T,F,N", [(257, 1, 128), (511, 1, 256), (512, 7, 16), (1000, 3, 144), (1700, 12, 208),
-                                   (4096, 8, 256), (5000, 25, 160), (9000, 1, 256), (300, 51, 256), (385, 77, 112),
-                                   (3969, 52, 256), (32700, 40, 256)])
+@pytest.mark.parametrize("T,F,N", [(2100, 1, 64), (2177, 1, 16), (4096, 8, 256), (4097, 12, 208), (5000, 25, 160),
+                                   (9000, 1, 256), (2000, 256, 112), (3969, 52, 256), (5000, 110, 256),
+                                   (32700, 40, 256)])
 def test_small_items_shared_whole_or_cut(T, F, N):
     rng = np.random.default_rng(T + F + N)
     blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
@@ -115,10 +115,12 @@ def test_small_items_shared_whole_or_cut(T, F, N):
     assert np.array_equal(correlate(blk, pieces=[T // 3])[keep], want)
 
 
-# Launches whose kernel is chosen by their shape: a few stages over many pairs (one
-# pass, N = 128 and 256 too), one round (one pass) and, at N = 512 x 26 channels, 78
+# Launches whose kernel is chosen by their shape: a few stages (one pass, N <= 256
+# too, where sharing or cutting its items would take longer), one round (one pass) and, at N = 512 x 26 channels, 78
 # items for 76 clusters: 25 channels by the pair kernel, the last by the one pass.
-@pytest.mark.parametrize("T,F,N", [(130, 40, 512), (1500, 26, 512), (700, 3, 1024), (200, 300, 128), (256, 90, 256)])
+@pytest.mark.parametrize("T,F,N", [(130, 40, 512), (1500, 26, 512), (700, 3, 1024), (200, 300, 128), (256, 90, 256),
+                                   (1, 1, 16), (511, 7, 208), (1000, 3, 144), (2048, 8, 256), (4000, 150, 128),
+                                   (4096, 48, 256)])
 def test_kernel_by_launch_shape(T, F, N):
     rng = np.random.default_rng(T * 3 + F + N)
     blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
