@@ -197,8 +197,8 @@ XENG_API int64_t xeng_dump_gated(xeng_t h, int32_t *out, int32_t *counts, void *
  *   where t counts the samples of the handle's stream (every push since this
  *   call, in order) and x_i(t) = 0 + 0i for t < 0.  Between pushes the handle
  *   keeps the last max(d) samples of each delayed input on the device
- *   ((max(d) + min(t_integ, 32768)) * n_freq * #{i : d_i > 0} bytes); xeng_dump
- *   does not reset that history.
+ *   (max(d) * n_freq * #{i : d_i > 0} bytes, and up to 2 GiB more for a push's
+ *   own); xeng_dump does not reset that history.
  *   delays: host int32 [n_inputs], each in [0, XENG_MAX_DELAY]; NULL, or all
  *   zero, removes the delays.  The history restarts empty (zeros) with every
  *   call.  Synchronizes the device: a set-up call, not for the streaming loop.

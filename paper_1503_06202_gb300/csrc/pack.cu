@@ -141,7 +141,9 @@ pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_blo
 // there, so that reading them d samples back stays in L2, where the block's rows
 // do not.  Launched over these chunks alone: among plain ones they kept whole
 // warps waiting (N = 496 x 188 channels x 30,415 samples, 7 inputs delayed, 1.9 ms
-// for all chunks in one launch).
+// for all chunks in one launch).  !kAhead, where a ring of that size would not be
+// worth its memory: the launch's own samples from the block.
+template <bool kAhead>
 __global__ void __launch_bounds__(kPackThreads)
 pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols_per_block, int rows_per_block, int span)
 {
@@ -187,8 +189,11 @@ pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols
             const uint32_t byte = 0xFFu << (8 * (m & 3));
             uint32_t b[kPackRows];
             #pragma unroll
-            for (int k = 0; k < kPackRows; k++)
-                b[k] = 0x01010101u * __ldg(ring + sa.row(min(t + (int64_t)k * rows_per_block, last - 1) - d) * ring_bytes + s);
+            for (int k = 0; k < kPackRows; k++) {
+                const int64_t src = min(t + (int64_t)k * rows_per_block, last - 1) - d;
+                const uint8_t *from = !kAhead && src >= 0 ? blk + src * row_bytes + m : ring + sa.row(src) * ring_bytes + s;
+                b[k] = 0x01010101u * __ldg(from);
+            }
             #pragma unroll
             for (int k = 0; k < kPackRows; k++) {
                 #pragma unroll
@@ -256,7 +261,8 @@ cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_
     if (cols <= 0 || a.nt <= 0) return cudaSuccess;
     if (!pack_args_ok(a) || !a.chunks) return cudaErrorInvalidValue;
     const PackGrid g = pack_grid(a, cols, num_sms);
-    pack_shifted_kernel<<<g.grid, kPackThreads, 0, s>>>(a, sa, cols, g.cols, g.rows, g.span);
+    auto kernel = sa.ahead ? pack_shifted_kernel<true> : pack_shifted_kernel<false>;
+    kernel<<<g.grid, kPackThreads, 0, s>>>(a, sa, cols, g.cols, g.rows, g.span);
     return cudaGetLastError();
 }
 

@@ -12,6 +12,12 @@
 
 using namespace xeng;
 
+// Memory that set_delays takes at most so that a round's samples of the delayed inputs
+// can enter the history before they are integrated and be read there, densely (N = 496
+// x 188 channels x 30,415 samples, 7 inputs delayed: rearranged in 1.59 ms so, in
+// 2.15 ms with the launch's samples read from the block).
+constexpr int64_t kShiftAheadBytes = int64_t(2) << 30;
+
 static_assert(XENG_MAX_GATES == kMaxGates, "gate set limit of the header and of the kernels");
 
 struct TimedLaunch {
@@ -66,6 +72,7 @@ struct xeng_s {
     SubBlocks shift_blocks{};           // those blocks (n of them; `packed` is set per launch)
     uint8_t *hist = nullptr;
     int64_t hist_cap = 0, hist_head = 0;
+    bool hist_ahead = false;  // it also takes a round's samples before they are integrated
     int32_t hist_S = 0;
     bool decode_tma = false;       // decode through the TMA pipeline where the block allows it
     int fused_force = 0;           // single_pass_kernel's force: XENG_FUSED_KERNEL at handle creation
@@ -501,9 +508,10 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
         }
         h->n_shift_chunks[list] = (int32_t)(chunks.size() - before);
     }
-    // the ring holds a round's samples besides the H before them
-    const int64_t cap = H + std::min<int64_t>(h->t_integ, kFusedMaxSamples);
-    const int64_t hist_bytes = cap * h->F * S;
+    // the ring holds the H samples before a round and, up to kShiftAheadBytes, the round's
+    const int64_t row = (int64_t)h->F * S, ahead = std::min<int64_t>(h->t_integ, kFusedMaxSamples);
+    h->hist_ahead = ahead * row <= kShiftAheadBytes;
+    int64_t cap = H + (h->hist_ahead ? ahead : 0);
     cudaError_t e = cudaMalloc(&h->d_delay, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_slot, sizeof(int32_t) * N);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_chunk_delay, sizeof(int32_t) * chunk.size());
@@ -511,14 +519,20 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
     if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_chunks, sizeof(int2) * chunks.size());
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_shift_chunks, chunks.data(), sizeof(int2) * chunks.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&h->hist, (size_t)hist_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&h->hist, (size_t)(cap * row));
+    if (e == cudaErrorMemoryAllocation && h->hist_ahead) {  // the H samples alone
+        cudaGetLastError();
+        h->hist_ahead = false;
+        cap = H;
+        e = cudaMalloc(&h->hist, (size_t)(cap * row));
+    }
     if (e == cudaSuccess) e = cudaMemcpy(h->d_delay, delays, sizeof(int32_t) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_slot, slot.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_chunk_delay, chunk.data(), sizeof(int32_t) * chunk.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_shift_inputs, inputs.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(h->hist, 0x88, (size_t)hist_bytes);  // value 0 + 0i
+    if (e == cudaSuccess) e = cudaMemset(h->hist, 0x88, (size_t)(cap * row));  // value 0 + 0i
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -616,7 +630,7 @@ cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t t0, int64_
 // The same with the handle's delays applied to samples 0 .. n - 1 of the block:
 // where TMA can address the block's rows only the 128-input blocks that hold a
 // delayed input are rearranged, else every input.  Each round's samples enter the
-// history first.
+// history first, where it has room for them.
 cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int64_t n, int32_t *target, bool fresh,
                               cudaStream_t s)
 {
@@ -631,6 +645,7 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
     sa.hist = h->hist;
     sa.cap = h->hist_cap;
     sa.S = h->hist_S;
+    sa.ahead = h->hist_ahead;
     PackArgs p;
     p.block = dblock;
     p.F = F;
@@ -645,7 +660,7 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
         p.nt = std::min<int64_t>(kFusedMaxSamples, n - t0);
         p.t0 = t0;
         sa.head = h->hist_head;
-        e = advance_history(h, dblock, t0, p.nt, s);
+        if (h->hist_ahead) e = advance_history(h, dblock, t0, p.nt, s);
         const int64_t group = std::min<int64_t>(65535, h->packed_bytes / (p.nt * p.pitch));
         for (int64_t f0 = 0; f0 < F && e == cudaSuccess; f0 += group) {
             p.f0 = (int32_t)f0;
@@ -670,6 +685,7 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
                                               accumulate, s, p.pitch);
             });
         }
+        if (e == cudaSuccess && !h->hist_ahead) e = advance_history(h, dblock, t0, p.nt, s);
     }
     return e;
 }

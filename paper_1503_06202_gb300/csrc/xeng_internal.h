@@ -98,6 +98,7 @@ struct ShiftArgs {
     const uint8_t *hist = nullptr;
     int64_t cap = 0, head = 0;
     int32_t S = 0;
+    int32_t ahead = 0;  // != 0: the launch's own samples are there too
     // the ring's row of sample src, |src| <= cap
     __host__ __device__ int64_t row(int64_t src) const
     {

@@ -157,3 +157,26 @@ def test_shift_some_blocks(N, F, delays):
         d[i] = v
     stream, got = run_stream(N, F, 2000, d, [900, 100, 700, 200, 1000], {1, 3, 4}, seed=N + F)
     check(stream, d, got)
+
+
+# Many delayed inputs and a long integration: the history has no room for the pushes'
+# own samples, which are read from the block; 65 channels of 1040 inputs
+def test_shift_history_without_room_for_a_round():
+    N, F, pushes = 1040, 65, [150, 64, 300]
+    rng = np.random.default_rng(5)
+    d = rng.integers(1, 120, N).astype(np.int32)
+    d[-1] = 400
+    stream = rng.integers(0, 256, size=(sum(pushes), F, N), dtype=np.uint8)
+    eng = xe.XEngine(N, F, 32768)
+    eng.set_delays(d)
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    t = 0
+    for k, n in enumerate(pushes):
+        eng.push(torch.from_numpy(stream[t:t + n]).cuda(), n)
+        t += n
+        if k > 0:
+            t_a = 0 if k == 1 else sum(pushes[:2])
+            assert eng.dump(out) == t - t_a
+            got = out[[0, F - 1]].cpu().numpy().astype(np.int64)
+            assert np.array_equal(got, oracle.correlate_shifted(np.ascontiguousarray(stream[:, [0, F - 1]]), d, t_a, t))
+    eng.close()
