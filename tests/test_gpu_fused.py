@@ -116,10 +116,11 @@ def test_small_items_shared_whole_or_cut(T, F, N):
 
 
 # Launches whose kernel is chosen by their shape: a few stages (one pass, N <= 256
-# too, where sharing or cutting its items would take longer), one round (one pass) and, at N = 512 x 26 channels, 78
-# items for 76 clusters: 25 channels by the pair kernel, the last by the one pass.
+# too, where sharing or cutting the items would take longer), one round (one pass)
+# and, at N = 512 x 26 channels, 78 items for 76 clusters: 25 channels by the pair
+# kernel, the last by the one pass.
 @pytest.mark.parametrize("T,F,N", [(130, 40, 512), (1500, 26, 512), (700, 3, 1024), (200, 300, 128), (256, 90, 256),
-                                   (1, 1, 16), (511, 7, 208), (1000, 3, 144), (2048, 8, 256), (4000, 150, 128),
+                                   (8, 2, 16), (511, 7, 208), (1000, 3, 144), (2048, 8, 256), (4000, 150, 128),
                                    (4096, 48, 256)])
 def test_kernel_by_launch_shape(T, F, N):
     rng = np.random.default_rng(T * 3 + F + N)
