@@ -63,10 +63,10 @@ __device__ __forceinline__ void pack_column(const PackArgs &a, int64_t col, int 
 }
 
 // kAligned: every source chunk is 16-byte aligned.  Thread = (row of the block's
-// rows, chunk of a sample).
+// rows, chunk of a sample); blockIdx.z: set.
 template <bool kAligned, bool kValid>
 __global__ void __launch_bounds__(kPackThreads)
-pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_block, int span)
+pack_kernel(const __grid_constant__ PackArgs a, int64_t cols, int cols_per_block, int rows_per_block, int span)
 {
     constexpr int kRows = !kAligned && kValid ? kPackRows / 2 : kPackRows;  // registers
     const int64_t col = (int64_t)blockIdx.x * cols_per_block + threadIdx.x % cols_per_block;
@@ -77,10 +77,14 @@ pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_blo
     const int n = min(16, a.N - ic);
     const int64_t row_bytes = (int64_t)a.F * a.N;
     const int64_t off = (int64_t)(a.f0 + c) * a.N + ic;
-    const int64_t out_row = (int64_t)a.nf * a.pitch;
+    const int set = (int)blockIdx.z;
+    const int32_t *idx = a.sets ? a.idx + a.set_first[set] : a.idx;
+    const int64_t have = a.sets ? a.set_first[set + 1] - a.set_first[set] : a.nt;
+    const int64_t out_row = (int64_t)a.nf * a.pitch * max(a.sets, 1);
     const int64_t first = (int64_t)blockIdx.y * span * rows_per_block + rsub;
-    const int64_t last = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
-    uint8_t *out = a.out + (int64_t)c * a.pitch + j * 16;
+    const int64_t end = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
+    const int64_t last = min(have, end);
+    uint8_t *out = a.out + ((int64_t)set * a.nf + c) * a.pitch + j * 16;
     uint32_t acc[4] = {0, 0, 0, 0};                       // usable samples, a byte per input
     uint32_t acc16[8] = {0, 0, 0, 0, 0, 0, 0, 0};         // the same, 16-bit lanes
     int rows = 0, pending = 0;
@@ -99,7 +103,7 @@ pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_blo
         for (int k = 0; k < kRows; k++) {
             const int64_t tk = t + (int64_t)k * rows_per_block;
             if (tk >= last) break;
-            const int64_t src = (a.idx ? (int64_t)__ldg(a.idx + tk) : a.t0 + tk) * row_bytes + off;
+            const int64_t src = (idx ? (int64_t)__ldg(idx + tk) : a.t0 + tk) * row_bytes + off;
             if (kAligned) x[k].lo = __ldg(reinterpret_cast<const uint4 *>(a.block + src));
             else x[k] = load16(a.block + src, n);
             if (kValid && kAligned) v[k].lo = __ldg(reinterpret_cast<const uint4 *>(a.valid + src));
@@ -126,9 +130,15 @@ pack_kernel(const PackArgs a, int64_t cols, int cols_per_block, int rows_per_blo
         }
         if (kValid && (pending += kRows) > 240 - kRows) widen();
     }
+    if (have < end) {  // value 0 + 0i past the set's samples
+        int64_t t = first;
+        if (t < have) t += (have - t + rows_per_block - 1) / rows_per_block * rows_per_block;
+        for (; t < end; t += rows_per_block)
+            *reinterpret_cast<uint4 *>(out + t * out_row) = make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);
+    }
     if (!a.counts) return;
     if (kValid) widen();
-    int32_t *cnt = a.counts + (int64_t)c * a.N + ic;
+    int32_t *cnt = a.counts + ((int64_t)set * a.nf + c) * a.N + ic;
     #pragma unroll
     for (int m = 0; m < 16; m++) {
         const int usable = kValid ? (int)((acc16[2 * (m >> 2) + (m & 1)] >> (16 * ((m >> 1) & 1))) & 0xFFFFu) : rows;
@@ -225,11 +235,11 @@ PackGrid pack_grid(const PackArgs &a, int64_t cols, int num_sms)
     PackGrid g;
     g.cols = (int)(cols < kPackThreads ? cols : kPackThreads);
     g.rows = kPackThreads / g.cols;
-    const int64_t bx = (cols + g.cols - 1) / g.cols;
+    const int64_t bx = (cols + g.cols - 1) / g.cols, bz = a.sets > 0 ? a.sets : 1;
     g.span = kPackSpan;
-    while (g.span > 2 * kPackRows && bx * ((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)) < 16 * num_sms)
+    while (g.span > 2 * kPackRows && bz * bx * ((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)) < 16 * num_sms)
         g.span /= 2;
-    g.grid = dim3((unsigned)bx, (unsigned)((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)));
+    g.grid = dim3((unsigned)bx, (unsigned)((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)), (unsigned)bz);
     return g;
 }
 
@@ -245,7 +255,7 @@ cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s)
 {
     const int64_t cols = (int64_t)a.nf * (a.chunks ? a.n_chunks : a.pitch / 16);
     if (cols <= 0 || a.nt <= 0) return cudaSuccess;
-    if (!pack_args_ok(a) || (!a.chunks && a.pitch < a.N)) return cudaErrorInvalidValue;
+    if (!pack_args_ok(a) || (!a.chunks && a.pitch < a.N) || a.sets > kMaxGates || (a.sets > 0 && !a.idx)) return cudaErrorInvalidValue;
     const PackGrid g = pack_grid(a, cols, num_sms);
     const bool aligned = a.N % 16 == 0 && (reinterpret_cast<uintptr_t>(a.block) & 15) == 0 &&
                          (reinterpret_cast<uintptr_t>(a.valid) & 15) == 0;

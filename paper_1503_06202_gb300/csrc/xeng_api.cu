@@ -616,6 +616,51 @@ cudaError_t integrate_packed(xeng_s *h, int kernel, const uint8_t *dblock, int32
     return e;
 }
 
+// The samples of G gate sets, listed in idx[cnt[g] .. cnt[g + 1] - 1], as one launch
+// of G * F channels into the consecutive sets at `target`, the shorter sets' missing
+// samples 0 + 0i: rearranging and correlating G short lists one after another leaves
+// most SMs idle (GB300, a push and dump, one by one / together: N = 160 x 2 channels, 7
+// gates of 640 samples with flags 207 / 63 us; 512 x 16, 8 of 1000 316 / 175; 256 x 256,
+// 2 of 8192 with flags 988 / 926).  Returns false, with nothing done, where the sets are
+// too unequal for that, or too large.
+bool integrate_sets(xeng_s *h, int kernel, const uint8_t *dblock, int32_t G, const std::vector<int64_t> &cnt,
+                    const int32_t *idx, const uint8_t *valid, int32_t *counts, int32_t *target, bool fresh, cudaStream_t s,
+                    cudaError_t *e)
+{
+    if (G < 2 || G > kMaxGates || (int64_t)G * h->F > 65535) return false;
+    const int64_t stage = kTile, b1 = (h->N + 127) / 128;
+    int64_t longest = 0, stages = 0;
+    for (int g = 0; g < G; g++) {
+        const int64_t n = cnt[g + 1] - cnt[g];
+        if (n == 0) return false;
+        longest = std::max(longest, n);
+        stages += (n + stage - 1) / stage;
+    }
+    PackArgs p;
+    p.pitch = (int32_t)round_up(h->N, 16);
+    if (longest > kFusedMaxSamples || longest * G * h->F * p.pitch > h->packed_bytes) return false;
+    // the stages that it adds (770 ns per 128 x 128 inputs on an SM) against 8 us per
+    // pair of launches
+    const int64_t more = G * ((longest + stage - 1) / stage) - stages;
+    if (more * h->F * (b1 * (b1 + 1) / 2) * 770 / h->num_sms > 8000 * (int64_t)(G - 1)) return false;
+    p.block = dblock;
+    p.F = p.nf = h->F;
+    p.N = h->N;
+    p.nt = longest;
+    p.idx = idx;
+    p.valid = valid;
+    p.counts = counts;
+    p.out = h->packed;
+    p.sets = G;
+    for (int g = 0; g <= G; g++) p.set_first[g] = (int32_t)cnt[g];
+    *e = timed_launch(h, 0, s, [&] { return launch_pack(p, h->num_sms, s); });
+    if (*e != cudaSuccess) return true;
+    *e = timed_launch(h, 1, s, [&] {
+        return launch_shaped(h, kernel, h->packed, p.nt, 0, p.nt, G * h->F, 0, G * h->F, target, fresh ? 0 : 1, s, p.pitch);
+    });
+    return true;
+}
+
 // Samples t0 .. t0 + n - 1 of the block into the history of the delayed inputs (the
 // last of them, where it holds no more).
 cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t t0, int64_t n, cudaStream_t s)
@@ -1071,7 +1116,9 @@ int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samples, cons
     e = cudaMemcpyAsync(h->gidx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // idx is pageable and goes out of scope
     if (e == cudaSuccess && counts) e = cudaMemsetAsync(counts, 0, (size_t)(n_gates * F * N * 4), s);
-    for (int g = 0; g < n_gates && e == cudaSuccess; g++) {
+    const bool together = e == cudaSuccess && pk &&
+                          integrate_sets(h, pk, block, n_gates, cnt, h->gidx, valid, counts, out, true, s, &e);
+    for (int g = together ? n_gates : 0; g < n_gates && e == cudaSuccess; g++) {
         const int64_t Tg = cnt[g + 1] - cnt[g];
         int32_t *out_g = out + (int64_t)g * F * nb2;
         if (Tg == 0) {
@@ -1270,9 +1317,20 @@ int xeng_push_gated(xeng_t h, const uint8_t *block, int64_t n_samples, const int
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->gidx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // idx is pageable and goes out of scope
+    bool alike = true;  // every set stores, or every set adds
+    for (int g = 1; g < G; g++) alike = alike && set_fresh(h, g) == set_fresh(h, 0);
+    const bool together = e == cudaSuccess && pk && alike &&
+                          integrate_sets(h, pk, block, G, cnt, h->gidx, valid, valid ? h->counts : nullptr, h->acc,
+                                         set_fresh(h, 0), s, &e);
     for (int g = 0; g < G && e == cudaSuccess; g++) {
         const int64_t Tg = cnt[g + 1] - cnt[g];
         if (Tg == 0) continue;
+        if (together) {
+            mark_set_used(h, g);
+            if (valid) h->counts_dirty = true;
+            else h->gate_base[g] += Tg;
+            continue;
+        }
         int32_t *set = h->acc + (int64_t)g * F * nb2;
         if (pk) {
             e = integrate_packed(h, pk, block, (int32_t)F, 0, (int32_t)F, Tg, h->gidx + cnt[g], valid,
@@ -1329,7 +1387,12 @@ int64_t xeng_dump_gated(xeng_t h, int32_t *out, int32_t *counts, void *stream)
     const int64_t counts_bytes = (int64_t)G * h->F * h->N * 4;
     cudaError_t e = cudaSuccess;
     if (!dev_out || (counts && !dev_counts)) e = cudaStreamSynchronize(s);  // host memory is written below
-    for (int g = 0; g < G && e == cudaSuccess; g++) {
+    bool all = true;  // every set holds something: one copy
+    for (int g = 0; g < G; g++) all = all && !set_fresh(h, g);
+    if (e == cudaSuccess && all)
+        e = cudaMemcpyAsync(out, h->acc, (size_t)(G * set_bytes), dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                            s);
+    for (int g = all ? G : 0; g < G && e == cudaSuccess; g++) {
         const bool fresh = set_fresh(h, g);
         int32_t *dst = out + (int64_t)g * (set_bytes / 4);
         if (fresh) {

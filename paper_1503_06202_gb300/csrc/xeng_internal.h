@@ -162,7 +162,10 @@ cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0
 // (position in the packed row, 16-input chunk of the block); null: chunk k is
 // chunk k.  launch_pack_shifted takes the chunks that hold delayed inputs and
 // applies the delays of `sa`, whose ring has to hold the launch's samples already
-// (head: row of sample t0).  nt <= kMaxChunkSamples.
+// (head: row of sample t0) where sa.ahead.  nt <= kMaxChunkSamples.  launch_pack with
+// sets > 0: that many lists of samples side by side, out[nt][sets][nf][pitch] and
+// counts[sets][nf][N], set k's samples idx[set_first[k]] .. idx[set_first[k + 1] - 1],
+// its rows past them 0x88.
 struct PackArgs {
     const uint8_t *block = nullptr;
     int64_t t0 = 0, nt = 0;
@@ -174,6 +177,8 @@ struct PackArgs {
     int32_t n_chunks = 0;
     int32_t pitch = 0;
     uint8_t *out = nullptr;
+    int32_t sets = 0;
+    int32_t set_first[kMaxGates + 1];
 };
 cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s);
 cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_sms, cudaStream_t s);

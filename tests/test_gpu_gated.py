@@ -153,3 +153,33 @@ def test_gate_sets_flags_on_plain_integration_and_argument_checks():
     assert (o[0] == 0).all()                                          # set 0 received nothing
     assert np.array_equal(o[1], oracle.correlate(blk[:10]))
     eng.close()
+
+
+# Gate sets of unlike lengths side by side in one launch, or one after another where a
+# set is empty or far longer than the others: 1 sample, a stage more than the others,
+# 64 sets, rows off 16 bytes, two rounds (more than 32,768 samples of a set)
+@pytest.mark.parametrize("N,F,sizes", [(160, 2, (640, 641, 1, 639)), (61, 3, (5,) * 64), (272, 2, (300, 128, 129)),
+                                       (1040, 1, (200, 90)), (128, 5, (3000, 1, 2)), (48, 40, (9, 0, 4)),
+                                       (32, 1, (33000, 32900))])
+def test_gate_sets_of_unlike_lengths(N, F, sizes):
+    G, T = len(sizes), sum(sizes) + 7
+    rng = np.random.default_rng(N + F + G)
+    gate = np.concatenate([np.full(n, g) for g, n in enumerate(sizes)] + [np.full(7, -1)]).astype(np.int32)
+    rng.shuffle(gate)
+    blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    valid = (rng.random((T, F, N)) > 0.1).astype(np.uint8)
+    want, want_counts = oracle.correlate_gated(blk, gate, G, valid)
+    d, v = torch.from_numpy(blk).cuda(), torch.from_numpy(valid).cuda()
+    eng = xe.XEngine(N, F, 2 * T)
+    got, counts = gated(eng, d, gate, G, v) if T <= 32768 else (want, want_counts)
+    assert np.array_equal(got, want) and np.array_equal(counts, want_counts)
+    # a push that stores and one that adds
+    assert xe.xeng_set_gates(eng.h, G) == xe.XENG_OK
+    out = torch.full((G, F, N * (N + 1) // 2, 2), 77, dtype=torch.int32, device="cuda")
+    cnt = torch.full((G, F, N), -1, dtype=torch.int32, device="cuda")
+    for _ in range(2):
+        assert xe.xeng_push_gated(eng.h, d, T, gate, v) == xe.XENG_OK
+    assert xe.xeng_dump_gated(eng.h, out, cnt) == 2 * T
+    assert np.array_equal(out.cpu().numpy().astype(np.int64), 2 * want)
+    assert np.array_equal(cnt.cpu().numpy().astype(np.int64), 2 * want_counts)
+    eng.close()
