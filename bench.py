@@ -46,10 +46,10 @@ METRIC = "Correlation TOPS (8 ops per complex MAC, bit-exact int32 visibilities)
 # channels.  Keyed by (kernel, N, T); re-take (or remove) an entry whenever its
 # kernel changes.
 DRAM_BYTES_PER_CHANNEL = {
-    ("correlate_pair", 2048, 8192): (300.792576e6 + 217.08416e6) / 16,  # 256-input block pairs, 16-channel slice
+    ("correlate_pair", 2048, 8192): (299.8336e6 + 216.72832e6) / 16,  # 256-input block pairs, 16-channel slice
     ("correlate_tc", 2048, 8192): (607.22048e6 + 240.377344e6) / 16,   # planes engine, 16-channel slice
-    ("correlate_small", 256, 32768): (821.3591e6 + 19.01209e6) / 64,  # N <= 256 kernel, 64-channel slice
-    ("correlate_onepass", 640, 8192): (676.018944e6 + 184.502016e6) / 128,  # one pass, 128-channel slice
+    ("correlate_small", 256, 32768): (822.181632e6 + 20.4864e6) / 64,  # N <= 256 kernel, 64-channel slice
+    ("correlate_onepass", 640, 8192): (673.741056e6 + 183.711744e6) / 128,  # one pass, 128-channel slice
 }
 
 
@@ -684,7 +684,7 @@ def main():
                   "correlate_ms_per_step": gst["correlate_ms"] / greps,
                   "value": whole_job_rate(useful_ops(T, F, N), max_over_ranks(g_ms, dist) * 1e-3, world) / 1e12,
                   "unit": "TOPS", "ungated_ms_per_step": ms,
-                  "kernels": "decode_gather_kernel (gate rows, flags, counts) + correlate_tc_kernel per gate"}
+                  "kernels": "pack_kernel (gate rows, flags, counts) + single-pass kernel"}
         del valid, gout, gcounts
         torch.cuda.synchronize()
     # beamforming (Sec. IV-C-3): 16 beams over the same block, int8 weights;

@@ -64,20 +64,21 @@ extern "C" {
 #define XENG_MAX_T_INTEG  16777215LL
 
 /* Correlation engines (all give identical bits). */
-#define XENG_ENGINE_TENSOR        0  /* tcgen05 tensor cores (default): for N <= 3584 a multiple of 16 (block
-                                        16-byte aligned) one kernel splits the raw bytes in shared memory and
-                                        correlates them -- N <= 256: single CTAs over 128-input blocks
-                                        (scratch of 256 KB per SM, allocated at the first such call); above:
-                                        single CTAs over 128-input block pairs or 2-CTA clusters over
-                                        256-input block pairs, whichever does less padded work for N.  The
-                                        environment variable XENG_FUSED_KERNEL=onepass or =pair (read by
-                                        xeng_create) forces one of the two for every such N.  Otherwise as
-                                        XENG_ENGINE_TENSOR_PLANES                                            */
+#define XENG_ENGINE_TENSOR        0  /* tcgen05 tensor cores (default): for N <= 3584 one kernel splits the raw
+                                        bytes in shared memory and correlates them -- single CTAs over items of
+                                        two 128-input blocks (N <= 256; scratch of 256 KB per SM, allocated at
+                                        the first such call), single CTAs over 128-input block pairs or 2-CTA
+                                        clusters over 256-input block pairs, whichever takes least for N and
+                                        the launch's channels and samples.  Blocks that TMA cannot address (N
+                                        not a multiple of 16, or not 16-byte aligned), gated and delayed
+                                        samples are rearranged first (buffer of up to 16 GiB, allocated at the
+                                        first such call).  The environment variable XENG_FUSED_KERNEL=onepass
+                                        or =pair (read by xeng_create) forces one of the two for every such N.
+                                        Otherwise as XENG_ENGINE_TENSOR_PLANES                               */
 #define XENG_ENGINE_DP4A          1  /* plain CUDA-core kernel: int8 dp4a straight from the bytes            */
 #define XENG_ENGINE_TENSOR_PLANES 2  /* two passes: decode to FP8 planes in HBM, then the tensor-core GEMM
                                         (decode buffer of up to 16 GiB, allocated at the first such call)    */
-#define XENG_ENGINE_TENSOR_FUSED  3  /* the default engine's single pass for every N that is a multiple of
-                                        16 (block 16-byte aligned), also above the N up to which the default
+#define XENG_ENGINE_TENSOR_FUSED  3  /* the default engine's single pass also above the N up to which the default
                                         engine takes it (the build parameter XENG_FUSED_MAX_N, 3584): no
                                         decode buffer, about 2% slower than two passes at N = 4096           */
 
@@ -169,7 +170,7 @@ XENG_API int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samp
  *   gate: host int32 [n_samples], a set per sample (values outside
  *   [0, n_gates) drop the sample), or NULL for set 0; valid: device uint8
  *   [n_samples][F][N] (0 = missing or saturated), or NULL for all usable.
- *   Any length (rounds of at most 65,536 samples per set); every sample
+ *   Any length (rounds of at most 32,768 samples per set, 65,536 with planes); every sample
  *   counts against t_integ (XENG_ERR_OVERFLOW, nothing done).  Tensor engine
  *   only (else XENG_ERR_ARG), not while delays are set (XENG_ERR_UNSUPPORTED).
  *   Reads `gate` before returning and synchronizes `stream` (it uploads the

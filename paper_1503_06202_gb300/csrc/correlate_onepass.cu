@@ -6,10 +6,12 @@
 // A separate decode writes two plane bytes per input byte to HBM and the
 // correlation reads them back.  Converting in shared memory instead takes the
 // converter warps' time: each 128 x 128 block pair converts two raw tiles per
-// 1024 MMA cycles (per 128-sample stage), so this kernel runs
-// at about 60% of the MMA rate -- ahead of the two passes while the decode is a
-// large share of the step; the library runs it for N > 256 where ceil(N / 128)
-// is odd (there the 2-CTA kernel over 256-input block pairs pads N the most).
+// 1024 MMA cycles (per 128-sample stage), so this kernel runs at about 70% of the
+// MMA rate (N = 640 x 128 channels x 8192 samples, 615 us; 689 with the MMA and TMA
+// issue in diverged warps and integer offsets) -- ahead of the two passes while the
+// decode is a large share of the step.  Its items are the smallest of the three
+// kernels' and its epilogue overlaps the next item, so it also takes launches of few
+// rounds or few stages whatever N is (single_pass_by_shape).
 // Each CTA (one per SM, cta_group::1) takes upper-triangle tile pairs (I <= J)
 // of 128-input blocks of a channel, channel-major and round-robin over the
 // CTAs, so the CTAs at work at any time share one or two channels' raw bytes in

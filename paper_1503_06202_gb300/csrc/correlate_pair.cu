@@ -18,7 +18,9 @@
 // which with A = x_j, B = x_i is Im of x_i conj(x_j) (each CTA supplies its
 // 128 rows of A and its half of B, so per MMA a CTA reads 8 KB of operands for
 // 128 x 256 x 32 multiply-adds; per stage it converts two 16 KB tiles for 16
-// MMAs, about 2048 tensor cycles).  The 256 x 256 complex accumulator fills
+// MMAs, about 2048 tensor cycles; 2048 inputs x 256 channels x 8192 samples: a stage
+// takes about 2200, an item of 64 stages 155,700 cycles of which the MMAs are 131,000
+// and 12,000 its epilogue).  The 256 x 256 complex accumulator fills
 // all 512 TMEM columns of both CTAs; the epilogue (tcgen05.ld -> int32
 // triangle) follows each pair and cannot overlap the next pair's MMAs, so its
 // stores are laid out for the memory system: per column i, a warp's 32 lanes

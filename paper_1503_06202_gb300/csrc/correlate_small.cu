@@ -32,8 +32,9 @@
 // the others' partial blocks to its own.  A cooperative launch keeps every CTA
 // resident, so the waits end.  Bound by latency where calls are small: N = 256
 // x 8 channels x 4096 samples (12 items of 32 stages) takes 25 us on 144 CTAs,
-// 54-61 us on the 12 that pieces of 32 stages at least allowed; x 64 channels x
-// 1024 samples 23 us (86 us on 24 CTAs).
+// 54-61 us on the 12 that pieces of 32 stages at least allowed.  Where the exchange
+// of partial blocks (about 10 us) would cost more than it saves, the one pass over
+// 128-input block pairs runs instead (single_pass_by_shape).
 //
 // The TMA writes raw tiles with a 128-byte swizzle: rows are samples, each 128
 // input bytes -- the canonical MN-major layout of an 8-bit tcgen05 operand

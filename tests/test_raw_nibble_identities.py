@@ -107,3 +107,30 @@ def test_raw_nibble_sums_stay_exact_in_f32():
     assert np.array_equal(k.astype(np.float32).astype(np.int64), k)
     N = 4096                          # beamformer: 2N K positions of u (<= 15) times a part (<= 15)
     assert 2 * N * 15 * 15 < 2 ** 22  # also inside the float-bit read-out's range
+
+
+# raw_offset.cuh: terms = M + 128 n - 8 S_j, then - 8 S_i, each in f32, one rounding of
+# 2^18 acc + terms, and the float's bits less M's are the integer (both signs of Im)
+@pytest.mark.parametrize("n", [1, 127, 4097, 32768])
+def test_visibilities_from_float_bits(n):
+    f32, M = np.float32, np.float32(12582912.0)
+    ends = np.array([[a, b, c, d] for a in (0, 8, 15) for b in (0, 15) for c in (0, 7, 15) for d in (0, 15)])
+    a, b, c, d = ends.T.astype(np.int64)  # constant nibbles over the launch
+    p, q, pj, qj = a * n, b * n, c * n, d * n
+    raw_re, raw_im = n * (a * c + b * d), n * (b * c - a * d)
+    S_i, D_i, S_j, D_j = p + q, p - q, pj + qj, pj - qj
+    want_re = n * ((a - 8) * (c - 8) + (b - 8) * (d - 8))
+    want_im = n * ((b - 8) * (c - 8) - (a - 8) * (d - 8))
+
+    def bits(raw, scale, terms):  # one rounding, as a fused multiply-add
+        acc = (raw / 2.0 ** 18).astype(f32)
+        assert (acc.astype(np.float64) * 2.0 ** 18 == raw).all()
+        v = (scale * acc.astype(np.float64) + terms.astype(np.float64)).astype(f32)
+        return (v.view(np.uint32) - np.uint32(0x4B400000)).view(np.int32)
+
+    re_j = (M + f32(128 * n)) + f32(-8) * S_j.astype(f32)
+    im_j = M - f32(8) * D_j.astype(f32)
+    terms_re, terms_im = re_j + f32(-8) * S_i.astype(f32), im_j + f32(8) * D_i.astype(f32)
+    assert np.array_equal(bits(raw_re, 2.0 ** 18, terms_re), want_re)
+    assert np.array_equal(bits(raw_im, 2.0 ** 18, terms_im), want_im)
+    assert np.array_equal(bits(-raw_im, -2.0 ** 18, terms_im), want_im)
