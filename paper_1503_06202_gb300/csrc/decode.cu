@@ -17,6 +17,8 @@
 // 1024.0, so the half value is 1024 + u, minus 1032 gives u - 8 exactly) and
 // packs pairs to E4M3 with the hardware converter.  HBM-bound: 1 byte read,
 // 2 bytes written per (input, sample).
+#include <algorithm>
+
 #include "nibble.cuh"
 #include "xeng_internal.h"
 
@@ -228,6 +230,7 @@ decode_shifted_kernel(const uint8_t *__restrict__ block, int64_t t0, int64_t nt,
     const int fl = blockIdx.z;
     const int64_t f = f0 + fl;
     const int tid = threadIdx.x;
+    const int64_t head = sa.head();
     for (int ch = tid; ch < 128 * 8; ch += kDecThreads) {
         const int t = ch >> 3, c = ch & 7;
         const int64_t tt = t0 + tr0 + t;  // sample of the block before the shift
@@ -244,7 +247,7 @@ decode_shifted_kernel(const uint8_t *__restrict__ block, int64_t t0, int64_t nt,
                     if (i >= N) break;
                     const int64_t src = tt - sa.delay[i];
                     const uint32_t byte = src >= 0 ? block[(src * F + f) * N + i]
-                                                   : sa.hist[(sa.row(src) * F + f) * sa.S + sa.slot[i]];
+                                                   : sa.hist[(sa.row(head, src) * F + f) * sa.S + sa.slot[i]];
                     w[m >> 2] = (w[m >> 2] & ~(0xFFu << (8 * (m & 3)))) | (byte << (8 * (m & 3)));
                 }
             }
@@ -266,7 +269,7 @@ __global__ void shift_fixup_kernel(const uint8_t *__restrict__ block, int64_t t0
                                    int32_t f0, int32_t nf, const ShiftArgs sa, const int32_t *__restrict__ inputs,
                                    uint8_t *__restrict__ planes, int64_t t_pad, int64_t n_pad)
 {
-    const int64_t total = (int64_t)nf * sa.S * nt;
+    const int64_t total = (int64_t)nf * sa.S * nt, head = sa.head();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t t = k % nt;
         const int32_t sl = (int32_t)((k / nt) % sa.S);
@@ -274,29 +277,41 @@ __global__ void shift_fixup_kernel(const uint8_t *__restrict__ block, int64_t t0
         const int64_t f = f0 + fl;
         const int32_t i = inputs[sl];
         const int64_t src = t0 + t - sa.delay[i];
-        const uint32_t byte = src >= 0 ? block[(src * F + f) * N + i] : sa.hist[(sa.row(src) * F + f) * sa.S + sl];
+        const uint32_t byte = src >= 0 ? block[(src * F + f) * N + i] : sa.hist[(sa.row(head, src) * F + f) * sa.S + sl];
         const uint32_t codes = nib2_to_e4m3(byte | (byte << 12));  // low nibble -> byte 0, high nibble -> byte 1
         planes[((fl * 2 + 0) * n_pad + i) * t_pad + t] = (uint8_t)(codes >> 8);  // real part: high nibble
         planes[((fl * 2 + 1) * n_pad + i) * t_pad + t] = (uint8_t)(codes & 0xFFu);
     }
 }
 
-// Block sample t0 + k of the delayed inputs goes to the ring's row (head + k) %
-// cap, k < m: a push writes its own samples, whatever the delays (N = 16, 183
+// Block sample t0 + k of the delayed inputs goes to the row k after the last append's
+// end, k < m: a push writes its own samples, whatever the delays (N = 16, 183
 // channels, 4048 samples, 13 inputs delayed 11,662: 100 us of the push when every
-// row of the history was moved).  One row per block in y.
-__global__ void shift_history_kernel(uint8_t *__restrict__ hist, const uint8_t *__restrict__ block, int64_t t0,
-                                     int64_t m, int32_t F, int32_t N, const int32_t *__restrict__ inputs, int32_t S,
-                                     int64_t cap, int64_t head)
+// row of the history was moved).  The last block to finish, every block having read
+// the state, makes this append the last one.  Int: m F S fits.
+template <typename Int>
+__global__ void __launch_bounds__(256)
+shift_history_kernel(uint8_t *__restrict__ hist, const uint8_t *__restrict__ block, int64_t t0,
+                     int64_t m, int32_t F, int32_t N, const int32_t *__restrict__ inputs, int32_t S,
+                     int64_t cap, int64_t *state)
 {
-    const int64_t cols = (int64_t)F * S;
-    for (int64_t k = blockIdx.y; k < m; k += gridDim.y) {
-        const uint8_t *src = block + (t0 + k) * F * N;
+    const Int cols = (Int)F * (Int)S, total = (Int)m * cols;
+    int64_t head = state[0] + state[1];
+    if (head >= cap) head -= cap;
+    #pragma unroll 4
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < (int64_t)total; e += (int64_t)gridDim.x * blockDim.x) {
+        const Int k = (Int)e / cols, c = (Int)e - k * cols, f = c / (Int)S;
         const int64_t r = head + k;
-        uint8_t *dst = hist + (r >= cap ? r - cap : r) * cols;
-        for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < cols; c += (int64_t)gridDim.x * blockDim.x) {
-            const int64_t f = c / S;
-            dst[c] = src[f * N + inputs[c - f * S]];
+        hist[(r >= cap ? r - cap : r) * (int64_t)cols + c] = block[((t0 + k) * F + f) * N + inputs[c - f * S]];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        unsigned long long *ticket = reinterpret_cast<unsigned long long *>(state + 2);
+        if (atomicAdd(ticket, 1ull) == (unsigned long long)gridDim.x - 1) {
+            state[0] = head;
+            state[1] = m;
+            *ticket = 0;
         }
     }
 }
@@ -327,17 +342,14 @@ cudaError_t launch_shift_fixup(const uint8_t *block, int64_t t0, int64_t nt, int
 }
 
 cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0, int64_t m, int32_t F, int32_t N,
-                                 const int32_t *inputs, int32_t S, int64_t cap, int64_t head, cudaStream_t s)
+                                 const int32_t *inputs, int32_t S, int64_t cap, int64_t *state, cudaStream_t s)
 {
     const int64_t cols = (int64_t)F * S;
     if (m <= 0 || cols <= 0) return cudaSuccess;
-    if (m > cap || head < 0 || head >= cap) return cudaErrorInvalidValue;
-    const int threads = cols < 256 ? (int)round_up(cols, 32) : 256;
-    int64_t bx = (cols + threads - 1) / threads;
-    if (bx > 1024) bx = 1024;
-    const int64_t by = m < 65535 ? m : 65535;
-    shift_history_kernel<<<dim3((unsigned)bx, (unsigned)by), threads, 0, s>>>(hist, block, t0, m, F, N, inputs, S, cap,
-                                                                              head);
+    if (m > cap) return cudaErrorInvalidValue;
+    const int64_t total = m * cols, blocks = std::min<int64_t>((total + 1023) / 1024, 4096);  // a ticket a block
+    auto kernel = total < 0x80000000LL ? shift_history_kernel<uint32_t> : shift_history_kernel<uint64_t>;
+    kernel<<<(unsigned)blocks, 256, 0, s>>>(hist, block, t0, m, F, N, inputs, S, cap, state);
     return cudaGetLastError();
 }
 

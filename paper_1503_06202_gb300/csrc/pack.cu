@@ -177,6 +177,7 @@ pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols
             delayed |= 1u << m;
         }
     const uint8_t *ring = sa.hist + f * sa.S + slot0;
+    const int64_t head = sa.head();
     uint8_t *out = a.out + (int64_t)c * a.pitch + j * 16;
     for (int64_t t = first; t < last; t += (int64_t)kPackRows * rows_per_block) {
         Loaded16 x[kPackRows];
@@ -201,7 +202,7 @@ pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols
             #pragma unroll
             for (int k = 0; k < kPackRows; k++) {
                 const int64_t src = min(t + (int64_t)k * rows_per_block, last - 1) - d;
-                const uint8_t *from = !kAhead && src >= 0 ? blk + src * row_bytes + m : ring + sa.row(src) * ring_bytes + s;
+                const uint8_t *from = !kAhead && src >= 0 ? blk + src * row_bytes + m : ring + sa.row(head, src) * ring_bytes + s;
                 b[k] = 0x01010101u * __ldg(from);
             }
             #pragma unroll

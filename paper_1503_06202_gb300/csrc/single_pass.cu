@@ -210,6 +210,11 @@ cudaError_t launch_single_pass_shaped(int kernel, const uint8_t *block, int64_t 
                                       SmallScratch *sc, int *err, int num_sms, cudaStream_t s, int32_t pitch,
                                       const SubBlocks *sub, int64_t *launches)
 {
+    if (kernel == kSingleSmall) {
+        // with the first launch, whichever kernel that takes: a later one may be captured
+        const cudaError_t e0 = small_scratch_alloc(sc, num_sms, s);
+        if (e0 != cudaSuccess) return e0;
+    }
     const int k = single_pass_by_shape(kernel, N, nf, nt, accumulate, num_sms);
     const int32_t cut = k == kSinglePair ? pair_rounds_cut(N, nf, nt, accumulate, num_sms) : 0;
     const int32_t first = cut ? cut : nf;

@@ -71,7 +71,8 @@ struct xeng_s {
     int32_t n_shift_chunks[4] = {0, 0, 0, 0};
     SubBlocks shift_blocks{};           // those blocks (n of them; `packed` is set per launch)
     uint8_t *hist = nullptr;
-    int64_t hist_cap = 0, hist_head = 0;
+    int64_t hist_cap = 0;
+    int64_t *hist_state = nullptr;  // ShiftArgs::state
     bool hist_ahead = false;  // it also takes a round's samples before they are integrated
     int32_t hist_S = 0;
     bool decode_tma = false;       // decode through the TMA pipeline where the block allows it
@@ -133,13 +134,14 @@ void free_shift(xeng_s *h)
     cudaFree(h->d_shift_inputs);
     cudaFree(h->d_shift_chunks);
     cudaFree(h->hist);
+    cudaFree(h->hist_state);
     h->d_delay = h->d_slot = h->d_chunk_delay = h->d_shift_inputs = nullptr;
     h->d_shift_chunks = nullptr;
     h->hist = nullptr;
+    h->hist_state = nullptr;
     h->shifted = false;
     h->hist_cap = 0;
     h->hist_S = 0;
-    h->hist_head = 0;
 }
 
 int cuda_status(cudaError_t e)
@@ -532,6 +534,8 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
         e = cudaMemcpy(h->d_chunk_delay, chunk.data(), sizeof(int32_t) * chunk.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_shift_inputs, inputs.data(), sizeof(int32_t) * S, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&h->hist_state, 3 * sizeof(int64_t));
+    if (e == cudaSuccess) e = cudaMemset(h->hist_state, 0, 3 * sizeof(int64_t));
     if (e == cudaSuccess) e = cudaMemset(h->hist, 0x88, (size_t)(cap * row));  // value 0 + 0i
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
@@ -666,10 +670,8 @@ bool integrate_sets(xeng_s *h, int kernel, const uint8_t *dblock, int32_t G, con
 cudaError_t advance_history(xeng_s *h, const uint8_t *dblock, int64_t t0, int64_t n, cudaStream_t s)
 {
     const int64_t m = std::min(n, h->hist_cap);
-    cudaError_t e = launch_shift_history(h->hist, dblock, t0 + n - m, m, h->F, h->N, h->d_shift_inputs, h->hist_S,
-                                         h->hist_cap, h->hist_head, s);
-    if (e == cudaSuccess) h->hist_head = (h->hist_head + m) % h->hist_cap;
-    return e;
+    return launch_shift_history(h->hist, dblock, t0 + n - m, m, h->F, h->N, h->d_shift_inputs, h->hist_S, h->hist_cap,
+                                h->hist_state, s);
 }
 
 // The same with the handle's delays applied to samples 0 .. n - 1 of the block:
@@ -690,6 +692,7 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
     sa.hist = h->hist;
     sa.cap = h->hist_cap;
     sa.S = h->hist_S;
+    sa.state = h->hist_state;
     sa.ahead = h->hist_ahead;
     PackArgs p;
     p.block = dblock;
@@ -704,7 +707,6 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
     for (int64_t t0 = 0; t0 < n && e == cudaSuccess; t0 += kFusedMaxSamples) {
         p.nt = std::min<int64_t>(kFusedMaxSamples, n - t0);
         p.t0 = t0;
-        sa.head = h->hist_head;
         if (h->hist_ahead) e = advance_history(h, dblock, t0, p.nt, s);
         const int64_t group = std::min<int64_t>(65535, h->packed_bytes / (p.nt * p.pitch));
         for (int64_t f0 = 0; f0 < F && e == cudaSuccess; f0 += group) {
@@ -783,7 +785,7 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
                 sa.chunk_delay = h->d_chunk_delay;
                 sa.hist = h->hist;
                 sa.cap = h->hist_cap;
-                sa.head = h->hist_head;
+                sa.state = h->hist_state;
                 sa.S = h->hist_S;
                 e = timed_launch(h, 0, s, [&] {
                     if (h->decode_tma && decode_tma_ok(src, (int32_t)N)) {

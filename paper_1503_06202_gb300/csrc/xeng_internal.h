@@ -93,14 +93,22 @@ struct ShiftArgs {
     const int32_t *slot = nullptr;         // [N] history column of input i (-1: not delayed), in the inputs' order
     const int32_t *chunk_delay = nullptr;  // [ceil(N/16)] delay shared by inputs 16c..16c+15, or -1
     // [cap][F][S] samples of the delayed inputs, a ring of rows: sample 0 of the
-    // block (or of the launch, see launch_pack_shifted) belongs at row head, and
+    // block (or of the launch, see launch_pack_shifted) belongs at row head(), and
     // every sample from max(delay) before it on is there
     const uint8_t *hist = nullptr;
-    int64_t cap = 0, head = 0;
+    // where: {row of the last append's first sample, its rows, a ticket}, in device
+    // memory, so that captured pushes go on from where the ring is when they run
+    const int64_t *state = nullptr;
+    int64_t cap = 0;
     int32_t S = 0;
-    int32_t ahead = 0;  // != 0: the launch's own samples are there too
-    // the ring's row of sample src, |src| <= cap
-    __host__ __device__ int64_t row(int64_t src) const
+    int32_t ahead = 0;  // != 0: the launch's own samples are there too, appended last
+    __device__ int64_t head() const
+    {
+        const int64_t r = state[0] + (ahead ? 0 : state[1]);
+        return r >= cap ? r - cap : r;
+    }
+    // the row of sample src, |src| <= cap
+    __device__ int64_t row(int64_t head, int64_t src) const
     {
         const int64_t r = head + src;
         return r < 0 ? r + cap : r >= cap ? r - cap : r;
@@ -148,10 +156,10 @@ cudaError_t launch_decode_tma_batch(const CUtensorMap *maps, const DecTmaJob *jo
 cudaError_t launch_shift_fixup(const uint8_t *block, int64_t t0, int64_t nt, int32_t F, int32_t N, int32_t f0,
                                int32_t nf, const ShiftArgs &sa, const int32_t *inputs, uint8_t *planes, int64_t t_pad,
                                int64_t n_pad, cudaStream_t s);
-// Samples t0 .. t0 + m - 1 of the block's S delayed inputs, listed in `inputs`,
-// into the ring's rows head, head + 1, ... (modulo cap; m <= cap).
+// Appends samples t0 .. t0 + m - 1 of the block's S delayed inputs, listed in
+// `inputs`, to the ring (m <= cap) and updates its state (ShiftArgs).
 cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0, int64_t m, int32_t F, int32_t N,
-                                 const int32_t *inputs, int32_t S, int64_t cap, int64_t head, cudaStream_t s);
+                                 const int32_t *inputs, int32_t S, int64_t cap, int64_t *state, cudaStream_t s);
 
 // Raw samples rearranged into rows of `pitch` bytes (a multiple of 16) per
 // channel, out[nt][nf][pitch], for a single-pass launch: row t is the block's
@@ -161,8 +169,8 @@ cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0
 // may be null.  `chunks` (device memory): only these 16-byte chunks of the rows, as
 // (position in the packed row, 16-input chunk of the block); null: chunk k is
 // chunk k.  launch_pack_shifted takes the chunks that hold delayed inputs and
-// applies the delays of `sa`, whose ring has to hold the launch's samples already
-// (head: row of sample t0) where sa.ahead.  nt <= kMaxChunkSamples.  launch_pack with
+// applies the delays of `sa` (head(): row of sample t0), whose ring has to hold the
+// launch's samples already where sa.ahead.  nt <= kMaxChunkSamples.  launch_pack with
 // sets > 0: that many lists of samples side by side, out[nt][sets][nf][pitch] and
 // counts[sets][nf][N], set k's samples idx[set_first[k]] .. idx[set_first[k + 1] - 1],
 // its rows past them 0x88.

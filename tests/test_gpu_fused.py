@@ -302,3 +302,25 @@ def test_default_engine_at_its_single_pass_bound(N):
     assert np.array_equal(got, oracle.correlate(blk))
     if N > 3584:
         assert np.array_equal(correlate(blk, engine=FUSED), got)
+
+
+# A short first launch takes the one pass, but has the N <= 256 kernel's scratch made:
+# a long one may be captured next
+def test_long_launch_captured_after_a_short_one():
+    T, F, N = 6000, 2, 256
+    blk = np.random.default_rng(3).integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    block = torch.from_numpy(blk).cuda()
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    eng = xe.XEngine(N, F, T)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    eng.correlate(block, out, 128, s.cuda_stream)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        eng.correlate(block, out, T, s.cuda_stream)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk))
+    eng.close()

@@ -180,3 +180,33 @@ def test_shift_history_without_room_for_a_round():
             got = out[[0, F - 1]].cpu().numpy().astype(np.int64)
             assert np.array_equal(got, oracle.correlate_shifted(np.ascontiguousarray(stream[:, [0, F - 1]]), d, t_a, t))
     eng.close()
+
+
+# A captured push and dump, replayed: every replay goes on from where the history's
+# ring is, pushes of 300 samples shorter than the delays, an odd number of replays
+def test_shift_captured_pushes():
+    N, F, n = 272, 2, 300
+    d = np.zeros(N, np.int32)
+    d[[3, 130]] = 700, 41
+    stream = np.random.default_rng(8).integers(0, 256, size=(6 * n, F, N), dtype=np.uint8)
+    eng = xe.XEngine(N, F, 4096)
+    eng.set_delays(d)
+    block = torch.from_numpy(stream[:n]).cuda()
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    eng.push(block, n, side.cuda_stream)
+    assert eng.dump(out, side.cuda_stream) == n
+    side.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        eng.push(block, n, side.cuda_stream)
+        eng.dump(out, side.cuda_stream)
+    for k in range(1, 6):
+        block.copy_(torch.from_numpy(stream[k * n:(k + 1) * n]))
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        want = oracle.correlate_shifted(stream[:(k + 1) * n], d, k * n, (k + 1) * n)
+        assert np.array_equal(out.cpu().numpy().astype(np.int64), want), k
+    eng.close()
