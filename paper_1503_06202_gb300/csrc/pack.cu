@@ -22,6 +22,30 @@ constexpr int kPackThreads = 256;
 constexpr int kPackRows = 4;       // rows loaded before any is stored
 constexpr int kPackSpan = 256;     // rows per thread at most (byte-lane counts are widened every 240)
 
+// Blocks of 256 threads over the `all` columns of a row (all of them, or 256) and,
+// where a row is shorter, several rows; each thread walks at most kPackSpan rows, fewer
+// where that would leave SMs without a few blocks each.
+struct PackGrid {
+    int64_t all = 0;
+    int cols = 1, rows = 1, span = 1, nx = 0, ny = 0;  // nx * ny blocks a set
+};
+
+PackGrid pack_grid(const PackArgs &a, int64_t all, int num_sms)
+{
+    PackGrid g;
+    if (all <= 0) return g;
+    g.all = all;
+    g.cols = (int)(all < kPackThreads ? all : kPackThreads);
+    g.rows = kPackThreads / g.cols;
+    const int64_t nx = (all + g.cols - 1) / g.cols, sets = a.sets > 0 ? a.sets : 1;
+    auto ny = [&]() { return (a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows); };
+    g.span = kPackSpan;
+    while (g.span > 2 * kPackRows && sets * nx * ny() < 16 * num_sms) g.span /= 2;
+    g.nx = (int)nx;
+    g.ny = (int)ny();
+    return g;
+}
+
 // The 16 bytes at p, any alignment, of which the first n are wanted (the rest
 // may come out as anything): only 16-byte words that hold a wanted byte are read.
 // Without branches, so that several rows' loads are in flight at once.
@@ -63,13 +87,14 @@ __device__ __forceinline__ void pack_column(const PackArgs &a, int64_t col, int 
 }
 
 // kAligned: every source chunk is 16-byte aligned.  Thread = (row of the block's
-// rows, chunk of a sample); blockIdx.z: set.
+// rows, chunk of a sample); block (bx, by) of set `set`.
 template <bool kAligned, bool kValid>
-__global__ void __launch_bounds__(kPackThreads)
-pack_kernel(const __grid_constant__ PackArgs a, int64_t cols, int cols_per_block, int rows_per_block, int span)
+__device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, int bx, int by, int set)
 {
+    const int64_t cols = g.all;
+    const int cols_per_block = g.cols, rows_per_block = g.rows, span = g.span;
     constexpr int kRows = !kAligned && kValid ? kPackRows / 2 : kPackRows;  // registers
-    const int64_t col = (int64_t)blockIdx.x * cols_per_block + threadIdx.x % cols_per_block;
+    const int64_t col = (int64_t)bx * cols_per_block + threadIdx.x % cols_per_block;
     const int rsub = threadIdx.x / cols_per_block;
     if (col >= cols || rsub >= rows_per_block) return;
     int c, j, ic;
@@ -77,12 +102,11 @@ pack_kernel(const __grid_constant__ PackArgs a, int64_t cols, int cols_per_block
     const int n = min(16, a.N - ic);
     const int64_t row_bytes = (int64_t)a.F * a.N;
     const int64_t off = (int64_t)(a.f0 + c) * a.N + ic;
-    const int set = (int)blockIdx.z;
     const int32_t *idx = a.sets ? a.idx + a.set_first[set] : a.idx;
     const int64_t have = a.sets ? a.set_first[set + 1] - a.set_first[set] : a.nt;
     const int64_t out_row = (int64_t)a.nf * a.pitch * max(a.sets, 1);
-    const int64_t first = (int64_t)blockIdx.y * span * rows_per_block + rsub;
-    const int64_t end = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
+    const int64_t first = (int64_t)by * span * rows_per_block + rsub;
+    const int64_t end = min(a.nt, ((int64_t)by + 1) * span * rows_per_block);
     const int64_t last = min(have, end);
     uint8_t *out = a.out + ((int64_t)set * a.nf + c) * a.pitch + j * 16;
     uint32_t acc[4] = {0, 0, 0, 0};                       // usable samples, a byte per input
@@ -149,15 +173,16 @@ pack_kernel(const __grid_constant__ PackArgs a, int64_t cols, int cols_per_block
 // The chunks that hold a delayed input: copied, with the delayed inputs' samples
 // from the history's ring, which holds the launch's too -- their rows are dense
 // there, so that reading them d samples back stays in L2, where the block's rows
-// do not.  Launched over these chunks alone: among plain ones they kept whole
-// warps waiting (N = 496 x 188 channels x 30,415 samples, 7 inputs delayed, 1.9 ms
-// for all chunks in one launch).  !kAhead, where a ring of that size would not be
+// do not.  In blocks of their own: among plain ones they kept whole warps waiting
+// (N = 496 x 188 channels x 30,415 samples, 7 inputs delayed, 1.9 ms with the two
+// mixed, 1.58 as two launches, 1.52 as the blocks of one).  !kAhead, where a ring of that size would not be
 // worth its memory: the launch's own samples from the block.
 template <bool kAhead>
-__global__ void __launch_bounds__(kPackThreads)
-pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols_per_block, int rows_per_block, int span)
+__device__ __forceinline__ void pack_shifted_rows(const PackArgs &a, const ShiftArgs &sa, const PackGrid &g, int bx, int by)
 {
-    const int64_t col = (int64_t)blockIdx.x * cols_per_block + threadIdx.x % cols_per_block;
+    const int64_t cols = g.all;
+    const int cols_per_block = g.cols, rows_per_block = g.rows, span = g.span;
+    const int64_t col = (int64_t)bx * cols_per_block + threadIdx.x % cols_per_block;
     const int rsub = threadIdx.x / cols_per_block;
     if (col >= cols || rsub >= rows_per_block) return;
     int c, j, ic;
@@ -167,8 +192,8 @@ pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols
     const int64_t row_bytes = (int64_t)a.F * a.N, ring_bytes = (int64_t)a.F * sa.S;
     const uint8_t *blk = a.block + a.t0 * row_bytes + f * a.N + ic;
     const int64_t out_row = (int64_t)a.nf * a.pitch;
-    const int64_t first = (int64_t)blockIdx.y * span * rows_per_block + rsub;
-    const int64_t last = min(a.nt, ((int64_t)blockIdx.y + 1) * span * rows_per_block);
+    const int64_t first = (int64_t)by * span * rows_per_block + rsub;
+    const int64_t last = min(a.nt, ((int64_t)by + 1) * span * rows_per_block);
     int slot0 = -1;        // ring column of the chunk's first delayed input
     uint32_t delayed = 0;  // its delayed inputs
     for (int m = 0; m < n; m++)
@@ -223,25 +248,21 @@ pack_shifted_kernel(const PackArgs a, const ShiftArgs sa, int64_t cols, int cols
     }
 }
 
-// Blocks of 256 threads over the `cols` columns of a row (all of them, or 256) and,
-// where a row is shorter, several rows; each thread walks at most kPackSpan rows, fewer
-// where that would leave SMs without a few blocks each.
-struct PackGrid {
-    dim3 grid;
-    int cols, rows, span;
-};
-
-PackGrid pack_grid(const PackArgs &a, int64_t cols, int num_sms)
+template <bool kAligned, bool kValid>
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ PackArgs a, const PackGrid g)
 {
-    PackGrid g;
-    g.cols = (int)(cols < kPackThreads ? cols : kPackThreads);
-    g.rows = kPackThreads / g.cols;
-    const int64_t bx = (cols + g.cols - 1) / g.cols, bz = a.sets > 0 ? a.sets : 1;
-    g.span = kPackSpan;
-    while (g.span > 2 * kPackRows && bz * bx * ((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)) < 16 * num_sms)
-        g.span /= 2;
-    g.grid = dim3((unsigned)bx, (unsigned)((a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows)), (unsigned)bz);
-    return g;
+    pack_rows<kAligned, kValid>(a, g, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
+}
+
+// The chunks of `a` and, after their blocks, those of `b`, which hold delayed inputs.
+template <bool kAligned, bool kAhead>
+__global__ void __launch_bounds__(kPackThreads)
+pack_shifted_kernel(const __grid_constant__ PackArgs a, const __grid_constant__ PackArgs b,
+                    const __grid_constant__ ShiftArgs sa, const PackGrid ga, const PackGrid gb)
+{
+    const int na = ga.nx * ga.ny, x = (int)blockIdx.x;
+    if (x < na) pack_rows<kAligned, false>(a, ga, x % ga.nx, x / ga.nx, 0);
+    else pack_shifted_rows<kAhead>(b, sa, gb, (x - na) % gb.nx, (x - na) / gb.nx);
 }
 
 bool pack_args_ok(const PackArgs &a)
@@ -250,30 +271,44 @@ bool pack_args_ok(const PackArgs &a)
            (reinterpret_cast<uintptr_t>(a.out) & 15) == 0;
 }
 
+bool rows_aligned(const PackArgs &a)
+{
+    return a.N % 16 == 0 && (reinterpret_cast<uintptr_t>(a.block) & 15) == 0 &&
+           (reinterpret_cast<uintptr_t>(a.valid) & 15) == 0;
+}
+
 }  // namespace
 
 cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s)
 {
-    const int64_t cols = (int64_t)a.nf * (a.chunks ? a.n_chunks : a.pitch / 16);
+    const int64_t cols = (int64_t)a.nf * (a.pitch / 16);
     if (cols <= 0 || a.nt <= 0) return cudaSuccess;
-    if (!pack_args_ok(a) || (!a.chunks && a.pitch < a.N) || a.sets > kMaxGates || (a.sets > 0 && !a.idx)) return cudaErrorInvalidValue;
+    if (!pack_args_ok(a) || a.chunks || a.pitch < a.N || a.sets > kMaxGates || (a.sets > 0 && !a.idx))
+        return cudaErrorInvalidValue;
     const PackGrid g = pack_grid(a, cols, num_sms);
-    const bool aligned = a.N % 16 == 0 && (reinterpret_cast<uintptr_t>(a.block) & 15) == 0 &&
-                         (reinterpret_cast<uintptr_t>(a.valid) & 15) == 0;
+    const bool aligned = rows_aligned(a);
     auto kernel = a.valid ? (aligned ? pack_kernel<true, true> : pack_kernel<false, true>)
                           : (aligned ? pack_kernel<true, false> : pack_kernel<false, false>);
-    kernel<<<g.grid, kPackThreads, 0, s>>>(a, cols, g.cols, g.rows, g.span);
+    kernel<<<dim3((unsigned)g.nx, (unsigned)g.ny, a.sets > 0 ? a.sets : 1), kPackThreads, 0, s>>>(a, g);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_sms, cudaStream_t s)
+cudaError_t launch_pack_shifted(const PackArgs &a, int32_t n_shifted, const ShiftArgs &sa, int num_sms, cudaStream_t s)
 {
-    const int64_t cols = (int64_t)a.nf * a.n_chunks;
-    if (cols <= 0 || a.nt <= 0) return cudaSuccess;
-    if (!pack_args_ok(a) || !a.chunks) return cudaErrorInvalidValue;
-    const PackGrid g = pack_grid(a, cols, num_sms);
-    auto kernel = sa.ahead ? pack_shifted_kernel<true> : pack_shifted_kernel<false>;
-    kernel<<<g.grid, kPackThreads, 0, s>>>(a, sa, cols, g.cols, g.rows, g.span);
+    if (a.nf <= 0 || a.nt <= 0 || a.n_chunks + n_shifted <= 0) return cudaSuccess;
+    if (!pack_args_ok(a) || !a.chunks || a.n_chunks < 0 || n_shifted < 0 || a.valid || a.idx || a.sets)
+        return cudaErrorInvalidValue;
+    PackArgs b = a;
+    b.chunks = a.chunks + a.n_chunks;
+    b.n_chunks = n_shifted;
+    const PackGrid ga = pack_grid(a, (int64_t)a.nf * a.n_chunks, num_sms);
+    const PackGrid gb = pack_grid(b, (int64_t)b.nf * b.n_chunks, num_sms);
+    const int64_t blocks = (int64_t)ga.nx * ga.ny + (int64_t)gb.nx * gb.ny;
+    if (blocks > 2147483647LL) return cudaErrorInvalidValue;
+    const bool aligned = rows_aligned(a);
+    auto kernel = sa.ahead ? (aligned ? pack_shifted_kernel<true, true> : pack_shifted_kernel<false, true>)
+                           : (aligned ? pack_shifted_kernel<true, false> : pack_shifted_kernel<false, false>);
+    kernel<<<(unsigned)blocks, kPackThreads, 0, s>>>(a, b, sa, ga, gb);
     return cudaGetLastError();
 }
 

@@ -713,16 +713,9 @@ cudaError_t integrate_shifted(xeng_s *h, int kernel, const uint8_t *dblock, int6
             p.f0 = (int32_t)f0;
             p.nf = (int32_t)std::min<int64_t>(group, F - f0);
             const int accumulate = fresh && t0 == 0 ? 0 : 1;
-            e = timed_launch(h, 0, s, [&] {
-                p.chunks = plain;
-                p.n_chunks = nc[0];
-                const cudaError_t e2 = launch_pack(p, h->num_sms, s);
-                if (e2 != cudaSuccess) return e2;
-                if (nc[0] > 0) h->stats.launches++;
-                p.chunks = plain + nc[0];
-                p.n_chunks = nc[1];
-                return launch_pack_shifted(p, sa, h->num_sms, s);
-            });
+            p.chunks = plain;
+            p.n_chunks = nc[0];
+            e = timed_launch(h, 0, s, [&] { return launch_pack_shifted(p, nc[1], sa, h->num_sms, s); });
             if (e != cudaSuccess) break;
             sub.F = p.nf;
             e = timed_launch(h, 1, s, [&] {

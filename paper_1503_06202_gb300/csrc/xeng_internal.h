@@ -166,11 +166,12 @@ cudaError_t launch_shift_history(uint8_t *hist, const uint8_t *block, int64_t t0
 // sample t0 + t, or idx[t] where idx (device memory) is given; channels
 // f0 .. f0 + nf - 1.  launch_pack (pitch >= N) also replaces samples whose
 // `valid` byte is 0 by 0x88 and adds the usable samples to counts[nf][N]; both
-// may be null.  `chunks` (device memory): only these 16-byte chunks of the rows, as
-// (position in the packed row, 16-input chunk of the block); null: chunk k is
-// chunk k.  launch_pack_shifted takes the chunks that hold delayed inputs and
-// applies the delays of `sa` (head(): row of sample t0), whose ring has to hold the
-// launch's samples already where sa.ahead.  nt <= kMaxChunkSamples.  launch_pack with
+// may be null.  launch_pack_shifted takes two lists of 16-byte chunks, `chunks`
+// (device memory; position in the packed row, 16-input chunk of the block): n_chunks
+// that are copied and then n_shifted that hold delayed inputs, to which it applies the
+// delays of `sa` (head(): row of sample t0), whose ring has to hold the launch's
+// samples already where sa.ahead; the others of the row are left as they are.  nt <=
+// kMaxChunkSamples.  launch_pack with
 // sets > 0: that many lists of samples side by side, out[nt][sets][nf][pitch] and
 // counts[sets][nf][N], set k's samples idx[set_first[k]] .. idx[set_first[k + 1] - 1],
 // its rows past them 0x88.
@@ -189,7 +190,7 @@ struct PackArgs {
     int32_t set_first[kMaxGates + 1];
 };
 cudaError_t launch_pack(const PackArgs &a, int num_sms, cudaStream_t s);
-cudaError_t launch_pack_shifted(const PackArgs &a, const ShiftArgs &sa, int num_sms, cudaStream_t s);
+cudaError_t launch_pack_shifted(const PackArgs &a, int32_t n_shifted, const ShiftArgs &sa, int num_sms, cudaStream_t s);
 
 // What the three single-pass launches below share.  A block's rows are `pitch`
 // bytes per channel (0: N), a multiple of 16; N itself need not be one.  With
