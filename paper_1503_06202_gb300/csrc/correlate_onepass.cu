@@ -46,6 +46,7 @@
 //   warps 2..9   converters: raw slot -> Im and Re planes of a plane stage, nibble sums
 //   warps 10..17 epilogue: TMEM -> packed int32 triangle, two warps per TMEM lane
 //                quadrant taking alternate 8-column chunks
+//   warp 18      (adding launches, 608 threads) the next item's triangle, to L2
 #include <cstring>
 
 #include "raw_offset.cuh"
@@ -86,7 +87,12 @@ constexpr int kOPlanes = XENG_ONEPASS_PLANE_STAGES, kORaws = XENG_ONEPASS_RAW_SL
 #endif
 constexpr int kOConvWarp0 = 2, kOConvWarps = XENG_ONEPASS_CONV_WARPS;
 constexpr int kOEpiWarp0 = kOConvWarp0 + kOConvWarps, kOEpiWarps = XENG_ONEPASS_EPI_WARPS;
-constexpr int kOThreads = 32 * (kOEpiWarp0 + kOEpiWarps);
+// Adding launches: a warp more, which fetches the triangle of the next item to L2
+// (issued by the epilogue's own warps, 2900 of an item's 13,000 cycles at two stages:
+// N = 512 x 256 channels x 256 samples 121 us a push, 110 so; bulk prefetches instead
+// 109, but 27 us for 25 at N = 128 x 512 channels).
+constexpr int kOAheadWarp = kOEpiWarp0 + kOEpiWarps;
+__host__ __device__ constexpr int onepass_threads(bool add) { return 32 * (kOAheadWarp + (add ? 1 : 0)); }
 constexpr int kOCT = 16 * kOConvWarps;        // converter threads per tile
 constexpr int kOChunks = kOBox / 16 / kOCT;   // 16-byte chunks of a tile per converter thread and stage
 static_assert(kOConvWarps == 8 || kOConvWarps == 16, "8 or 16 converter warps");
@@ -160,7 +166,7 @@ __device__ __forceinline__ OnepassItem onepass_item(const OnepassArgs &a, int it
 // instead of storing it; a separate instantiation, so the storing epilogue
 // keeps two chunks' TMEM words in registers without spilling.
 template <bool kAdd>
-__global__ void __launch_bounds__(kOThreads, 1)
+__global__ void __launch_bounds__(onepass_threads(kAdd), 1)
 correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap sub_map,
                          const __grid_constant__ OnepassArgs a)
 {
@@ -204,7 +210,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(accf(b), 1);
-            mbar_init(acce(b), kOEpiWarps);
+            mbar_init(acce(b), kOEpiWarps + (kAdd ? 1 : 0));
         }
         mbar_init(drain, 1);
         for (int par = 0; par < 2; par++) {
@@ -214,7 +220,7 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(&raw_map) : "memory");
     }
-    for (int k = threadIdx.x; k < 2 * kOSumPar; k += kOThreads) sums[k] = make_int2(0, 0);
+    for (int k = threadIdx.x; k < 2 * kOSumPar; k += onepass_threads(kAdd)) sums[k] = make_int2(0, 0);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(kOTmemCols));
@@ -322,6 +328,24 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
             // Drain: every MMA issued above has finished once this completes.
             if (elect_one()) mma_commit(drain);
             (void)mbar_wait(drain, 0u, err, kDevTimeoutMma);
+        }
+    } else if (kAdd && warp == kOAheadWarp) {
+        // ---------------- the triangle of the items to come, to L2 (adding launches) ----------------
+        int local = 0;
+        for (int it = it_begin; it < a.n_items; it += it_step, ++local) {
+            const OnepassItem w = onepass_item(a, it);
+            const int2 *out = reinterpret_cast<const int2 *>(a.acc) + (int64_t)w.fl * ((int64_t)a.N * (a.N + 1) / 2);
+            // (a long launch's first item: its fetches would only meet the epilogue's own)
+            #pragma unroll 1
+            for (int q = 0; q < 4 && (local > 0 || n_k < 32); q++)
+                prefetch_triangle(out, a.N, w.J * 128 + 32 * q, w.I * 128, w.I * 128 + 128, 8, lane);
+            // one item ahead of the epilogue; the accumulator goes back only with this
+            // arrival too, so that no phase of its barrier passes unseen
+            const int ab = local & 1;
+            if (!__all_sync(0xffffffffu,
+                            mbar_wait_backoff(accf(ab), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128)))
+                break;
+            if (lane == 0) mbar_arrive(acce(ab));
         }
     } else if (warp < kOEpiWarp0) {
         // ---------------- converters ----------------
@@ -491,11 +515,6 @@ correlate_onepass_kernel(const __grid_constant__ CUtensorMap raw_map, const __gr
                 }
             };
             int2 old0[8], old1[8];  // of the warp's next two chunks
-            if (kAdd && it + it_step < a.n_items) {  // the next pair's values, to L2
-                const OnepassItem nx = onepass_item(a, it + it_step);
-                prefetch_triangle(reinterpret_cast<const int2 *>(a.acc) + (int64_t)nx.fl * nb2, N, nx.J * 128 + q * 32,
-                                  nx.I * 128 + 8 * half, nx.I * 128 + 128, 8 * kPerQuad, lane);
-            }
             if (kAdd && chunk_ok(8 * half)) load_old(8 * half, old0);  // under the wait for the accumulator
             if (kAdd && chunk_ok(8 * half + 8 * kPerQuad)) load_old(8 * half + 8 * kPerQuad, old1);
             bool ok = mbar_wait_backoff(accf(ab), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
@@ -665,7 +684,7 @@ cudaError_t launch_correlate_onepass(const uint8_t *block, int64_t T_block, int6
     a.sub_f0 = sub ? sub->f0 : 0;
     if (sub) memcpy(a.slot, sub->slot, sizeof a.slot);
     const int grid = n_items < num_sms ? (int)n_items : num_sms;
-    kernel<<<grid, kOThreads, kOSmem, s>>>(map, sub_map, a);
+    kernel<<<grid, onepass_threads(accumulate != 0), kOSmem, s>>>(map, sub_map, a);
     return cudaGetLastError();
 }
 
