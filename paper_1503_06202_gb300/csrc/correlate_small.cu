@@ -31,7 +31,7 @@
 // owner, the CTA holding its first stages (which reaches them last), which adds
 // the others' partial blocks to its own.  A cooperative launch keeps every CTA
 // resident, so the waits end.  Bound by latency where calls are small: N = 256
-// x 8 channels x 4096 samples (12 items of 32 stages) takes 25 us on 144 CTAs,
+// x 8 channels x 4096 samples (12 items of 32 stages) takes 23-24 us on 144 CTAs,
 // 54-61 us on the 12 that pieces of 32 stages at least allowed.  Where the exchange
 // of partial blocks (about 10 us) would cost more than it saves, the one pass over
 // 128-input block pairs runs instead (single_pass_by_shape).
@@ -66,7 +66,8 @@
 //   warp 1       TMEM allocation; MMA issuer
 //   warps 2..9   converters: raw slot -> Re and Im planes of a plane stage, nibble sums
 //   warps 10..17 epilogue: TMEM -> packed int32 triangle, one warp per TMEM lane
-//                quadrant and block of the item
+//                quadrant and block of the item (items shared by up to 14 CTAs: the
+//                converters too, their one piece done)
 #include <cstring>
 
 #include "tc_ptx.cuh"
@@ -119,6 +120,7 @@ constexpr int kSMinPiece = 32;  // evenly cut items: stages per CTA at least
 #ifndef XENG_SMALL_MAX_SHARED
 #define XENG_SMALL_MAX_SHARED 32
 #endif
+constexpr int kSJoin = 14;  // CTAs an item at most for the converters to join its epilogue
 constexpr int kSMinShared = XENG_SMALL_MIN_SHARED, kSMaxShared = XENG_SMALL_MAX_SHARED;
 constexpr int kSChunks = 2 * kSBox / 16 / (32 * kSConvWarps);  // 16-byte chunks per converter thread and stage
 static_assert(kSChunks * 32 * kSConvWarps * 16 == 2 * kSBox, "the converter threads cover both tiles");
@@ -230,9 +232,10 @@ __device__ __forceinline__ SmallItem small_item(const SmallArgs &a, int it)
 }
 
 // kAdd: add into acc (a.accumulate != 0) instead of storing; kShared: several
-// CTAs per item (a.split >= 2).  Templates so that each launch carries only its
+// CTAs per item (a.split >= 2); kJoin: there the converter warps take half of the
+// epilogue (a.split <= kSJoin).  Templates so that each launch carries only its
 // own epilogue (the adding one needs more registers).
-template <bool kAdd, bool kShared>
+template <bool kAdd, bool kShared, bool kJoin>
 __global__ void __launch_bounds__(kSThreads, 1)
 correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap diag_map,
                        const __grid_constant__ CUtensorMap sub_map, const __grid_constant__ SmallArgs a)
@@ -298,6 +301,241 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    bool conv_ok = true;  // a converter's
+    auto epilogue = [&]() {
+        constexpr int warp0 = kJoin ? kSConvWarp0 : kSEpiWarp0;
+        constexpr int tail = 32 * (kSEpiWarp0 + kSEpiWarps - warp0);  // its threads
+        const int q = warp & 3;                     // TMEM lane quadrant this warp may access
+        const int et = (int)threadIdx.x - 32 * warp0;
+        const int h = kJoin ? et >> 7 & 1 : et >> 7;  // the item's block: columns 128h.. of Re and Im
+        constexpr int halves = kJoin ? 2 : 1;       // warps a quadrant and block
+        const int half = kJoin ? et >> 8 : 0;
+        const int row = q * 32 + lane;              // TMEM lane: input j within its 128-input block
+        const int N = a.N;                          // <= 256
+        const int nt = (int)a.nt;
+        const int64_t nb = (int64_t)N * (N + 1) / 2;
+        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
+        // partial blocks in ws: [CTA][block h][chunk c / 8][column pair][row], 16 bytes each,
+        // so that a warp's 32 rows are one 512-byte run
+        constexpr int kWs = 2 * 16 * 4 * 128;    // 16-byte words per CTA
+        const int wsi = h * 16 * 4 * 128 + row;  // + (c / 8) * 512 + 128 per column pair
+        int4 *const ws = reinterpret_cast<int4 *>(a.ws);
+        uint32_t uses = 0;
+        int local = 0;
+        int x = lo;
+        Piece pc;
+        while (next_piece(a, x, hi, pc)) {
+            const SmallItem w = small_item(a, pc.it);
+            const int par = local & 1;
+            // the piece's samples inside the launch: 64 n from each of the two products
+            const float n128 = (float)(128 * ((pc.k1 * kSKc < nt ? pc.k1 * kSKc : nt) - pc.k0 * kSKc));
+            const bool owner = pc.k0 == 0;
+            // an owner whose item runs on: the CTAs after it that hold the rest
+            // (shared items: the item's other CTAs, which this one meets later)
+            const int c_lo = kShared ? pc.it * a.split : (int)blockIdx.x + 1;
+            const int c_hi = kShared ? c_lo + a.split - 1
+                                    : owner && pc.k1 < a.n_k ? stage_cta(a, (pc.it + 1) * a.n_k - 1) : 0;
+            // Block h: column items' inputs j = 128.. against i = 128h..; diagonal items'
+            // channel fx or fy, both 0..127.  Sums: X tile at 0, Y tile at 128.
+            const int fl = w.col ? w.fx : (h ? w.fy : w.fx);
+            const int j_warp = (w.col ? 128 : 0) + q * 32;
+            const int j = j_warp + lane;
+            const int i_base = w.col ? 128 * h : 0;
+            const bool lane_ok = j < N;
+            const bool warp_ok = fl >= 0 && j_warp < N;
+            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
+            // warp-uniform: columns inside the channel and up to some lane's diagonal
+            auto chunk_ok = [&](const int c) { return c < 128 && i_base + c < N && i_base + c <= j_warp + 31; };
+            // the triangle's values of columns c .. c + 7 (adding launches): pair (i, j) sits
+            // at i*N - i*(i-1)/2 + (j - i) in the channel's triangle and row i + 1 starts
+            // N - i - 1 pairs after row i, so per column the warp's 32 consecutive inputs j
+            // are one 256-byte run
+            auto load_old = [&](const int c, int2 (&o)[8]) {
+                const int i0 = i_base + c;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last) o[e] = __ldcg(out + off);
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            int2 old[8];
+            if (kAdd && !kShared) {
+                int nx = x;
+                Piece np;
+                if (next_piece(a, nx, hi, np)) {  // the next item's values, to L2
+                    const SmallItem nw = small_item(a, np.it);
+                    const int nfl = nw.col ? nw.fx : (h ? nw.fy : nw.fx);
+                    if (nfl >= 0 && np.k0 == 0)
+                        prefetch_triangle(reinterpret_cast<const int2 *>(a.acc) + (int64_t)nfl * nb, N,
+                                          (nw.col ? 128 : 0) + q * 32, nw.col ? 128 * h : 0,
+                                          min(N, nw.col ? 128 * h + 128 : 128), 8, lane);
+                }
+                if (owner && warp_ok && chunk_ok(0)) load_old(0, old);  // under the wait for the accumulator
+            }
+            bool ok = (!kJoin || conv_ok) && mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
+            ok = ok && mbar_wait_backoff(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
+            if (et == 0 && !kShared)
+                for (int b = c_lo; ok && b <= c_hi; b++) ok = flag_wait(a.flags + b, *s_epoch, err, kDevTimeoutEpilogue);
+            // the barrier ORs the warps' failures, so they leave together
+            if (bar_any(2, tail, !ok)) break;
+            ++uses;
+            fence_after();
+            // every input's offset terms in place of its sums (read by all the warps)
+            if (!kJoin || et < 256) {
+                const int m = par * kSSumPar + sum_slot(et);
+                terms[m] = offset_terms(sums[m]);
+            }
+            named_bar_sync(2, tail);
+            const float2 *ci = terms + par * kSSumPar + sum_slot(128 * h);  // inputs i of the columns
+            const float2 tj = terms[par * kSSumPar + sum_slot((w.col ? 128 : 128 * h) + row)];
+            const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
+            // TMEM columns of the block: column items Re at 128h.., Im at 256 + 128h..;
+            // diagonal items Re at 256h.., Im (negated) at 256h + 128..
+            const uint32_t tre = taddr + (w.col ? 128u * h : 256u * h);
+            const uint32_t tim = tre + (w.col ? 256u : 128u);
+            const float im_scale = w.col ? kRawScale : -kRawScale;
+            // the piece's visibilities in place of the accumulator words of columns c .. c + 7
+            auto correct = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + sum_slot(c) + e);  // the same for every lane: a broadcast
+                    vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
+                    vim[e] = raw_to_int(vim[e], im_scale, im_j + t2.y);
+                    vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
+                    vim[e + 1] = raw_to_int(vim[e + 1], im_scale, im_j + t2.w);
+                }
+            };
+            auto put_partial = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                int4 *d = ws + (int64_t)blockIdx.x * kWs + wsi + (c >> 3) * 512;
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2)
+                    __stcg(d + e * 64, make_int4((int)vre[e], (int)vim[e], (int)vre[e + 1], (int)vim[e + 1]));
+            };
+            auto add_partial = [&](const int b, const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                const int4 *src = ws + (int64_t)b * kWs + wsi + (c >> 3) * 512;
+                #pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    const int4 v = __ldcg(src + e * 64);
+                    vre[e] += (uint32_t)v.x;
+                    vim[e] += (uint32_t)v.y;
+                    vre[e + 1] += (uint32_t)v.z;
+                    vim[e + 1] += (uint32_t)v.w;
+                }
+            };
+            // Stores columns c .. c + 7, or adds them to the values in `old`.
+            auto put_chunk = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                const int i0 = i_base + c;
+                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;  // elements e <= last are pairs of the triangle
+                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
+                #pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    if (e <= last)
+                        __stcs(out + off, kAdd ? make_int2(old[e].x + (int)vre[e], old[e].y + (int)vim[e])
+                                               : make_int2((int)vre[e], (int)vim[e]));
+                    off += N - (i0 + e) - 1;
+                }
+            };
+            // Calls fn(c, re, im) with the corrected values of the chunks c = c0, c0 + step, ...
+            // Where registers allow, in two sets: the next chunk's TMEM loads run under this
+            // chunk's stores.
+            auto for_chunks = [&](const int c0, const int step, auto &&fn) {
+                if (kAdd || kShared) {
+                    // adding: the next chunk's old values are loaded under this chunk's TMEM
+                    // loads and stores
+                    for (int c = c0; warp_ok && chunk_ok(c); c += step) {
+                        uint32_t vre[8], vim[8];
+                        int2 next[8];
+                        tmem_ld8(tre + c, vre);
+                        tmem_ld8(tim + c, vim);
+                        if (kAdd && !kShared && owner && chunk_ok(c + step)) load_old(c + step, next);
+                        tmem_ld_wait();
+                        correct(c, vre, vim);
+                        fn(c, vre, vim);
+                        if (kAdd && !kShared) {
+                            #pragma unroll
+                            for (int e = 0; e < 8; e++) old[e] = next[e];
+                        }
+                    }
+                    return;
+                }
+                uint32_t ra[8], ia[8], rb[8], ib[8];
+                int c = c0;
+                if (!warp_ok || !chunk_ok(c)) return;
+                tmem_ld8(tre + c, ra);
+                tmem_ld8(tim + c, ia);
+                tmem_ld_wait();
+                for (;;) {
+                    const int c1 = c + step;
+                    const bool ok1 = chunk_ok(c1);
+                    if (ok1) {
+                        tmem_ld8(tre + c1, rb);
+                        tmem_ld8(tim + c1, ib);
+                    }
+                    correct(c, ra, ia);
+                    fn(c, ra, ia);
+                    if (!ok1) break;
+                    tmem_ld_wait();
+                    c = c1 + step;
+                    const bool ok2 = chunk_ok(c);
+                    if (ok2) {
+                        tmem_ld8(tre + c, ra);
+                        tmem_ld8(tim + c, ia);
+                    }
+                    correct(c1, rb, ib);
+                    fn(c1, rb, ib);
+                    if (!ok2) break;
+                    tmem_ld_wait();
+                }
+            };
+            if (kShared) {
+                // chunk c of block h is finished by the item's CTA (16 h + c / 8) % split, its
+                // chunks of a block by the halves in turn
+                const int part = (int)blockIdx.x - c_lo;
+                for_chunks(8 * half, 8 * halves, [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
+                    if (lane_ok && (16 * h + (c >> 3)) % a.split != part) put_partial(c, vre, vim);
+                });
+                __threadfence();  // the partials are visible at GPU scope before the flag below
+                named_bar_sync(2, tail);
+                if (et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
+                ok = et >= a.split || flag_wait(a.flags + c_lo + et, *s_epoch, err, kDevTimeoutEpilogue);
+                if (bar_any(2, tail, !ok)) break;
+                const int first = (part + a.split - 16 * h % a.split) % a.split;  // 16 h + first = part (mod split)
+                for_chunks(8 * (first + half * a.split), 8 * halves * a.split, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                    if (!lane_ok) return;
+                    if (kAdd) load_old(c, old);
+                    #pragma unroll 4
+                    for (int p = 1; p < a.split; p++)
+                        add_partial(c_lo + (part + p < a.split ? part + p : part + p - a.split), c, vre, vim);
+                    put_chunk(c, vre, vim);
+                });
+            } else {
+                for_chunks(0, 8, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
+                    if (!owner) {  // a later piece of the item: the partial goes to this CTA's slot
+                        if (lane_ok) put_partial(c, vre, vim);
+                        return;
+                    }
+                    // the item's later pieces (none for a whole item)
+                    for (int b = c_lo; lane_ok && b <= c_hi; b++) add_partial(b, c, vre, vim);
+                    put_chunk(c, vre, vim);
+                });
+            }
+            if (!owner && !kShared) __threadfence();  // the partial is visible at GPU scope before the flag below
+            // every epilogue thread is done with this parity's sums: clear them for
+            // the piece after next, then hand TMEM and the buffer back
+            named_bar_sync(2, tail);
+            if (!owner && !kShared && et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
+            for (int k = et; k < kSSumPar; k += tail) sums[par * kSSumPar + k] = make_int2(0, 0);
+            fence_before();
+            __syncwarp();
+            if (lane == 0 && warp >= kSEpiWarp0) {
+                mbar_arrive(acce);
+                mbar_arrive(sums_empty(par));
+            }
+            ++local;
+        }
+    };
     if (warp == 0) {
         {
             // ---------------- TMA producer (the whole warp, one elected lane issuing) ----------------
@@ -433,7 +671,7 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
         const int nt = (int)a.nt;                               // <= kFusedMaxSamples
         int rs = 0, ps = 0, local = 0;
         uint32_t rph = 0, pph = 0;
-        bool ok = true;
+        bool &ok = conv_ok;
         int x = lo;
         Piece pc;
         for (; ok && next_piece(a, x, hi, pc); ++local) {
@@ -551,236 +789,10 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
             __syncwarp();
             if (lane == 0) mbar_arrive(sums_full(par));
         }
-    } else {
-        // ---------------- epilogue ----------------
-        const int q = warp & 3;                     // TMEM lane quadrant this warp may access
-        const int h = (warp - kSEpiWarp0) >> 2;     // the item's block: columns 128h.. of Re and Im
-        const int et = (warp - kSEpiWarp0) * 32 + lane;
-        const int row = q * 32 + lane;              // TMEM lane: input j within its 128-input block
-        const int N = a.N;                          // <= 256
-        const int nt = (int)a.nt;
-        const int64_t nb = (int64_t)N * (N + 1) / 2;
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
-        // partial blocks in ws: [CTA][block h][chunk c / 8][column pair][row], 16 bytes each,
-        // so that a warp's 32 rows are one 512-byte run
-        constexpr int kWs = 2 * 16 * 4 * 128;    // 16-byte words per CTA
-        const int wsi = h * 16 * 4 * 128 + row;  // + (c / 8) * 512 + 128 per column pair
-        int4 *const ws = reinterpret_cast<int4 *>(a.ws);
-        uint32_t uses = 0;
-        int local = 0;
-        int x = lo;
-        Piece pc;
-        while (next_piece(a, x, hi, pc)) {
-            const SmallItem w = small_item(a, pc.it);
-            const int par = local & 1;
-            // the piece's samples inside the launch: 64 n from each of the two products
-            const float n128 = (float)(128 * ((pc.k1 * kSKc < nt ? pc.k1 * kSKc : nt) - pc.k0 * kSKc));
-            const bool owner = pc.k0 == 0;
-            // an owner whose item runs on: the CTAs after it that hold the rest
-            // (shared items: the item's other CTAs, which this one meets later)
-            const int c_lo = kShared ? pc.it * a.split : (int)blockIdx.x + 1;
-            const int c_hi = kShared ? c_lo + a.split - 1
-                                    : owner && pc.k1 < a.n_k ? stage_cta(a, (pc.it + 1) * a.n_k - 1) : 0;
-            // Block h: column items' inputs j = 128.. against i = 128h..; diagonal items'
-            // channel fx or fy, both 0..127.  Sums: X tile at 0, Y tile at 128.
-            const int fl = w.col ? w.fx : (h ? w.fy : w.fx);
-            const int j_warp = (w.col ? 128 : 0) + q * 32;
-            const int j = j_warp + lane;
-            const int i_base = w.col ? 128 * h : 0;
-            const bool lane_ok = j < N;
-            const bool warp_ok = fl >= 0 && j_warp < N;
-            int2 *out = reinterpret_cast<int2 *>(a.acc) + (int64_t)fl * nb;
-            // warp-uniform: columns inside the channel and up to some lane's diagonal
-            auto chunk_ok = [&](const int c) { return c < 128 && i_base + c < N && i_base + c <= j_warp + 31; };
-            // the triangle's values of columns c .. c + 7 (adding launches): pair (i, j) sits
-            // at i*N - i*(i-1)/2 + (j - i) in the channel's triangle and row i + 1 starts
-            // N - i - 1 pairs after row i, so per column the warp's 32 consecutive inputs j
-            // are one 256-byte run
-            auto load_old = [&](const int c, int2 (&o)[8]) {
-                const int i0 = i_base + c;
-                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;
-                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
-                #pragma unroll
-                for (int e = 0; e < 8; e++) {
-                    if (e <= last) o[e] = __ldcg(out + off);
-                    off += N - (i0 + e) - 1;
-                }
-            };
-            int2 old[8];
-            if (kAdd && !kShared) {
-                int nx = x;
-                Piece np;
-                if (next_piece(a, nx, hi, np)) {  // the next item's values, to L2
-                    const SmallItem nw = small_item(a, np.it);
-                    const int nfl = nw.col ? nw.fx : (h ? nw.fy : nw.fx);
-                    if (nfl >= 0 && np.k0 == 0)
-                        prefetch_triangle(reinterpret_cast<const int2 *>(a.acc) + (int64_t)nfl * nb, N,
-                                          (nw.col ? 128 : 0) + q * 32, nw.col ? 128 * h : 0,
-                                          min(N, nw.col ? 128 * h + 128 : 128), 8, lane);
-                }
-                if (owner && warp_ok && chunk_ok(0)) load_old(0, old);  // under the wait for the accumulator
-            }
-            bool ok = mbar_wait_backoff(accf, uses & 1u, err, kDevTimeoutEpilogue, 128);
-            ok = ok && mbar_wait_backoff(sums_full(par), (uint32_t)((local >> 1) & 1), err, kDevTimeoutEpilogue, 128);
-            if (et == 0 && !kShared)
-                for (int b = c_lo; ok && b <= c_hi; b++) ok = flag_wait(a.flags + b, *s_epoch, err, kDevTimeoutEpilogue);
-            // the barrier ORs the eight warps' failures, so they leave together
-            if (bar_any(2, kSEpiWarps * 32, !ok)) break;
-            ++uses;
-            fence_after();
-            // every input's offset terms in place of its sums (read by all the warps)
-            {
-                const int m = par * kSSumPar + sum_slot(et);
-                terms[m] = offset_terms(sums[m]);
-            }
-            named_bar_sync(2, kSEpiWarps * 32);
-            const float2 *ci = terms + par * kSSumPar + sum_slot(128 * h);  // inputs i of the columns
-            const float2 tj = terms[par * kSSumPar + sum_slot((w.col ? 128 : 128 * h) + row)];
-            const float re_j = kFloatToInt + n128 + tj.x, im_j = kFloatToInt - tj.y;
-            // TMEM columns of the block: column items Re at 128h.., Im at 256 + 128h..;
-            // diagonal items Re at 256h.., Im (negated) at 256h + 128..
-            const uint32_t tre = taddr + (w.col ? 128u * h : 256u * h);
-            const uint32_t tim = tre + (w.col ? 256u : 128u);
-            const float im_scale = w.col ? kRawScale : -kRawScale;
-            // the piece's visibilities in place of the accumulator words of columns c .. c + 7
-            auto correct = [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
-                #pragma unroll
-                for (int e = 0; e < 8; e += 2) {
-                    const float4 t2 = *reinterpret_cast<const float4 *>(ci + sum_slot(c) + e);  // the same for every lane: a broadcast
-                    vre[e] = raw_to_int(vre[e], kRawScale, re_j + t2.x);
-                    vim[e] = raw_to_int(vim[e], im_scale, im_j + t2.y);
-                    vre[e + 1] = raw_to_int(vre[e + 1], kRawScale, re_j + t2.z);
-                    vim[e + 1] = raw_to_int(vim[e + 1], im_scale, im_j + t2.w);
-                }
-            };
-            auto put_partial = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
-                int4 *d = ws + (int64_t)blockIdx.x * kWs + wsi + (c >> 3) * 512;
-                #pragma unroll
-                for (int e = 0; e < 8; e += 2)
-                    __stcg(d + e * 64, make_int4((int)vre[e], (int)vim[e], (int)vre[e + 1], (int)vim[e + 1]));
-            };
-            auto add_partial = [&](const int b, const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
-                const int4 *src = ws + (int64_t)b * kWs + wsi + (c >> 3) * 512;
-                #pragma unroll
-                for (int e = 0; e < 8; e += 2) {
-                    const int4 v = __ldcg(src + e * 64);
-                    vre[e] += (uint32_t)v.x;
-                    vim[e] += (uint32_t)v.y;
-                    vre[e + 1] += (uint32_t)v.z;
-                    vim[e + 1] += (uint32_t)v.w;
-                }
-            };
-            // Stores columns c .. c + 7, or adds them to the values in `old`.
-            auto put_chunk = [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
-                const int i0 = i_base + c;
-                const int last = lane_ok ? min(j - i0, N - 1 - i0) : -1;  // elements e <= last are pairs of the triangle
-                int off = i0 * N - i0 * (i0 - 1) / 2 - i0 + j;
-                #pragma unroll
-                for (int e = 0; e < 8; e++) {
-                    if (e <= last)
-                        __stcs(out + off, kAdd ? make_int2(old[e].x + (int)vre[e], old[e].y + (int)vim[e])
-                                               : make_int2((int)vre[e], (int)vim[e]));
-                    off += N - (i0 + e) - 1;
-                }
-            };
-            // Calls fn(c, re, im) with the corrected values of the chunks c = c0, c0 + step, ...
-            // Where registers allow, in two sets: the next chunk's TMEM loads run under this
-            // chunk's stores.
-            auto for_chunks = [&](const int c0, const int step, auto &&fn) {
-                if (kAdd || kShared) {
-                    // adding: the next chunk's old values are loaded under this chunk's TMEM
-                    // loads and stores
-                    for (int c = c0; warp_ok && chunk_ok(c); c += step) {
-                        uint32_t vre[8], vim[8];
-                        int2 next[8];
-                        tmem_ld8(tre + c, vre);
-                        tmem_ld8(tim + c, vim);
-                        if (kAdd && !kShared && owner && chunk_ok(c + step)) load_old(c + step, next);
-                        tmem_ld_wait();
-                        correct(c, vre, vim);
-                        fn(c, vre, vim);
-                        if (kAdd && !kShared) {
-                            #pragma unroll
-                            for (int e = 0; e < 8; e++) old[e] = next[e];
-                        }
-                    }
-                    return;
-                }
-                uint32_t ra[8], ia[8], rb[8], ib[8];
-                int c = c0;
-                if (!warp_ok || !chunk_ok(c)) return;
-                tmem_ld8(tre + c, ra);
-                tmem_ld8(tim + c, ia);
-                tmem_ld_wait();
-                for (;;) {
-                    const int c1 = c + step;
-                    const bool ok1 = chunk_ok(c1);
-                    if (ok1) {
-                        tmem_ld8(tre + c1, rb);
-                        tmem_ld8(tim + c1, ib);
-                    }
-                    correct(c, ra, ia);
-                    fn(c, ra, ia);
-                    if (!ok1) break;
-                    tmem_ld_wait();
-                    c = c1 + step;
-                    const bool ok2 = chunk_ok(c);
-                    if (ok2) {
-                        tmem_ld8(tre + c, ra);
-                        tmem_ld8(tim + c, ia);
-                    }
-                    correct(c1, rb, ib);
-                    fn(c1, rb, ib);
-                    if (!ok2) break;
-                    tmem_ld_wait();
-                }
-            };
-            if (kShared) {
-                // chunk c of block h is finished by the item's CTA (16 h + c / 8) % split
-                const int part = (int)blockIdx.x - c_lo;
-                for_chunks(0, 8, [&](const int c, const uint32_t (&vre)[8], const uint32_t (&vim)[8]) {
-                    if (lane_ok && (16 * h + (c >> 3)) % a.split != part) put_partial(c, vre, vim);
-                });
-                __threadfence();  // the partials are visible at GPU scope before the flag below
-                named_bar_sync(2, kSEpiWarps * 32);
-                if (et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
-                ok = et >= a.split || flag_wait(a.flags + c_lo + et, *s_epoch, err, kDevTimeoutEpilogue);
-                if (bar_any(2, kSEpiWarps * 32, !ok)) break;
-                const int first = (part + a.split - 16 * h % a.split) % a.split;  // 16 h + first = part (mod split)
-                for_chunks(8 * first, 8 * a.split, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
-                    if (!lane_ok) return;
-                    if (kAdd) load_old(c, old);
-                    #pragma unroll 4
-                    for (int p = 1; p < a.split; p++)
-                        add_partial(c_lo + (part + p < a.split ? part + p : part + p - a.split), c, vre, vim);
-                    put_chunk(c, vre, vim);
-                });
-            } else {
-                for_chunks(0, 8, [&](const int c, uint32_t (&vre)[8], uint32_t (&vim)[8]) {
-                    if (!owner) {  // a later piece of the item: the partial goes to this CTA's slot
-                        if (lane_ok) put_partial(c, vre, vim);
-                        return;
-                    }
-                    // the item's later pieces (none for a whole item)
-                    for (int b = c_lo; lane_ok && b <= c_hi; b++) add_partial(b, c, vre, vim);
-                    put_chunk(c, vre, vim);
-                });
-            }
-            if (!owner && !kShared) __threadfence();  // the partial is visible at GPU scope before the flag below
-            // every epilogue thread is done with this parity's sums: clear them for
-            // the piece after next, then hand TMEM and the buffer back
-            named_bar_sync(2, kSEpiWarps * 32);
-            if (!owner && !kShared && et == 0) st_release_gpu(a.flags + blockIdx.x, *s_epoch);
-            for (int k = et; k < kSSumPar; k += kSEpiWarps * 32) sums[par * kSSumPar + k] = make_int2(0, 0);
-            fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(acce);
-                mbar_arrive(sums_empty(par));
-            }
-            ++local;
-        }
+    } else if (!kJoin) {
+        epilogue();
     }
+    if (kJoin && warp >= kSConvWarp0) epilogue();
 
     __syncwarp();
     fence_before();
@@ -887,8 +899,15 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     }
     int32_t split = 0;
     const int grid = small_split(n_items, n_k, num_sms, &split);
-    auto kern = split >= 2 ? (accumulate ? correlate_small_kernel<true, true> : correlate_small_kernel<false, true>)
-                           : (accumulate ? correlate_small_kernel<true, false> : correlate_small_kernel<false, false>);
+    // Shared items: the converters join the epilogue, their one piece done, where each CTA
+    // finishes two 8-column chunks or more (us, without / with: N = 256 x 8 channels x 4096
+    // samples, 12 CTAs an item, 25.1 / 23.6, adding 30.3 / 26.3; 160 x 24 x 4096, 4 an item,
+    // 29.2 / 26.0; 256 x 6 x 8192, 16 an item, 25.4 / 25.8; 64 x 1 x 32,768, 32, 27.2 / 28.5).
+    auto kern = accumulate ? correlate_small_kernel<true, false, false> : correlate_small_kernel<false, false, false>;
+    if (split > kSJoin)
+        kern = accumulate ? correlate_small_kernel<true, true, false> : correlate_small_kernel<false, true, false>;
+    else if (split >= 2)
+        kern = accumulate ? correlate_small_kernel<true, true, true> : correlate_small_kernel<false, true, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSSmem);
     if (e != cudaSuccess) return e;
     SmallArgs a;
