@@ -148,3 +148,46 @@ def test_beams_repeat_the_same_bits():
     want = oracle.beamform(np.ascontiguousarray(blk[torch.from_numpy(ts).cuda()].cpu().numpy()), w_re, w_im)
     assert np.array_equal(first[torch.from_numpy(ts).cuda()].cpu().numpy().astype(np.int64), want)
     bf.close()
+
+
+def beams_64bit(blk, w_re, w_im):
+    """The beams of a device block as 64-bit products give them, int32 [T][F][B][2]."""
+    T, F, N = blk.shape
+    out = torch.empty((T, F, w_re.shape[1], 2), dtype=torch.int32, device="cuda")
+    for f in range(F):
+        re, im = (blk[:, f] >> 4).double() - 8, (blk[:, f] & 15).double() - 8
+        wr, wi = w_re[f].double().T, w_im[f].double().T
+        out[:, f, :, 0] = (re @ wr - im @ wi).to(torch.int32)  # integers below 2^53: exact
+        out[:, f, :, 1] = (re @ wi + im @ wr).to(torch.int32)
+    return out
+
+
+def test_beams_every_value_of_passes_among_others():
+    # passes over two handles' blocks with nothing waiting in between, as a loop runs
+    # them, copies on another stream taking memory time from some: every value of every
+    # beam is what 64 bits give
+    T, F, N, B = 16384, 128, 256, 32
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    cases = []
+    for _ in range(2):
+        blk = torch.randint(0, 256, (T, F, N), dtype=torch.uint8, device="cuda", generator=g)
+        w = torch.randint(-128, 128, (2, F, B, N), dtype=torch.int8, device="cuda", generator=g)
+        bf = xe.XBeam(N, F, B)
+        bf.set_weights(w[0], w[1])
+        cases.append((bf, blk, torch.empty((T, F, B, 2), dtype=torch.int32, device="cuda"), beams_64bit(blk, *w)))
+    side, a = torch.cuda.Stream(), torch.zeros(1 << 28, dtype=torch.uint8, device="cuda")
+    b = torch.empty_like(a)
+    torch.cuda.synchronize()
+    for k in range(200):
+        with torch.cuda.stream(side):
+            for _ in range(k % 4):
+                b.copy_(a)
+        for c in (0, 1, 0):
+            bf, blk, out, _ = cases[c]
+            bf.run(blk, out)
+        for _, _, out, want in cases:
+            assert torch.equal(out, want), k
+    torch.cuda.synchronize()
+    for bf, *_ in cases:
+        bf.close()
