@@ -30,9 +30,9 @@
 // One persistent CTA per SM; work items = (channel, 128-sample tile):
 //   warp 0        TMA producer of the 128-input slices of both weight
 //                 operands (L2-resident) into a deep shared-memory ring
-//   warp 1        TMEM allocation and the single-thread MMA issuer; the MMA
-//                 reads its A operand (the decoded samples) from tensor memory
-//                 and only B (the weights) from shared memory
+//   warp 1        TMEM allocation and the MMA issuer (the whole warp, one elected
+//                 lane issuing); the MMA reads its A operand (the decoded samples)
+//                 from tensor memory and only B (the weights) from shared memory
 //   warps 2..13   converters in three groups of four warps (one per TMEM lane
 //                 quadrant); group g takes the steps g, g + 3, ...: each thread
 //                 reads one sample row (128 inputs) of the step's raw tile from
@@ -42,7 +42,8 @@
 //   warps 14..21  epilogue: TMEM -> int32 beams [T][F][B][2] in HBM, two warps per
 //                 TMEM lane quadrant taking half the beams each
 //   warp 22       TMA producer of the raw tiles (128 samples x 128 inputs of one
-//                 channel, 128-byte swizzle) into a six-slot ring
+//                 channel, 128-byte swizzle) into a ring of six slots (three above 32
+//                 beams, whose weights and staged rows take the rest)
 // Shared memory then carries only the weight slices; decoded planes written to
 // and read back from shared memory made the MMAs shared-memory bound at small
 // beam counts.  Two TMEM accumulators (one above 32 beams) let the epilogue of
@@ -80,7 +81,8 @@ constexpr uint32_t kXCols = 64;                      // one K chunk of 128 input
 constexpr float kMagic = 196608.0f;                  // 1.5 * 2^17: its binade has the spacing 2^-6
 constexpr uint32_t kMagicBits = 0x48400000u;         // bit pattern of kMagic
 
-template <int kBp>
+// kStaged: the epilogue stages its beams in shared memory (beam_staged).
+template <int kBp, bool kStaged>
 struct BfCfg {
     static constexpr int kN = 4 * kBp;                           // MMA N: hi/lo x Re/Im x beams
     static constexpr int kWBytes = kN * 128;                     // one 128-byte-wide box of the weight operand
@@ -95,7 +97,7 @@ struct BfCfg {
     static constexpr int kMine = kBp >= 8 ? kBp / 2 : kBp;       // beams of an epilogue warp: half, but all of four
     static constexpr int kG = kMine < 16 ? kMine : 16;           // ... formed at once
     static constexpr int kRowBytes = 8 * kG;
-    static constexpr int kOutBytes = kEpiWarps * 32 * kRowBytes;
+    static constexpr int kOutBytes = kStaged ? kEpiWarps * 32 * kRowBytes : 0;
     // raw ring: a multiple of the groups, so each slot has one user
     static constexpr int kRFit =
         (232448 - 1024 - 512 - 2 * kBp * 8 - kOutBytes - 2 * kWStageBytes) / kRawBytes / kGroups * kGroups;
@@ -150,12 +152,12 @@ __device__ __forceinline__ void bf_item(const BfArgs &a, int it, int &f, int &tt
     }
 }
 
-template <int kBp>
+template <int kBp, bool kStaged>
 __global__ void __launch_bounds__(kBfThreads, 1)
 beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_constant__ CUtensorMap w_map,
                 const __grid_constant__ CUtensorMap out_map, const __grid_constant__ BfArgs a)
 {
-    using C = BfCfg<kBp>;
+    using C = BfCfg<kBp, kStaged>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t rbase = (raw + 1023u) & ~1023u;                  // raw ring
@@ -360,9 +362,9 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
         constexpr int kMine = C::kMine;
         // its staging rows; their 16-byte chunks swizzled as the output's map says (by the
         // 128-byte lines of the tile: rows of 128, 64 or 32 bytes)
-        const uint32_t stage = obase + (uint32_t)((warp - kEpiWarp0) * 32 * C::kRowBytes);
-        uint8_t *const srow = smem_raw + (stage - raw) + lane * C::kRowBytes;
-        const int sw_row = C::kRowBytes == 128 ? lane & 7 : C::kRowBytes == 64 ? (lane >> 1) & 3 : (lane >> 2) & 1;
+        [[maybe_unused]] const uint32_t stage = obase + (uint32_t)((warp - kEpiWarp0) * 32 * C::kRowBytes);
+        [[maybe_unused]] uint8_t *const srow = smem_raw + (stage - raw) + lane * C::kRowBytes;
+        [[maybe_unused]] const int sw_row = C::kRowBytes == 128 ? lane & 7 : C::kRowBytes == 64 ? (lane >> 1) & 3 : (lane >> 2) & 1;
         const int bb = (warp - kEpiWarp0) >> 2 ? kBp / 2 : 0;
         const bool idle = kBp < 8 && bb != 0;
         const bool stager = warp == kEpiWarp0;
@@ -419,9 +421,10 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                     tmem_ld4(ta + 3 * kBp + b0 + c, *reinterpret_cast<uint32_t(*)[4]>(lim + c));
                 }
                 tmem_ld_wait();
-                // the rows staged last time have been read
-                if (a.tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                __syncwarp();
+                if (kStaged) {  // the rows staged last time have been read
+                    if (a.tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
+                }
                 {
                     // An accumulator holds S / 64 for an integer |S| < 2^22; adding 1.5 * 2^17
                     // (ulp 2^-6) is exact and leaves S + kMagicBits in the sum's bit pattern,
@@ -442,6 +445,32 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                         const uint32_t bli = __float_as_uint(__uint_as_float(lim[e]) + kMagic);
                         y[e] = make_int2((int)(16u * bhr + blr - (uint32_t)c.x), (int)(16u * bhi + bli - (uint32_t)c.y));
                     }
+                    const int64_t t_warp = (int64_t)tt * 128 + q * 32;
+                    if constexpr (!kStaged) {
+                        const int64_t t = t_warp + lane;
+                        int2 *o = reinterpret_cast<int2 *>(a.out) + (t * a.F + f) * a.B + b0;
+                        if (t >= a.T) {
+                        } else if (G >= 4 && a.vec == 4) {  // four beams, a 32-byte sector, per store
+                            #pragma unroll
+                            for (int e = 0; e + 3 < G; e += 4)
+                                if (b0 + e < a.B)
+                                    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                                 ::"l"(o + e), "r"(y[e].x), "r"(y[e].y), "r"(y[e + 1].x), "r"(y[e + 1].y),
+                                                   "r"(y[e + 2].x), "r"(y[e + 2].y), "r"(y[e + 3].x), "r"(y[e + 3].y)
+                                                 : "memory");
+                        } else if (a.vec >= 2) {
+                            #pragma unroll
+                            for (int e = 0; e < G; e += 2)
+                                if (b0 + e < a.B)
+                                    *reinterpret_cast<int4 *>(o + e) = make_int4(y[e].x, y[e].y, y[e + 1].x, y[e + 1].y);
+                        } else {
+                            #pragma unroll
+                            for (int e = 0; e < G; e++)
+                                if (b0 + e < a.B) o[e] = y[e];
+                        }
+                        __syncwarp();
+                        continue;
+                    }
                     // Staged, then stored in whole runs of a row: a lane's own row is F * B beams
                     // from the next lane's.  By TMA where rows are multiples of 16 bytes (B even);
                     // rows past T and beams past B are clipped.
@@ -449,7 +478,6 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
                     for (int e = 0; e < G; e += 2)
                         *reinterpret_cast<int4 *>(srow + (((e >> 1) ^ sw_row) << 4)) =
                             make_int4(y[e].x, y[e].y, y[e + 1].x, y[e + 1].y);
-                    const int64_t t_warp = (int64_t)tt * 128 + q * 32;
                     if (a.tma_out) {
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
@@ -475,9 +503,9 @@ beamform_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid_consta
             fence_before();
             mbar_arrive(acce(ab));
         }
-        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // staging read, beams written
+        if (kStaged && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // staging read, beams written
     } else if (lane == 0) {
-        // ---------------- TMA producer: raw tiles (warp 18) ----------------
+        // ---------------- TMA producer: raw tiles (warp 22) ----------------
         int r = 0, issued = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -601,13 +629,36 @@ __global__ void beam_corr_kernel(const int8_t *__restrict__ w_re, const int8_t *
     }
 }
 
-template <int kBp>
+// Whether the beams are staged in shared memory and stored in whole runs of a row, or
+// straight from registers, each lane its own row.  Staging makes the epilogue cheap
+// however B divides; direct stores leave its 32 KB to the weight ring (17 to 32 beams:
+// four stages instead of three), which pays where an item has many K chunks, the
+// sooner the wider the stores.  At 5 to 16 and above 32 beams staging is level or
+// better at every size tried.  GB300, us, staged / direct, 128 channels x 8192 samples:
+//   N = 512 (4 chunks)   B = 20 144 / 148, 32 159 / 179
+//   N = 640 (5)          B = 20 176 / 165, 28 186 / 181, 32 190 / 193
+//   N = 768 (6)          B = 18 207 / 212, 32 219 / 213
+//   N = 1024 (8)         B = 18 276 / 265, 26 287 / 290, 32 288 / 273
+//   N = 2048 (16)        B = 17 475 / 467, 22 476 / 451, 26 483 / 467, 31 500 / 590, 32 489 / 445
+//                        (256 channels x 4096 samples)
+//   N = 4096 (32)        B = 30 254 / 236, 31 257 / 252, 32 253 / 229 (64 x 4096)
+// Up to 4 beams a lane's row is one sector or part of one, and only B = 3, three
+// stores of 8 bytes, gains from staging, at one chunk (N = 16 x 256 channels x 8192
+// samples 89 / 95; B = 1 89 / 74, 4 75 / 73; N = 256 x 128 x 16,384: B = 3 104 / 101).
+bool beam_staged(const BfArgs &a)
+{
+    if (a.B <= 4) return a.B == 3 && a.n_kc == 1;
+    if (a.B <= 16 || a.B > 32) return true;
+    return a.n_kc < (a.vec == 4 ? (a.B > 28 ? 6 : 5) : a.vec == 2 ? (a.B < 20 ? 7 : a.B - 12) : a.B - 5);
+}
+
+template <int kBp, bool kStaged>
 cudaError_t launch_bf(const CUtensorMap &rm, const CUtensorMap &wm, const BfArgs &a, int grid, cudaStream_t s)
 {
-    using C = BfCfg<kBp>;
+    using C = BfCfg<kBp, kStaged>;
     CUtensorMap om;
     memset(&om, 0, sizeof om);
-    if (a.tma_out) {
+    if (kStaged && a.tma_out) {
         // beams as int32: dims (2 B, channel, sample), boxes of one warp's rows
         cuuint64_t dims[3] = {(cuuint64_t)(2 * a.B), (cuuint64_t)a.F, (cuuint64_t)a.T};
         cuuint64_t strides[2] = {(cuuint64_t)a.B * 8, (cuuint64_t)a.F * a.B * 8};
@@ -621,10 +672,10 @@ cudaError_t launch_bf(const CUtensorMap &rm, const CUtensorMap &wm, const BfArgs
                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    cudaError_t e = cudaFuncSetAttribute(beamform_kernel<kBp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(beamform_kernel<kBp, kStaged>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)C::kSmem);
     if (e != cudaSuccess) return e;
-    beamform_kernel<kBp><<<grid, kBfThreads, C::kSmem, s>>>(rm, wm, om, a);
+    beamform_kernel<kBp, kStaged><<<grid, kBfThreads, C::kSmem, s>>>(rm, wm, om, a);
     return cudaGetLastError();
 }
 
@@ -691,14 +742,15 @@ cudaError_t launch_beamform(const uint8_t *block, const uint8_t *wdev, const int
     a.block = block;
     const uintptr_t oa = reinterpret_cast<uintptr_t>(a.out);
     a.tma_out = a.B % 2 == 0 && (oa & 15) == 0 ? 1 : 0;  // TMA rows are 16-byte multiples
+    a.vec = a.B % 4 == 0 && (oa & 31) == 0 ? 4 : a.tma_out ? 2 : 1;
     if (a.n_items > 2147483647LL) return cudaErrorInvalidValue;  // more than the device's memory could hold
     const int grid = (int)(a.n_items < num_sms ? a.n_items : num_sms);
     switch (bp) {
-        case 4: return launch_bf<4>(rm, wm, a, grid, s);
-        case 8: return launch_bf<8>(rm, wm, a, grid, s);
-        case 16: return launch_bf<16>(rm, wm, a, grid, s);
-        case 32: return launch_bf<32>(rm, wm, a, grid, s);
-        default: return launch_bf<64>(rm, wm, a, grid, s);
+        case 4: return beam_staged(a) ? launch_bf<4, true>(rm, wm, a, grid, s) : launch_bf<4, false>(rm, wm, a, grid, s);
+        case 8: return launch_bf<8, true>(rm, wm, a, grid, s);
+        case 16: return launch_bf<16, true>(rm, wm, a, grid, s);
+        case 32: return beam_staged(a) ? launch_bf<32, true>(rm, wm, a, grid, s) : launch_bf<32, false>(rm, wm, a, grid, s);
+        default: return launch_bf<64, true>(rm, wm, a, grid, s);
     }
 }
 

@@ -325,7 +325,8 @@ struct BfArgs {
     int32_t n_tt = 0;       // 128-sample tiles
     int64_t n_items = 0;    // F * n_tt
     int32_t f_fastest = 0;  // item order: channel fastest, else sample tile fastest
-    int32_t tma_out = 0;    // B even, out 16-byte aligned: beams staged in shared memory and stored by TMA
+    int32_t tma_out = 0;    // B even, out 16-byte aligned: staged beams are stored by TMA
+    int32_t vec = 1;        // beams per direct store: 4 (B % 4 == 0, out 32-byte aligned), 2 (as tma_out) or 1
     const uint8_t *block = nullptr;  // [T][F][N]
     int32_t *out = nullptr; // [T][F][B][2]
     const int32_t *corr = nullptr;  // [F][Bp][2] offset terms (8 sum(w_re - w_im), 8 sum(w_re + w_im))

@@ -191,3 +191,24 @@ def test_beams_every_value_of_passes_among_others():
     torch.cuda.synchronize()
     for bf, *_ in cases:
         bf.close()
+
+
+# Beams staged and stored by TMA, staged and stored by threads (odd B, or out on an
+# 8-byte but not a 16-byte boundary) or stored straight from registers, four, two or one
+# at a time: both sides of every line of the choice, ragged samples
+@pytest.mark.parametrize("N,B,off", [(16, 1, 0), (16, 2, 8), (16, 3, 0), (144, 3, 8), (144, 4, 16), (16, 4, 0),
+                                     (16, 8, 8), (256, 16, 8), (256, 32, 8), (256, 64, 8), (512, 28, 0), (640, 28, 0),
+                                     (640, 32, 0), (656, 32, 0), (768, 18, 0), (784, 18, 0), (768, 32, 16), (2304, 30, 0),
+                                     (1408, 17, 0), (1536, 17, 0), (3328, 32, 8), (3328, 31, 0), (2048, 20, 8)])
+def test_beams_staged_and_direct_stores(N, B, off):
+    T, F = 300, 2
+    blk, w_re, w_im = random_case(N + B + off, T, F, N, B)
+    flat = torch.full((T * F * B * 2 + 64,), 77, dtype=torch.int32, device="cuda")
+    lo, n = 8 + off // 4, T * F * B * 2
+    bf = xe.XBeam(N, F, B)
+    bf.set_weights(np.ascontiguousarray(w_re, np.int8), np.ascontiguousarray(w_im, np.int8))
+    bf.run(torch.from_numpy(blk).cuda(), flat[lo:lo + n].view(T, F, B, 2))
+    got = flat.cpu().numpy().astype(np.int64)
+    bf.close()
+    assert np.array_equal(got[lo:lo + n].reshape(T, F, B, 2), oracle.beamform(blk, w_re, w_im))
+    assert (got[:lo] == 77).all() and (got[lo + n:] == 77).all()
