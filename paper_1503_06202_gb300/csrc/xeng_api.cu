@@ -502,8 +502,8 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
         for (int32_t c = 0; c * 16 < N; c++) {
             const int8_t b = sub.slot[c * 16 / kTile];
             if (list < 2 && b < 0) continue;
-            // the chunks of a 64-byte line go together: parts of it written by two launches
-            // are read back from HBM in between
+            // the chunks of a 64-byte line go together: parts of it written by blocks far
+            // apart are read back from HBM in between
             bool has = false;
             for (int32_t i = c / 4 * 64; i < std::min(N, c / 4 * 64 + 64); i++) has = has || delays[i] > 0;
             if (has == (list % 2 == 1)) chunks.push_back(make_int2(list < 2 ? b * (kTile / 16) + c % (kTile / 16) : c, c));
@@ -521,12 +521,14 @@ int xeng_set_delays(xeng_t h, const int32_t *delays)
     if (e == cudaSuccess) e = cudaMalloc(&h->d_shift_chunks, sizeof(int2) * chunks.size());
     if (e == cudaSuccess)
         e = cudaMemcpy(h->d_shift_chunks, chunks.data(), sizeof(int2) * chunks.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&h->hist, (size_t)(cap * row));
-    if (e == cudaErrorMemoryAllocation && h->hist_ahead) {  // the H samples alone
-        cudaGetLastError();
-        h->hist_ahead = false;
-        cap = H;
+    if (e == cudaSuccess) {
         e = cudaMalloc(&h->hist, (size_t)(cap * row));
+        if (e == cudaErrorMemoryAllocation && h->hist_ahead) {  // the H samples alone
+            cudaGetLastError();
+            h->hist_ahead = false;
+            cap = H;
+            e = cudaMalloc(&h->hist, (size_t)(cap * row));
+        }
     }
     if (e == cudaSuccess) e = cudaMemcpy(h->d_delay, delays, sizeof(int32_t) * N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_slot, slot.data(), sizeof(int32_t) * N, cudaMemcpyHostToDevice);
