@@ -340,8 +340,9 @@ typedef struct {
 
 typedef struct {
     int32_t n_jobs;
-    int64_t n_items;             /* work items of the persistent launch                  */
-    int32_t grid;                /* persistent CTAs (one per SM)                         */
+    int64_t n_items;             /* work items of the persistent launch over planes      */
+    int32_t grid;                /* its CTAs (at most one per SM); 0 where no job is on
+                                    planes, and there is no such launch                  */
     int64_t decode_ctas;         /* 128 x 128 tiles the decode launches convert per run  */
     int64_t planes_bytes;        /* decode scratch owned by the batch                    */
     int32_t max_chunks_per_item;

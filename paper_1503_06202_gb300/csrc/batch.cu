@@ -610,7 +610,7 @@ int xeng_batch_info(xeng_batch_t b, xeng_batch_info_t *info)
     if (!b || !info) return XENG_ERR_ARG;
     info->n_jobs = (int32_t)b->jobs.size();
     info->n_items = b->n_items;
-    info->grid = b->grid ? b->grid : b->num_sms;  // no planned launch: the single-pass kernels' own
+    info->grid = b->grid;
     info->decode_ctas = b->dec_ctas + b->dtiles;
     info->planes_bytes = b->planes_bytes;
     info->max_chunks_per_item = b->opts.max_chunks_per_item;

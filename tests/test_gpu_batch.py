@@ -58,7 +58,7 @@ def test_batch_matches_oracle_and_alone(batch_path):
     b.run()
     torch.cuda.synchronize()
     info = b.info()
-    assert info["n_jobs"] == len(jobs) and info["grid"] >= 1
+    assert info["n_jobs"] == len(jobs) and info["n_items"] > 0 and info["grid"] >= 1
     for (T, F, N), blk, (d, out) in zip(SMALL_MIX, host, jobs):
         got = out.cpu().numpy().astype(np.int64)
         assert np.array_equal(got, oracle.correlate(blk)), (T, F, N)
@@ -162,4 +162,19 @@ def test_batch_listed_pair_launch_and_long_jobs():
     for (T, F, N), blk, (d, out) in zip(shapes, host, jobs):
         assert torch.equal(out, alone(d)), (T, F, N)
         assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk)), (T, F, N)
+    b.close()
+
+
+def test_batch_info_without_planes_jobs():
+    """The planned launch is the one over planes: with every job on a single-pass
+    kernel there is none, and its CTAs are 0."""
+    _, jobs = make_jobs([(300, 2, 256), (500, 1, 512)], seed=45)
+    b = xe.XBatch(jobs)
+    info = b.info()
+    assert info["n_jobs"] == 2 and info["n_items"] == 0 and info["grid"] == 0
+    b.close()
+    _, jobs = make_jobs([(300, 2, 256), (500, 1, 20)], seed=45)  # the second on planes
+    b = xe.XBatch(jobs)
+    info = b.info()
+    assert info["n_items"] == 1 and info["grid"] == 1
     b.close()
