@@ -112,16 +112,7 @@ constexpr int kSBars = 2 * kSRaws + 2 * kSPlanes + 3 + 4;
 constexpr size_t kSSmem =
     1024 + (size_t)kSPlanes * kSPlaneBytes + (size_t)kSRaws * kSRawBytes + kSSums + kSBars * 8 + 16;
 static_assert(kSSmem <= 232448, "shared memory over the per-CTA limit");
-constexpr int kSMinPiece = 32;  // evenly cut items: stages per CTA at least
-// Shared items: stages per CTA at least, CTAs per item at most.
-#ifndef XENG_SMALL_MIN_SHARED
-#define XENG_SMALL_MIN_SHARED 2
-#endif
-#ifndef XENG_SMALL_MAX_SHARED
-#define XENG_SMALL_MAX_SHARED 32
-#endif
 constexpr int kSJoin = 14;  // CTAs an item at most for the converters to join its epilogue
-constexpr int kSMinShared = XENG_SMALL_MIN_SHARED, kSMaxShared = XENG_SMALL_MAX_SHARED;
 constexpr int kSChunks = 2 * kSBox / 16 / (32 * kSConvWarps);  // 16-byte chunks per converter thread and stage
 static_assert(kSChunks * 32 * kSConvWarps * 16 == 2 * kSBox, "the converter threads cover both tiles");
 constexpr int kSWiden = 16 / kSChunks;  // stages between widenings of the byte-lane sums (<= 240)
@@ -821,36 +812,6 @@ correlate_small_kernel(const __grid_constant__ CUtensorMap raw_map, const __grid
 bool small_ok(const uint8_t *block, int32_t N, int32_t pitch)
 {
     return N >= 1 && N <= 256 && (pitch ? pitch : N) % 16 == 0 && (reinterpret_cast<uintptr_t>(block) & 15) == 0;
-}
-
-namespace {
-
-}  // namespace
-
-int small_split(int64_t n_items, int n_k, int num_sms, int32_t *split)
-{
-    // Few items: as many CTAs per item as there are SMs for, each with at least
-    // kSMinShared stages -- unless an even cut would leave a CTA over 16 stages
-    // less to do (GB300, N = 256 x 40 channels x 32,768 samples, 60 items: 162 us
-    // with two CTAs per item on 120 SMs, 159 cut evenly over 152).
-    const int64_t total = n_items * n_k;
-    int64_t s = num_sms / n_items;
-    if (s > n_k / kSMinShared) s = n_k / kSMinShared;
-    if (s > kSMaxShared) s = kSMaxShared;
-    if (s >= 2 && n_k / s <= total / num_sms + 16) {
-        *split = (int32_t)s;
-        return (int)(n_items * s);
-    }
-    // Short items: whole ones, since a partial block costs as much as the stages
-    // that an even cut saves (GB300, N = 256 x 128 channels x 256 samples: 25 us;
-    // cut evenly into pieces of kSMinPiece stages, 209).
-    if (n_k < kSMinPiece) {
-        *split = kSmallWhole;
-        return (int)(n_items < num_sms ? n_items : num_sms);
-    }
-    *split = kSmallEven;
-    const int64_t grid = total / kSMinPiece;
-    return (int)(grid < num_sms ? grid : num_sms);
 }
 
 size_t small_ws_bytes(int num_sms) { return (size_t)num_sms * 2 * 16 * 128 * 8 * sizeof(int2); }

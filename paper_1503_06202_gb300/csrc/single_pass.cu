@@ -7,8 +7,6 @@
 #include "tc_ptx.cuh"
 #include "xeng_internal.h"
 
-namespace xeng {
-
 // Up to 256 inputs: single CTAs over the upper-triangle 128-input blocks
 // (correlate_small.cu).  0 disables it (such blocks decode to planes).
 #ifndef XENG_FUSED_SMALL
@@ -25,7 +23,8 @@ namespace xeng {
 // 3.22; 512 3.66 / 3.26; 640 5.26 / 6.75; 768 7.50 / 6.75; 896 9.79 / 11.05;
 // 1024 13.06 / 11.09; 1152 15.98 / 16.96; 1408 23.15 / 23.90; 1664 32.13 /
 // 33.70; 1920 51.88 / 42.12; 2176 67.87 / 53.46: the ratio of the two costs
-// must lie between 3.25 and 3.33).  A cost of 0 forces that kernel.
+// must lie between 3.25 and 3.33).  A cost of 0 forces that kernel, for every
+// launch shape too (launch_rule.h).
 #ifndef XENG_PAIR_COST
 #define XENG_PAIR_COST 118
 #endif
@@ -41,16 +40,9 @@ namespace xeng {
 #ifndef XENG_FUSED_MAX_N
 #define XENG_FUSED_MAX_N 3584
 #endif
+#include "launch_rule.h"
 
-namespace {
-
-bool use_pair_kernel(int32_t N)
-{
-    const int64_t b2 = (N + 255) / 256, b1 = (N + 127) / 128;
-    return (int64_t)XENG_PAIR_COST * (b2 * (b2 + 1) / 2) < (int64_t)XENG_ONEPASS_COST * (b1 * (b1 + 1) / 2);
-}
-
-}  // namespace
+namespace xeng {
 
 cudaError_t status_alloc(int **d_err, int **h_err)
 {
@@ -98,70 +90,6 @@ int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded,
     case kSinglePair: return pair_ok(block, N, pitch) ? k : 0;
     default: return onepass_ok(block, N, pitch) ? k : 0;
     }
-}
-
-namespace {
-
-// Channels whose block pairs fill whole rounds of the pair kernel, where the rest
-// takes less than another round in the one pass (5 us for the second launch); 0:
-// one launch for all.  GB300, N = 1024 x 64 channels x 8192 samples, 640 items on
-// 76 clusters: 717 us in nine rounds, 690 as eight and a launch of four channels.
-int32_t pair_rounds_cut(int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms)
-{
-    const int64_t n_k = (nt + 127) / 128, units = num_sms / 2;
-    const int64_t b2 = (N + 255) / 256, per = b2 * (b2 + 1) / 2, b1 = (N + 127) / 128, per1 = b1 * (b1 + 1) / 2;
-    const int64_t full = nf * per / units, cut = full * units / per;
-    if (cut <= 0 || cut >= nf) return 0;
-    const int64_t ones = ((nf - cut) * per1 + num_sms - 1) / num_sms;
-    const int64_t t_round = 1200 * n_k + (accumulate ? 12300 : 7400);
-    return ones * (770 * n_k + (accumulate ? 3200 : 1600)) + 5000 < t_round ? (int32_t)cut : 0;
-}
-
-}  // namespace
-
-int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms)
-{
-    // Rounds of the grid times an item's time in ns, fitted to launches of 2 .. 256
-    // stages of 128 samples (GB300; us per item at 2 / 8 / 64 / 256 stages, storing:
-    // pair kernel 8.4 / 16.8 / 83.5 / 314, one pass 3.0 / 7.8 / 52 / 204, N <= 256
-    // kernel 7.9 / 14.9 / --; adding: 14.7 / -- / 87 / --, 5.3 / 9.3 / 55 / --,
-    // 14.9 / 24.8 / --).  At 64 stages and many rounds the first two are in the ratio
-    // of XENG_PAIR_COST and XENG_ONEPASS_COST.  A few rounds, and short launches,
-    // favour the one pass, whose items are the smallest and whose epilogue overlaps
-    // the next item (us a call, the N-only choice / the one pass: N = 1024 x 4
-    // channels x 32,768 samples 322 / 207; 512 x 256 x 256 100 / 65; 256 x 256 x 256
-    // 32 / 25); above about 1900 inputs and many channels its items take a quarter
-    // longer.
-    const int64_t n_k = (nt + 127) / 128;
-    auto rounds = [](int64_t items, int64_t units) { return (items + units - 1) / units; };
-    const int64_t b2 = (N + 255) / 256, b1 = (N + 127) / 128;
-    const int64_t ones = rounds(nf * (b1 * (b1 + 1) / 2), num_sms);
-    int64_t t_one = ones * (770 * n_k + (accumulate ? 3200 : 1600));
-    if (N > 1900 && ones > 8 && n_k > 32) t_one += t_one / 4;
-    if (kernel == kSingleSmall) {
-        // By how it cuts its items: between CTAs (an exchange of partial blocks, then
-        // the stages of one CTA) or whole.  The exchange costs more than the stages it
-        // takes off the CTAs of a short launch (us a call, the N <= 256 kernel / the
-        // one pass: N = 256 x 8 channels x 1024 samples 22.3 / 14.3, x 2048 22.5 / 19.2,
-        // x 4096 26.1 / 30.6; 256 x 48 x 4096 37.9 / 31.3, x 8192 56.0 / 54.4; 160 x 2
-        // x 256 15.0 / 9.0; 128 x 152 x 4096 39.5 / 27.7, x 32,768 168 / 191).
-        const int64_t items = N > 128 ? nf + (nf + 1) / 2 : (nf + 1) / 2;
-        const int64_t n_one = accumulate ? 3200 : 1600;
-        int32_t split;
-        const int grid = small_split(items, (int)n_k, num_sms, &split);
-        int64_t t_small;
-        if (split == kSmallWhole)
-            t_small = 2000 + rounds(items, num_sms) * (1100 * n_k + (accumulate ? 13500 : 5000));
-        else if (split == kSmallEven)  // one item a CTA is as good as whole
-            t_small = (grid == items ? 6000 : 18000) + 1200 * (items * n_k / grid) + (accumulate ? 11000 * items / grid : 0);
-        else
-            t_small = 9000 + 25 * N + 1100 * n_k / split + (accumulate ? 5500 : 0);
-        return t_small <= ones * ((N > 128 ? 770 : 680) * n_k + n_one) ? kernel : kSingleOnepass;
-    }
-    if (kernel != kSinglePair && kernel != kSingleOnepass) return kernel;
-    return rounds(nf * (b2 * (b2 + 1) / 2), num_sms / 2) * (1200 * n_k + (accumulate ? 12300 : 7400)) < t_one
-               ? kSinglePair
-               : kSingleOnepass;
 }
 
 cudaError_t small_scratch_alloc(SmallScratch *sc, int num_sms, cudaStream_t s)
@@ -216,7 +144,7 @@ cudaError_t launch_single_pass_shaped(int kernel, const uint8_t *block, int64_t 
         if (e0 != cudaSuccess) return e0;
     }
     const int k = single_pass_by_shape(kernel, N, nf, nt, accumulate, num_sms);
-    const int32_t cut = k == kSinglePair ? pair_rounds_cut(N, nf, nt, accumulate, num_sms) : 0;
+    const int32_t cut = single_pass_cut(k, N, nf, nt, accumulate, num_sms);
     const int32_t first = cut ? cut : nf;
     cudaError_t e = launch_single_pass(k, block, T_block, t0, nt, F, N, f0, first, acc, accumulate, sc, err, num_sms, s,
                                        nullptr, 0, pitch, sub);

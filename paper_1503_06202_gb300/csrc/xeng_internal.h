@@ -284,6 +284,9 @@ int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded,
 // block pairs, or (kernel = kSingleSmall) of that one and the one pass.  All three
 // read the same stages.
 int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);
+// Channels that a launch of the pair kernel (by shape) takes before the one pass takes
+// the others; 0: all.
+int32_t single_pass_cut(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);
 // How a launch of the N <= 256 kernel cuts its items (n_k stages each) over the
 // CTAs, at most one per SM: *split CTAs share each item (2 or more), or all stages
 // are cut evenly (kSmallEven), or the items stay whole (kSmallWhole); returns the grid.

@@ -3,9 +3,12 @@ that kernel's DRAM figure for the roofline) from its own copy of the library's
 choice between the two single-pass kernels above 256 inputs.  These checks keep
 that copy equal to the library's build defaults and to the winners measured on
 GB300 (1024 channels, 8192 samples, both kernels forced in turn)."""
+import ctypes
 import importlib.util
 import os
 import re
+import shutil
+import subprocess
 
 import pytest
 
@@ -59,3 +62,33 @@ def test_pair_when_block_count_is_even_above_384():
 def test_default_engine_path_by_n(N, kernel):
     # single pass for N a multiple of 16 up to the bound; decoded planes otherwise
     assert _bench().correlate_kernel("tensor", N)[0].startswith(kernel)
+
+
+# The two build parameters hold for every launch shape: a cost of 0 forces that kernel
+@pytest.mark.parametrize("pair,onepass", [(0, 36), (118, 0), (118, 36)])
+def test_a_cost_of_zero_forces_a_kernel(pair, onepass, tmp_path):
+    cuda = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+    if shutil.which("g++") is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        pytest.skip("needs g++ and the CUDA headers")
+    src, so = tmp_path / "rule.cpp", str(tmp_path / "rule.so")
+    src.write_text('#include "launch_rule.h"\nusing namespace xeng;\n'
+                   'extern "C" int choice(int N, long nf, long nt, int add, int *cut) {\n'
+                   '    const int k = single_pass_by_shape(use_pair_kernel(N) ? kSinglePair : kSingleOnepass, N, nf, nt, add, 152);\n'
+                   '    *cut = single_pass_cut(k, N, nf, nt, add, 152);\n    return k;\n}\n')
+    subprocess.check_call(["g++", "-std=c++17", "-fPIC", "-shared", "-I" + cuda, "-I" + os.path.dirname(SINGLE_PASS),
+                           "-DXENG_PAIR_COST=%d" % pair, "-DXENG_ONEPASS_COST=%d" % onepass, str(src), "-o", so])
+    lib = ctypes.CDLL(so)
+    lib.choice.argtypes = [ctypes.c_int, ctypes.c_long, ctypes.c_long, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    seen = set()
+    for N in (272, 512, 1024, 2048, 3584):
+        for F in (1, 4, 26, 64, 1024):
+            for T in (1, 200, 8192, 32768):
+                for add in (0, 1):
+                    cut = ctypes.c_int()
+                    k = lib.choice(N, F, T, add, ctypes.byref(cut))
+                    seen.add((k, cut.value > 0))
+    # 2: one pass, 3: pair kernel, and whether its last round goes to the one pass
+    if pair and onepass:
+        assert seen == {(3, False), (3, True), (2, False)}
+    else:
+        assert seen == {(2 if pair else 3, False)}
