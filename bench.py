@@ -53,10 +53,13 @@ DRAM_BYTES_PER_CHANNEL = {
 }
 
 
-# The library's choice between its two single-pass kernels above 256 inputs, at
-# its default build parameters: measured cost of one block pair (tens of us per
-# 1024 channels x 8192 samples) times the upper-triangle block pairs.
+# The library's choice by N alone between its two single-pass kernels above 256
+# inputs, which batches follow, at its default build parameters: measured cost of one
+# block pair (tens of us per 1024 channels x 8192 samples) times the upper-triangle
+# block pairs.
 PAIR_COST, ONEPASS_COST, FUSED_MAX_N = 118, 36, 3584
+# Bytes from which a batch rearranges a job whose rows TMA cannot address.
+BATCH_PACK_BYTES = 16 << 20
 
 
 def use_pair_kernel(N):
@@ -64,18 +67,28 @@ def use_pair_kernel(N):
     return PAIR_COST * (b2 * (b2 + 1) // 2) < ONEPASS_COST * (b1 * (b1 + 1) // 2)
 
 
-def correlate_kernel(engine, N):
-    """(name, tile) of the correlation kernel an engine runs for N inputs (tile:
-    the square of inputs one work item computes, lower halves of diagonal
-    items included)."""
-    fused = N % 16 == 0 and (engine == "fused" or (engine == "tensor" and N <= FUSED_MAX_N))
-    if fused and N <= 256:
-        return "correlate_small_kernel (decode fused; upper-triangle 128-input blocks, one CTA each)", 128
-    if fused and use_pair_kernel(N):
-        return "correlate_pair_kernel (decode fused; 256-input block pairs, 2-CTA clusters)", 256
-    if fused:
-        return "correlate_onepass_kernel (decode fused; 128-input block pairs, one CTA each)", 128
-    return "correlate_tc_kernel (decoded planes; 128-input tile pairs)", 128
+def correlate_kernel(engine, N, F=1024, T=8192, num_sms=152, accumulate=False):
+    """(name, executed) of the correlation kernel that an engine runs for N inputs, F
+    channels and T samples (the first launch's, up to 32,768), as the library says:
+    its name, and the input pairs that it computes per channel -- whole tiles, lower
+    halves of diagonal items and padding included -- over the N (N + 1) / 2 useful ones."""
+    import paper_1503_06202_gb300 as xe
+
+    number = {"tensor": xe.XENG_ENGINE_TENSOR, "planes": xe.XENG_ENGINE_TENSOR_PLANES, "fused": xe.XENG_ENGINE_TENSOR_FUSED}
+    kind, first = xe.xeng_kernel_choice(number[engine], N, F, min(T, 32768), accumulate, num_sms)
+    if kind < 0:
+        raise ValueError("no kernel for N=%d F=%d T=%d: %d" % (N, F, T, kind))
+    name = {xe.XENG_KERNEL_SMALL: "correlate_small_kernel (decode fused; upper-triangle 128-input blocks, one CTA each)",
+            xe.XENG_KERNEL_ONEPASS: "correlate_onepass_kernel (decode fused; 128-input block pairs, one CTA each)",
+            xe.XENG_KERNEL_PAIR: "correlate_pair_kernel (decode fused; 256-input block pairs, 2-CTA clusters)",
+            xe.XENG_KERNEL_PLANES: "correlate_tc_kernel (decoded planes; 128-input tile pairs)"}[kind]
+
+    def pairs(tile):
+        nt = -(-N // tile)
+        return nt * (nt + 1) // 2 * tile * tile
+
+    done = first * pairs(256 if kind == xe.XENG_KERNEL_PAIR else 128) + (F - first) * pairs(128)
+    return name, done / (F * N * (N + 1) / 2)
 
 
 def max_over_ranks(x, dist=None):
@@ -232,13 +245,14 @@ def batch_launches(recipes):
     """Kernel launches of one batched run, as the library plans them: one
     persistent launch over every block pair of the jobs the 2-CTA pair kernel
     takes (up to 32,768 samples), one single-pass launch per 32,768 samples of
-    each other job a single-pass kernel takes, and for the rest the TMA decode
+    each other job a single-pass kernel takes (two for a job of other N from
+    BATCH_PACK_BYTES on, which is rearranged first), and for the rest the TMA decode
     (N % 16 == 0 above FUSED_MAX_N), the thread-per-row decode (other N), the
     nibble-sums pass (with the TMA decode) and one listed tensor-core launch."""
-    single = [r for r in recipes if r.N % 16 == 0 and r.N <= FUSED_MAX_N]
-    listed = [r for r in single if r.N > 256 and use_pair_kernel(r.N) and r.T <= 32768]
+    single = [r for r in recipes if r.N <= FUSED_MAX_N and (r.N % 16 == 0 or r.T * r.F * r.N >= BATCH_PACK_BYTES)]
+    listed = [r for r in single if r.N % 16 == 0 and r.N > 256 and use_pair_kernel(r.N) and r.T <= 32768]
     rest = [r for r in recipes if r not in single]
-    n = (1 if listed else 0) + sum(-(-r.T // 32768) for r in single if r not in listed)
+    n = (1 if listed else 0) + sum((2 if r.N % 16 else 1) * -(-r.T // 32768) for r in single if r not in listed)
     tma = any(r.N % 16 == 0 for r in rest)
     if rest:
         n += (2 if tma else 0) + (1 if any(r.N % 16 for r in rest) else 0) + 1
@@ -484,7 +498,7 @@ def main():
     ap.add_argument("--workload", default="chime_full", choices=sorted(WORKLOADS))
     ap.add_argument("--engine", default="tensor", choices=["tensor", "dp4a", "planes", "fused"],
                     help="tensor: the default engine; planes: always decode to HBM planes, then correlate; "
-                         "fused: single pass (raw bytes split in shared memory) wherever N is a multiple of 16")
+                         "fused: single pass (raw bytes split in shared memory) for every N")
     ap.add_argument("--no-engine-compare", "--no-fused-compare", dest="no_engine_compare", action="store_true",
                     help="skip timing the two-pass (planes) engine beside the default one")
     ap.add_argument("--e2e-steps", type=int, default=3)
@@ -779,7 +793,7 @@ def main():
     flops_per_launch = ops / launches_per_step
     if tensor_engine:
         peak = 2.0 * peaks["bf16_tflops_sustained"]
-        kernel, tile = correlate_kernel(args.engine, N)
+        kernel, executed = correlate_kernel(args.engine, N, F, T, torch.cuda.get_device_properties(local_rank).multi_processor_count)
         peak_note = ("fp8 dense = 2 x %s sustained bf16 %.1f TFLOP/s (nominal fp8:bf16 = 4.5:2.25); "
                      "sm_103a has no tcgen05 kind::i8; the bf16 figure was sustained at a power-capped clock, "
                      "so frac can exceed 1 -- the fp8 probes measured in this run (peak_probe_*) are the "
@@ -800,9 +814,7 @@ def main():
             roof["peak_probe_fp8"] = probes["tc_f8f6f4"]
             roof["frac_of_probe_fp8"] = roof["achieved"] / probes["tc_f8f6f4"]
             # useful ops exclude the lower halves of diagonal tiles (and the padding past N)
-            # the MMAs also compute: nt (nt + 1) / 2 tiles of tile x tile per channel
-            nt = -(-N // tile)
-            executed = (nt * (nt + 1) // 2 * tile * tile) / (N * (N + 1) / 2)
+            # the MMAs also compute
             roof["executed_over_useful"] = executed
             roof["frac_executed_of_probe_fp8"] = roof["achieved"] * executed / probes["tc_f8f6f4"]
         if probes and probes.get("tc_f8f6f4_live_data"):
@@ -822,12 +834,15 @@ def main():
                 "traffic": None, "frac": None}
     roof["avg_launch_ms"] = corr_ms
     roof["decode_ms_per_step"] = st["decode_ms"] / args.steps
-    # the decode stage (HBM-bound): 1 byte read + 2 plane bytes written per (input, sample, channel)
+    # the stage before the correlation (HBM-bound): 1 byte read + 2 plane bytes written per
+    # (input, sample, channel), or 1 read + 1 written where the samples are only rearranged
     decode_roof = None
     if tensor_engine and st["decode_ms"] > 0:
         dec_ms = st["decode_ms"] / args.steps
-        dec_bytes = 3 * T * F * N
-        decode_roof = {"kernel": "decode_tma_kernel" if N % 16 == 0 else "decode_kernel", "bound": "hbm",
+        planes = kernel.startswith("correlate_tc")
+        dec_bytes = (3 * N if planes else N + -(-N // 16) * 16) * T * F
+        decode_roof = {"kernel": ("decode_tma_kernel" if N % 16 == 0 else "decode_kernel") if planes else "pack_kernel",
+                       "bound": "hbm",
                        "ms_per_step": dec_ms, "algorithmic_bytes": dec_bytes,
                        "achieved": dec_bytes / (dec_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                        "frac": dec_bytes / (dec_ms * 1e-3) / 1e9 / peaks["hbm_gbs"], "peak_source": peak_src}

@@ -1,6 +1,7 @@
 /*
- * xeng_peaks.h -- dense-throughput probes (part of libxeng.so) that measure
- * the roofline denominators for the correlator on the GPU at hand.
+ * xeng_peaks.h -- for measurements of the correlator (part of libxeng.so):
+ * dense-throughput probes that measure the roofline denominators on the GPU at
+ * hand, and which kernel a launch takes.
  *
  * The paper's cost measure is complex multiply-accumulates, Eq. 1, at 8 real
  * operations each (Sec. II: 4 TFLOPS ~ 0.5 TcMAC/s); these probes give the
@@ -50,6 +51,23 @@ extern "C" {
  *   error) or -6 (a device-side wait timed out).  Allocates a 4-byte flag.
  */
 XENG_API int xeng_peak_probe(int32_t kind, int64_t iters, double *tflops, double *ms);
+
+#define XENG_KERNEL_PLANES  0  /* decode to planes, then 128-input tile pairs       */
+#define XENG_KERNEL_SMALL   1  /* N <= 256: items of two 128-input blocks           */
+#define XENG_KERNEL_ONEPASS 2  /* 128-input block pairs, single CTAs                */
+#define XENG_KERNEL_PAIR    3  /* 256-input block pairs, clusters of two CTAs       */
+
+/*
+ * xeng_kernel_choice -- the correlation kernel that a handle created now with a
+ *   tensor engine (XENG_ENGINE_*) takes for a launch of n_freq channels x
+ *   n_samples samples (a call's samples go in launches of at most 32,768) of
+ *   n_inputs inputs, storing or adding, on num_sms SMs; plain, rearranged and
+ *   delayed samples alike.  *first_channels (may be NULL): channels that it
+ *   takes; the one pass takes the others in a second launch.  Host code only, no
+ *   device needed.  Returns XENG_KERNEL_*, -1 (bad argument) or -2 (bad size).
+ */
+XENG_API int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t n_samples, int32_t accumulate,
+                                int32_t num_sms, int32_t *first_channels);
 
 #ifdef __cplusplus
 }

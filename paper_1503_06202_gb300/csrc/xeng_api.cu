@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/xeng.h"
+#include "../../include/xeng_peaks.h"
 #include "xeng_internal.h"
 
 using namespace xeng;
@@ -19,6 +20,8 @@ using namespace xeng;
 constexpr int64_t kShiftAheadBytes = int64_t(2) << 30;
 
 static_assert(XENG_MAX_GATES == kMaxGates, "gate set limit of the header and of the kernels");
+static_assert(XENG_KERNEL_SMALL == kSingleSmall && XENG_KERNEL_ONEPASS == kSingleOnepass && XENG_KERNEL_PAIR == kSinglePair,
+              "kernel numbers of the header and of the library");
 
 struct TimedLaunch {
     int kind;  // 0 = decode, 1 = correlate
@@ -289,14 +292,15 @@ cudaError_t launch_fused(xeng_s *h, const uint8_t *block, int64_t T_block, int64
 
 // The single-pass kernel for samples that are rearranged first (pack.cu), so
 // that neither N nor the block's alignment matters; 0: decode to planes.
-int packed_kernel(const xeng_s *h)
+int packed_kernel(int32_t engine, int32_t N, int force)
 {
-    const int32_t pitch = (int32_t)round_up(h->N, 16);
-    if (h->engine == XENG_ENGINE_TENSOR) return single_pass_kernel(nullptr, h->N, h->fused_force, true, pitch);
-    if (h->engine == XENG_ENGINE_TENSOR_FUSED)
-        return single_pass_kernel(nullptr, h->N, h->fused_force == kSingleNone ? 0 : h->fused_force, false, pitch);
+    const int32_t pitch = (int32_t)round_up(N, 16);
+    if (engine == XENG_ENGINE_TENSOR) return single_pass_kernel(nullptr, N, force, true, pitch);
+    if (engine == XENG_ENGINE_TENSOR_FUSED)
+        return single_pass_kernel(nullptr, N, force == kSingleNone ? 0 : force, false, pitch);
     return 0;
 }
+int packed_kernel(const xeng_s *h) { return packed_kernel(h->engine, h->N, h->fused_force); }
 
 cudaError_t ensure_packed(xeng_s *h)
 {
@@ -1474,6 +1478,25 @@ int xeng_selftest_wait_timeout(int64_t limit_ns, int32_t *status, int32_t *threa
     *status = st;
     *threads_left = left;
     return XENG_OK;
+}
+
+int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t n_samples, int32_t accumulate,
+                       int32_t num_sms, int32_t *first_channels)
+{
+    if (engine != XENG_ENGINE_TENSOR && engine != XENG_ENGINE_TENSOR_PLANES && engine != XENG_ENGINE_TENSOR_FUSED)
+        return XENG_ERR_ARG;
+    if (n_inputs < 1 || n_inputs > XENG_MAX_INPUTS || n_freq < 1 || n_samples < 1 || n_samples > kFusedMaxSamples ||
+        num_sms < 2)
+        return XENG_ERR_RANGE;
+    const int force = single_pass_force_from_env();
+    int kernel = packed_kernel(engine, n_inputs, force);
+    int32_t cut = 0;
+    if (kernel && !force) {  // as launch_shaped
+        kernel = single_pass_by_shape(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);
+        cut = single_pass_cut(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);
+    }
+    if (first_channels) *first_channels = cut ? cut : n_freq;
+    return kernel;
 }
 
 int xeng_set_profiling(xeng_t h, int32_t on)

@@ -359,6 +359,23 @@ def xeng_peak_probe(kind: int, iters: int):
     return rc, tf.value, ms.value
 
 
+XENG_KERNEL_PLANES, XENG_KERNEL_SMALL, XENG_KERNEL_ONEPASS, XENG_KERNEL_PAIR = 0, 1, 2, 3
+
+
+def xeng_kernel_choice(engine: int, n_inputs: int, n_freq: int, n_samples: int, accumulate: bool = False,
+                       num_sms: int = 152):
+    """Returns (kernel or status, channels it takes before the one pass takes the rest): include/xeng_peaks.h."""
+    L = lib()
+    if not getattr(L.xeng_kernel_choice, "_typed", False):
+        i32 = ctypes.c_int32
+        L.xeng_kernel_choice.argtypes = [i32, i32, i32, ctypes.c_int64, i32, i32, ctypes.POINTER(i32)]
+        L.xeng_kernel_choice.restype = ctypes.c_int
+        L.xeng_kernel_choice._typed = True
+    first = ctypes.c_int32()
+    rc = L.xeng_kernel_choice(engine, n_inputs, n_freq, n_samples, 1 if accumulate else 0, num_sms, ctypes.byref(first))
+    return rc, first.value
+
+
 # ------------------------------------------------------------------ batches --
 
 XENG_SCHED_LPT = 0

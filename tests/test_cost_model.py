@@ -1,8 +1,10 @@
-"""The bench names the correlation kernel the default engine runs (and takes
-that kernel's DRAM figure for the roofline) from its own copy of the library's
-choice between the two single-pass kernels above 256 inputs.  These checks keep
-that copy equal to the library's build defaults and to the winners measured on
-GB300 (1024 channels, 8192 samples, both kernels forced in turn)."""
+"""Which kernel takes a launch.  Batches choose by N alone between the two
+single-pass kernels above 256 inputs, and the bench counts their launches from its
+own copy of that choice: equal to the library's build defaults and to the winners
+measured on GB300 (1024 channels, 8192 samples, both kernels forced in turn).
+Handles and the streaming service choose by the launch's channels and samples too;
+the bench names the kernel (and takes its DRAM figure for the roofline) as the
+library says it, checked here against measured winners."""
 import ctypes
 import importlib.util
 import os
@@ -11,6 +13,8 @@ import shutil
 import subprocess
 
 import pytest
+
+import paper_1503_06202_gb300 as xe
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SINGLE_PASS = os.path.join(ROOT, "paper_1503_06202_gb300", "csrc", "single_pass.cu")
@@ -58,10 +62,64 @@ def test_pair_when_block_count_is_even_above_384():
 @pytest.mark.parametrize("N,kernel", [(16, "correlate_small"), (256, "correlate_small"),
                                       (272, "correlate_onepass"), (2048, "correlate_pair"),
                                       (3584, "correlate_pair"), (3600, "correlate_tc"),
-                                      (4096, "correlate_tc"), (250, "correlate_tc"), (1000, "correlate_tc")])
+                                      (4096, "correlate_tc"), (250, "correlate_small"), (1000, "correlate_pair")])
 def test_default_engine_path_by_n(N, kernel):
-    # single pass for N a multiple of 16 up to the bound; decoded planes otherwise
+    # 1024 channels x 8192 samples: single pass for every N up to the bound (rows that
+    # TMA cannot address are rearranged first); decoded planes above
     assert _bench().correlate_kernel("tensor", N)[0].startswith(kernel)
+
+
+# (N, channels, samples) and the faster kernel, us a call with the N-only choice / the
+# one pass; 256 x 8 x 4096 the N <= 256 kernel's 24 against 31
+MEASURED_SHAPE = [(1024, 4, 32768, "onepass"),   # 322 / 207
+                  (512, 256, 256, "onepass"),    # 100 / 65
+                  (256, 256, 256, "onepass"),    # 32 / 25
+                  (256, 8, 1024, "onepass"),     # 22.3 / 14.3
+                  (256, 8, 2048, "onepass"),     # 22.5 / 19.2
+                  (256, 8, 4096, "small"),
+                  (256, 48, 4096, "onepass"),    # 37.9 / 31.3
+                  (160, 2, 256, "onepass"),      # 15.0 / 9.0
+                  (128, 152, 4096, "onepass"),   # 39.5 / 27.7
+                  (128, 152, 32768, "small"),    # 168 / 191
+                  (256, 1024, 32768, "small"), (1024, 1024, 8192, "pair"), (2048, 256, 8192, "pair")]
+
+
+@pytest.mark.parametrize("N,F,T,kernel", MEASURED_SHAPE)
+def test_choice_by_launch_shape_matches_measured_winner(N, F, T, kernel, monkeypatch):
+    monkeypatch.delenv("XENG_FUSED_KERNEL", raising=False)
+    assert _bench().correlate_kernel("tensor", N, F, T)[0].startswith("correlate_" + kernel)
+
+
+# Above 256 inputs the last channels may go to the one pass: 1024 x 64 x 8192 is 640
+# items on 76 clusters, eight rounds (60 channels) and 40 items
+def test_last_round_of_few_items_goes_to_the_one_pass(monkeypatch):
+    monkeypatch.delenv("XENG_FUSED_KERNEL", raising=False)
+    for accumulate in (False, True):
+        assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, 1024, 64, 8192, accumulate) == (xe.XENG_KERNEL_PAIR, 60)
+        assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, 2048, 1024, 8192, accumulate) == (xe.XENG_KERNEL_PAIR, 1023)
+    # 76 channels: ten whole rounds
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, 1024, 76, 8192) == (xe.XENG_KERNEL_PAIR, 76)
+    monkeypatch.setenv("XENG_FUSED_KERNEL", "pair")
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, 1024, 64, 8192) == (xe.XENG_KERNEL_PAIR, 64)
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, 1024, 4, 32768) == (xe.XENG_KERNEL_PAIR, 4)
+
+
+def test_executed_work_counts_whole_tiles():
+    b, useful = _bench(), 512 * 513 / 2  # 1216 channels: 48 whole rounds
+    assert b.correlate_kernel("tensor", 512, 1216, 8192)[1] == 3 * 256 ** 2 / useful
+    assert b.correlate_kernel("planes", 512)[1] == 10 * 128 ** 2 / useful
+    useful = 1024 * 1025 / 2
+    assert b.correlate_kernel("tensor", 1024, 64, 8192)[1] == pytest.approx(
+        (60 * 10 * 256 ** 2 + 4 * 36 * 128 ** 2) / 64 / useful, rel=1e-12)
+
+
+def test_choice_argument_checks():
+    T = xe.XENG_ENGINE_TENSOR
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_DP4A, 64, 1, 1)[0] == xe.XENG_ERR_ARG
+    for args in ((0, 1, 1), (4097, 1, 1), (64, 0, 1), (64, 1, 0), (64, 1, 32769)):
+        assert xe.xeng_kernel_choice(T, *args)[0] == xe.XENG_ERR_RANGE
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_PLANES, 64, 1, 1)[0] == xe.XENG_KERNEL_PLANES
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_FUSED, 4096, 256, 8192)[0] == xe.XENG_KERNEL_PAIR
 
 
 # The two build parameters hold for every launch shape: a cost of 0 forces that kernel
@@ -87,8 +145,9 @@ def test_a_cost_of_zero_forces_a_kernel(pair, onepass, tmp_path):
                     cut = ctypes.c_int()
                     k = lib.choice(N, F, T, add, ctypes.byref(cut))
                     seen.add((k, cut.value > 0))
-    # 2: one pass, 3: pair kernel, and whether its last round goes to the one pass
+                    if pair and onepass:
+                        assert (k, cut.value or F) == xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, T, add)
     if pair and onepass:
-        assert seen == {(3, False), (3, True), (2, False)}
+        assert seen == {(xe.XENG_KERNEL_PAIR, False), (xe.XENG_KERNEL_PAIR, True), (xe.XENG_KERNEL_ONEPASS, False)}
     else:
-        assert seen == {(2 if pair else 3, False)}
+        assert seen == {(xe.XENG_KERNEL_ONEPASS if pair else xe.XENG_KERNEL_PAIR, False)}
