@@ -178,3 +178,24 @@ def test_batch_info_without_planes_jobs():
     info = b.info()
     assert info["n_items"] == 1 and info["grid"] == 1
     b.close()
+
+
+def test_batch_rearranged_jobs():
+    """Jobs of 16 MiB and more whose rows TMA cannot address (N not a multiple of 16, a
+    block off a 16-byte boundary) are rearranged and take a single-pass kernel, in rounds
+    of 32,768 samples; below that they go through the planes.  Every job as the oracle."""
+    shapes = [(42000, 4, 100), (8400, 10, 200), (29000, 1, 600), (40000, 1, 1001), (33000, 2, 256), (1000, 1, 100),
+              (2100, 4, 2005)]
+    host, jobs = make_jobs(shapes, seed=46)
+    k, n = 4, host[4].size  # N = 256 off a 16-byte boundary
+    flat = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
+    flat[8:8 + n] = jobs[k][0].flatten()
+    jobs[k] = (flat[8:8 + n].view(host[k].shape), jobs[k][1])
+    b = xe.XBatch(jobs)
+    assert b.info()["n_items"] == 1  # of the one job on planes
+    for _ in range(2):  # a second run overwrites
+        b.run()
+    torch.cuda.synchronize()
+    for (T, F, N), blk, (_, out) in zip(shapes, host, jobs):
+        assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk)), (T, F, N)
+    b.close()

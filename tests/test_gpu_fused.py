@@ -1,4 +1,4 @@
-"""The fused decode + correlation (N a multiple of 16).  Up to 256 inputs, single
+"""The fused decode + correlation.  Up to 256 inputs, single
 CTAs over 128-input blocks: bit-exact against the oracle for tiny N (tiles
 mostly padding), up to and above 128 inputs (diagonal items of two channels;
 row items and diagonal items of the upper input halves), odd channel counts (a
@@ -115,10 +115,8 @@ def test_small_items_shared_whole_or_cut(T, F, N):
     assert np.array_equal(correlate(blk, pieces=[T // 3])[keep], want)
 
 
-# Launches whose kernel is chosen by their shape: a few stages (one pass, N <= 256
-# too, where sharing or cutting the items would take longer), one round (one pass)
-# and, at N = 512 x 26 channels, 78 items for 76 clusters: 25 channels by the pair
-# kernel, the last by the one pass.
+# Launches whose kernel is chosen by their shape: a few stages or rounds (one pass, N <=
+# 256 too, where sharing or cutting the items would take longer).
 @pytest.mark.parametrize("T,F,N", [(130, 40, 512), (1500, 26, 512), (700, 3, 1024), (200, 300, 128), (256, 90, 256),
                                    (8, 2, 16), (511, 7, 208), (1000, 3, 144), (2048, 8, 256), (4000, 150, 128),
                                    (4096, 48, 256)])
@@ -130,6 +128,36 @@ def test_kernel_by_launch_shape(T, F, N):
     assert np.array_equal(correlate(blk)[keep], want)
     # the later pushes add, the last of them a few samples
     assert np.array_equal(correlate(blk, pieces=[T // 2, T // 2 - 3])[keep], want)
+
+
+# Above 256 inputs a last round of the pair kernel with few items goes to the one pass,
+# as a second launch: 2048 x 7 channels (252 items on 76 clusters, six channels fill
+# three rounds), 1280 x 17 (255, 15 channels).  A call and a push store, a second push
+# adds; the channels on both sides of the cut against the oracle.
+@pytest.mark.parametrize("N,F", [(2048, 7), (1280, 17)])
+def test_last_round_of_the_pair_kernel_by_the_one_pass(N, F):
+    T, sms = 6000, torch.cuda.get_device_properties(0).multi_processor_count
+    kernel, cut = xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, T, False, sms)
+    assert kernel == xe.XENG_KERNEL_PAIR and 0 < cut < F
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, T, True, sms) == (kernel, cut)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N)
+    block = torch.randint(0, 256, (T, F, N), dtype=torch.uint8, device="cuda", generator=g)
+    eng = xe.XEngine(N, F, 2 * T)
+    out = torch.full((F, N * (N + 1) // 2, 2), 77, dtype=torch.int32, device="cuda")
+    eng.correlate(block, out)
+    st = eng.stats(reset=True)
+    assert st["correlate_launches"] == 1 and st["launches"] == 2
+    keep = sorted({0, cut - 1, cut, F - 1})
+    want = torch.from_numpy(oracle.correlate(np.ascontiguousarray(block[:, keep].cpu().numpy())))
+    assert torch.equal(out[keep].cpu().to(torch.int64), want)
+    for _ in range(2):
+        eng.push(block)
+    assert eng.stats(reset=True)["launches"] == 4
+    added = torch.full_like(out, 77)
+    assert eng.dump(added) == 2 * T
+    assert torch.equal(added, 2 * out)
+    eng.close()
 
 
 # Samples rearranged first (pack.cu): rows off 16 bytes, fewer inputs than a chunk,
@@ -265,13 +293,15 @@ def test_fused_raw_int32_beyond_f32_range(fused_kernel):
     assert (out[..., 0] == 128 * T).all() and (out[..., 1] == 0).all()
 
 
-@pytest.mark.parametrize("N", [272, 512])
-def test_single_pass_host_pipeline_channel_groups(N):
+@pytest.mark.parametrize("N,force", [(272, None), (512, None), (512, "pair")])
+def test_single_pass_host_pipeline_channel_groups(N, force, monkeypatch):
     # host in, host out through the channel-group pipeline (at least two groups of
     # about 400 KB rows, each correlated and downloaded in four channel sub-ranges)
-    # with the single-pass kernels (one pass over 128-input block pairs at 272 inputs,
-    # 256-input block pairs at 512): the same bits as device buffers, sampled channels
-    # as the oracle
+    # with the single-pass kernels (the one pass over 128-input block pairs, which such
+    # short launches take, and 256-input block pairs): the same bits as device buffers,
+    # sampled channels as the oracle
+    if force:
+        monkeypatch.setenv("XENG_FUSED_KERNEL", force)
     rng = np.random.default_rng(N + 5)
     T, F = 160, 2 * 409600 // N + 3
     blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
@@ -292,9 +322,11 @@ def test_single_pass_host_pipeline_channel_groups(N):
 
 @pytest.mark.parametrize("N", [3584, 3600])
 def test_default_engine_at_its_single_pass_bound(N):
-    # the default engine takes the single pass up to 3584 inputs (here the pair
-    # kernel) and decodes to planes above: both exact against the oracle on a
+    # the default engine takes the single pass up to 3584 inputs (here, two stages, the
+    # one pass) and decodes to planes above: both exact against the oracle on a
     # few sampled channels, and the same bits as the single-pass engine at 3600
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, 2, 160)[0] == (
+        xe.XENG_KERNEL_ONEPASS if N == 3584 else xe.XENG_KERNEL_PLANES)
     rng = np.random.default_rng(N + 7)
     T, F = 160, 2
     blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)

@@ -157,10 +157,11 @@ def test_gate_sets_flags_on_plain_integration_and_argument_checks():
 
 # Gate sets of unlike lengths side by side in one launch, or one after another where a
 # set is empty or far longer than the others: 1 sample, a stage more than the others,
-# 64 sets, rows off 16 bytes, two rounds (more than 32,768 samples of a set)
+# 64 sets, rows off 16 bytes, two rounds (more than 32,768 samples of a set; the call
+# that takes a block whole refuses more than 65,536)
 @pytest.mark.parametrize("N,F,sizes", [(160, 2, (640, 641, 1, 639)), (61, 3, (5,) * 64), (272, 2, (300, 128, 129)),
                                        (1040, 1, (200, 90)), (128, 5, (3000, 1, 2)), (48, 40, (9, 0, 4)),
-                                       (32, 1, (33000, 32900))])
+                                       (32, 1, (33000, 32000)), (24, 2, (40000, 3)), (32, 1, (33000, 32900))])
 def test_gate_sets_of_unlike_lengths(N, F, sizes):
     G, T = len(sizes), sum(sizes) + 7
     rng = np.random.default_rng(N + F + G)
@@ -171,8 +172,13 @@ def test_gate_sets_of_unlike_lengths(N, F, sizes):
     want, want_counts = oracle.correlate_gated(blk, gate, G, valid)
     d, v = torch.from_numpy(blk).cuda(), torch.from_numpy(valid).cuda()
     eng = xe.XEngine(N, F, 2 * T)
-    got, counts = gated(eng, d, gate, G, v) if T <= 32768 else (want, want_counts)
-    assert np.array_equal(got, want) and np.array_equal(counts, want_counts)
+    if T <= 65536:
+        got, counts = gated(eng, d, gate, G, v)
+        assert np.array_equal(got, want) and np.array_equal(counts, want_counts)
+    else:
+        untouched = torch.full((G, F, N * (N + 1) // 2, 2), 77, dtype=torch.int32, device="cuda")
+        assert xe.xeng_correlate_gated(eng.h, d, T, gate, G, v, untouched, None) == xe.XENG_ERR_RANGE
+        assert (untouched == 77).all()
     # a push that stores and one that adds
     assert xe.xeng_set_gates(eng.h, G) == xe.XENG_OK
     out = torch.full((G, F, N * (N + 1) // 2, 2), 77, dtype=torch.int32, device="cuda")

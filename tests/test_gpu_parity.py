@@ -137,11 +137,12 @@ RAW_LAUNCH = 32768
 
 
 # N = 256: the single-pass kernel of up to 256 inputs; N = 272: the single pass
-# over 128-input block pairs; N = 1024: the single pass over 256-input block
-# pairs, and at N = 1040 (a ragged last block) forced by XENG_FUSED_KERNEL; the
-# TMA decode's raw planes + tensor correlator (planes engine)
+# over 128-input block pairs; N = 1024 and 1040 (a ragged last block): the single
+# pass over 256-input block pairs, forced by XENG_FUSED_KERNEL, since one or two
+# channels would take the other; the TMA decode's raw planes + tensor correlator
+# (planes engine)
 RAW_CASES = [(256, xe.XENG_ENGINE_TENSOR, None), (272, xe.XENG_ENGINE_TENSOR, None),
-             (1024, xe.XENG_ENGINE_TENSOR, None), (1040, xe.XENG_ENGINE_TENSOR, "pair"),
+             (1024, xe.XENG_ENGINE_TENSOR, "pair"), (1040, xe.XENG_ENGINE_TENSOR, "pair"),
              (1040, xe.XENG_ENGINE_TENSOR_PLANES, None)]
 
 

@@ -147,7 +147,7 @@ def test_shift_argument_checks_and_removal():
 
 # Delayed inputs in some 128-input blocks only (copied, the others read in place),
 # whole 16-input chunks and single inputs, pushes longer and shorter than the
-# delays and across the ring's end; 26 channels of 512 inputs run as two launches
+# delays and across the ring's end
 @pytest.mark.parametrize("N,F,delays", [(512, 26, {0: 5, 130: 700, 131: 700}), (272, 2, {i: 40 for i in range(16, 32)}),
                                         (256, 3, {3: 1, 255: 999}), (1040, 1, {1039: 300, 500: 1}),
                                         (61, 4, {60: 17, 0: 1000})])
@@ -157,6 +157,47 @@ def test_shift_some_blocks(N, F, delays):
         d[i] = v
     stream, got = run_stream(N, F, 2000, d, [900, 100, 700, 200, 1000], {1, 3, 4}, seed=N + F)
     check(stream, d, got)
+
+
+# The same through the kernel over 256-input block pairs: substituted blocks in either
+# CTA's half, both or neither, in the rows and the columns of diagonal pairs and others,
+# in a last block of 16 inputs
+@pytest.mark.parametrize("N,F,delays", [(1040, 3, {5: 700, 300: 1, 640: 41, 1039: 300}), (512, 2, {200: 33}),
+                                        (528, 1, {0: 9, 128: 800, 256: 2, 384: 7, 520: 64}), (2048, 1, {1900: 500})])
+def test_shift_some_blocks_by_pair_kernel(N, F, delays, monkeypatch):
+    monkeypatch.setenv("XENG_FUSED_KERNEL", "pair")
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, 900)[0] == xe.XENG_KERNEL_PAIR
+    d = np.zeros(N, np.int32)
+    for i, v in delays.items():
+        d[i] = v
+    stream, got = run_stream(N, F, 2000, d, [900, 100, 700, 200], {1, 3}, seed=N + F)
+    check(stream, d, got)
+
+
+# Substituted blocks across the cut of a launch whose last round goes to the one pass:
+# 1280 x 17 channels, 15 by the pair kernel; a push that stores and one that adds
+def test_shift_across_the_cut_of_a_launch():
+    N, F, T, sms = 1280, 17, 6000, torch.cuda.get_device_properties(0).multi_processor_count
+    kernel, cut = xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, T, False, sms)
+    assert kernel == xe.XENG_KERNEL_PAIR and 0 < cut < F
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR, N, F, T, True, sms) == (kernel, cut)
+    d = np.zeros(N, np.int32)
+    d[[5, 300, 700, 701, 1279]] = 7000, 1, 41, 5999, 300
+    g = torch.Generator(device="cuda")
+    g.manual_seed(9)
+    stream = torch.randint(0, 256, (2 * T, F, N), dtype=torch.uint8, device="cuda", generator=g)
+    eng = xe.XEngine(N, F, 2 * T)
+    eng.set_delays(d)
+    for k in range(2):
+        eng.push(stream[k * T:(k + 1) * T])
+        st = eng.stats(reset=True)
+        assert st["correlate_launches"] == 1 and st["launches"] == 3  # rearranged, then two
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    assert eng.dump(out) == 2 * T
+    eng.close()
+    keep = [0, cut - 1, cut, F - 1]
+    want = oracle.correlate_shifted(np.ascontiguousarray(stream[:, keep].cpu().numpy()), d, 0, 2 * T)
+    assert np.array_equal(out[keep].cpu().numpy().astype(np.int64), want)
 
 
 # Many delayed inputs and a long integration: the history has no room for the pushes'
