@@ -21,6 +21,7 @@ namespace {
 constexpr int kPackThreads = 256;
 constexpr int kPackRows = 4;       // rows loaded before any is stored
 constexpr int kPackSpan = 256;     // rows per thread at most (byte-lane counts are widened every 240)
+constexpr int kPackCountSpan = 32; // rows per thread, where a block adds its counts to memory, unless SMs idle
 
 // Blocks of 256 threads over the `all` columns of a row (all of them, or 256) and,
 // where a row is shorter, several rows; each thread walks at most kPackSpan rows, fewer
@@ -40,7 +41,10 @@ PackGrid pack_grid(const PackArgs &a, int64_t all, int num_sms)
     const int64_t nx = (all + g.cols - 1) / g.cols, sets = a.sets > 0 ? a.sets : 1;
     auto ny = [&]() { return (a.nt + (int64_t)g.span * g.rows - 1) / ((int64_t)g.span * g.rows); };
     g.span = kPackSpan;
-    while (g.span > 2 * kPackRows && sets * nx * ny() < 16 * num_sms) g.span /= 2;
+    auto few = [&]() {
+        return sets * nx * ny() < (a.valid && a.counts && g.span <= kPackCountSpan ? 2 : 16) * (int64_t)num_sms;
+    };
+    while (g.span > 2 * kPackRows && few()) g.span /= 2;
     g.nx = (int)nx;
     g.ny = (int)ny();
     return g;
@@ -86,15 +90,21 @@ __device__ __forceinline__ void pack_column(const PackArgs &a, int64_t col, int 
     ic = 16 * (a.chunks ? a.chunks[k].y : k);
 }
 
+// Where a block keeps the usable samples of input m of its column `lc`, so that the
+// lanes of a warp, each with its own column, meet two to a bank.
+__device__ __forceinline__ int count_slot(int lc, int m) { return lc * 16 + ((m + lc) & 15); }
+
 // kAligned: every source chunk is 16-byte aligned.  Thread = (row of the block's
-// rows, chunk of a sample); block (bx, by) of set `set`.
+// rows, chunk of a sample); block (bx, by) of set `set`.  kValid: the usable samples
+// per input are added up in `count` (shared memory, 16 a column, zeroed by the caller).
 template <bool kAligned, bool kValid>
-__device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, int bx, int by, int set)
+__device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, int bx, int by, int set, int *count)
 {
     const int64_t cols = g.all;
     const int cols_per_block = g.cols, rows_per_block = g.rows, span = g.span;
     constexpr int kRows = !kAligned && kValid ? kPackRows / 2 : kPackRows;  // registers
-    const int64_t col = (int64_t)bx * cols_per_block + threadIdx.x % cols_per_block;
+    const int lc = threadIdx.x % cols_per_block;
+    const int64_t col = (int64_t)bx * cols_per_block + lc;
     const int rsub = threadIdx.x / cols_per_block;
     if (col >= cols || rsub >= rows_per_block) return;
     int c, j, ic;
@@ -111,7 +121,7 @@ __device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, 
     uint8_t *out = a.out + ((int64_t)set * a.nf + c) * a.pitch + j * 16;
     uint32_t acc[4] = {0, 0, 0, 0};                       // usable samples, a byte per input
     uint32_t acc16[8] = {0, 0, 0, 0, 0, 0, 0, 0};         // the same, 16-bit lanes
-    int rows = 0, pending = 0;
+    int pending = 0;
     auto widen = [&]() {
         #pragma unroll
         for (int k = 0; k < 4; k++) {
@@ -149,7 +159,6 @@ __device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, 
                     acc[j] += ~z & 0x01010101u;
                 }
             }
-            ++rows;
             *reinterpret_cast<uint4 *>(out + tk * out_row) = make_uint4(w[0], w[1], w[2], w[3]);
         }
         if (kValid && (pending += kRows) > 240 - kRows) widen();
@@ -161,12 +170,14 @@ __device__ __forceinline__ void pack_rows(const PackArgs &a, const PackGrid &g, 
             *reinterpret_cast<uint4 *>(out + t * out_row) = make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);
     }
     if (!a.counts) return;
-    if (kValid) widen();
-    int32_t *cnt = a.counts + ((int64_t)set * a.nf + c) * a.N + ic;
-    #pragma unroll
-    for (int m = 0; m < 16; m++) {
-        const int usable = kValid ? (int)((acc16[2 * (m >> 2) + (m & 1)] >> (16 * ((m >> 1) & 1))) & 0xFFFFu) : rows;
-        if (m < n && usable) atomicAdd(cnt + m, usable);
+    if (kValid) {
+        widen();
+        #pragma unroll
+        for (int m = 0; m < 16; m++)
+            atomicAdd(count + count_slot(lc, m), (int)((acc16[2 * (m >> 2) + (m & 1)] >> (16 * ((m >> 1) & 1))) & 0xFFFFu));
+    } else if (by == 0 && rsub == 0) {  // every sample usable: the first block adds the set's
+        int32_t *cnt = a.counts + ((int64_t)set * a.nf + c) * a.N + ic;
+        for (int m = 0; m < n; m++) atomicAdd(cnt + m, (int)have);
     }
 }
 
@@ -248,10 +259,34 @@ __device__ __forceinline__ void pack_shifted_rows(const PackArgs &a, const Shift
     }
 }
 
+// A block's counts go to memory from shared memory, consecutive inputs by consecutive
+// threads: added by each thread, 16 inputs apart, they took longer than the samples where
+// a row is short and its blocks many (GB300, one gate with flags, N = 560 x 5 channels x
+// 26,713 samples 278 us and so 46; without flags, N = 256 x 64 x 8192, 277 and 43 with
+// the samples counted once).  Blocks an SM: unaligned rows, without flags, 42 us with
+// four and 47 with three (N = 203 x 64 x 10,007).
 template <bool kAligned, bool kValid>
-__global__ void __launch_bounds__(kPackThreads) pack_kernel(const __grid_constant__ PackArgs a, const PackGrid g)
+__global__ void __launch_bounds__(kPackThreads, kValid ? 3 : kAligned ? 0 : 4)
+pack_kernel(const __grid_constant__ PackArgs a, const PackGrid g)
 {
-    pack_rows<kAligned, kValid>(a, g, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z);
+    if constexpr (!kValid) {
+        pack_rows<kAligned, false>(a, g, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, nullptr);
+    } else {
+        __shared__ int count[16 * kPackThreads];
+        for (int k = threadIdx.x; k < 16 * g.cols; k += kPackThreads) count[k] = 0;
+        __syncthreads();
+        pack_rows<kAligned, true>(a, g, (int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, count);
+        __syncthreads();
+        if (!a.counts) return;
+        // the block's columns from its first on: channel c0, chunk k0
+        const int per = a.pitch / 16, m = threadIdx.x & 15;
+        const int64_t col0 = (int64_t)blockIdx.x * g.cols, c0 = col0 / per;
+        const int k0 = (int)(col0 - c0 * per), cols = (int)min((int64_t)g.cols, g.all - col0);
+        for (int lc = threadIdx.x >> 4; lc < cols; lc += kPackThreads / 16) {
+            const int c = (k0 + lc) / per, ic = 16 * (k0 + lc - c * per), usable = count[count_slot(lc, m)];
+            if (ic + m < a.N && usable) atomicAdd(a.counts + ((int64_t)blockIdx.z * a.nf + c0 + c) * a.N + ic + m, usable);
+        }
+    }
 }
 
 // The chunks of `a` and, after their blocks, those of `b`, which hold delayed inputs.
@@ -261,7 +296,7 @@ pack_shifted_kernel(const __grid_constant__ PackArgs a, const __grid_constant__ 
                     const __grid_constant__ ShiftArgs sa, const PackGrid ga, const PackGrid gb)
 {
     const int na = ga.nx * ga.ny, x = (int)blockIdx.x;
-    if (x < na) pack_rows<kAligned, false>(a, ga, x % ga.nx, x / ga.nx, 0);
+    if (x < na) pack_rows<kAligned, false>(a, ga, x % ga.nx, x / ga.nx, 0, nullptr);
     else pack_shifted_rows<kAhead>(b, sa, gb, (x - na) % gb.nx, (x - na) / gb.nx);
 }
 

@@ -189,3 +189,26 @@ def test_gate_sets_of_unlike_lengths(N, F, sizes):
     assert np.array_equal(out.cpu().numpy().astype(np.int64), 2 * want)
     assert np.array_equal(cnt.cpu().numpy().astype(np.int64), 2 * want_counts)
     eng.close()
+
+
+# Usable samples per (set, channel, input), with flags and without: columns of several
+# channels in a block, blocks that begin inside a channel, fewer columns than a block has
+# threads, a set in two rounds (more than 32,768 samples) and sets one after another
+@pytest.mark.parametrize("N,F,T,G", [(200, 30, 700, 1), (200, 30, 700, 3), (16, 1, 40000, 1), (40, 2, 300, 2),
+                                     (61, 90, 2100, 2), (272, 5, 9000, 1)])
+def test_gated_counts(N, F, T, G):
+    rng = np.random.default_rng(N + T)
+    blk = rng.integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    gate = np.minimum(rng.integers(-1, 4 * G, T), G - 1).astype(np.int32)  # the last set far longer
+    valid = (rng.random((T, F, N)) > 0.2).astype(np.uint8) * rng.integers(1, 256, size=(T, F, N), dtype=np.uint8)
+    d, v = torch.from_numpy(blk).cuda(), torch.from_numpy(valid).cuda()
+    eng = xe.XEngine(N, F, T)
+    for flags in (v, None):
+        got, counts = gated(eng, d, gate, G, flags)
+        use = (valid != 0).astype(np.uint8) if flags is not None else np.ones_like(valid)
+        assert np.array_equal(counts, np.stack([use[gate == g].sum(axis=0, dtype=np.int64) for g in range(G)]))
+        for f in (0, F - 1):
+            want, _ = oracle.correlate_gated(np.ascontiguousarray(blk[:, f:f + 1]), gate, G,
+                                             np.ascontiguousarray(use[:, f:f + 1]))
+            assert np.array_equal(got[:, f:f + 1], want)
+    eng.close()
