@@ -62,7 +62,8 @@ XENG_API int xeng_peak_probe(int32_t kind, int64_t iters, double *tflops, double
  *   tensor engine (XENG_ENGINE_*) takes for a launch of n_freq channels x
  *   n_samples samples (a call's samples go in launches of at most 32,768) of
  *   n_inputs inputs, storing or adding, on num_sms SMs; plain, rearranged and
- *   delayed samples alike.  *first_channels (may be NULL): channels that it
+ *   delayed samples alike (but 8192 rearranged or delayed samples and more of few
+ *   channels, above 256 inputs, decode to planes).  *first_channels (may be NULL): channels that it
  *   takes; the one pass takes the others in a second launch.  Host code only, no
  *   device needed.  Returns XENG_KERNEL_*, -1 (bad argument) or -2 (bad size).
  */

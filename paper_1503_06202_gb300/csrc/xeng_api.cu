@@ -302,15 +302,38 @@ int packed_kernel(int32_t engine, int32_t N, int force)
 }
 int packed_kernel(const xeng_s *h) { return packed_kernel(h->engine, h->N, h->fused_force); }
 
+// Many samples of few channels, above 256 inputs, decode to planes after all: their
+// items leave SMs idle either way, so a call takes as long as one item, at 0.6 us a
+// stage of 128 samples from planes and 0.75-0.88 split on the way, and decoding few
+// rows costs little (GB300, us rearranged / planes: N = 713 x 2 channels x 99,296
+// samples 739 / 619, 354 x 2 x 28,340 182 / 155, 364 x 2 x 14,662 99 / 86, two inputs of
+// 484 x 1 x 34,956 delayed 245 / 204; past the line 280 x 3 x 6214 48 / 46, 1252 x 2 x
+// 27,363 204 / 205, 372 x 11 x 83,069 599 / 759, delayed 1184 x 2 x 19,769 131 / 152).
+// The line: channels times inputs in whole 128-input blocks, and samples; delayed
+// inputs only through the TMA decode (379 x 3 x 45,877 308 / 327).
+constexpr int64_t kPlanesRows = 1536, kPlanesSamples = 8192;
+bool decodes_long_calls(const xeng_s *h)
+{
+    return h->engine == XENG_ENGINE_TENSOR && !h->fused_force && h->N > 256 &&
+           h->F * round_up(h->N, kTile) <= kPlanesRows && h->t_integ >= kPlanesSamples;
+}
+int packed_kernel(const xeng_s *h, int64_t n_samples)
+{
+    return n_samples >= kPlanesSamples && decodes_long_calls(h) ? 0 : packed_kernel(h);
+}
+
+// Both buffers where a longer call may decode to planes: it may be captured.
 cudaError_t ensure_packed(xeng_s *h)
 {
-    if (h->packed) return cudaSuccess;
-    cudaError_t e = cudaMalloc(&h->packed, (size_t)h->packed_bytes);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        h->packed = nullptr;
+    if (!h->packed) {
+        cudaError_t e = cudaMalloc(&h->packed, (size_t)h->packed_bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h->packed = nullptr;
+            return e;
+        }
     }
-    return e;
+    return decodes_long_calls(h) ? ensure_planes(h) : cudaSuccess;
 }
 
 // Run one kernel launch, bracketed by events when profiling.
@@ -762,13 +785,14 @@ cudaError_t integrate(xeng_s *h, const uint8_t *dblock, int64_t n_samples, int32
         }
         return e;
     }
-    if (const int kernel = packed_kernel(h)) {
+    const bool may_decode = !apply_shift || (h->decode_tma && decode_tma_ok(dblock, h->N));
+    if (const int kernel = may_decode ? packed_kernel(h, n_samples) : packed_kernel(h)) {
         if (!apply_shift)
             return integrate_packed(h, kernel, dblock, (int32_t)F, 0, (int32_t)F, n_samples, nullptr, nullptr, nullptr,
                                     target, fresh, s);
         return integrate_shifted(h, kernel, dblock, n_samples, target, fresh, s);
     }
-    e = ensure_planes(h);
+    e = packed_kernel(h) ? ensure_packed(h) : ensure_planes(h);
     for (int64_t t0 = 0; t0 < n_samples && e == cudaSuccess; t0 += h->chunk_t) {
         const int64_t nt = (n_samples - t0) < h->chunk_t ? (n_samples - t0) : h->chunk_t;
         const int64_t t_pad = round_up(nt, kTile);
@@ -1126,7 +1150,7 @@ int xeng_correlate_gated(xeng_t h, const uint8_t *block, int64_t n_samples, cons
             e = cudaMemsetAsync(out_g, 0, (size_t)(F * nb2 * 4), s);
             continue;
         }
-        if (pk) {
+        if (pk && packed_kernel(h, Tg)) {
             e = integrate_packed(h, pk, block, (int32_t)F, 0, (int32_t)F, Tg, h->gidx + cnt[g], valid,
                                  counts ? counts + (int64_t)g * F * N : nullptr, out_g, true, s);
             continue;
@@ -1333,7 +1357,7 @@ int xeng_push_gated(xeng_t h, const uint8_t *block, int64_t n_samples, const int
             continue;
         }
         int32_t *set = h->acc + (int64_t)g * F * nb2;
-        if (pk) {
+        if (pk && packed_kernel(h, Tg)) {
             e = integrate_packed(h, pk, block, (int32_t)F, 0, (int32_t)F, Tg, h->gidx + cnt[g], valid,
                                  valid ? h->counts + (int64_t)g * F * N : nullptr, set, set_fresh(h, g), s);
             mark_set_used(h, g);

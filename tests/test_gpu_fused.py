@@ -356,3 +356,32 @@ def test_long_launch_captured_after_a_short_one():
     torch.cuda.synchronize()
     assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk))
     eng.close()
+
+
+# Long calls of few channels, above 256 inputs, decode to planes where samples would be
+# rearranged (from 8192 samples, up to 1536 channels x inputs in 128-input blocks): both
+# sides of both lines, one call, pushes of both kinds, and one captured after a short call
+@pytest.mark.parametrize("N,F", [(283, 4), (283, 5), (1025, 1), (257, 1)])
+def test_long_unaligned_calls_of_few_channels(N, F):
+    T = 8192 + 8191
+    blk = np.random.default_rng(N + F).integers(0, 256, size=(T, F, N), dtype=np.uint8)
+    want = oracle.correlate(blk)
+    assert np.array_equal(correlate(blk[:8191]), oracle.correlate(blk[:8191]))
+    assert np.array_equal(correlate(blk), want)
+    for pieces in ([8191], [8192], [100, 9000]):
+        assert np.array_equal(correlate(blk, pieces=pieces), want)
+    block = torch.from_numpy(blk).cuda()
+    out = torch.empty((F, N * (N + 1) // 2, 2), dtype=torch.int32, device="cuda")
+    eng = xe.XEngine(N, F, T)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    eng.correlate(block, out, 128, s.cuda_stream)
+    s.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        eng.correlate(block, out, T, s.cuda_stream)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy().astype(np.int64), want)
+    eng.close()

@@ -158,10 +158,12 @@ def test_gate_sets_flags_on_plain_integration_and_argument_checks():
 # Gate sets of unlike lengths side by side in one launch, or one after another where a
 # set is empty or far longer than the others: 1 sample, a stage more than the others,
 # 64 sets, rows off 16 bytes, two rounds (more than 32,768 samples of a set; the call
-# that takes a block whole refuses more than 65,536)
+# that takes a block whole refuses more than 65,536), a set that decodes to planes (8192
+# samples and more of few channels) beside ones that are rearranged
 @pytest.mark.parametrize("N,F,sizes", [(160, 2, (640, 641, 1, 639)), (61, 3, (5,) * 64), (272, 2, (300, 128, 129)),
                                        (1040, 1, (200, 90)), (128, 5, (3000, 1, 2)), (48, 40, (9, 0, 4)),
-                                       (32, 1, (33000, 32000)), (24, 2, (40000, 3)), (32, 1, (33000, 32900))])
+                                       (32, 1, (33000, 32000)), (24, 2, (40000, 3)), (32, 1, (33000, 32900)),
+                                       (272, 4, (8192, 8191, 5)), (289, 1, (70000, 300))])
 def test_gate_sets_of_unlike_lengths(N, F, sizes):
     G, T = len(sizes), sum(sizes) + 7
     rng = np.random.default_rng(N + F + G)

@@ -251,3 +251,15 @@ def test_shift_captured_pushes():
         want = oracle.correlate_shifted(stream[:(k + 1) * n], d, k * n, (k + 1) * n)
         assert np.array_equal(out.cpu().numpy().astype(np.int64), want), k
     eng.close()
+
+
+# Pushes that are rearranged and pushes that decode to planes (8192 samples and more of
+# few channels) in one stream: the history goes on from one to the other, pushes longer
+# than it and shorter than the delays among them
+@pytest.mark.parametrize("N,F,delays", [(272, 2, {3: 700, 130: 9500, 271: 1}), (512, 3, {200: 20000, 511: 40})])
+def test_shift_pushes_rearranged_and_decoded(N, F, delays):
+    d = np.zeros(N, np.int32)
+    for i, v in delays.items():
+        d[i] = v
+    stream, got = run_stream(N, F, 30000, d, [900, 8192, 100, 300, 9000, 8191, 8500, 700], {1, 2, 4, 5, 7}, seed=N + F)
+    check(stream, d, got)
