@@ -426,8 +426,10 @@ int xeng_create(int32_t n_inputs, int32_t n_freq, int64_t t_integ, xeng_t *out_h
     h->planes_bytes = g * per_ch;
     {
         // the same budget for rearranged samples: rounds of channels x at most
-        // kFusedMaxSamples samples x whole 128-input blocks
-        const int64_t per = std::min<int64_t>(h->chunk_t, kFusedMaxSamples) * round_up(n_inputs, kTile);
+        // kFusedMaxSamples samples x whole 128-input blocks, and an eighth and a tile more
+        // samples, since gate sets side by side all take as many as the longest
+        const int64_t samples = std::min<int64_t>(h->chunk_t, kFusedMaxSamples);
+        const int64_t per = (samples + samples / 8 + kTile) * round_up(n_inputs, kTile);
         h->packed_bytes = std::min<int64_t>(n_freq, std::max<int64_t>(1, budget / per)) * per;
     }
 

@@ -214,3 +214,19 @@ def test_gated_counts(N, F, T, G):
                                              np.ascontiguousarray(use[:, f:f + 1]))
             assert np.array_equal(got[:, f:f + 1], want)
     eng.close()
+
+
+# Sets whose longest, taken that many times, is more than the block: still side by side
+def test_gate_sets_longer_together_than_the_block():
+    N, F, sizes = 292, 8, (60, 20, 20, 20)
+    rng = np.random.default_rng(3)
+    gate = np.repeat(np.arange(4), sizes).astype(np.int32)
+    rng.shuffle(gate)
+    blk = rng.integers(0, 256, size=(len(gate), F, N), dtype=np.uint8)
+    eng = xe.XEngine(N, F, len(gate))
+    got, counts = gated(eng, torch.from_numpy(blk).cuda(), gate, 4)
+    st = eng.stats()
+    assert st["decode_launches"] == 1 and st["correlate_launches"] == 1
+    want, want_counts = oracle.correlate_gated(blk, gate, 4)
+    assert np.array_equal(got, want) and np.array_equal(counts, want_counts)
+    eng.close()
