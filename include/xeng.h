@@ -72,15 +72,17 @@ extern "C" {
                                         the launch's channels and samples.  Blocks that TMA cannot address (N
                                         not a multiple of 16, or not 16-byte aligned), gated and delayed
                                         samples are rearranged first (buffer of up to 16 GiB, allocated at the
-                                        first such call).  The environment variable XENG_FUSED_KERNEL=onepass
-                                        or =pair (read by xeng_create) forces one of the two for every such N.
+                                        first such call; long calls of few channels decode to planes).  The
+                                        environment variable XENG_FUSED_KERNEL=onepass or =pair (read by
+                                        xeng_create) forces that kernel for every such N.
                                         Otherwise as XENG_ENGINE_TENSOR_PLANES                               */
 #define XENG_ENGINE_DP4A          1  /* plain CUDA-core kernel: int8 dp4a straight from the bytes            */
 #define XENG_ENGINE_TENSOR_PLANES 2  /* two passes: decode to FP8 planes in HBM, then the tensor-core GEMM
                                         (decode buffer of up to 16 GiB, allocated at the first such call)    */
 #define XENG_ENGINE_TENSOR_FUSED  3  /* the default engine's single pass also above the N up to which the default
-                                        engine takes it (the build parameter XENG_FUSED_MAX_N, 3584): no
-                                        decode buffer, about 2% slower than two passes at N = 4096           */
+                                        engine takes it (the build parameter XENG_FUSED_MAX_N, 3584), where N is
+                                        a multiple of 16 and the block 16-byte aligned: no decode buffer, about
+                                        2% slower than two passes at N = 4096                                */
 
 typedef struct xeng_s *xeng_t;
 

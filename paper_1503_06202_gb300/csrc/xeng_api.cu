@@ -261,13 +261,13 @@ cudaError_t run_decode(xeng_s *h, const uint8_t *src, int64_t nt, int32_t F, int
 // apply to this block: launches of at most kFusedMaxSamples samples over all
 // channels, no planes in HBM.  The default engine takes them up to the build's
 // XENG_FUSED_MAX_N inputs, XENG_ENGINE_TENSOR_FUSED for every N they cover.
-int fused_kernel(const xeng_s *h, const uint8_t *block)
+int fused_kernel(int32_t engine, const uint8_t *block, int32_t N, int force)
 {
-    if (h->engine == XENG_ENGINE_TENSOR) return single_pass_kernel(block, h->N, h->fused_force, true);
-    if (h->engine == XENG_ENGINE_TENSOR_FUSED)
-        return single_pass_kernel(block, h->N, h->fused_force == kSingleNone ? 0 : h->fused_force, false);
+    if (engine == XENG_ENGINE_TENSOR) return single_pass_kernel(block, N, force, true);
+    if (engine == XENG_ENGINE_TENSOR_FUSED) return single_pass_kernel(block, N, force == kSingleNone ? 0 : force, false);
     return 0;
 }
+int fused_kernel(const xeng_s *h, const uint8_t *block) { return fused_kernel(h->engine, block, h->N, h->fused_force); }
 
 bool fused_ok(const xeng_s *h, const uint8_t *block) { return fused_kernel(h, block) != 0; }
 
@@ -291,13 +291,16 @@ cudaError_t launch_fused(xeng_s *h, const uint8_t *block, int64_t T_block, int64
 }
 
 // The single-pass kernel for samples that are rearranged first (pack.cu), so
-// that neither N nor the block's alignment matters; 0: decode to planes.
+// that neither N nor the block's alignment matters; 0: decode to planes, above
+// XENG_FUSED_MAX_N inputs with the single-pass engine too, whose promise is for
+// blocks read in place (GB300, N = 4001 x 8 channels x 2048 samples rearranged 436 us,
+// on planes 410).
 int packed_kernel(int32_t engine, int32_t N, int force)
 {
     const int32_t pitch = (int32_t)round_up(N, 16);
     if (engine == XENG_ENGINE_TENSOR) return single_pass_kernel(nullptr, N, force, true, pitch);
     if (engine == XENG_ENGINE_TENSOR_FUSED)
-        return single_pass_kernel(nullptr, N, force == kSingleNone ? 0 : force, false, pitch);
+        return single_pass_kernel(nullptr, N, force == kSingleNone ? 0 : force, true, pitch);
     return 0;
 }
 int packed_kernel(const xeng_s *h) { return packed_kernel(h->engine, h->N, h->fused_force); }
@@ -1515,7 +1518,8 @@ int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t
         num_sms < 2)
         return XENG_ERR_RANGE;
     const int force = single_pass_force_from_env();
-    int kernel = packed_kernel(engine, n_inputs, force);
+    int kernel = fused_kernel(engine, nullptr, n_inputs, force);  // where N lets TMA read the block in place
+    if (!kernel) kernel = packed_kernel(engine, n_inputs, force);
     int32_t cut = 0;
     if (kernel && !force) {  // as launch_shaped
         kernel = single_pass_by_shape(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);

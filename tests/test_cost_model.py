@@ -119,7 +119,10 @@ def test_choice_argument_checks():
     for args in ((0, 1, 1), (4097, 1, 1), (64, 0, 1), (64, 1, 0), (64, 1, 32769)):
         assert xe.xeng_kernel_choice(T, *args)[0] == xe.XENG_ERR_RANGE
     assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_PLANES, 64, 1, 1)[0] == xe.XENG_KERNEL_PLANES
+    # the single-pass engine above the bound: blocks that TMA reads in place
     assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_FUSED, 4096, 256, 8192)[0] == xe.XENG_KERNEL_PAIR
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_FUSED, 4001, 256, 8192)[0] == xe.XENG_KERNEL_PLANES
+    assert xe.xeng_kernel_choice(xe.XENG_ENGINE_TENSOR_FUSED, 3583, 256, 8192)[0] == xe.XENG_KERNEL_PAIR
 
 
 # The two build parameters hold for every launch shape: a cost of 0 forces that kernel

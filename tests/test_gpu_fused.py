@@ -385,3 +385,13 @@ def test_long_unaligned_calls_of_few_channels(N, F):
     torch.cuda.synchronize()
     assert np.array_equal(out.cpu().numpy().astype(np.int64), want)
     eng.close()
+
+
+# The single-pass engine with rows that TMA cannot address: rearranged up to 3584 inputs,
+# decoded to planes above, gates and delays too
+@pytest.mark.parametrize("N", [3583, 3601, 4001])
+def test_single_pass_engine_unaligned(N):
+    blk = np.random.default_rng(N).integers(0, 256, size=(140, 1, N), dtype=np.uint8)
+    want = oracle.correlate(blk)
+    assert np.array_equal(correlate(blk, engine=FUSED), want)
+    assert np.array_equal(correlate(blk, pieces=[70], engine=FUSED), want)
