@@ -58,8 +58,6 @@ DRAM_BYTES_PER_CHANNEL = {
 # block pair (tens of us per 1024 channels x 8192 samples) times the upper-triangle
 # block pairs.
 PAIR_COST, ONEPASS_COST, FUSED_MAX_N = 118, 36, 3584
-# Bytes from which a batch rearranges a job whose rows TMA cannot address.
-BATCH_PACK_BYTES = 16 << 20
 
 
 def use_pair_kernel(N):
@@ -241,15 +239,30 @@ def run_reference(args, rank, world):
     print(json.dumps(line), flush=True)
 
 
-def batch_launches(recipes):
+def batch_rearranges(r, num_sms=152):
+    """Whether a batch rearranges a job whose rows TMA cannot address, as the library
+    decides it: from 16 MiB on, where its own two launches take less than a share of
+    the launches over planes."""
+    import paper_1503_06202_gb300 as xe
+
+    if r.N > FUSED_MAX_N or r.T * r.F * r.N < 16 << 20:
+        return False
+    ns = sum(xe.xeng_kernel_time(xe.XENG_ENGINE_TENSOR, r.N, r.F, min(32768, r.T - t0), t0 > 0, num_sms)[2]
+             for t0 in range(0, r.T, 32768))
+    b1 = -(-r.N // 128)
+    kb, items, n_k = (r.T * r.F * 128 * b1) >> 10, r.F * (b1 * (b1 + 1) // 2), -(-r.T // 128)
+    return ns + 15000 + kb * 292 // 1000 < items * (583 * n_k + 2100) // num_sms + kb * 870 // 1000
+
+
+def batch_launches(recipes, num_sms=152):
     """Kernel launches of one batched run, as the library plans them: one
     persistent launch over every block pair of the jobs the 2-CTA pair kernel
     takes (up to 32,768 samples), one single-pass launch per 32,768 samples of
-    each other job a single-pass kernel takes (two for a job of other N from
-    BATCH_PACK_BYTES on, which is rearranged first), and for the rest the TMA decode
+    each other job a single-pass kernel takes (two for a job of other N that is
+    rearranged first), and for the rest the TMA decode
     (N % 16 == 0 above FUSED_MAX_N), the thread-per-row decode (other N), the
     nibble-sums pass (with the TMA decode) and one listed tensor-core launch."""
-    single = [r for r in recipes if r.N <= FUSED_MAX_N and (r.N % 16 == 0 or r.T * r.F * r.N >= BATCH_PACK_BYTES)]
+    single = [r for r in recipes if (r.N % 16 == 0 and r.N <= FUSED_MAX_N) or (r.N % 16 and batch_rearranges(r, num_sms))]
     listed = [r for r in single if r.N % 16 == 0 and r.N > 256 and use_pair_kernel(r.N) and r.T <= 32768]
     rest = [r for r in recipes if r not in single]
     n = (1 if listed else 0) + sum((2 if r.N % 16 else 1) * -(-r.T // 32768) for r in single if r not in listed)
@@ -331,7 +344,7 @@ def batched_record(args, steps, warmup, local_rank):
                          "of every job it takes; single-pass launches for the other jobs with N % 16 == 0 (N <= 256: "
                          "on a side branch); the rest decoded to planes, then one persistent listed tensor-core "
                          "launch)",
-            "gpu_launches": batch_launches(recipes) * steps,
+            "gpu_launches": batch_launches(recipes, torch.cuda.get_device_properties(local_rank).multi_processor_count) * steps,
             "autotune": {"opts": opts.as_dict(), "tuned_ms": tuned_ms, "from_cache": rc == 1, "fixed": rc == 2,
                          "tune_s": tune_s},
             "plan": info,

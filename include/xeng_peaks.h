@@ -64,11 +64,12 @@ XENG_API int xeng_peak_probe(int32_t kind, int64_t iters, double *tflops, double
  *   n_inputs inputs, storing or adding, on num_sms SMs; plain, rearranged and
  *   delayed samples alike (but 8192 rearranged or delayed samples and more of few
  *   channels, above 256 inputs, decode to planes).  *first_channels (may be NULL): channels that it
- *   takes; the one pass takes the others in a second launch.  Host code only, no
- *   device needed.  Returns XENG_KERNEL_*, -1 (bad argument) or -2 (bad size).
+ *   takes; the one pass takes the others in a second launch.  *ns (may be NULL): the
+ *   time that the choice goes by, 0 for planes.  Host code only, no device needed.
+ *   Returns XENG_KERNEL_*, -1 (bad argument) or -2 (bad size).
  */
 XENG_API int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t n_samples, int32_t accumulate,
-                                int32_t num_sms, int32_t *first_channels);
+                                int32_t num_sms, int32_t *first_channels, int64_t *ns);
 
 #ifdef __cplusplus
 }

@@ -91,10 +91,20 @@ struct xeng_batch_s {
 namespace {
 
 // From this many bytes on, a job whose rows TMA cannot address is rearranged
-// (pack.cu) and takes a single-pass kernel: two launches of its own, 15 us, where
-// decoding it with the others costs it about 1 us per MB more (GB300, N = 203 x 64
-// channels x 10007 samples, 130 MB: 146 us against 269).
+// (pack.cu) and takes a single-pass kernel, where that takes less: two launches of its
+// own, 15 us, while decoding it with the others costs about 0.6 us per MB more but
+// lets its items share the SMs with theirs (GB300, N = 203 x 64 channels x 10007
+// samples, 130 MB: 146 us against 269; four jobs of 1000 x 8 x 4096: 434 us, on planes
+// 299).
 constexpr int64_t kBatchPackBytes = (int64_t)16 << 20;
+// 0.285 and 0.85 ns per KB of rearranged and decoded samples, 583 ns a stage of a plane
+// item and 2100 an item.
+bool rearranged_pays(const xeng_job_t &jb, int64_t single_ns, int num_sms)
+{
+    const int64_t b1 = (jb.n_inputs + 127) / 128, kb = jb.n_samples * jb.n_freq * 128 * b1 >> 10;
+    const int64_t items = jb.n_freq * (b1 * (b1 + 1) / 2), n_k = (jb.n_samples + 127) / 128;
+    return single_ns + 15000 + kb * 292 / 1000 < items * (583 * n_k + 2100) / num_sms + kb * 870 / 1000;
+}
 
 int status_of(cudaError_t e)
 {
@@ -264,8 +274,18 @@ int plan(xeng_batch_s *b)
         }
         const xeng_job_t &jb = b->jobs[j];
         const int32_t pitch = (int32_t)round_up(jb.n_inputs, 16);
-        const int kp = single_pass_kernel(nullptr, jb.n_inputs, force, true, pitch);
+        int kp = single_pass_kernel(nullptr, jb.n_inputs, force, true, pitch);
         if (kp && jb.n_samples * jb.n_freq * jb.n_inputs >= kBatchPackBytes) {
+            // its launches are its own: the kernel by their shape, as a handle's
+            int64_t ns = 0;
+            int by_shape = kp;
+            for (int64_t t0 = 0; t0 < jb.n_samples; t0 += kFusedMaxSamples)
+                ns += single_pass_ns(kp, jb.n_inputs, jb.n_freq, std::min<int64_t>(kFusedMaxSamples, jb.n_samples - t0),
+                                     t0 > 0 ? 1 : 0, b->num_sms, &by_shape);
+            if (!force && !rearranged_pays(jb, ns, b->num_sms)) continue;
+            if (!force)
+                kp = single_pass_by_shape(kp, jb.n_inputs, jb.n_freq, std::min<int64_t>(jb.n_samples, kFusedMaxSamples), 0,
+                                          b->num_sms);
             single[j] = 1;
             b->single.push_back({j, kp});
             b->packed[j] = total;

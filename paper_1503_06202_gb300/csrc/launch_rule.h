@@ -2,6 +2,7 @@
 // sizes alone: host code without CUDA calls, part of single_pass.cu, which defines the
 // build parameters XENG_PAIR_COST and XENG_ONEPASS_COST.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 #include "xeng_internal.h"
@@ -73,7 +74,7 @@ int32_t single_pass_cut(int kernel, int32_t N, int64_t nf, int64_t nt, int accum
     return ones * (kOnepassStageNs * n_k + (accumulate ? 3200 : 1600)) + 5000 < t_round ? (int32_t)cut : 0;
 }
 
-int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms)
+int64_t single_pass_ns(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms, int *best)
 {
     // Rounds of the grid times an item's time in ns, fitted to launches of 2 .. 256
     // stages of 128 samples (GB300; us per item at 2 / 8 / 64 / 256 stages, storing:
@@ -110,12 +111,21 @@ int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accu
             t_small = (grid == items ? 6000 : 18000) + 1200 * (items * n_k / grid) + (accumulate ? 11000 * items / grid : 0);
         else
             t_small = 9000 + 25 * N + 1100 * n_k / split + (accumulate ? 5500 : 0);
-        return t_small <= ones * ((N > 128 ? 770 : 680) * n_k + n_one) ? kernel : kSingleOnepass;
+        const int64_t t = ones * ((N > 128 ? 770 : 680) * n_k + n_one);
+        *best = t_small <= t ? kernel : kSingleOnepass;
+        return std::min(t_small, t);
     }
-    if ((kernel != kSinglePair && kernel != kSingleOnepass) || kCostForces) return kernel;
-    return rounds(nf * (b2 * (b2 + 1) / 2), num_sms / 2) * (kPairStageNs * n_k + (accumulate ? 12300 : 7400)) < t_one
-               ? kSinglePair
-               : kSingleOnepass;
+    const int64_t t_pair = rounds(nf * (b2 * (b2 + 1) / 2), num_sms / 2) * (kPairStageNs * n_k + (accumulate ? 12300 : 7400));
+    *best = kCostForces ? kernel : t_pair < t_one ? kSinglePair : kSingleOnepass;
+    return *best == kSinglePair ? t_pair : t_one;
+}
+
+int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms)
+{
+    if (kernel != kSingleSmall && kernel != kSinglePair && kernel != kSingleOnepass) return kernel;
+    int best = 0;
+    single_pass_ns(kernel, N, nf, nt, accumulate, num_sms, &best);
+    return best;
 }
 
 }  // namespace xeng

@@ -1510,7 +1510,7 @@ int xeng_selftest_wait_timeout(int64_t limit_ns, int32_t *status, int32_t *threa
 }
 
 int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t n_samples, int32_t accumulate,
-                       int32_t num_sms, int32_t *first_channels)
+                       int32_t num_sms, int32_t *first_channels, int64_t *ns)
 {
     if (engine != XENG_ENGINE_TENSOR && engine != XENG_ENGINE_TENSOR_PLANES && engine != XENG_ENGINE_TENSOR_FUSED)
         return XENG_ERR_ARG;
@@ -1521,9 +1521,13 @@ int xeng_kernel_choice(int32_t engine, int32_t n_inputs, int32_t n_freq, int64_t
     int kernel = fused_kernel(engine, nullptr, n_inputs, force);  // where N lets TMA read the block in place
     if (!kernel) kernel = packed_kernel(engine, n_inputs, force);
     int32_t cut = 0;
-    if (kernel && !force) {  // as launch_shaped
-        kernel = single_pass_by_shape(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);
-        cut = single_pass_cut(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);
+    if (ns) *ns = 0;
+    if (kernel) {  // as launch_shaped
+        int best = 0;
+        const int64_t t = single_pass_ns(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms, &best);
+        if (!force) kernel = best;
+        if (!force) cut = single_pass_cut(kernel, n_inputs, n_freq, n_samples, accumulate, num_sms);
+        if (ns) *ns = t;
     }
     if (first_channels) *first_channels = cut ? cut : n_freq;
     return kernel;

@@ -284,6 +284,8 @@ int single_pass_kernel(const uint8_t *block, int32_t N, int force, bool bounded,
 // block pairs, or (kernel = kSingleSmall) of that one and the one pass.  All three
 // read the same stages.
 int single_pass_by_shape(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);
+// The time that this choice, *best, takes by the same rule, in ns.
+int64_t single_pass_ns(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms, int *best);
 // Channels that a launch of the pair kernel (by shape) takes before the one pass takes
 // the others; 0: all.
 int32_t single_pass_cut(int kernel, int32_t N, int64_t nf, int64_t nt, int accumulate, int num_sms);

@@ -365,15 +365,23 @@ XENG_KERNEL_PLANES, XENG_KERNEL_SMALL, XENG_KERNEL_ONEPASS, XENG_KERNEL_PAIR = 0
 def xeng_kernel_choice(engine: int, n_inputs: int, n_freq: int, n_samples: int, accumulate: bool = False,
                        num_sms: int = 152):
     """Returns (kernel or status, channels it takes before the one pass takes the rest): include/xeng_peaks.h."""
+    return xeng_kernel_time(engine, n_inputs, n_freq, n_samples, accumulate, num_sms)[:2]
+
+
+def xeng_kernel_time(engine: int, n_inputs: int, n_freq: int, n_samples: int, accumulate: bool = False,
+                     num_sms: int = 152):
+    """The same and the ns that the choice goes by."""
     L = lib()
     if not getattr(L.xeng_kernel_choice, "_typed", False):
         i32 = ctypes.c_int32
-        L.xeng_kernel_choice.argtypes = [i32, i32, i32, ctypes.c_int64, i32, i32, ctypes.POINTER(i32)]
+        L.xeng_kernel_choice.argtypes = [i32, i32, i32, ctypes.c_int64, i32, i32, ctypes.POINTER(i32),
+                                         ctypes.POINTER(ctypes.c_int64)]
         L.xeng_kernel_choice.restype = ctypes.c_int
         L.xeng_kernel_choice._typed = True
-    first = ctypes.c_int32()
-    rc = L.xeng_kernel_choice(engine, n_inputs, n_freq, n_samples, 1 if accumulate else 0, num_sms, ctypes.byref(first))
-    return rc, first.value
+    first, ns = ctypes.c_int32(), ctypes.c_int64()
+    rc = L.xeng_kernel_choice(engine, n_inputs, n_freq, n_samples, 1 if accumulate else 0, num_sms, ctypes.byref(first),
+                              ctypes.byref(ns))
+    return rc, first.value, ns.value
 
 
 # ------------------------------------------------------------------ batches --

@@ -182,17 +182,17 @@ def test_batch_info_without_planes_jobs():
 
 def test_batch_rearranged_jobs():
     """Jobs of 16 MiB and more whose rows TMA cannot address (N not a multiple of 16, a
-    block off a 16-byte boundary) are rearranged and take a single-pass kernel, in rounds
-    of 32,768 samples; below that they go through the planes.  Every job as the oracle."""
-    shapes = [(42000, 4, 100), (8400, 10, 200), (29000, 1, 600), (40000, 1, 1001), (33000, 2, 256), (1000, 1, 100),
-              (2100, 4, 2005)]
+    block off a 16-byte boundary) are rearranged where their own launches take less, the
+    N <= 256 kernel's and the one pass's, in rounds of 32,768 samples; the others go
+    through the planes.  Every job as the oracle."""
+    shapes = [(34000, 20, 100), (10000, 64, 203), (33000, 12, 256), (2000, 126, 300), (8400, 10, 200), (1000, 1, 100)]
     host, jobs = make_jobs(shapes, seed=46)
-    k, n = 4, host[4].size  # N = 256 off a 16-byte boundary
+    k, n = 2, host[2].size  # N = 256 off a 16-byte boundary
     flat = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
     flat[8:8 + n] = jobs[k][0].flatten()
     jobs[k] = (flat[8:8 + n].view(host[k].shape), jobs[k][1])
     b = xe.XBatch(jobs)
-    assert b.info()["n_items"] == 1  # of the one job on planes
+    assert b.info()["n_items"] == 3 * 10 + 1  # of the last two jobs, on planes
     for _ in range(2):  # a second run overwrites
         b.run()
     torch.cuda.synchronize()
