@@ -75,6 +75,7 @@ struct xeng_batch_s {
     int n_pjobs = 0;
     int64_t p_items = 0;
     SmallScratch small;                         // the N <= 256 kernel's scratch, if a job takes it
+    bool small_beside = false;                  // ... on few CTAs each, beside longer work on the others
     int grid = 0;
     int64_t n_items = 0;
     double max_load = 0, mean_load = 0;
@@ -104,6 +105,15 @@ bool rearranged_pays(const xeng_job_t &jb, int64_t single_ns, int num_sms)
     const int64_t b1 = (jb.n_inputs + 127) / 128, kb = jb.n_samples * jb.n_freq * 128 * b1 >> 10;
     const int64_t items = jb.n_freq * (b1 * (b1 + 1) / 2), n_k = (jb.n_samples + 127) / 128;
     return single_ns + 15000 + kb * 292 / 1000 < items * (583 * n_k + 2100) / num_sms + kb * 870 / 1000;
+}
+
+// CTAs of a launch of the N <= 256 kernel that runs beside others: 16 stages each, or
+// its items where those are short.
+int beside_ctas(const xeng_job_t &jb, int64_t nt, int num_sms)
+{
+    const int64_t items = jb.n_inputs > 128 ? (int64_t)jb.n_freq + (jb.n_freq + 1) / 2 : (int64_t)(jb.n_freq + 1) / 2;
+    const int64_t n_k = (nt + 127) / 128;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(num_sms, n_k < 32 ? items : items * n_k / 16));
 }
 
 int status_of(cudaError_t e)
@@ -170,6 +180,7 @@ cudaError_t enqueue_run(xeng_batch_s *b, cudaStream_t s)
             const xeng_job_t &jb = b->jobs[jk.first];
             for (int64_t t0 = 0; t0 < jb.n_samples && e == cudaSuccess; t0 += kFusedMaxSamples) {
                 const int64_t nt = std::min<int64_t>(kFusedMaxSamples, jb.n_samples - t0);
+                const int ctas = small && b->side && b->small_beside ? beside_ctas(jb, nt, b->num_sms) : 0;
                 if (b->packed[jk.first] >= 0) {
                     PackArgs p;
                     p.block = jb.block;
@@ -182,11 +193,13 @@ cudaError_t enqueue_run(xeng_batch_s *b, cudaStream_t s)
                     e = launch_pack(p, b->num_sms, st);
                     if (e == cudaSuccess)
                         e = launch_single_pass(jk.second, p.out, nt, 0, nt, jb.n_freq, jb.n_inputs, 0, jb.n_freq, jb.out,
-                                               t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st, nullptr, 0, p.pitch);
+                                               t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st, nullptr, 0, p.pitch,
+                                               nullptr, ctas);
                     continue;
                 }
                 e = launch_single_pass(jk.second, jb.block, jb.n_samples, t0, nt, jb.n_freq, jb.n_inputs, 0,
-                                       jb.n_freq, jb.out, t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st);
+                                       jb.n_freq, jb.out, t0 > 0 ? 1 : 0, &b->small, b->d_err, b->num_sms, st, nullptr, 0, 0,
+                                       nullptr, ctas);
             }
         }
     };
@@ -324,7 +337,7 @@ int plan(xeng_batch_s *b)
         b->n_pjobs = (int)pj.size();
         b->p_items = item0;
     }
-    int64_t ptotal = 0, stotal = 0;
+    int64_t ptotal = 0, stotal = 0, decoded_kb = 0;
     for (int j = 0; j < n; j++) {
         if (single[j]) continue;
         const xeng_job_t &jb = b->jobs[j];
@@ -332,6 +345,7 @@ int plan(xeng_batch_s *b)
         t_pad[j] = round_up(jb.n_samples, kTile);
         off[j] = total;
         total += round_up((int64_t)jb.n_freq * 2 * n_pad[j] * t_pad[j], 1024);
+        decoded_kb += (int64_t)jb.n_freq * n_pad[j] * t_pad[j] >> 10;
         if (decode_tma_ok(jb.block, jb.n_inputs)) {  // raw-nibble planes: room for the nibble sums
             poff[j] = ptotal;
             soff[j] = stotal;
@@ -504,6 +518,24 @@ int plan(xeng_batch_s *b)
     b->grid = cand.empty() ? 0 : P;
     b->max_load = mx;
     b->mean_load = P ? sum / P : 0;
+
+    // The N <= 256 kernel's jobs on few CTAs each where their time so is well less than
+    // what the other branch takes: on all SMs each is shorter, but the two branches then
+    // wait for one another (GB300, us on all SMs / on few: two jobs of 16 inputs and three
+    // ragged ones 151 / 123; 3, 1 and 11 of up to 480 inputs 611 / 497).
+    int64_t beside = 0, others = (int64_t)(mx * 583) + decoded_kb * 870 / 1000;
+    for (const auto &jk : b->single) {
+        const xeng_job_t &jb = b->jobs[jk.first];
+        for (int64_t t0 = 0; t0 < jb.n_samples; t0 += kFusedMaxSamples) {
+            const int64_t nt = std::min<int64_t>(kFusedMaxSamples, jb.n_samples - t0), n_k = (nt + 127) / 128;
+            int best = 0;
+            const int64_t ns = single_pass_ns(jk.second, jb.n_inputs, jb.n_freq, nt, t0 > 0 ? 1 : 0, b->num_sms, &best);
+            if (jk.second != kSingleSmall) others += ns;
+            else if (beside_ctas(jb, nt, b->num_sms) >= b->num_sms) beside += ns;
+            else beside += n_k < 32 ? 7000 + 1100 * n_k : 37000;
+        }
+    }
+    b->small_beside = 4 * others > 5 * beside;
 
     e = upload(&b->d_maps, maps);
     if (e == cudaSuccess) e = upload(&b->d_jobs, jd);

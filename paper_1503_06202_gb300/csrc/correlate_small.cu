@@ -823,7 +823,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
                                    int32_t f0, int32_t nf, int32_t *acc, int accumulate, int2 *ws, int *flags,
                                    int *err, int num_sms, cudaStream_t s,
                                    const CUtensorMap *maps, int32_t spb,
-                                   int32_t pitch, const SubBlocks *sub)
+                                   int32_t pitch, const SubBlocks *sub, int max_ctas)
 {
     if (nf <= 0 || nt <= 0) return cudaSuccess;
     if (!small_ok(maps ? nullptr : block, N, pitch) || (sub && maps) || (maps && (spb < 1 || t0 != 0)) || nt > kFusedMaxSamples ||
@@ -836,11 +836,11 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     if (n_items * n_k > 2147483647LL) {  // stages are counted in 32 bits
         const int32_t half = nf / 4 * 2;
         const cudaError_t e = launch_correlate_small(block, T_block, t0, nt, F, N, f0, half, acc, accumulate, ws, flags,
-                                                     err, num_sms, s, maps, spb, pitch, nullptr);
+                                                     err, num_sms, s, maps, spb, pitch, nullptr, max_ctas);
         if (e != cudaSuccess) return e;
         return launch_correlate_small(block, T_block, t0, nt, F, N, f0 + half, nf - half,
                                       acc + (int64_t)half * N * (N + 1), accumulate, ws, flags, err, num_sms, s, maps,
-                                      spb, pitch, nullptr);
+                                      spb, pitch, nullptr, max_ctas);
     }
     CUtensorMap map, diag_map, sub_map;
     memset(&map, 0, sizeof map);  // not read with `maps`: the stages take the blocks' maps
@@ -859,7 +859,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
         if (e0 != cudaSuccess) return e0;
     }
     int32_t split = 0;
-    const int grid = small_split(n_items, n_k, num_sms, &split);
+    const int grid = small_split(n_items, n_k, max_ctas > 0 && max_ctas < num_sms ? max_ctas : num_sms, &split);
     // Shared items: the converters join the epilogue, their one piece done, where each CTA
     // finishes two 8-column chunks or more (us, without / with: N = 256 x 8 channels x 4096
     // samples, 12 CTAs an item, 25.1 / 23.6, adding 30.3 / 26.3; 160 x 24 x 4096, 4 an item,

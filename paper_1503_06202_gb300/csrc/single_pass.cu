@@ -116,13 +116,13 @@ void small_scratch_free(SmallScratch *sc)
 cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, SmallScratch *sc,
                                int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps, int32_t spb,
-                               int32_t pitch, const SubBlocks *sub)
+                               int32_t pitch, const SubBlocks *sub, int max_ctas)
 {
     if (kernel == kSingleSmall) {
         cudaError_t e = small_scratch_alloc(sc, num_sms, s);
         if (e != cudaSuccess) return e;
         return launch_correlate_small(block, T_block, t0, nt, F, N, f0, nf, acc, accumulate, sc->ws, sc->flags, err,
-                                      num_sms, s, maps, spb, pitch, sub);
+                                      num_sms, s, maps, spb, pitch, sub, max_ctas);
     }
     if (kernel == kSinglePair)
         return launch_correlate_pair(block, T_block, t0, nt, F, N, f0, nf, acc, accumulate, err, num_sms, s, maps,

@@ -220,6 +220,7 @@ cudaError_t encode_raw_map(CUtensorMap *map, const uint8_t *block, int64_t T_blo
 // and flags (small_flags_bytes(num_sms), zeroed once: a flag per CTA, the
 // count of launches on them and an arrival counter, with which the last CTA of
 // each launch advances the count, so replays of a captured launch stay apart).
+// max_ctas (0: num_sms): CTAs at most, where others are to run beside them.
 bool small_ok(const uint8_t *block, int32_t N, int32_t pitch = 0);
 size_t small_ws_bytes(int num_sms);
 size_t small_flags_bytes(int num_sms);
@@ -227,7 +228,7 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
                                    int32_t f0, int32_t nf, int32_t *acc, int accumulate, int2 *ws, int *flags,
                                    int *err, int num_sms, cudaStream_t s,
                                    const CUtensorMap *maps = nullptr, int32_t spb = 0,
-                                   int32_t pitch = 0, const SubBlocks *sub = nullptr);
+                                   int32_t pitch = 0, const SubBlocks *sub = nullptr, int max_ctas = 0);
 int small_stage_samples();  // its stage
 
 // One pass over the raw bytes for N up to 4096 (rows of 16-byte multiples, block
@@ -306,11 +307,12 @@ void small_scratch_free(SmallScratch *sc);
 // (nt <= kFusedMaxSamples) and channels f0 .. f0 + nf - 1 of the block.  With
 // `maps` (device memory, 64-byte aligned), the samples come instead from
 // consecutive blocks of spb stages each, block k through maps[k] (made by
-// encode_raw_map); block is then unused and t0 must be 0.
+// encode_raw_map); block is then unused and t0 must be 0.  max_ctas: of the N <= 256
+// kernel.
 cudaError_t launch_single_pass(int kernel, const uint8_t *block, int64_t T_block, int64_t t0, int64_t nt, int32_t F,
                                int32_t N, int32_t f0, int32_t nf, int32_t *acc, int accumulate, SmallScratch *sc,
                                int *err, int num_sms, cudaStream_t s, const CUtensorMap *maps = nullptr,
-                               int32_t spb = 0, int32_t pitch = 0, const SubBlocks *sub = nullptr);
+                               int32_t spb = 0, int32_t pitch = 0, const SubBlocks *sub = nullptr, int max_ctas = 0);
 // The same launch with the kernel chosen by its shape (single_pass_by_shape); what
 // would be a last round of the pair kernel with few items may go to the one pass,
 // as a second launch (counted in *launches).

@@ -199,3 +199,21 @@ def test_batch_rearranged_jobs():
     for (T, F, N), blk, (_, out) in zip(shapes, host, jobs):
         assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk)), (T, F, N)
     b.close()
+
+
+@pytest.mark.parametrize("others", [[(9000, 3, 1024)], [(20000, 20, 250)], [(300, 1, 272)]])
+def test_batch_small_jobs_beside_others(others):
+    """The N <= 256 kernel's jobs on a few CTAs each beside longer work of the other
+    kernels, or on all SMs where that is short: a few stages, items cut and shared,
+    several launches of one job."""
+    shapes = [(4000, 9, 64), (200, 5, 256), (33000, 2, 256), (6000, 20, 16), (1, 1, 128)] + others
+    host, jobs = make_jobs(shapes, seed=47)
+    b = xe.XBatch(jobs)
+    for _ in range(3):
+        for _, out in jobs:
+            out.fill_(-3)
+        b.run()
+        torch.cuda.synchronize()
+        for (T, F, N), blk, (_, out) in zip(shapes, host, jobs):
+            assert np.array_equal(out.cpu().numpy().astype(np.int64), oracle.correlate(blk)), (T, F, N)
+    b.close()
