@@ -251,7 +251,7 @@ def batch_rearranges(r, num_sms=152):
              for t0 in range(0, r.T, 32768))
     b1 = -(-r.N // 128)
     kb, items, n_k = (r.T * r.F * 128 * b1) >> 10, r.F * (b1 * (b1 + 1) // 2), -(-r.T // 128)
-    return ns + 15000 + kb * 292 // 1000 < items * (583 * n_k + 2100) // num_sms + kb * 870 // 1000
+    return 4 * (ns + 15000 + kb * 292 // 1000) < 5 * (items * (583 * n_k + 2100) // num_sms + kb * 870 // 1000)
 
 
 def batch_launches(recipes, num_sms=152):

@@ -99,12 +99,14 @@ namespace {
 // 299).
 constexpr int64_t kBatchPackBytes = (int64_t)16 << 20;
 // 0.285 and 0.85 ns per KB of rearranged and decoded samples, 583 ns a stage of a plane
-// item and 2100 an item.
+// item and 2100 an item; a quarter more, since the launches over planes hold every SM
+// while they run (seven jobs of up to 238 inputs, 293 us rearranged, 361 on planes by
+// the bare sums).
 bool rearranged_pays(const xeng_job_t &jb, int64_t single_ns, int num_sms)
 {
     const int64_t b1 = (jb.n_inputs + 127) / 128, kb = jb.n_samples * jb.n_freq * 128 * b1 >> 10;
     const int64_t items = jb.n_freq * (b1 * (b1 + 1) / 2), n_k = (jb.n_samples + 127) / 128;
-    return single_ns + 15000 + kb * 292 / 1000 < items * (583 * n_k + 2100) / num_sms + kb * 870 / 1000;
+    return 4 * (single_ns + 15000 + kb * 292 / 1000) < 5 * (items * (583 * n_k + 2100) / num_sms + kb * 870 / 1000);
 }
 
 // CTAs of a launch of the N <= 256 kernel that runs beside others: 16 stages each, or
