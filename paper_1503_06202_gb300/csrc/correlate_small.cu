@@ -860,8 +860,8 @@ cudaError_t launch_correlate_small(const uint8_t *block, int64_t T_block, int64_
     }
     int32_t split = 0;
     const int grid = small_split(n_items, n_k, max_ctas > 0 && max_ctas < num_sms ? max_ctas : num_sms, &split);
-    // Shared items: the converters join the epilogue, their one piece done, where each CTA
-    // finishes two 8-column chunks or more (us, without / with: N = 256 x 8 channels x 4096
+    // Shared items: up to 14 CTAs an item the converters join the epilogue, their one piece
+    // done: 4 and 12 an item gain, 16 and 32 lose (us, without / with: N = 256 x 8 channels x 4096
     // samples, 12 CTAs an item, 25.1 / 23.6, adding 30.3 / 26.3; 160 x 24 x 4096, 4 an item,
     // 29.2 / 26.0; 256 x 6 x 8192, 16 an item, 25.4 / 25.8; 64 x 1 x 32,768, 32, 27.2 / 28.5).
     auto kern = accumulate ? correlate_small_kernel<true, false, false> : correlate_small_kernel<false, false, false>;
